@@ -62,6 +62,7 @@ typedef int32_t pgm_status;
 #define PGM_FLAG_CONTRADICTION 1u /* a message or belief had every state at -inf */
 #define PGM_FLAG_NAN 2u           /* a NaN reached a belief */
 #define PGM_FLAG_INDEX 4u         /* checked mode: an index array entry out of range (pgm_checked_report) */
+#define PGM_FLAG_TIMEOUT 8u       /* a one-launch run gave up waiting for another of its blocks (msgs undefined) */
 
 /* Limits of this build (checked by pgm_build). */
 #define PGM_MAX_STATES 256        /* states per variable */
@@ -522,16 +523,21 @@ pgm_status pgm_run_bp_until_members(pgm_graph *g, const float *log_pot, const fl
  * shared memories together hold the run's state, for at most 1,024 C variables and 2,048 C
  * factors: C = 16 where the device places a cluster of 16 such blocks (GB300: up to 16,384
  * variables), else 8 where it places 8, else no cluster form. 2 takes the cluster at every
- * size up to its limits. The launch converts msgs, runs
- * every iteration with the exchanged arrays in shared memory (24 bytes per variable) and a
- * block or cluster barrier after each pass, and writes msgs back, instead of 2 launches per
- * iteration plus 3. The arithmetic per variable and per factor is that of the multi-launch
- * iterations, so the messages and flags are bitwise the same. 0 turns it off. Per-pass
+ * size up to its limits. Above the cluster's limits pgm_run_bp is one cooperative launch of
+ * up to one block per SM while 24 bytes per variable fit the SMs' shared memories (152 SMs:
+ * up to 1.45 million variables) and few enough factors join two blocks' ranges of
+ * consecutive variables that the graph's scratch holds the exchange; pgm_run_bp_multi runs
+ * chunks of samples in one such launch each. The launch converts msgs, runs every iteration
+ * with the messages in shared memory, and writes msgs back, instead of 2 launches per
+ * iteration plus 3; such calls are launched directly, not recorded as CUDA graphs. The
+ * arithmetic per variable and per factor is that of the multi-launch
+ * iterations, so the messages and flags are bitwise the same. 0 turns all of it off. Per-pass
  * profiling (pgm_set_profiling) keeps the multi-launch form, which is also the one that
  * launches_per_iter and pgm_launch_info describe. Changing it drops the cached CUDA
  * graphs. pgm_get_option returns the setting where a log-ratio run of the graph takes
- * this form, else 0 (it asks the device once whether the cluster fits). Values outside
- * 0..2: PGM_EINVAL.
+ * the one-block or cluster form, else 0 (it asks the device once whether the cluster fits).
+ * A block's wait for another block is bounded; one that runs out raises PGM_FLAG_TIMEOUT.
+ * Values outside 0..2: PGM_EINVAL.
  */
 #define PGM_OPT_SMALL_RUN 6
 pgm_status pgm_set_option(pgm_graph *g, int32_t option, int64_t value);

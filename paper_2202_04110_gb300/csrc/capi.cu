@@ -72,9 +72,9 @@ struct pgm_graph {
     float *b = nullptr;
     float *lr_d = nullptr, *lr_lam = nullptr;  // Plan::lr: log-ratio arrays (lr_slots each)
     float *lr_prm = nullptr;                    // Plan::lr: table differences [3F] (per run)
-    // pgm_run_bp_multi buffers for up to ms_cap samples (allocated on first use)
+    // pgm_run_bp_multi buffers (allocated on first use)
     void *ms_mem = nullptr;
-    int32_t ms_cap = 0;
+    size_t ms_bytes = 0;
     float2 *ms_ev = nullptr, *ms_Dv = nullptr;
     float *ms_d = nullptr, *ms_lam = nullptr, *ms_prm = nullptr;
     // pgm_run_bp_until: the messages before a chunk's last iteration [ES] and the residual
@@ -253,6 +253,43 @@ std::vector<int32_t> lr_slot_map(const HostLayout &H) {
         for (int64_t k = 0; k < H.E; ++k) pos[H.vin_es[k] >> 1] = (int32_t)k;
     }
     return pos;
+}
+
+// The grid form of a one-launch run: blocks of Vc consecutive variables; each block's first
+// whole item (factors between two of its variables) and split item (edges whose factor's
+// other variable is another block's), ending with the totals.
+std::vector<int2> lr_grid_plan(const HostLayout &H, LrGridPlan *g) {
+    *g = LrGridPlan{};
+    std::vector<int2> off;
+    const int nb = H.V <= kLrBlockAutoV || H.V >= (1 << 24) ? 0 : lr_grid_blocks((int)H.V);
+    if (nb == 0) return off;
+    g->nb = nb;
+    g->Vc = (int32_t)((H.V + nb - 1) / nb);
+    off.assign((size_t)nb + 1, make_int2(0, 0));
+    // v / Vc by a multiplication: exact for v < 2^24, Vc < 2^14
+    const uint64_t mul = (((uint64_t)1 << 40) + g->Vc - 1) / g->Vc;
+    const int32_t *vs = H.edge_vs.data();
+    for (int64_t e = 0; e < H.E; e += 2) {
+        const uint32_t b0 = (uint32_t)(((uint64_t)(vs[e] >> 1) * mul) >> 40);
+        const uint32_t b1 = (uint32_t)(((uint64_t)(vs[e + 1] >> 1) * mul) >> 40);
+        if (b0 == b1) {
+            ++off[b0].x;
+        } else {
+            ++off[b0].y;
+            ++off[b1].y;
+        }
+    }
+    int2 sum = make_int2(0, 0);
+    for (int2 &o : off) {
+        g->f_max = std::max(g->f_max, o.x);
+        g->h_max = std::max(g->h_max, o.y);
+        const int2 n = o;
+        o = sum;
+        sum.x += n.x;
+        sum.y += n.y;
+    }
+    g->n_split = sum.y;
+    return off;
 }
 
 // Block-per-factor enumeration launch (kEnumBlock) with `threads` threads: each segment's
@@ -661,6 +698,11 @@ static pgm_status build_from_layout(const HostLayout &H, pgm_graph **out, cudaSt
         g->lr_slots = lr_slot_count(H);
         o_lr_pos = pk.add(pos.data(), pos.size());
     }
+    size_t o_grid = 0;
+    if (g->P.lr && !H.vin_tab4.empty()) {
+        const std::vector<int2> off = lr_grid_plan(H, &g->P.grid);
+        if (g->P.grid.nb > 0) o_grid = pk.add(off.data(), off.size());
+    }
     g->ordered = ordered;
     g->alloc_stream = s;
     char *dmem = nullptr;
@@ -757,6 +799,7 @@ static pgm_status build_from_layout(const HostLayout &H, pgm_graph **out, cudaSt
             max_smem = std::max(max_smem, L.smem);
         }
     }
+    if (g->P.grid.nb > 0) g->P.grid.off = reinterpret_cast<const int2 *>(dmem + o_grid);
     if (g->adj_seg_off != (size_t)-1) g->adj_launch.segs = dmem + g->adj_seg_off;
     if (g->adj_block_seg_off != (size_t)-1) g->adj_block_launch.segs = dmem + g->adj_block_seg_off;
     if (g->adj_logic_seg_off != (size_t)-1) g->adj_logic_launch.segs = dmem + g->adj_logic_seg_off;
@@ -813,7 +856,8 @@ int64_t pgm::layout_device_bytes(const HostLayout &H) {
     size_t es_bytes = align_up(std::max<int64_t>(H.ES, 1) * sizeof(float), 256);
     if (lr_eligible(H))  // the slot map, the two log-ratio arrays and the table differences
         idx += H.E * sizeof(int32_t) + 2 * align_up((size_t)lr_slot_count(H) * sizeof(float), 256) +
-               align_up((size_t)3 * (H.E / 2) * sizeof(float), 256);
+               align_up((size_t)3 * (H.E / 2) * sizeof(float), 256) +
+               (H.vin_tab4.empty() ? 0 : ((size_t)lr_grid_blocks((int)H.V) + 1) * sizeof(int2));
     const size_t vs_bytes = align_up(std::max<int64_t>(H.VS, 1) * sizeof(float), 256);
     // the high-degree variables' tile list (index memory), tile totals and tickets (scratch)
     int64_t n_tiles = 0, tot = 0;
@@ -946,6 +990,13 @@ static bool small_run_used(const pgm_graph *g) {
     return small_run_cluster(g) ? lr_cluster_fits(V, F) : lr_block_fits(V, F);
 }
 
+// Whether a log-ratio run of this graph takes the cooperative-grid form: graphs above the
+// small forms, with the option on. (PGM_OPT_SMALL_RUN 0 keeps the launches at every size.)
+static bool grid_run_used(const pgm_graph *g) {
+    return g->small_run != 0 && g->P.lr && g->P.grid.nb > 0 && !small_run_used(g) &&
+           lr_grid_fits(g->P.grid, g->G.V, g->G.E / 2);
+}
+
 static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const float *evidence, float T,
                                      float damping, int32_t n_iters, float *msgs, cudaStream_t s,
                                      bool profile) {
@@ -957,8 +1008,8 @@ static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const f
     float2 *Dv = reinterpret_cast<float2 *>(g->b);
     // a small graph: the whole run in one launch (per-pass profiling keeps the passes)
     if (lr && small_run_used(g) && !(profile && g->profiling > 0)) {
-        cudaError_t e = launch_lr_small_run(g->G, g->P, log_pot, evidence, msgs, lam, T, damping, n_iters,
-                                            small_run_cluster(g), s);
+        cudaError_t e = launch_lr_small_run(g->G, g->P, log_pot, evidence, msgs, lam, reinterpret_cast<int32_t *>(d), T,
+                                            damping, n_iters, small_run_cluster(g), s);
         if (e != cudaSuccess) return cuda_fail(e, "small-graph run launch");
         return PGM_OK;
     }
@@ -1125,26 +1176,34 @@ static void drop_cached_runs(pgm_graph *g) {
     g->runs.clear();
 }
 
-// pgm_run_bp_multi's buffers for S samples: transposed evidence (V S float2), packed
-// messages and flagged-variable lam (4V S each), per-variable totals (V S float2), table
-// differences (3F S: room for per-sample tables).
-static pgm_status ms_reserve(pgm_graph *g, int32_t S) {
-    if (g->ms_cap >= S) return PGM_OK;
-    const size_t V = (size_t)g->info.n_vars, F = (size_t)g->info.n_edges / 2;
-    const size_t b_ev = align_up(V * S * sizeof(float2), 256), b_d = align_up(4 * V * S * sizeof(float), 256);
-    const size_t b_prm = align_up(3 * F * S * sizeof(float), 256);
+// pgm_run_bp_multi's buffers: at least n bytes at ms_mem, kept with the graph.
+static pgm_status multi_reserve(pgm_graph *g, size_t n) {
+    if (g->ms_bytes >= n) return PGM_OK;
     if (g->ms_mem) {
         cudaError_t e = cudaDeviceSynchronize();  // the old buffers may still be in use
         if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
         cudaFree(g->ms_mem);
         g->ms_mem = nullptr;
-        g->ms_cap = 0;
+        g->ms_bytes = 0;
     }
-    char *mem = nullptr;
-    if (cudaMalloc(&mem, 2 * b_ev + 2 * b_d + b_prm) != cudaSuccess)
+    if (cudaMalloc(&g->ms_mem, n) != cudaSuccess) {
+        g->ms_mem = nullptr;
+        cudaGetLastError();
         return fail(PGM_ENOMEM, "cudaMalloc(multi-sample buffers)");
-    g->ms_mem = mem;
-    g->ms_cap = S;
+    }
+    g->ms_bytes = n;
+    return PGM_OK;
+}
+
+// The multi-launch form's buffers for S samples: transposed evidence (V S float2), packed
+// messages and flagged-variable lam (4V S each), per-variable totals (V S float2), table
+// differences (3F S: room for per-sample tables).
+static pgm_status ms_reserve(pgm_graph *g, int32_t S) {
+    const size_t V = (size_t)g->info.n_vars, F = (size_t)g->info.n_edges / 2;
+    const size_t b_ev = align_up(V * S * sizeof(float2), 256), b_d = align_up(4 * V * S * sizeof(float), 256);
+    const size_t b_prm = align_up(3 * F * S * sizeof(float), 256);
+    if (pgm_status st = multi_reserve(g, 2 * b_ev + 2 * b_d + b_prm); st != PGM_OK) return st;
+    char *mem = static_cast<char *>(g->ms_mem);
     g->ms_ev = reinterpret_cast<float2 *>(mem);
     g->ms_Dv = reinterpret_cast<float2 *>(mem + b_ev);
     g->ms_d = reinterpret_cast<float *>(mem + 2 * b_ev);
@@ -1224,6 +1283,22 @@ pgm_status pgm_run_bp_multi(pgm_graph *g, int32_t n_samples, const float *log_po
     if (!dg.ok) return fail(PGM_ECUDA, "cudaSetDevice failed");
     if (!ms)  // any other graph: edge-state iterations with the samples side by side
         return run_multi_es(g, n_samples, log_pot, pot_per_sample, evidence, T, damping, n_iters, msgs, stream);
+    // One launch for a chunk of samples, every iteration inside it, where the device takes it
+    // (and, when a sample needs several blocks, few factors join two of them: at most half)
+    if (g->small_run != 0) {
+        const bool local = g->P.grid.nb > 0 && g->P.grid.n_split <= g->info.n_edges / 2;
+        const LrMultiPlan p = lr_multi_plan((int)g->info.n_vars, n_samples, local);
+        if (p.S > 1 && multi_reserve(g, p.sample_bytes * p.S) == PGM_OK) {
+            for (int32_t s0 = 0; s0 < n_samples; s0 += p.S) {
+                cudaError_t e = launch_lr_multi_run(
+                    g->G, g->P, p, std::min(p.S, n_samples - s0), pot_per_sample ? P : 0,
+                    log_pot + (pot_per_sample ? (size_t)s0 * P : 0), evidence + (size_t)s0 * VS, msgs + (size_t)s0 * ES,
+                    static_cast<char *>(g->ms_mem), T, damping, n_iters, static_cast<cudaStream_t>(stream));
+                if (e != cudaSuccess) return cuda_fail(e, "multi-sample run launch");
+            }
+            return PGM_OK;
+        }
+    }
     // Samples run together in chunks whose per-iteration exchange arrays (messages and
     // per-variable totals, plus their table differences and evidence) fit in half the
     // L2, so that the factor pass finds them there; a sample that alone needs more runs
@@ -1745,6 +1820,15 @@ pgm_status pgm_run_bp(pgm_graph *g, const float *log_pot, const float *evidence,
     DeviceGuard dg(g->device);
     if (!dg.ok) return fail(PGM_ECUDA, "cudaSetDevice failed");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (g->profiling == 0 && log_ratio_run(g, n_iters)) {  // one launch: nothing to record
+        if (grid_run_used(g)) {
+            cudaError_t e = launch_lr_grid_run(g->G, g->P, g->P.grid, log_pot, evidence, msgs, g->lr_lam, g->m_tmp, g->b,
+                                               g->lr_d, g->lr_prm, T, damping, n_iters, s);
+            if (e != cudaSuccess) return cuda_fail(e, "grid run launch");
+            return PGM_OK;
+        }
+        if (small_run_used(g)) return enqueue_iterations(g, log_pot, evidence, T, damping, n_iters, msgs, s, false);
+    }
     if (g->use_cuda_graph && n_iters >= 2) {
         cudaGraphExec_t exec = nullptr;
         pgm_graph::CachedRun *run = nullptr;

@@ -41,15 +41,11 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "lr_math.cuh"
 #include "pgm_internal.h"
 
 namespace pgm {
 namespace {
-
-constexpr uint32_t kFlagContradiction = 1u;
-constexpr uint32_t kFlagNaN = 2u;
-
-#define kNegInf (-CUDART_INF_F)
 
 // Programmatic dependent launch (griddepcontrol): a kernel launched with the
 // programmatic-serialization attribute may be scheduled before the previous kernel of
@@ -134,42 +130,6 @@ __device__ __forceinline__ void store_n(float *__restrict__ p, const float (&s)[
     }
 #pragma unroll
     for (int i = 0; i < N; ++i) p[i] = s[i];
-}
-
-// ---- compensated (float-float) sums ----------------------------------------------------
-// A value hi + lo with |lo| << |hi|: TwoSum keeps the rounding error of every addition,
-// giving about 44 significant bits at FP32 speed (FP64 is a small fraction of the FP32
-// rate on this GPU). Infinite sums keep lo = 0.
-struct FF {
-    float hi, lo;
-};
-
-__device__ __forceinline__ FF ff_make(float v) { return FF{v, 0.f}; }
-
-__device__ __forceinline__ FF ff_add(FF a, float v) {
-    const float s = a.hi + v;
-    if (!isfinite(s)) return FF{s, 0.f};
-    const float bp = s - a.hi;
-    const float e = (a.hi - (s - bp)) + (v - bp);
-    return FF{s, a.lo + e};
-}
-
-__device__ __forceinline__ FF ff_add(FF a, FF b) {
-    FF r = ff_add(a, b.hi);
-    if (!isfinite(r.hi)) return r;
-    r.lo += b.lo;
-    return r;
-}
-
-__device__ __forceinline__ FF ff_shfl_down(FF v, int d) {
-    return FF{__shfl_down_sync(0xffffffffu, v.hi, d), __shfl_down_sync(0xffffffffu, v.lo, d)};
-}
-
-// a - b for float-float values, rounded to FP32 (exact up to that rounding when a and b
-// are close). -inf - finite = -inf.
-__device__ __forceinline__ float ff_diff(FF a, FF b) {
-    if (!isfinite(a.hi) || !isfinite(b.hi)) return a.hi - b.hi;
-    return (a.hi - b.hi) + (a.lo - b.lo);
 }
 
 // a > b, compared exactly on the float-float values
@@ -3688,8 +3648,6 @@ __global__ void __launch_bounds__(128) k_adj_var(DevGraph G, const float *__rest
 // (contradictory evidence) is stored as the NaN pattern kLamBothNegInf; FP32 arithmetic
 // on this GPU returns the canonical NaN 0x7fffffff, never this pattern.
 
-constexpr uint32_t kLamBothNegInf = 0x7fc00001u;
-
 // Programmatic dependent launch between the passes of a log-ratio run (the kernels are
 // launched with cudaLaunchAttributeProgrammaticStreamSerialization): each pass lets the
 // next one be scheduled as soon as all of its own blocks have started, loads only inputs
@@ -3697,51 +3655,6 @@ constexpr uint32_t kLamBothNegInf = 0x7fc00001u;
 // passes exchange only after it. pdl_wait() returns once the previous kernel of the
 // stream has completed and its writes are visible (at once when there is none); as
 // that kernel waited the same way, every earlier one has completed too.
-
-__device__ __forceinline__ float2 lr_decode(float d) {
-    return d > 0.f ? make_float2(-d, 0.f) : make_float2(0.f, d);
-}
-
-__device__ __forceinline__ float lr_encode(float m0, float m1) { return m1 - m0; }
-
-__device__ __forceinline__ float2 lam_decode(float l) {
-    if (__float_as_uint(l) == kLamBothNegInf) return make_float2(kNegInf, kNegInf);
-    return lr_decode(l);
-}
-
-__device__ __forceinline__ float lam_encode(FF l0, FF l1) {
-    if (l0.hi == kNegInf && l1.hi == kNegInf) return __uint_as_float(kLamBothNegInf);
-    return ff_diff(l1, l0);
-}
-
-// ff_add for operands known to be finite: an overflow shows as a non-finite result,
-// which the caller tests.
-__device__ __forceinline__ FF ff_add_nc(FF a, float v) {
-    const float s = a.hi + v;
-    const float bp = s - a.hi;
-    const float e = (a.hi - (s - bp)) + (v - bp);
-    return FF{s, a.lo + e};
-}
-
-// Variable-to-factor log-ratios of one variable: the leave-one-out value of edge k is
-//   lam_k = l_k(1) - l_k(0) = (e(1) - e(0)) + sum over j != k of d_j = D - d_k,
-// linear in the stored log-ratios, with D = (e(1) - e(0)) + sum_j d_j kept float-float
-// (the evidence difference exactly, by TwoSum), so lam_k is exact up to its final
-// rounding. lr_var_slow handles a variable with an infinite evidence entry or message
-// (hard constraints) by the per-state explicit sums l_k(x) instead (d = 0 of an unused
-// slot decodes to (0, 0) and adds nothing there either).
-__device__ __noinline__ void lr_var_slow(float2 e, const float *dk, const int *pos, int n, float *lam) {
-    for (int k = 0; k < n; ++k) {
-        FF l0 = ff_make(e.x), l1 = ff_make(e.y);
-        for (int j = 0; j < n; ++j) {
-            if (j == k) continue;
-            const float2 q = lr_decode(dk[j]);
-            l0 = ff_add(l0, q.x);
-            l1 = ff_add(l1, q.y);
-        }
-        lam[pos[k]] = lam_encode(l0, l1);
-    }
-}
 
 // Variable pass, at most 4 factors per variable: thread per variable, slot k of variable
 // v at k V + v; four coalesced loads of d and one store per variable, no index. It
@@ -3751,13 +3664,6 @@ __device__ __noinline__ void lr_var_slow(float2 e, const float *dk, const int *p
 // variable whose lam would not come out finite this way (an infinite evidence entry or
 // message; an overflow) gets its four lam by the per-state explicit sums in lam, and
 // the pattern kDvSlow in Dv[v].x so that the factor pass reads them there.
-constexpr uint32_t kDvSlow = 0x7fc00002u;
-
-__device__ __forceinline__ float lr_lam_from_D(float2 D, float dk) {
-    const FF l = ff_add_nc(FF{D.x, D.y}, -dk);
-    return l.hi + l.lo;
-}
-
 __global__ void __launch_bounds__(256) k_var_slot4_lr(int V, const float *__restrict__ ev,
                                                       const float *__restrict__ d, float2 *__restrict__ Dv,
                                                       float *__restrict__ lam) {
@@ -3830,96 +3736,10 @@ __global__ void __launch_bounds__(256) k_var_csr_lr(DevGraph G, const int32_t *_
     }
 }
 
-// LSE_T of two values for the log-ratio factor pass:
-//   max + T ln(1 + e^((min - max) / T)) = max + (T ln 2) log2(1 + 2^((min - max) k)),
-// k = log2(e) / T, on the SFU's base-2 exponential and logarithm (flush-to-zero forms;
-// the argument of log2 lies in [1, 2], the result's absolute error is below 3e-7 T).
-__device__ __forceinline__ float lse2_fast(float a, float b, float k, float Tln2) {
-    const float mx = fmaxf(a, b), mn = fminf(a, b);
-    float p, l;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"((mn - mx) * k));
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(1.f + p));
-    return fmaf(Tln2, l, mx);
-}
-
-// The same with the -inf case (both values -inf) returning -inf.
-template <bool MAXP>
-__device__ __forceinline__ float lse2_lr(float a, float b, float k, float Tln2) {
-    if constexpr (MAXP) return fmaxf(a, b);
-    if (fmaxf(a, b) == kNegInf) return kNegInf;
-    return lse2_fast(a, b, k, Tln2);
-}
-
-template <bool MAXP>
-__device__ __forceinline__ float lse2_fast_t(float a, float b, float k, float Tln2) {
-    if constexpr (MAXP) return fmaxf(a, b);
-    else return lse2_fast(a, b, k, Tln2);
-}
-
-// The normalise-damp-normalise epilogue (finish_k) in log-ratio form: from the factor's
-// values a(0), a(1) and the stored message d_old, the new message's log-ratio. The
-// decoded pairs are those finish_k sees, so the result is the one it would store; a
-// contradiction (both entries -inf) gives zeros and the flag.
-__device__ __forceinline__ float lr_finish(float a0, float a1, float d_old, float damping, uint32_t *flags) {
-    float dt;
-    if (a0 == kNegInf && a1 == kNegInf) {
-        atomicOr(flags, kFlagContradiction);
-        dt = 0.f;
-    } else {
-        dt = a1 - a0;
-    }
-    if (damping == 0.f) return dt;
-    const float2 o = lr_decode(dt), mo = lr_decode(d_old);
-    const float w = 1.f - damping;
-    const float t0 = damping * mo.x + w * o.x, t1 = damping * mo.y + w * o.y;
-    if (t0 == kNegInf && t1 == kNegInf) {
-        atomicOr(flags, kFlagContradiction);
-        return 0.f;
-    }
-    return t1 - t0;
-}
-
-// One factor's two new log-ratio messages with every special case handled: a
-// variable-to-factor pair that is -inf in both states, table entries of -inf, infinite
-// stored messages, damping 0 (the update of finish_k, decoded pair by pair).
-template <bool MAXP>
-__device__ __noinline__ float2 pair2_lr_exact(const float *phi, float l0, float l1, float mo0, float mo1,
-                                              float k, float Tln2, float damping, uint32_t *flags) {
-    const float2 v0 = lam_decode(l0), v1 = lam_decode(l1);
-    const float a0 = lse2_lr<MAXP>(phi[0] + v1.x, phi[1] + v1.y, k, Tln2);
-    const float a1 = lse2_lr<MAXP>(phi[2] + v1.x, phi[3] + v1.y, k, Tln2);
-    const float c0 = lse2_lr<MAXP>(phi[0] + v0.x, phi[2] + v0.y, k, Tln2);
-    const float c1 = lse2_lr<MAXP>(phi[1] + v0.x, phi[3] + v0.y, k, Tln2);
-    return make_float2(lr_finish(a0, a1, mo0, damping, flags), lr_finish(c0, c1, mo1, damping, flags));
-}
-
-// The segment of global factor g (segments in factor order, segment i starting at
-// factor segs[i].edge_base / 2).
-__device__ __forceinline__ int lr_seg_of(const EnumSeg *__restrict__ segs, int n_seg, int g) {
-    int lo = 0, hi = n_seg - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((__ldg(&segs[mid].edge_base) >> 1) <= g) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-// The table of global factor g: its own 4 entries, or the segment's shared table.
-__device__ __forceinline__ float4 lr_table(const EnumSeg *__restrict__ segs, int n_seg,
-                                           const float *__restrict__ pot, int g) {
-    const EnumSeg *S = segs + lr_seg_of(segs, n_seg, g);
-    const int shared = __ldg(&S->shared);
-    const float *t = pot + __ldg(&S->pot_base) + (shared ? 0 : (size_t)4 * (g - (__ldg(&S->edge_base) >> 1)));
-    if ((reinterpret_cast<uintptr_t>(t) & 15u) == 0)
-        return shared ? __ldg(reinterpret_cast<const float4 *>(t)) : __ldcs(reinterpret_cast<const float4 *>(t));
-    return make_float4(__ldg(t), __ldg(t + 1), __ldg(t + 2), __ldg(t + 3));
-}
-
 // Per run: each factor's table as the three numbers the log-ratio update depends on,
 // c = phi(1,0) - phi(0,0), al = phi(1,1) - phi(1,0), be = phi(0,1) - phi(0,0), at
-// prm[g], prm[F + g], prm[2F + g]. A table with a non-finite entry gets c = NaN, which
-// sends its factor to the exact path (that reads the table itself).
+// prm[g], prm[F + g], prm[2F + g]. A table with a non-finite entry gets NaNs, which
+// send both its messages to the exact path (that reads the table itself).
 __global__ void __launch_bounds__(256) k_lr_params(const EnumSeg *__restrict__ segs, int n_seg, int F,
                                                    const float *__restrict__ pot, float *__restrict__ prm) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
@@ -3927,23 +3747,8 @@ __global__ void __launch_bounds__(256) k_lr_params(const EnumSeg *__restrict__ s
     const float4 t = lr_table(segs, n_seg, pot, g);
     const bool fin = isfinite(t.x) & isfinite(t.y) & isfinite(t.z) & isfinite(t.w);
     prm[g] = fin ? t.z - t.x : CUDART_NAN_F;
-    prm[F + g] = t.w - t.z;
-    prm[2 * (size_t)F + g] = t.y - t.x;
-}
-
-// sp_T(x) = T ln(1 + e^(x / T)) = max(x, 0) + (T ln 2) log2(1 + 2^(-|x| k)), k = log2(e) / T,
-// on the SFU's base-2 exponential and logarithm (flush-to-zero forms; the argument of
-// log2 lies in [1, 2], absolute error below 3e-7 T); max(x, 0) for T = 0.
-template <bool MAXP>
-__device__ __forceinline__ float softplus_t(float x, float k, float Tln2) {
-    if constexpr (MAXP) {
-        return fmaxf(x, 0.f);
-    } else {
-        float p, l;
-        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(-fabsf(x) * k));
-        asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(1.f + p));
-        return fmaf(Tln2, l, fmaxf(x, 0.f));
-    }
+    prm[F + g] = fin ? t.w - t.z : CUDART_NAN_F;
+    prm[2 * (size_t)F + g] = fin ? t.y - t.x : CUDART_NAN_F;
 }
 
 // Factor pass, 2 x 2 tables, persistent: thread-stride loop over the global factors
@@ -3954,17 +3759,7 @@ __device__ __forceinline__ float softplus_t(float x, float k, float Tln2) {
 // arithmetic, so the index stream's latency overlaps the gathers'. d is updated in place
 // (a slot belongs to one factor).
 //
-// With the variable-to-factor log-ratios l0, l1 and the table numbers (k_lr_params),
-// LSE_T over the other variable's states gives the new log-ratios
-//   to variable 0: c  + sp_T(al + l1) - sp_T(be + l1),
-//   to variable 1: be + sp_T(al + c - be + l0) - sp_T(c + l0)   (al + c - be = phi(1,1) - phi(0,1)).
-// With o, mo the decoded new and stored messages (one entry of each exactly 0), the damped
-// pair t = damping mo + (1 - damping) o has log-ratio damping d_old + (1 - damping) dt,
-// since min(x, 0) + max(x, 0) = x; the final normalisation does not change it. Every
-// input that needs the guarded arithmetic (a non-finite table entry, an infinite
-// variable-to-factor value or stored message, damping 0 against an infinite stored
-// message) makes a result non-finite; that and a NaN lam (the contradiction pattern)
-// send the factor to pair2_lr_exact with its table.
+// The two messages by lr_dir, each with its own way to the guarded arithmetic.
 template <bool MAXP, bool FROM_D>
 __global__ void __launch_bounds__(256) k_pair2_lr(const EnumSeg *__restrict__ segs, int n_seg, int F, int V,
                                                   const int2 *__restrict__ lr_pos2, const float *__restrict__ prm,
@@ -4002,13 +3797,13 @@ __global__ void __launch_bounds__(256) k_pair2_lr(const EnumSeg *__restrict__ se
             l0 = __ldcg(lam + p.x);
             l1 = __ldcg(lam + p.y);
         }
-        const float dt0 = c + softplus_t<MAXP>(al + l1, k, Tln2) - softplus_t<MAXP>(be + l1, k, Tln2);
-        const float dt1 = be + softplus_t<MAXP>(al + c - be + l0, k, Tln2) - softplus_t<MAXP>(c + l0, k, Tln2);
-        float2 dn = make_float2(fmaf(damping, mo0, w * dt0), fmaf(damping, mo1, w * dt1));
-        if (!(isfinite(dn.x) && isfinite(dn.y) && l0 == l0 && l1 == l1)) {
+        float2 dn = make_float2(lr_dir<MAXP>(c, al, be, l1, mo0, k, Tln2, damping, w),
+                                lr_dir<MAXP>(be, al + c - be, c, l0, mo1, k, Tln2, damping, w));
+        if (lr_dir_rare(dn.x, l1) || lr_dir_rare(dn.y, l0)) {
             const float4 t = lr_table(segs, n_seg, pot, g);
             const float t4[4] = {t.x, t.y, t.z, t.w};
-            dn = pair2_lr_exact<MAXP>(t4, l0, l1, mo0, mo1, k, Tln2, damping, flags);
+            if (lr_dir_rare(dn.x, l1)) dn.x = lr_dir_exact<MAXP>(t4, 0, l1, mo0, k, Tln2, damping, flags);
+            if (lr_dir_rare(dn.y, l0)) dn.y = lr_dir_exact<MAXP>(t4, 1, l0, mo1, k, Tln2, damping, flags);
         }
         d[p.x] = dn.x;
         d[p.y] = dn.y;
@@ -4119,8 +3914,8 @@ __global__ void __launch_bounds__(256) k_ms_params(const EnumSeg *__restrict__ s
     const float4 q = lr_table(segs, n_seg, pot + (size_t)sp * P, g);
     const bool fin = isfinite(q.x) & isfinite(q.y) & isfinite(q.z) & isfinite(q.w);
     prm[t] = fin ? q.z - q.x : CUDART_NAN_F;
-    prm[n + t] = q.w - q.z;
-    prm[2 * n + t] = q.y - q.x;
+    prm[n + t] = fin ? q.w - q.z : CUDART_NAN_F;
+    prm[2 * n + t] = fin ? q.y - q.x : CUDART_NAN_F;
 }
 
 // Variable pass (k_var_slot4_lr per sample): item t = v S + s.
@@ -4189,13 +3984,13 @@ __global__ void __launch_bounds__(256) k_ms_pair(const EnumSeg *__restrict__ seg
         const float2 D0 = __ldcg(Dv + (size_t)v0 * S + s), D1 = __ldcg(Dv + (size_t)v1 * S + s);
         const float l0 = __float_as_uint(D0.x) == kDvSlow ? __ldcg(lam + px) : lr_lam_from_D(D0, mo0);
         const float l1 = __float_as_uint(D1.x) == kDvSlow ? __ldcg(lam + py) : lr_lam_from_D(D1, mo1);
-        const float dt0 = c + softplus_t<MAXP>(al + l1, k, Tln2) - softplus_t<MAXP>(be + l1, k, Tln2);
-        const float dt1 = be + softplus_t<MAXP>(al + c - be + l0, k, Tln2) - softplus_t<MAXP>(c + l0, k, Tln2);
-        float2 dn = make_float2(fmaf(damping, mo0, w * dt0), fmaf(damping, mo1, w * dt1));
-        if (!(isfinite(dn.x) && isfinite(dn.y) && l0 == l0 && l1 == l1)) {
+        float2 dn = make_float2(lr_dir<MAXP>(c, al, be, l1, mo0, k, Tln2, damping, w),
+                                lr_dir<MAXP>(be, al + c - be, c, l0, mo1, k, Tln2, damping, w));
+        if (lr_dir_rare(dn.x, l1) || lr_dir_rare(dn.y, l0)) {
             const float4 tq = lr_table(segs, n_seg, pot + (Sp > 1 ? (size_t)s * P : 0), g);
             const float t4[4] = {tq.x, tq.y, tq.z, tq.w};
-            dn = pair2_lr_exact<MAXP>(t4, l0, l1, mo0, mo1, k, Tln2, damping, flags);
+            if (lr_dir_rare(dn.x, l1)) dn.x = lr_dir_exact<MAXP>(t4, 0, l1, mo0, k, Tln2, damping, flags);
+            if (lr_dir_rare(dn.y, l0)) dn.y = lr_dir_exact<MAXP>(t4, 1, l0, mo1, k, Tln2, damping, flags);
         }
         d[px] = dn.x;
         d[py] = dn.y;
@@ -4359,291 +4154,6 @@ __global__ void k_until_control(cudaGraphConditionalHandle h, const unsigned *__
     *done = d;
     const float r = __uint_as_float(*res);
     cudaGraphSetConditional(h, ((r > tol) || (r != r)) && d < limit ? 1u : 0u);
-}
-
-// =====================================================================================
-// Small binary pairwise graphs: one block for the whole run (Plan::lr, 4-slot layout)
-// =====================================================================================
-//
-// On a graph of up to a few thousand variables the log-ratio run is bound by its
-// launches, not by memory: each pass is one short wave of blocks, two dependent launches
-// per iteration plus the conversions around the run. Here one block (below) or a cluster
-// of blocks (further below) does the whole run in one launch. The block: it converts the messages into log-ratios in shared memory (as
-// k_lr_pack_slot4), forms its factors' table numbers in registers (as k_lr_params), runs
-// every iteration with block barriers between the steps, and writes the messages back (as
-// k_lr_unpack). Per iteration a variable pass (thread t owns variable t; the totals Dv in
-// shared memory) and a factor pass (thread t owns factor t, or factors t and t + n_t when
-// there are more factors than a block has threads, and keeps their slot pairs and table
-// numbers in registers for the whole run), with a block barrier after each. A thread with
-// two factors loads both factors' shared-memory inputs before it computes and stores
-// either (a factor's slots belong to that factor alone), so their latencies overlap. The
-// per-item arithmetic is that of k_var_slot4_lr and k_pair2_lr step for step, so the
-// messages are bitwise those of the multi-launch run. A variable on the explicit-sum path
-// (an infinite evidence entry or message) writes its four lam (lr_var_slow) to global
-// memory, which the factor pass reads after the barrier. (A schedule with one barrier per
-// iteration, each factor forming its variables' totals itself into a second copy of d,
-// measured the same on a 10 x 10 grid and up to 1.9x slower on larger ones.)
-
-// Prologue: the log-ratios of msgs into d, as k_lr_pack_slot4 (msgs through L2: the
-// epilogue writes it).
-__device__ __forceinline__ void lr_small_pack(const DevGraph &G, const float *m, float *d) {
-    const int V = G.V;
-    for (int v = threadIdx.x; v < V; v += blockDim.x) {
-        const int4 t = __ldg(G.vin_tab4 + v);
-        const int es[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            d[q * V + v] = es[q] >= 0 ? lr_encode(__ldcg(m + es[q]), __ldcg(m + es[q] + 1)) : 0.f;
-        }
-    }
-}
-
-// Epilogue: every edge's two entries from its slot of d, as k_lr_unpack.
-__device__ __forceinline__ void lr_small_unpack(const DevGraph &G, const float *d, float *m) {
-    for (int e = threadIdx.x; e < G.E; e += blockDim.x) {
-        const float2 q = lr_decode(d[__ldg(G.lr_pos + e)]);
-        m[2 * (size_t)e] = q.x;
-        m[2 * (size_t)e + 1] = q.y;
-    }
-}
-
-// Factor g's slot pair and table numbers, as k_lr_params.
-struct LrSmallFactor {
-    int2 p;
-    float c, al, be;
-};
-__device__ __forceinline__ LrSmallFactor lr_small_factor(const DevGraph &G, const EnumSeg *segs, int n_seg,
-                                                         const float *pot, int g, int F) {
-    LrSmallFactor r{make_int2(0, 0), 0.f, 0.f, 0.f};
-    if (g >= F) return r;
-    r.p = __ldg(reinterpret_cast<const int2 *>(G.lr_pos) + g);
-    const float4 t = lr_table(segs, n_seg, pot, g);
-    const bool fin = isfinite(t.x) & isfinite(t.y) & isfinite(t.z) & isfinite(t.w);
-    r.c = fin ? t.z - t.x : CUDART_NAN_F;
-    r.al = t.w - t.z;
-    r.be = t.y - t.x;
-    return r;
-}
-
-// The factor update of k_pair2_lr from the variable-to-factor log-ratios l0, l1 and the
-// stored messages mo0, mo1.
-template <bool MAXP>
-__device__ __forceinline__ float2 lr_small_update(const LrSmallFactor &f, const EnumSeg *segs, int n_seg,
-                                                  const float *pot, int g, float l0, float l1, float mo0,
-                                                  float mo1, float k, float Tln2, float damping, float w,
-                                                  uint32_t *flags) {
-    const float dt0 = f.c + softplus_t<MAXP>(f.al + l1, k, Tln2) - softplus_t<MAXP>(f.be + l1, k, Tln2);
-    const float dt1 = f.be + softplus_t<MAXP>(f.al + f.c - f.be + l0, k, Tln2) - softplus_t<MAXP>(f.c + l0, k, Tln2);
-    float2 dn = make_float2(fmaf(damping, mo0, w * dt0), fmaf(damping, mo1, w * dt1));
-    if (!(isfinite(dn.x) && isfinite(dn.y) && l0 == l0 && l1 == l1)) {
-        const float4 t = lr_table(segs, n_seg, pot, g);
-        const float t4[4] = {t.x, t.y, t.z, t.w};
-        dn = pair2_lr_exact<MAXP>(t4, l0, l1, mo0, mo1, k, Tln2, damping, flags);
-    }
-    return dn;
-}
-
-// The variable pass of k_var_slot4_lr for one variable: its total into *Dv, or kDvSlow
-// and its four lam (lr_var_slow) into global lam.
-__device__ __forceinline__ void lr_small_var(float2 e, const float (&dk)[4], int v, int V, float2 *Dv,
-                                             float *lam) {
-    bool fin = isfinite(e.x) & isfinite(e.y);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) fin &= isfinite(dk[q]);
-    if (fin) {
-        FF D = ff_add_nc(ff_make(e.y), -e.x);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) D = ff_add_nc(D, dk[q]);
-        const float2 Df = make_float2(D.hi, D.lo);
-        bool ok = true;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) ok &= isfinite(lr_lam_from_D(Df, dk[q]));
-        if (ok) {
-            *Dv = Df;
-            return;
-        }
-    }
-    const int pos[4] = {v, V + v, 2 * V + v, 3 * V + v};
-    lr_var_slow(e, dk, pos, 4, lam);
-    *Dv = make_float2(__uint_as_float(kDvSlow), 0.f);
-}
-
-template <bool MAXP, int NF>
-__global__ void __launch_bounds__(kLrSmallThreads)
-k_lr_small(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float *__restrict__ pot,
-            const float *__restrict__ ev, float *__restrict__ msgs, float *__restrict__ lam, float k, float Tln2,
-            float damping, int n_iters) {
-    extern __shared__ __align__(16) float lr_sm[];
-    const int V = G.V, F = G.E / 2, tid = threadIdx.x, nt = blockDim.x;
-    float2 *Dv = reinterpret_cast<float2 *>(lr_sm);  // V float2 (8-byte aligned at the base)
-    float *d = lr_sm + 2 * (size_t)V;                // 4 V floats
-    lr_small_pack(G, msgs, d);
-    const float2 e = tid < V ? __ldg(reinterpret_cast<const float2 *>(ev) + tid) : make_float2(0.f, 0.f);
-    LrSmallFactor f[NF];
-#pragma unroll
-    for (int j = 0; j < NF; ++j) f[j] = lr_small_factor(G, segs, n_seg, pot, tid + j * nt, F);
-    const float w = 1.f - damping;
-    __syncthreads();
-    for (int it = 0; it < n_iters; ++it) {
-        if (tid < V) {  // variable pass (k_var_slot4_lr)
-            float dk[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) dk[q] = d[q * V + tid];
-            lr_small_var(e, dk, tid, V, Dv + tid, lam);
-        }
-        __syncthreads();
-        float mo0[NF], mo1[NF];  // factor pass (k_pair2_lr<MAXP, true>)
-        float2 D0[NF], D1[NF];
-#pragma unroll
-        for (int j = 0; j < NF; ++j) {
-            const int2 p = f[j].p;
-            mo0[j] = d[p.x];
-            mo1[j] = d[p.y];
-            D0[j] = Dv[p.x - V * ((p.x >= V) + (p.x >= 2 * V) + (p.x >= 3 * V))];
-            D1[j] = Dv[p.y - V * ((p.y >= V) + (p.y >= 2 * V) + (p.y >= 3 * V))];
-        }
-#pragma unroll
-        for (int j = 0; j < NF; ++j) {
-            const int g = tid + j * nt;
-            if (g >= F) continue;
-            const int2 p = f[j].p;
-            const float l0 = __float_as_uint(D0[j].x) == kDvSlow ? __ldcg(lam + p.x) : lr_lam_from_D(D0[j], mo0[j]);
-            const float l1 = __float_as_uint(D1[j].x) == kDvSlow ? __ldcg(lam + p.y) : lr_lam_from_D(D1[j], mo1[j]);
-            const float2 dn = lr_small_update<MAXP>(f[j], segs, n_seg, pot, g, l0, l1, mo0[j], mo1[j], k, Tln2,
-                                                    damping, w, G.flags);
-            d[p.x] = dn.x;
-            d[p.y] = dn.y;
-        }
-        __syncthreads();
-    }
-    lr_small_unpack(G, d, msgs);
-}
-
-// ---- a cluster of blocks: graphs of up to 16,384 variables -----------------------------
-//
-// Above one block's share the same run goes to a thread-block cluster of C blocks
-// (lr_cluster_size: 16 or 8; co-scheduled, one per SM) whose shared memories together hold d and the totals D,
-// distributed by variable: block r owns variables r Vc .. (r + 1) Vc - 1 (their four slots,
-// plane q at q Vc, and their totals) and factors r Fc .. (r + 1) Fc - 1. A factor reads and
-// writes its two slots, and reads its variables' totals, in whichever block holds them,
-// through the cluster's distributed shared memory (mapa: the generic address of the same
-// offset in another block). The passes are separated by cluster barriers (arrive with
-// release, wait with acquire, at cluster scope: they also order the explicit-sum path's
-// global lam), and a block leaves only after a last barrier, once no block reads another's
-// memory. Every thread of every block runs every barrier. The per-item arithmetic is that
-// of the multi-launch kernels, so the messages are bitwise theirs.
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-// The generic address of the same shared-memory location in block `rank` of the cluster.
-template <class Tp>
-__device__ __forceinline__ Tp *rank_ptr(Tp *p, uint32_t rank) {
-    uint64_t out;
-    asm volatile("mapa.u64 %0, %1, %2;" : "=l"(out) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
-    return reinterpret_cast<Tp *>(out);
-}
-
-// Slot p = k V + v of the 4-slot layout: the block that owns v and the slot's offset in its
-// d (k Vc + the variable's local index); also the local index of the variable.
-__device__ __forceinline__ void lr_slot_home(int p, int V, int Vc, uint32_t &rank, int &off, int &lv) {
-    const int k = (p >= V) + (p >= 2 * V) + (p >= 3 * V);
-    const int v = p - k * V;
-    rank = (uint32_t)(v / Vc);
-    lv = v - (int)rank * Vc;
-    off = k * Vc + lv;
-}
-
-template <bool MAXP, int NF>
-__global__ void __launch_bounds__(kLrSmallThreads)
-k_lr_cluster(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float *__restrict__ pot,
-             const float *__restrict__ ev, float *__restrict__ msgs, float *__restrict__ lam, float k, float Tln2,
-             float damping, int n_iters, int Vc, int Fc) {
-    extern __shared__ __align__(16) float lr_sm[];
-    const int V = G.V, F = G.E / 2, tid = threadIdx.x, nt = blockDim.x;
-    const uint32_t r = cluster_rank();
-    float2 *Dv = reinterpret_cast<float2 *>(lr_sm);  // Vc float2: this block's variables' totals
-    float *d = lr_sm + 2 * (size_t)Vc;               // 4 Vc floats: their slots
-    const int v0 = (int)r * Vc, nv = max(0, min(Vc, V - v0));
-    // this block's variables' slots from msgs (as k_lr_pack_slot4)
-    for (int lv = tid; lv < nv; lv += nt) {
-        const int4 t = __ldg(G.vin_tab4 + v0 + lv);
-        const int es[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            d[q * Vc + lv] = es[q] >= 0 ? lr_encode(__ldcg(msgs + es[q]), __ldcg(msgs + es[q] + 1)) : 0.f;
-    }
-    const bool hv = tid < nv;
-    const float2 e = hv ? __ldg(reinterpret_cast<const float2 *>(ev) + v0 + tid) : make_float2(0.f, 0.f);
-    // this thread's factors: table numbers and where their slots and totals live
-    LrSmallFactor f[NF];
-    float *s0[NF], *s1[NF];
-    const float2 *t0[NF], *t1[NF];
-    bool hf[NF];
-#pragma unroll
-    for (int j = 0; j < NF; ++j) {
-        const int i = tid + j * nt, g = (int)r * Fc + i;
-        hf[j] = i < Fc && g < F;
-        f[j] = lr_small_factor(G, segs, n_seg, pot, hf[j] ? g : F, F);  // (0, 0) for no factor
-        uint32_t ra, rb;
-        int oa, ob, la, lb;
-        lr_slot_home(f[j].p.x, V, Vc, ra, oa, la);
-        lr_slot_home(f[j].p.y, V, Vc, rb, ob, lb);
-        s0[j] = rank_ptr(d + oa, ra);
-        s1[j] = rank_ptr(d + ob, rb);
-        t0[j] = rank_ptr(Dv + la, ra);
-        t1[j] = rank_ptr(Dv + lb, rb);
-    }
-    const float w = 1.f - damping;
-    cluster_barrier();  // every block's slots are packed
-    for (int it = 0; it < n_iters; ++it) {
-        if (hv) {  // variable pass (k_var_slot4_lr), this block's variables
-            float dk[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) dk[q] = d[q * Vc + tid];
-            lr_small_var(e, dk, v0 + tid, V, Dv + tid, lam);
-        }
-        cluster_barrier();
-        float mo0[NF], mo1[NF];  // factor pass (k_pair2_lr<MAXP, true>), this block's factors
-        float2 D0[NF], D1[NF];
-#pragma unroll
-        for (int j = 0; j < NF; ++j) {
-            mo0[j] = *s0[j];
-            mo1[j] = *s1[j];
-            D0[j] = *t0[j];
-            D1[j] = *t1[j];
-        }
-#pragma unroll
-        for (int j = 0; j < NF; ++j) {
-            if (!hf[j]) continue;
-            const int2 p = f[j].p;
-            const float l0 = __float_as_uint(D0[j].x) == kDvSlow ? __ldcg(lam + p.x) : lr_lam_from_D(D0[j], mo0[j]);
-            const float l1 = __float_as_uint(D1[j].x) == kDvSlow ? __ldcg(lam + p.y) : lr_lam_from_D(D1[j], mo1[j]);
-            const float2 dn = lr_small_update<MAXP>(f[j], segs, n_seg, pot, (int)r * Fc + tid + j * nt, l0, l1,
-                                                    mo0[j], mo1[j], k, Tln2, damping, w, G.flags);
-            *s0[j] = dn.x;
-            *s1[j] = dn.y;
-        }
-        cluster_barrier();
-    }
-    // the edges of this block's factors back into msgs (as k_lr_unpack)
-    const int e_end = 2 * min(F, ((int)r + 1) * Fc);
-    for (int ei = 2 * (int)r * Fc + tid; ei < e_end; ei += nt) {
-        uint32_t ra;
-        int oa, la;
-        lr_slot_home(__ldg(G.lr_pos + ei), V, Vc, ra, oa, la);
-        const float2 q = lr_decode(*rank_ptr(d + oa, ra));
-        msgs[2 * (size_t)ei] = q.x;
-        msgs[2 * (size_t)ei + 1] = q.y;
-    }
-    cluster_barrier();  // no block leaves while another may still read its shared memory
 }
 
 }  // namespace
@@ -5011,95 +4521,6 @@ cudaError_t launch_lr_unpack(const DevGraph &G, const float *d, float *m, cudaSt
     const int blocks = (G.E + 255) / 256;
     if ((reinterpret_cast<uintptr_t>(m) & 7u) == 0) k_lr_unpack<true><<<blocks, 256, 0, s>>>(G, d, m);
     else k_lr_unpack<false><<<blocks, 256, 0, s>>>(G, d, m);
-    return cudaGetLastError();
-}
-
-// The cluster size of the cluster form on this device: 16 blocks of kLrSmallThreads threads
-// where the device places such a cluster (above the portable size of 8), else 8, else 0
-// (asked once per device).
-int lr_cluster_size() {
-    static int size[64];  // 0 unknown, else the size + 1
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (size[dev] == 0) {
-        void (*kerns[4])(DevGraph, const EnumSeg *, int, const float *, const float *, float *, float *, float,
-                         float, float, int, int, int) = {k_lr_cluster<false, 1>, k_lr_cluster<false, 2>,
-                                                         k_lr_cluster<true, 1>, k_lr_cluster<true, 2>};
-        for (auto kern : kerns) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        int found = 0;
-        for (int C : {kLrClusterMax, 8}) {
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3(C);
-            cfg.blockDim = dim3(kLrSmallThreads);
-            cfg.dynamicSmemBytes = (size_t)24 * kLrSmallMaxV;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = C;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            bool yes = true;
-            for (auto kern : kerns) {
-                int n = 0;
-                yes = yes && cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0;
-            }
-            cudaGetLastError();  // a refused query leaves no error behind
-            if (yes) {
-                found = C;
-                break;
-            }
-        }
-        size[dev] = found + 1;
-    }
-    return size[dev] - 1;
-}
-
-cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *log_pot, const float *ev,
-                                float *msgs, float *lam, float T, float damping, int n_iters, bool cluster,
-                                cudaStream_t s) {
-    const float k = T > 0.f ? (float)(1.4426950408889634 / (double)T) : 0.f;
-    const float Tln2 = (float)((double)T * 0.6931471805599453);
-    const int F = G.E / 2, V = G.V;
-    const bool block = !cluster;
-    if (!(block ? lr_block_fits(V, F) : lr_cluster_fits(V, F)) || G.vin_tab4 == nullptr || G.lr_pos == nullptr)
-        return cudaErrorInvalidValue;
-    for (const FactorLaunch &L : P.factor) {  // the one kPair2 launch: every factor
-        if (L.n_blocks == 0 || n_iters <= 0) continue;
-        const EnumSeg *segs = static_cast<const EnumSeg *>(L.segs);
-        if (block) {  // one block: one variable and one factor per thread, or two factors
-            const bool one = F <= kLrSmallThreads;
-            const int per = one ? std::max(V, F) : std::max(V, (F + 1) / 2);
-            const int threads = std::max(32, ((per + 31) / 32) * 32);
-            const size_t smem = (size_t)V * 6 * sizeof(float);
-            auto kern = T == 0.f ? (one ? k_lr_small<true, 1> : k_lr_small<true, 2>)
-                                 : (one ? k_lr_small<false, 1> : k_lr_small<false, 2>);
-            kern<<<1, threads, smem, s>>>(G, segs, L.n_seg, log_pot, ev, msgs, lam, k, Tln2, damping, n_iters);
-            continue;
-        }
-        // a cluster of C blocks: block r owns Vc variables and Fc factors
-        const int C = lr_cluster_size();
-        const int Vc = (V + C - 1) / C, Fc = (F + C - 1) / C;
-        const bool one = Fc <= kLrSmallThreads;
-        const int per = one ? std::max(Vc, Fc) : std::max(Vc, (Fc + 1) / 2);
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(C);
-        cfg.blockDim = dim3(std::max(32, ((per + 31) / 32) * 32));
-        cfg.dynamicSmemBytes = (size_t)Vc * 6 * sizeof(float);
-        cfg.stream = s;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = C;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        auto kern = T == 0.f ? (one ? k_lr_cluster<true, 1> : k_lr_cluster<true, 2>)
-                             : (one ? k_lr_cluster<false, 1> : k_lr_cluster<false, 2>);
-        cudaError_t e = cudaLaunchKernelEx(&cfg, kern, G, segs, L.n_seg, log_pot, ev, msgs, lam, k, Tln2, damping,
-                                           n_iters, Vc, Fc);
-        if (e != cudaSuccess) return e;
-    }
     return cudaGetLastError();
 }
 

@@ -1,0 +1,704 @@
+// One-launch runs of binary pairwise graphs (every variable binary with at most 4 factors,
+// every factor a 2 x 2 table): every iteration of a pgm_run_bp call inside one kernel, the
+// messages resident in shared memory from the first iteration to the last.
+//
+// Method: the log-ratio form of PGMax's damped flooding updates (arXiv 2202.04110, Sec. 3)
+// with the arithmetic of lr_math.cuh, item for item that of the multi-launch kernels, so
+// messages and flags are bitwise theirs.
+//
+// Why: the multi-launch run moves 112 bytes per variable and iteration through L2 and pays
+// two launch boundaries; on a 1000 x 1000 grid that took 17.4 us per iteration, on grids of
+// 10^4 .. 10^5 variables 3 .. 4 us, nearly all of it boundaries. A block here owns a
+// contiguous range of Vc variables: their incoming messages d (4 slots, 16 bytes) and totals
+// D (8 bytes) live in its shared memory (24 bytes per variable: 9,600 per SM, 1.45 million
+// on 152 SMs), factors between two variables of one block are updated in place, and only
+// the factors that join two blocks exchange anything: one variable-to-factor value in each
+// direction per iteration. Each of the two blocks computes the message to its own variable.
+//
+// One iteration of a block:
+//   1. totals: thread per variable, D = (e(1) - e(0)) + sum of its d (float-float);
+//   2. publish: for every split factor, its value D - d into the other block's inbox;
+//   3. whole factors: thread per factor, both messages in place;
+//   4. split factors: wait for the other block's value, one message in place;
+// with a block barrier after 1 and after 4. Step 3 runs while the values travel.
+// Measured against the multi-launch run (whole calls, GB300): 1000 x 1000, 200 iterations
+// 3.65 -> 2.16 ms (10.6 us per iteration), 317 x 241 max-product, 50 iterations 213 -> 93 us,
+// 32 evidence sets of 256 x 256, 100 iterations 4.22 -> 2.24 ms.
+//
+// Inbox words carry their iteration: one 8-byte store holds (value, iteration), and the
+// reader polls its own word until the iteration is the one it is in; no fence, flag or
+// grid-wide barrier is needed. Two parities suffice: a block can publish iteration t + 2
+// only after its own step 4 of t + 1, which waited for the other side's t + 1, which that
+// side published after it had finished reading t. Inboxes are cleared in the prologue,
+// before the one barrier of all blocks (per sample they exchange with; the launch's).
+//   - a cluster of up to 16 blocks (graphs of 701 .. 16,384 variables): the inboxes are in the
+//     reader's shared memory, written through distributed shared memory, so a poll is a
+//     local read;
+//   - a cooperative grid of up to one block per SM (above that): the inboxes are in global
+//     memory (L2).
+// Every wait is bounded: after kWaitLimit polls a block raises PGM_FLAG_TIMEOUT in the status
+// word, stops waiting and runs to its end.
+#include <algorithm>
+#include <cstdint>
+#include <mutex>
+
+#include <cuda_runtime.h>
+
+#include "lr_math.cuh"
+#include "pgm_internal.h"
+
+namespace pgm {
+namespace {
+
+constexpr uint32_t kFlagTimeout = PGM_FLAG_TIMEOUT;
+constexpr int kWaitLimit = 1 << 22;  // polls: about a second on a device-memory word
+
+// Where a block's items and exchanged values live.
+enum Exchange : int { kAlone = 0, kCluster = 1, kGrid = 2 };
+
+struct LrRun {
+    int32_t V, E;
+    const int4 *tab4;       // each variable's incoming edge-states (DevGraph::vin_tab4)
+    const int32_t *lr_pos;  // each edge's slot k V + v
+    const EnumSeg *segs;
+    int n_seg;
+    const float *pot, *ev;
+    float *msgs, *lam;      // lam: explicit sums of variables with infinite entries, [4 V] per sample
+    int64_t pot_stride, ev_stride, msg_stride;  // per sample (pot_stride 0: one table set)
+    uint32_t *flags;
+    float k, Tln2, damping;
+    int n_iters;
+    int nb, Vc;             // blocks per sample, variables per block
+    int f_cap, h_cap;       // items per block that the arrays below have room for
+    const int2 *off;        // kGrid, one sample: first whole / split item of each block; else null
+    int32_t *dir;           // [4 V] per sample: a split slot's item in its block
+    unsigned long long *box0, *box1;  // kGrid inboxes of the even / odd iterations
+    float4 *rec;            // whole factors' records when not in shared memory
+    float4 *hrec;           // split factors' records when not in shared memory
+    uint32_t *hdst;         // and the other block's inbox word
+    uint32_t *bar;          // launch-wide barrier: arrivals, generation
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// The shared::cluster address of the same shared-memory location in block `rank`.
+__device__ __forceinline__ uint32_t rank_addr(uint32_t a, uint32_t rank) {
+    uint32_t out;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(a), "r"(rank));
+    return out;
+}
+
+// (value, iteration) as one 8-byte word.
+__device__ __forceinline__ unsigned long long box_word(float v, uint32_t it) {
+    return ((unsigned long long)it << 32) | __float_as_uint(v);
+}
+
+// All blocks of the launch (co-resident: a cooperative launch), once. The last to arrive
+// resets the count and moves the generation on, so the words need no clearing between
+// launches.
+__device__ __forceinline__ bool grid_barrier_once(uint32_t *bar, uint32_t n_blocks, uint32_t *flags) {
+    bool ok = true;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        volatile uint32_t *gen = bar + 1;
+        const uint32_t g0 = *gen;
+        __threadfence();
+        if (atomicAdd(bar, 1u) == n_blocks - 1) {
+            atomicExch(bar, 0u);
+            __threadfence();
+            atomicAdd(bar + 1, 1u);
+        } else {
+            int polls = 0;
+            while (*gen == g0 && ++polls < kWaitLimit) __nanosleep(64);
+            if (*gen == g0) {
+                atomicOr(flags, kFlagTimeout);
+                ok = false;
+            }
+        }
+        __threadfence();
+    }
+    return __syncthreads_and(ok || threadIdx.x != 0);
+}
+
+// The message into slot (v, kk) with every special case handled: its factor's table, its side.
+template <bool MAXP>
+__device__ __noinline__ float run_exact(const LrRun &A, const float *pot, int v, int kk, float l, float mo) {
+    const int4 t = __ldg(A.tab4 + v);
+    const int es = kk == 0 ? t.x : kk == 1 ? t.y : kk == 2 ? t.z : t.w;
+    const float4 q = lr_table(A.segs, A.n_seg, pot, es >> 2);
+    const float phi[4] = {q.x, q.y, q.z, q.w};
+    return lr_dir_exact<MAXP>(phi, (es >> 1) & 1, l, mo, A.k, A.Tln2, A.damping, A.flags);
+}
+
+// A variable whose totals do not come out finite: its four values by the explicit sums, in
+// lam (through L2: other threads of the block read them after the barrier).
+__device__ __noinline__ void run_var_slow(const LrRun &A, float *lam, int v, float2 e, float d0, float d1, float d2,
+                                          float d3) {
+    const float dk[4] = {d0, d1, d2, d3};
+    const int pos[4] = {v, A.V + v, 2 * A.V + v, 3 * A.V + v};
+    lr_var_slow(e, dk, pos, 4, lam);
+}
+
+__device__ __forceinline__ bool is_slow(float2 D) { return __float_as_uint(D.x) == kDvSlow; }
+
+// A record: three table numbers and the slots packed as local variable (14 bits) | slot
+// index k (2 bits): the first neighbour's in the low half, the second's in the high half.
+__device__ __forceinline__ uint32_t pack_slot(int lv, int k) { return (uint32_t)lv | ((uint32_t)k << 14); }
+
+// X: how blocks exchange values; RES: the records (and evidence) are in shared memory too,
+// else they are streamed from L2 (16 bytes per whole factor and iteration, loaded one item
+// ahead; the loads do not depend on the messages, so the block barriers do not delay them).
+template <bool MAXP, int X, bool RES>
+__global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
+    extern __shared__ __align__(16) char lr_sm[];
+    __shared__ int s_n[2];
+    __shared__ int s_abort;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    const int V = A.V, Vc = A.Vc;
+    int b, smp;  // block within the sample, sample
+    if constexpr (X == kCluster) {
+        b = (int)cluster_rank();
+        smp = 0;
+    } else {
+        smp = (int)blockIdx.x / A.nb;
+        b = (int)blockIdx.x - smp * A.nb;
+    }
+    const int v0 = b * Vc, nv = max(0, min(Vc, V - v0));
+    const float *pot = A.pot + (size_t)smp * A.pot_stride;
+    const float2 *ev = reinterpret_cast<const float2 *>(A.ev + (size_t)smp * A.ev_stride) + v0;
+    float *msgs = A.msgs + (size_t)smp * A.msg_stride;
+    float *lam = A.lam + (size_t)smp * 4 * V;
+    int32_t *dir = A.dir + (size_t)smp * 4 * V;
+    // shared memory: [records, split records,] totals, [evidence,] [inbox,] slots, [addresses]
+    char *sp = lr_sm;
+    float4 *rec, *hrec;
+    uint32_t *hdst;
+    float2 *es_sh = nullptr;
+    unsigned long long *box = nullptr;
+    size_t f_base = 0, h_base = 0;  // this block's first item in the global arrays
+    if constexpr (X == kGrid) {
+        f_base = A.off ? (size_t)A.off[b].x : (size_t)blockIdx.x * A.f_cap;
+        h_base = A.off ? (size_t)A.off[b].y : (size_t)blockIdx.x * A.h_cap;
+    } else if (!RES) {
+        f_base = (size_t)blockIdx.x * A.f_cap;
+    }
+    if constexpr (RES) {
+        rec = reinterpret_cast<float4 *>(sp);
+        sp += 16 * (size_t)A.f_cap;
+        hrec = reinterpret_cast<float4 *>(sp);
+        sp += 16 * (size_t)A.h_cap;
+    } else {
+        rec = A.rec + f_base;
+        hrec = A.hrec + h_base;
+        hdst = A.hdst + h_base;
+    }
+    float2 *Dv = reinterpret_cast<float2 *>(sp);
+    sp += 8 * (size_t)Vc;
+    if constexpr (RES) {
+        es_sh = reinterpret_cast<float2 *>(sp);
+        sp += 8 * (size_t)Vc;
+    }
+    if constexpr (X == kCluster) {
+        box = reinterpret_cast<unsigned long long *>(sp);
+        sp += 16 * (size_t)A.h_cap;
+    }
+    float *d = reinterpret_cast<float *>(sp);
+    sp += 16 * (size_t)Vc;
+    if constexpr (RES) hdst = reinterpret_cast<uint32_t *>(sp);
+
+    // ---- prologue: slots from msgs, the block's items ----
+    if (tid < 2) s_n[tid] = 0;
+    if (tid == 0) s_abort = 0;
+    __syncthreads();
+    for (int l0 = 0; l0 < nv; l0 += nt) {
+        const int lv = l0 + tid, v = v0 + lv;
+        const int4 t = lv < nv ? __ldg(A.tab4 + v) : make_int4(-1, -1, -1, -1);
+        if (RES && lv < nv) es_sh[lv] = __ldg(ev + lv);
+        const int es[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool have = es[q] >= 0;
+            float m = 0.f;
+            int u = 0, uk = 0;
+            if (have) {
+                m = lr_encode(__ldcg(msgs + es[q]), __ldcg(msgs + es[q] + 1));
+                const int p = __ldg(A.lr_pos + ((es[q] >> 1) ^ 1));  // the factor's other slot
+                uk = (p >= V) + (p >= 2 * V) + (p >= 3 * V);
+                u = p - uk * V;
+            }
+            if (lv < nv) d[q * Vc + lv] = m;
+            const bool local = X == kAlone || (u >= v0 && u < v0 + nv);
+            const int side = (es[q] >> 1) & 1;
+            const bool whole = have && local && side == 0, split = have && !local;
+            float c = 0.f, al = 0.f, be = 0.f;
+            if (whole || split) {
+                const float4 tb = lr_table(A.segs, A.n_seg, pot, es[q] >> 2);
+                const bool fin = isfinite(tb.x) & isfinite(tb.y) & isfinite(tb.z) & isfinite(tb.w);
+                c = fin ? tb.z - tb.x : CUDART_NAN_F;  // as k_lr_params
+                al = fin ? tb.w - tb.z : CUDART_NAN_F;
+                be = fin ? tb.y - tb.x : CUDART_NAN_F;
+            }
+            // runs of consecutive variables stay together: coalesced, without bank conflicts
+            const unsigned mw = __ballot_sync(0xffffffffu, whole), mh = __ballot_sync(0xffffffffu, split);
+            int bw = 0, bh = 0;
+            if (lane == 0) {
+                if (mw) bw = atomicAdd(&s_n[0], __popc(mw));
+                if (mh) bh = atomicAdd(&s_n[1], __popc(mh));
+            }
+            bw = __shfl_sync(0xffffffffu, bw, 0) + __popc(mw & ((1u << lane) - 1u));
+            bh = __shfl_sync(0xffffffffu, bh, 0) + __popc(mh & ((1u << lane) - 1u));
+            if (whole)
+                rec[bw] = make_float4(c, al, be, __uint_as_float(pack_slot(lv, q) | (pack_slot(u - v0, uk) << 16)));
+            if (X != kAlone && split) {
+                hrec[bh] = side == 0 ? make_float4(c, al, be, __uint_as_float(pack_slot(lv, q)))
+                                     : make_float4(be, al + c - be, c, __uint_as_float(pack_slot(lv, q)));
+                __stcg(dir + (size_t)q * V + v, bh);
+            }
+        }
+    }
+    __syncthreads();
+    const int nF = s_n[0], nH = X == kAlone ? 0 : s_n[1];
+    bool ok = true;
+    if constexpr (X == kCluster) {
+        for (int h = tid; h < 2 * A.h_cap; h += nt) box[h] = 0;
+        cluster_barrier();
+    } else if constexpr (X == kGrid) {
+        for (int h = tid; h < nH; h += nt) {
+            __stcg(A.box0 + h_base + h, 0ull);
+            __stcg(A.box1 + h_base + h, 0ull);
+        }
+        ok = grid_barrier_once(A.bar, gridDim.x, A.flags);
+    }
+    if (X == kGrid && !ok) return;  // (a block that got past the barrier times out in its waits)
+    for (int h = tid; h < nH; h += nt) {  // where each split factor's value goes
+        const uint32_t pk = __float_as_uint(hrec[h].w);
+        const int lv = pk & 0x3fff, q = (pk >> 14) & 3;
+        const int4 t = __ldg(A.tab4 + v0 + lv);
+        const int es = q == 0 ? t.x : q == 1 ? t.y : q == 2 ? t.z : t.w;
+        const int p = __ldg(A.lr_pos + ((es >> 1) ^ 1));
+        const int u = p - V * ((p >= V) + (p >= 2 * V) + (p >= 3 * V));
+        const int ub = u / Vc, at = __ldcg(dir + p);
+        if constexpr (X == kCluster) hdst[h] = rank_addr(smem_addr(box + at), (uint32_t)ub);
+        else hdst[h] = (uint32_t)((A.off ? A.off[ub].y : (smp * A.nb + ub) * A.h_cap) + at);
+    }
+    __syncthreads();
+
+    // ---- iterations ----
+    const float k = A.k, Tln2 = A.Tln2, damping = A.damping, w = 1.f - damping;
+    for (int it = 1; it <= A.n_iters; ++it) {
+        // 1. totals
+        for (int lv = tid; lv < nv; lv += nt) {
+            const float2 e = RES ? es_sh[lv] : __ldg(ev + lv);
+            const float d0 = d[lv], d1 = d[Vc + lv], d2 = d[2 * Vc + lv], d3 = d[3 * Vc + lv];
+            FF D = ff_add_nc(ff_make(e.y), -e.x);
+            D = ff_add_nc(D, d0);
+            D = ff_add_nc(D, d1);
+            D = ff_add_nc(D, d2);
+            D = ff_add_nc(D, d3);
+            float2 Df = make_float2(D.hi, D.lo);
+            const float big = fmaxf(fmaxf(fabsf(d0), fabsf(d1)), fmaxf(fabsf(d2), fabsf(d3)));
+            if (!(fabsf(D.hi) + big < 1e38f)) {  // an infinite entry, NaN, or near overflow
+                bool fin = isfinite(e.x) && isfinite(e.y) && isfinite(d0) && isfinite(d1) && isfinite(d2) &&
+                           isfinite(d3);
+                fin = fin && isfinite(lr_lam_from_D(Df, d0)) && isfinite(lr_lam_from_D(Df, d1)) &&
+                      isfinite(lr_lam_from_D(Df, d2)) && isfinite(lr_lam_from_D(Df, d3));
+                if (!fin) {
+                    run_var_slow(A, lam, v0 + lv, e, d0, d1, d2, d3);
+                    Df = make_float2(__uint_as_float(kDvSlow), 0.f);
+                }
+            }
+            Dv[lv] = Df;
+        }
+        __syncthreads();
+        // 2. publish
+        if constexpr (X != kAlone) {
+            for (int h = tid; h < nH; h += nt) {
+                const uint32_t pk = __float_as_uint(RES ? hrec[h].w : __ldcg(&hrec[h].w));
+                const int lv = pk & 0x3fff, q = (pk >> 14) & 3;
+                const float2 D = Dv[lv];
+                const float l = is_slow(D) ? __ldcg(lam + (size_t)q * V + v0 + lv) : lr_lam_from_D(D, d[q * Vc + lv]);
+                const unsigned long long wd = box_word(l, (uint32_t)it);
+                if constexpr (X == kCluster) {
+                    const uint32_t a = hdst[h] + ((it & 1) ? 8u * (uint32_t)A.h_cap : 0u);
+                    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(wd) : "memory");
+                } else {
+                    unsigned long long *p = ((it & 1) ? A.box1 : A.box0) + (RES ? hdst[h] : __ldcg(hdst + h));
+                    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(wd) : "memory");
+                }
+            }
+        }
+        // 3. whole factors
+        {
+            int i = tid;
+            float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i < nF) r = RES ? rec[i] : __ldcg(rec + i);
+            while (i < nF) {
+                const int in = i + nt;
+                float4 rn = r;
+                if (!RES && in < nF) rn = __ldcg(rec + in);
+                const uint32_t pk = __float_as_uint(r.w);
+                const int lv0 = pk & 0x3fff, k0 = (pk >> 14) & 3, lv1 = (pk >> 16) & 0x3fff, k1 = pk >> 30;
+                const int s0 = k0 * Vc + lv0, s1 = k1 * Vc + lv1;
+                const float mo0 = d[s0], mo1 = d[s1];
+                const float2 D0 = Dv[lv0], D1 = Dv[lv1];
+                float l0 = lr_lam_from_D(D0, mo0), l1 = lr_lam_from_D(D1, mo1);
+                if (is_slow(D0)) l0 = __ldcg(lam + (size_t)k0 * V + v0 + lv0);
+                if (is_slow(D1)) l1 = __ldcg(lam + (size_t)k1 * V + v0 + lv1);
+                float n0 = lr_dir<MAXP>(r.x, r.y, r.z, l1, mo0, k, Tln2, damping, w);
+                float n1 = lr_dir<MAXP>(r.z, r.y + r.x - r.z, r.x, l0, mo1, k, Tln2, damping, w);
+                if (lr_dir_rare(n0, l1)) n0 = run_exact<MAXP>(A, pot, v0 + lv0, k0, l1, mo0);
+                if (lr_dir_rare(n1, l0)) n1 = run_exact<MAXP>(A, pot, v0 + lv1, k1, l0, mo1);
+                d[s0] = n0;
+                d[s1] = n1;
+                i = in;
+                if (RES) {
+                    if (i < nF) r = rec[i];
+                } else {
+                    r = rn;
+                }
+            }
+        }
+        // 4. split factors
+        if constexpr (X != kAlone) {
+            for (int h = tid; h < nH; h += nt) {
+                const float4 r = RES ? hrec[h] : __ldcg(hrec + h);
+                unsigned long long wd = 0;
+                int polls = 0;
+                while (true) {
+                    if constexpr (X == kCluster) {
+                        const uint32_t a = smem_addr(box + h) + ((it & 1) ? 8u * (uint32_t)A.h_cap : 0u);
+                        asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(wd) : "r"(a) : "memory");
+                    } else {
+                        const unsigned long long *p = ((it & 1) ? A.box1 : A.box0) + h_base + h;
+                        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(wd) : "l"(p) : "memory");
+                    }
+                    if ((uint32_t)(wd >> 32) == (uint32_t)it) break;
+                    if (*(volatile int *)&s_abort) break;
+                    if (++polls >= kWaitLimit) {
+                        atomicOr(A.flags, kFlagTimeout);
+                        *(volatile int *)&s_abort = 1;
+                        break;
+                    }
+                }
+                const float l = __uint_as_float((uint32_t)wd);
+                const uint32_t pk = __float_as_uint(r.w);
+                const int lv = pk & 0x3fff, q = (pk >> 14) & 3;
+                const float mo = d[q * Vc + lv];
+                float n = lr_dir<MAXP>(r.x, r.y, r.z, l, mo, k, Tln2, damping, w);
+                if (lr_dir_rare(n, l)) n = run_exact<MAXP>(A, pot, v0 + lv, q, l, mo);
+                d[q * Vc + lv] = n;
+            }
+        }
+        __syncthreads();
+    }
+
+    // ---- epilogue: every slot's two entries back into msgs (as k_lr_unpack) ----
+    const bool aligned = (reinterpret_cast<uintptr_t>(msgs) & 7u) == 0;
+    for (int lv = tid; lv < nv; lv += nt) {
+        const int4 t = __ldg(A.tab4 + v0 + lv);
+        const int es[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (es[q] < 0) continue;
+            const float2 o = lr_decode(d[q * Vc + lv]);
+            if (aligned) {
+                reinterpret_cast<float2 *>(msgs)[es[q] >> 1] = o;
+            } else {
+                msgs[es[q]] = o.x;
+                msgs[es[q] + 1] = o.y;
+            }
+        }
+    }
+    if constexpr (X == kCluster) cluster_barrier();  // no block leaves while another may write to its inbox
+}
+
+using RunKernel = void (*)(const LrRun);
+RunKernel run_kernel(bool maxp, int x, bool res) {
+    if (x == kAlone) return maxp ? (res ? k_lr_run<true, kAlone, true> : k_lr_run<true, kAlone, false>)
+                                 : (res ? k_lr_run<false, kAlone, true> : k_lr_run<false, kAlone, false>);
+    if (x == kCluster) return maxp ? k_lr_run<true, kCluster, true> : k_lr_run<false, kCluster, true>;
+    return maxp ? (res ? k_lr_run<true, kGrid, true> : k_lr_run<true, kGrid, false>)
+                : (res ? k_lr_run<false, kGrid, true> : k_lr_run<false, kGrid, false>);
+}
+
+// Shared memory of a block.
+size_t run_smem(int x, bool res, int Vc, int f_cap, int h_cap) {
+    size_t n = 24 * (size_t)Vc;
+    if (res) n += 8 * (size_t)Vc + 16 * (size_t)f_cap + 20 * (size_t)h_cap;
+    if (x == kCluster) n += 16 * (size_t)h_cap;
+    return n + 16;
+}
+
+// What the device offers, asked once: SMs, shared memory for a block, cluster size, whether
+// it takes cooperative launches. The kernels' attributes are set here too.
+struct RunDevice {
+    bool ready = false;
+    int n_sm = 0, smem = 0, cluster = 0;
+    bool coop = false;
+};
+const RunDevice &run_device() {
+    static RunDevice devs[64];
+    static std::mutex mu;
+    static const RunDevice none;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return none;
+    std::lock_guard<std::mutex> lk(mu);
+    RunDevice &R = devs[dev];
+    if (R.ready) return R;
+    int optin = 0, coop = 0;
+    if (cudaDeviceGetAttribute(&R.n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return none;
+    }
+    R.smem = optin - 256;  // less the kernels' static shared memory
+    for (int x = 0; x < 3; ++x)
+        for (int m = 0; m < 2; ++m)
+            for (int r = 0; r < 2; ++r) {
+                RunKernel kern = run_kernel(m, x, r);
+                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, R.smem);
+                if (x == kCluster) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            }
+    for (int C : {kLrClusterMax, 8}) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(C);
+        cfg.blockDim = dim3(kLrRunThreads);
+        cfg.dynamicSmemBytes = run_smem(kCluster, true, kLrSmallMaxV, 2 * kLrSmallMaxV, 4 * kLrSmallMaxV);
+        if ((int)cfg.dynamicSmemBytes > R.smem) break;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n0 = 0, n1 = 0;
+        if (cudaOccupancyMaxActiveClusters(&n0, k_lr_run<true, kCluster, true>, &cfg) == cudaSuccess && n0 > 0 &&
+            cudaOccupancyMaxActiveClusters(&n1, k_lr_run<false, kCluster, true>, &cfg) == cudaSuccess && n1 > 0) {
+            R.cluster = C;
+            break;
+        }
+    }
+    R.coop = coop != 0;
+    for (int m = 0; m < 2 && R.coop; ++m)
+        for (int r = 0; r < 2; ++r) {
+            int n = 0;
+            R.coop = R.coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, run_kernel(m, kGrid, r), kLrRunThreads,
+                                                                             R.smem) == cudaSuccess && n >= 1;
+        }
+    cudaGetLastError();  // a refused query leaves no error behind
+    R.ready = true;
+    return R;
+}
+
+int run_threads(int Vc, int items) {
+    const int per = std::max(Vc, items);
+    return std::min(kLrRunThreads, std::max(32, (per + 31) / 32 * 32));
+}
+
+cudaError_t launch(RunKernel kern, const LrRun &A, int blocks, int threads, size_t smem, int x, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    if (x == kCluster) {
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)blocks;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+    } else {
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = x == kAlone ? 0 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, A);
+}
+
+LrRun run_args(const DevGraph &G, const EnumSeg *segs, int n_seg, const float *pot, const float *ev, float *msgs,
+               float *lam, float T, float damping, int n_iters) {
+    LrRun A{};
+    A.V = G.V;
+    A.E = G.E;
+    A.tab4 = G.vin_tab4;
+    A.lr_pos = G.lr_pos;
+    A.segs = segs;
+    A.n_seg = n_seg;
+    A.pot = pot;
+    A.ev = ev;
+    A.msgs = msgs;
+    A.lam = lam;
+    A.flags = G.flags;
+    A.bar = G.flags + 16;
+    // softplus_t constants: k = log2(e) / T, T ln 2
+    A.k = T > 0.f ? (float)(1.4426950408889634 / (double)T) : 0.f;
+    A.Tln2 = (float)((double)T * 0.6931471805599453);
+    A.damping = damping;
+    A.n_iters = n_iters;
+    A.nb = 1;
+    A.Vc = G.V;
+    return A;
+}
+
+// The one launch that covers every factor of a log-ratio graph.
+const FactorLaunch *only_launch(const Plan &P) {
+    for (const FactorLaunch &L : P.factor)
+        if (L.n_blocks > 0) return &L;
+    return nullptr;
+}
+
+}  // namespace
+
+int lr_cluster_size() { return run_device().cluster; }
+
+cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *log_pot, const float *ev, float *msgs,
+                                float *lam, int32_t *dir, float T, float damping, int n_iters, bool cluster,
+                                cudaStream_t s) {
+    const int F = G.E / 2, V = G.V;
+    if (!(cluster ? lr_cluster_fits(V, F) : lr_block_fits(V, F)) || G.vin_tab4 == nullptr || G.lr_pos == nullptr)
+        return cudaErrorInvalidValue;
+    const FactorLaunch *L = only_launch(P);
+    if (L == nullptr || n_iters <= 0) return cudaSuccess;
+    run_device();  // the kernels' attributes
+    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, lam, T, damping, n_iters);
+    A.dir = dir;
+    if (!cluster) {
+        A.f_cap = F;
+        return launch(run_kernel(T == 0.f, kAlone, true), A, 1, run_threads(V, F), run_smem(kAlone, true, V, F, 0),
+                      kAlone, s);
+    }
+    const int C = lr_cluster_size();
+    A.nb = C;
+    A.Vc = (V + C - 1) / C;
+    A.f_cap = 2 * A.Vc;  // a block's variables have 4 slots each, a whole factor takes two
+    A.h_cap = 4 * A.Vc;
+    return launch(run_kernel(T == 0.f, kCluster, true), A, C, run_threads(A.Vc, (F + C - 1) / C),
+                  run_smem(kCluster, true, A.Vc, A.f_cap, A.h_cap), kCluster, s);
+}
+
+// ---- the grid form of one sample ----
+
+int lr_grid_blocks(int V) {
+    const RunDevice &R = run_device();
+    if (!R.coop || V < 2) return 0;
+    const int Vc = std::max((V + R.n_sm - 1) / R.n_sm, kLrGridMinV);
+    const int nb = (V + Vc - 1) / Vc;
+    return nb >= 2 && 24 * (int64_t)Vc + 16 <= R.smem && Vc < (1 << 14) ? nb : 0;
+}
+
+bool lr_grid_fits(const LrGridPlan &g, int V, int F) {
+    const RunDevice &R = run_device();
+    if (g.nb < 2 || !R.coop || g.nb > R.n_sm) return false;
+    const int64_t split = g.n_split;
+    // the workspace: see launch_lr_grid_run
+    if (run_smem(kGrid, true, g.Vc, g.f_max, g.h_max) <= (size_t)R.smem) return 2 * split <= 3 * (int64_t)F;
+    return 20 * split <= 12 * (int64_t)F && 16 * split <= 8 * (int64_t)V;
+}
+
+// Workspace from the graph's multi-launch scratch, which a one-launch run does not otherwise
+// use (bytes, F factors, V variables): m_tmp [16 F], b [8 V], d [16 V], prm [12 F]. The slot
+// directory (16 V) is in d. Records in shared memory: the inboxes (8 bytes per split slot
+// each) in m_tmp and prm. Records in global memory: whole factors' in m_tmp (16 each), split
+// factors' (16 + 4) in prm, the inboxes in b. lr_grid_fits has checked that they fit.
+cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPlan &g, const float *log_pot,
+                               const float *ev, float *msgs, float *lam, float *m_tmp, float *b, float *d, float *prm,
+                               float T, float damping, int n_iters, cudaStream_t s) {
+    const int F = G.E / 2, V = G.V;
+    if (!lr_grid_fits(g, V, F)) return cudaErrorInvalidValue;
+    const FactorLaunch *L = only_launch(P);
+    if (L == nullptr || n_iters <= 0) return cudaSuccess;
+    const RunDevice &R = run_device();
+    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, lam, T, damping, n_iters);
+    A.dir = reinterpret_cast<int32_t *>(d);
+    A.nb = g.nb;
+    A.Vc = g.Vc;
+    A.f_cap = g.f_max;
+    A.h_cap = g.h_max;
+    A.off = g.off;
+    const size_t smem = run_smem(kGrid, true, g.Vc, g.f_max, g.h_max);
+    const bool res = smem <= (size_t)R.smem;
+    if (res) {
+        A.box0 = reinterpret_cast<unsigned long long *>(m_tmp);
+        A.box1 = reinterpret_cast<unsigned long long *>(prm);
+    } else {
+        A.rec = reinterpret_cast<float4 *>(m_tmp);
+        A.hrec = reinterpret_cast<float4 *>(prm);
+        A.hdst = reinterpret_cast<uint32_t *>(prm) + 4 * g.n_split;
+        A.box0 = reinterpret_cast<unsigned long long *>(b);
+        A.box1 = A.box0 + g.n_split;
+    }
+    return launch(run_kernel(T == 0.f, kGrid, res), A, g.nb, run_threads(g.Vc, g.f_max),
+                  res ? smem : run_smem(kGrid, false, g.Vc, 0, 0), kGrid, s);
+}
+
+// ---- many samples of one graph ----
+
+LrMultiPlan lr_multi_plan(int V, int S, bool local) {
+    const RunDevice &R = run_device();
+    LrMultiPlan p;
+    if (R.n_sm < 1 || V < 1 || S < 1) return p;
+    const int v_max = std::min((1 << 14) - 1, (R.smem - 16) / 24);  // variables one block can own
+    const int nb_min = (V + v_max - 1) / v_max;
+    int nb = 1, Sc = S;
+    if (V > kLrAloneV && R.coop && local && nb_min <= R.n_sm) {
+        const int chunks = (S + R.n_sm / nb_min - 1) / (R.n_sm / nb_min);
+        Sc = (S + chunks - 1) / chunks;
+        nb = std::min(R.n_sm / Sc, (V + kLrGridMinV - 1) / kLrGridMinV);
+    } else if (nb_min > 1) {
+        return p;
+    }
+    p.Vc = (V + nb - 1) / nb;
+    p.nb = (V + p.Vc - 1) / p.Vc;
+    p.f_cap = 2 * p.Vc;
+    p.h_cap = p.nb > 1 ? 4 * p.Vc : 0;
+    const int x = p.nb > 1 ? kGrid : kAlone;
+    p.res = run_smem(x, true, p.Vc, p.f_cap, p.h_cap) <= (size_t)R.smem;
+    // per sample: lam and directory, then each block's items (run_multi's layout)
+    p.sample_bytes = 32 * (size_t)V + (size_t)p.nb * (16 * (size_t)p.h_cap + (p.res ? 0 : 16 * (size_t)p.f_cap + 20 * (size_t)p.h_cap));
+    if (p.nb == 1) Sc = (int)std::min<int64_t>(S, std::max<int64_t>(1, ((int64_t)1 << 28) / (int64_t)p.sample_bytes));
+    p.S = Sc;
+    return p;
+}
+
+cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiPlan &p, int S, int64_t pot_stride,
+                                const float *log_pot, const float *ev, float *msgs, char *work, float T, float damping,
+                                int n_iters, cudaStream_t s) {
+    const FactorLaunch *L = only_launch(P);
+    if (S < 1 || S > p.S || G.vin_tab4 == nullptr) return cudaErrorInvalidValue;
+    if (L == nullptr || n_iters <= 0) return cudaSuccess;
+    const size_t V = (size_t)G.V, blocks = (size_t)S * p.nb;
+    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, nullptr, T, damping, n_iters);
+    A.pot_stride = pot_stride;
+    A.ev_stride = G.VS;
+    A.msg_stride = G.ES;
+    A.nb = p.nb;
+    A.Vc = p.Vc;
+    A.f_cap = p.f_cap;
+    A.h_cap = p.h_cap;
+    // 16-byte records first, then 8-byte inboxes, then words
+    if (!p.res) {
+        A.rec = reinterpret_cast<float4 *>(work);
+        A.hrec = A.rec + blocks * p.f_cap;
+        work = reinterpret_cast<char *>(A.hrec + blocks * p.h_cap);
+    }
+    A.box0 = reinterpret_cast<unsigned long long *>(work);
+    A.box1 = A.box0 + blocks * p.h_cap;
+    A.hdst = reinterpret_cast<uint32_t *>(A.box1 + blocks * p.h_cap);
+    A.lam = reinterpret_cast<float *>(A.hdst + (p.res ? 0 : blocks * p.h_cap));
+    A.dir = reinterpret_cast<int32_t *>(A.lam + 4 * V * S);
+    const int x = p.nb > 1 ? kGrid : kAlone;
+    return launch(run_kernel(T == 0.f, x, p.res), A, (int)blocks, run_threads(p.Vc, (2 * G.V + p.nb - 1) / p.nb),
+                  p.res ? run_smem(x, true, p.Vc, p.f_cap, p.h_cap) : run_smem(x, false, p.Vc, 0, 0), x, s);
+}
+
+}  // namespace pgm

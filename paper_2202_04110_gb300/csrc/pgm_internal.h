@@ -178,6 +178,15 @@ struct VarLaunch {
     int32_t n_tiles;
 };
 
+// The grid form of a one-launch run of this graph (lr_run.cu): nb blocks of Vc variables,
+// the largest counts of whole and split factors (items) of a block, all split items, and
+// each block's first whole and split item (device).
+struct LrGridPlan {
+    int32_t nb = 0, Vc = 0, f_max = 0, h_max = 0;
+    int64_t n_split = 0;
+    const int2 *off = nullptr;
+};
+
 struct Plan {
     std::vector<FactorLaunch> factor;
     std::vector<VarLaunch> var;
@@ -185,6 +194,7 @@ struct Plan {
     // high-degree variable): iterations may keep one log-ratio per edge.
     bool lr = false;
     int32_t lr_blocks = 1;  // persistent log-ratio factor pass: blocks of 256 (8 per SM)
+    LrGridPlan grid;        // nb = 0: none
 };
 
 // Host-side result of the graph compiler (compile.cpp).
@@ -297,19 +307,16 @@ cudaError_t launch_pmp_perturb(int64_t VS, int S, const float *ev, const float *
 // Log-ratio pack (from the [2E] edge-state layout; unused slots 0) and unpack.
 cudaError_t launch_lr_pack(const DevGraph &G, const float *m, float *d, cudaStream_t s);
 cudaError_t launch_lr_unpack(const DevGraph &G, const float *d, float *m, cudaStream_t s);
-// One block, or a cluster of blocks sharing their shared memories, runs a whole log-ratio
-// run of a small graph (4-slot layout), msgs in and out: one block up to kLrSmallMaxV
-// variables and kLrSmallMaxF factors (one variable and one factor per thread, or two
-// factors above kLrSmallThreads of them; 24 V bytes of shared memory), a cluster of C blocks
-// up to C times that (the same per block on its share). C is 16 where the device places a
-// cluster of 16 such blocks (a non-portable size), else 8 where it places 8, else there is
-// no cluster form (lr_cluster_size, asked once per device).
-constexpr int kLrSmallThreads = 1024, kLrSmallMaxV = 1024, kLrSmallMaxF = 2048;
+// One-launch runs (lr_run.cu): a whole log-ratio run of a graph with the 4-slot layout in one
+// kernel, msgs in and out.
+// Small graphs: one block up to kLrSmallMaxV variables and kLrSmallMaxF factors, a cluster of C
+// blocks up to C times that. C is 16 where the device places a cluster of 16 such blocks (a
+// non-portable size), else 8 where it places 8, else there is no cluster form
+// (lr_cluster_size, asked once per device). dir: 4 V words of scratch.
+constexpr int kLrRunThreads = 1024, kLrSmallMaxV = 1024, kLrSmallMaxF = 2048;
 constexpr int kLrClusterMax = 16;
 int lr_cluster_size();
-// Setting 1 of PGM_OPT_SMALL_RUN: one block up to this many variables, the cluster above
-// (the cluster's two barriers per iteration cost about 1.1 us per iteration on a GB300; one
-// block was faster up to 24 x 24 grids, the cluster from 28 x 28).
+// Setting 1 of PGM_OPT_SMALL_RUN: one block up to this many variables, the cluster above.
 constexpr int kLrBlockAutoV = 700;
 inline bool lr_block_fits(int V, int F) { return V > 0 && V <= kLrSmallMaxV && F <= kLrSmallMaxF; }
 inline bool lr_cluster_fits(int V, int F) {
@@ -317,8 +324,31 @@ inline bool lr_cluster_fits(int V, int F) {
     return C > 0 && V > 0 && V <= C * kLrSmallMaxV && F <= C * kLrSmallMaxF;
 }
 cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *log_pot, const float *ev,
-                                float *msgs, float *lam, float T, float damping, int n_iters, bool cluster,
-                                cudaStream_t s);
+                                float *msgs, float *lam, int32_t *dir, float T, float damping, int n_iters,
+                                bool cluster, cudaStream_t s);
+// Larger graphs: a cooperative grid of nb blocks, block b owning variables b Vc ..
+// (b + 1) Vc - 1. lr_grid_blocks: nb for V variables on this device (0: none); the plan's
+// other fields are counted from the graph (capi.cu). lr_grid_fits: the device takes it and
+// the graph's scratch holds its workspace.
+constexpr int kLrGridMinV = 256;  // variables per block at least
+int lr_grid_blocks(int V);
+bool lr_grid_fits(const LrGridPlan &g, int V, int F);
+cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPlan &g, const float *log_pot,
+                               const float *ev, float *msgs, float *lam, float *m_tmp, float *b, float *d, float *prm,
+                               float T, float damping, int n_iters, cudaStream_t s);
+// S samples of one graph (pgm_run_bp_multi), nb blocks each, up to p.S samples a launch;
+// work: p.sample_bytes per sample. local: few factors join different blocks (LrGridPlan).
+constexpr int kLrAloneV = 1536;  // up to this many variables a sample takes one block
+struct LrMultiPlan {
+    int S = 0;  // samples per launch; 0: the device takes no such launch
+    int nb = 0, Vc = 0, f_cap = 0, h_cap = 0;
+    bool res = false;
+    size_t sample_bytes = 0;
+};
+LrMultiPlan lr_multi_plan(int V, int S, bool local);
+cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiPlan &p, int S, int64_t pot_stride,
+                                const float *log_pot, const float *ev, float *msgs, char *work, float T, float damping,
+                                int n_iters, cudaStream_t s);
 // Adjoint launchers (kernels.cu).
 cudaError_t launch_adj_beliefs(const DevGraph &G, const float *ev, const float *m, const float *gnb, float *d_ev,
                                float *adj, cudaStream_t s);
