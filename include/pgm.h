@@ -492,7 +492,9 @@ pgm_status pgm_run_bp_until_members(pgm_graph *g, const float *log_pot, const fl
 #define PGM_OPT_ENUM_BLOCK 3
 /*
  * PGM_OPT_PAIR_FORM (default 0): the kernel form of dense K-state pairwise groups (K = 4,
- * 8, 16). 0 the compiler's choice (a thread per factor), 1 a thread per factor, 2 K
+ * 8, 16). 0 the compiler's choice (the variable pass and the factor pass in one kernel where
+ * every group of the launch shares one table, is its member's only group and has variables
+ * with at most 4 factors; else a thread per factor), 1 a thread per factor, 2 K
  * lanes per factor, 3 K / 4 lanes per factor with four states each (K = 8, 16, for
  * launches whose groups all share their tables; else a thread per factor), 4 a thread per
  * factor and direction. The thread, K / 4-lane and direction forms give the same bits.
@@ -578,8 +580,9 @@ pgm_status pgm_autotune(pgm_graph *g, const float *log_pot, const float *evidenc
  * per factor, the default form, which pgm_autotune may exchange with 1..3, 11, 12 or
  * 13..15; 10 listed configurations with a block per run of factors; 11, 12 dense
  * pairwise K = 8, 16 with K / 4 lanes per factor, for shared tables; 13..15 dense
- * pairwise K = 4, 8, 16 with a thread per factor and direction); threads per block and
- * blocks. Any output pointer may be NULL.
+ * pairwise K = 4, 8, 16 with a thread per factor and direction; 16..18 dense pairwise K = 4,
+ * 8, 16 with the variable pass in the same kernel: the variable launch of that K is then
+ * listed but not made); threads per block and blocks (of the two-pass form for 16..18). Any output pointer may be NULL.
  */
 pgm_status pgm_launch_info(const pgm_graph *g, int32_t i, int32_t *kind, int32_t *variant,
                            int32_t *threads, int32_t *n_blocks);

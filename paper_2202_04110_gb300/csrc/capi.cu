@@ -141,6 +141,11 @@ struct pgm_graph {
     size_t adj_logic_seg_off = (size_t)-1;
     int32_t enum_block = 0;  // PGM_OPT_ENUM_BLOCK
     int32_t pair_form = 0;   // PGM_OPT_PAIR_FORM
+    struct Fused {           // factor launches with a fused form, the variable launch each
+        int factor, var;     // replaces, and its blocks in the index memory
+        size_t off;
+    };
+    std::vector<Fused> fused;
     // checked mode (PGM_OPT_CHECKED): the audit's work buffer (allocated on first use),
     // the pools' sizes, the last violation found
     int32_t checked = 0;
@@ -328,6 +333,60 @@ static int32_t plan_enum_block(EnumSeg *segs, int n_seg, int threads, int n_sm, 
     return blk;
 }
 
+// The fused form (pair_fused.cu) of each dense K-state pairwise launch, K = 4, 8, 16: taken
+// when every group of the launch shares one table and is its member's only group (so its
+// variables' factors are all its own) and none of its variables has more than 4 factors; its blocks go into the index
+// memory.
+void plan_fused(const HostLayout &H, pgm_graph *g, Packer &pk) {
+    Plan &P = g->P;
+    std::vector<int32_t> groups(H.members.size(), 0);
+    for (const HostEnumGroup &hg : H.enum_groups) groups[hg.seg.member] += hg.seg.n_fac > 0;
+    for (const HostLogicGroup &hg : H.logic_groups) groups[hg.seg.member] += hg.seg.n_fac > 0;
+    for (size_t li = 0; li < P.factor.size(); ++li) {
+        FactorLaunch &L = P.factor[li];
+        if (fused_variant(L.variant) < 0) continue;
+        const int kind = L.variant == kPairT4 ? kVarGroup4 : L.variant == kPairT8 ? kVarGroup8 : kVarGroup16;
+        const std::vector<int32_t> &bucket = H.var_bucket[kind];
+        size_t vi = 0;
+        while (vi < P.var.size() && P.var[vi].kind != kind) ++vi;
+        bool ok = vi < P.var.size();
+        // variables per block: one round of the block's teams (256 threads, K / 4 lanes each);
+        // more rounds would form the table less often, but a round's loads depend on one
+        // another and other blocks hide them better (K = 16 on the batch: 171 us with one
+        // round, 192 with two)
+        const int per = L.variant == kPairT4 ? 256 : L.variant == kPairT8 ? 128 : 64;
+        std::vector<FuseBlock> fs;
+        // (the variable launch goes as a whole: no other group may touch its variables)
+        int64_t all_edges = 0;
+        for (int32_t v : bucket) all_edges += H.vin_off[v + 1] - H.vin_off[v];
+        for (const HostEnumGroup &hg : H.enum_groups) {
+            if (hg.variant != L.variant) continue;
+            if (hg.seg.n_fac == 0 || !ok) continue;
+            const HostMember &m = H.members[hg.seg.member];
+            ok = ok && groups[hg.seg.member] == 1 && hg.seg.shared != 0;
+            const auto b0 = std::lower_bound(bucket.begin(), bucket.end(), (int32_t)m.var_off);
+            const auto b1 = std::lower_bound(b0, bucket.end(), (int32_t)(m.var_off + m.n_vars));
+            // every edge of the group belongs to a variable of the bucket
+            int64_t edges = 0;
+            for (auto it = b0; it != b1; ++it) {
+                const int32_t deg = H.vin_off[*it + 1] - H.vin_off[*it];
+                ok = ok && deg <= 4;
+                edges += deg;
+            }
+            ok = ok && edges == 2 * (int64_t)hg.seg.n_fac;
+            all_edges -= edges;
+            for (auto it = b0; it < b1; it += std::min<int64_t>(per, b1 - it))
+                fs.push_back({(int32_t)(it - bucket.begin()), (int32_t)std::min<int64_t>(per, b1 - it), hg.seg.es_base,
+                              hg.seg.pot_base, hg.seg.member, {0, 0, 0}});
+        }
+        if (!ok || fs.empty() || all_edges != 0) continue;
+        g->fused.push_back({(int)li, (int)vi, pk.add(fs.data(), fs.size())});
+        L.fuse_blocks = (int32_t)fs.size();
+        L.variant = fused_variant(L.base_variant);
+        P.var[vi].fused_by = (int32_t)li;
+    }
+}
+
 pgm_status build_plan(const HostLayout &H, pgm_graph *g, Packer &pk, std::vector<size_t> &seg_off,
                       std::vector<int> &seg_kind) {
     // variable pass: one launch per non-empty bucket of variables
@@ -337,6 +396,7 @@ pgm_status build_plan(const HostLayout &H, pgm_graph *g, Packer &pk, std::vector
         if (bucket.empty()) continue;
         VarLaunch L{};
         L.kind = kind;
+        L.fused_by = -1;
         L.n = (int32_t)bucket.size();
         L.threads = 256;
         L.n_blocks = (kind == kVarBlock) ? L.n : (int32_t)(((int64_t)L.n * var_lanes(kind) + 255) / 256);
@@ -492,6 +552,7 @@ pgm_status build_plan(const HostLayout &H, pgm_graph *g, Packer &pk, std::vector
                                              reinterpret_cast<const char *>(segs.data() + segs.size()));
         }
     }
+    plan_fused(H, g, pk);
     P.lr = lr_eligible(H);
     P.lr_blocks = std::max(1, g->n_sm * 8);
     return PGM_OK;
@@ -798,6 +859,11 @@ static pgm_status build_from_layout(const HostLayout &H, pgm_graph **out, cudaSt
             L.segs = dmem + seg_off[k];
             max_smem = std::max(max_smem, L.smem);
         }
+    }
+    for (const auto &f : g->fused) {
+        FactorLaunch &L = g->P.factor[f.factor];
+        L.fuse = reinterpret_cast<const FuseBlock *>(dmem + f.off);
+        L.fuse_list = g->P.var[f.var].list;
     }
     if (g->P.grid.nb > 0) g->P.grid.off = reinterpret_cast<const int2 *>(dmem + o_grid);
     if (g->adj_seg_off != (size_t)-1) g->adj_launch.segs = dmem + g->adj_seg_off;
@@ -1938,6 +2004,7 @@ pgm_status pgm_autotune(pgm_graph *g, const float *log_pot, const float *evidenc
     launch_var_pass(g->G, g->P, evidence, m_in, g->b, kVarIter, nullptr, s);
     for (size_t li = 0; li < g->P.factor.size(); ++li) {
         const int orig_variant = g->P.factor[li].variant;
+        if (is_fused(orig_variant)) continue;  // (it was faster than every two-pass form and has one shape)
         int best = g->P.factor[li].threads, best_variant = orig_variant;
         float best_ms = 1e30f;
         // the kernel forms that can run this launch's groups, each with its block shapes
@@ -2147,7 +2214,7 @@ static pgm_status enqueue_grad(pgm_graph *g, const float *log_pot, const float *
             // which its reverse step reads; the segment's last state needs one more pass
             for (int i = 1; i <= t1 - t0 && st == PGM_OK; ++i) {
                 const DevGraph Gs = step_G(i - 1);
-                e = launch_var_pass(Gs, g->P, evidence, recp(i - 1), step_b(i - 1), kVarIter, nullptr, s);
+                e = launch_var_pass(Gs, g->P, evidence, recp(i - 1), step_b(i - 1), kVarIter, nullptr, s, 1, nullptr, true);
                 if (e == cudaSuccess && i < t1 - t0)
                     e = launch_factor_pass(Gs, g->P, log_pot, step_b(i - 1), evidence, recp(i - 1), recp(i), T,
                                            damping, s);
@@ -2161,7 +2228,7 @@ static pgm_status enqueue_grad(pgm_graph *g, const float *log_pot, const float *
             const float *m_prev = recp(t - 1 - t0);
             const DevGraph Gs = keep ? step_G(t - 1 - t0) : g->G;
             float *bt = keep ? step_b(t - 1 - t0) : g->b;
-            e = keep ? cudaSuccess : launch_var_pass(Gs, g->P, evidence, m_prev, bt, kVarIter, nullptr, s);
+            e = keep ? cudaSuccess : launch_var_pass(Gs, g->P, evidence, m_prev, bt, kVarIter, nullptr, s, 1, nullptr, true);
             if (e == cudaSuccess)
                 e = launch_adj_factor(Gs, g->adj_launch, log_pot, bt, evidence, m_prev, adjA, dv, ddamp, d_log_pot,
                                       partials, g->adj_nc_max, T, damping, s);
@@ -2326,12 +2393,12 @@ pgm_status pgm_set_option(pgm_graph *g, int32_t option, int64_t value) {
                 bool all_shared = true;
                 const EnumSeg *sg = reinterpret_cast<const EnumSeg *>(g->factor_segs_host[li].data());
                 for (int i = 0; i < L.n_seg; ++i) all_shared = all_shared && sg[i].shared != 0;
-                const int want = value == 0 ? base : value == 1 ? thr : value == 2 ? lanes
+                const int want = value == 0 ? (L.fuse_blocks > 0 ? fused_variant(base) : base) : value == 1 ? thr : value == 2 ? lanes
                                  : value == 3 ? (all_shared ? quad : thr) : dir;
                 if (L.variant == want) continue;
                 const int old_variant = L.variant;
                 L.variant = want;
-                if (!replan_factor_launch(g, li, want == kPairT16 ? 128 : 256, nullptr)) {
+                if (!replan_factor_launch(g, li, want == kPairT16 || want == kPairF16 ? 128 : 256, nullptr)) {
                     L.variant = old_variant;
                     return fail(PGM_ECUDA, "re-planning a pairwise launch failed");
                 }

@@ -41,416 +41,17 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "bp_common.cuh"
 #include "lr_math.cuh"
+#include "pair_math.cuh"
 #include "pgm_internal.h"
 
 namespace pgm {
 namespace {
 
-// Programmatic dependent launch (griddepcontrol): a kernel launched with the
-// programmatic-serialization attribute may be scheduled before the previous kernel of
-// its stream has finished. pdl_wait() returns once that kernel has completed and its
-// writes are visible (at once for a kernel launched without the attribute);
-// pdl_launch_dependents() lets the next kernel be scheduled before this one ends.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-template <class Seg>
-__device__ __forceinline__ int find_seg(const Seg *__restrict__ segs, int n, int blk) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (__ldg(&segs[mid].block_begin) <= blk) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-// ---- vector loads / stores with a run-time alignment check -------------------------
-
-template <int N>
-__device__ __forceinline__ void load_n(float (&d)[N], const float *__restrict__ p) {
-    if constexpr (N % 4 == 0) {
-        if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
-#pragma unroll
-            for (int i = 0; i < N / 4; ++i) {
-                float4 q = __ldg(reinterpret_cast<const float4 *>(p) + i);
-                d[4 * i] = q.x; d[4 * i + 1] = q.y; d[4 * i + 2] = q.z; d[4 * i + 3] = q.w;
-            }
-            return;
-        }
-    }
-    if constexpr (N % 2 == 0) {
-        if ((reinterpret_cast<uintptr_t>(p) & 7u) == 0) {
-#pragma unroll
-            for (int i = 0; i < N / 2; ++i) {
-                float2 q = __ldg(reinterpret_cast<const float2 *>(p) + i);
-                d[2 * i] = q.x; d[2 * i + 1] = q.y;
-            }
-            return;
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < N; ++i) d[i] = __ldg(p + i);
-}
-
-// Streaming load of data read once per iteration (messages).
-template <int N>
-__device__ __forceinline__ void load_n_stream(float (&d)[N], const float *__restrict__ p) {
-    if constexpr (N % 4 == 0) {
-        if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
-#pragma unroll
-            for (int i = 0; i < N / 4; ++i) {
-                float4 q = __ldcs(reinterpret_cast<const float4 *>(p) + i);
-                d[4 * i] = q.x; d[4 * i + 1] = q.y; d[4 * i + 2] = q.z; d[4 * i + 3] = q.w;
-            }
-            return;
-        }
-    }
-    load_n<N>(d, p);
-}
-
-template <int N>
-__device__ __forceinline__ void store_n(float *__restrict__ p, const float (&s)[N]) {
-    if constexpr (N % 4 == 0) {
-        if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
-#pragma unroll
-            for (int i = 0; i < N / 4; ++i)
-                reinterpret_cast<float4 *>(p)[i] = make_float4(s[4 * i], s[4 * i + 1], s[4 * i + 2], s[4 * i + 3]);
-            return;
-        }
-    }
-    if constexpr (N % 2 == 0) {
-        if ((reinterpret_cast<uintptr_t>(p) & 7u) == 0) {
-#pragma unroll
-            for (int i = 0; i < N / 2; ++i)
-                reinterpret_cast<float2 *>(p)[i] = make_float2(s[2 * i], s[2 * i + 1]);
-            return;
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < N; ++i) p[i] = s[i];
-}
-
-// a > b, compared exactly on the float-float values
-__device__ __forceinline__ bool ff_gt(FF a, FF b) {
-    if (a.hi == kNegInf) return false;
-    if (b.hi == kNegInf) return true;
-    return ff_diff(a, b) > 0.f;
-}
-
-// What r = ff_diff(a, b) dropped: (a - b) - r, from the two-sum of the high parts plus
-// the low parts; 0 where a or b is not finite.
-__device__ __forceinline__ float ff_diff_lo(FF a, FF b, float r) {
-    if (!isfinite(a.hi) || !isfinite(b.hi)) return 0.f;
-    const float th = a.hi - b.hi, bb = th - a.hi;
-    const float te = (a.hi - (th - bb)) + (-b.hi - bb);
-    return (th - r) + (te + (a.lo - b.lo));
-}
-
-// Belief residuals of a binary variable whose relative beliefs (r0, r1) came from the
-// float-float sums (s0, s1): the larger state is exact (0), the other keeps what its
-// rounding dropped.
-__device__ __forceinline__ void write_b_lo2(float *p, FF s0, FF s1, float r0, float r1) {
-    float l0 = 0.f, l1 = 0.f;
-    if (r0 != 0.f || r1 != 0.f) {
-        if (r1 == 0.f) l0 = ff_diff_lo(s0, s1, r0);
-        else l1 = ff_diff_lo(s1, s0, r1);
-    }
-    reinterpret_cast<float2 *>(p)[0] = make_float2(l0, l1);
-}
-
-// ---- variable-to-factor value -------------------------------------------------------
-
-// Explicit leave-one-out values of one edge: v(x) = e_v(x) + sum over the variable's
-// other incoming edges of m(x), float-float summed, for all K states of the edge. Used
-// when b - m would be unreliable: a stored entry is -inf (-inf - -inf) or very large
-// (cancellation). Its per-edge constant differs from the fast path's, which the factor
-// update does not see (it is invariant to a constant added to one edge's values).
-constexpr float kExactThreshold = 128.f;
-
-__device__ __noinline__ void v2f_slow_edge(const DevGraph G, const float *__restrict__ ev,
-                                           const float *__restrict__ m, int vs, int es, int K,
-                                           float *__restrict__ out) {
-    int lo = 0, hi = G.V - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (G.vs_off[mid] <= vs) lo = mid;
-        else hi = mid - 1;
-    }
-    const int k0 = G.vin_off[lo], k1 = G.vin_off[lo + 1];
-    for (int x = 0; x < K; ++x) {
-        FF s = ff_make(ev[vs + x]);
-        for (int k = k0; k < k1; ++k) {
-            const int e2 = G.vin_es[k];
-            if (e2 != es) s = ff_add(s, m[e2 + x]);
-        }
-        out[x] = s.hi + s.lo;
-    }
-}
-
-__device__ __forceinline__ bool needs_exact(float mv) { return !(fabsf(mv) <= kExactThreshold); }
-
-// High-degree variables (more than kVarBlockDegree factors; their edges carry edge_vs
-// with the sign bit set, the variable's first state in the other bits): the variable pass
-// keeps, per state, the float-float sum of the finite evidence and incoming entries and
-// the count of the -inf ones (G.hd_b, float4 (hi, lo, count, 0)). An edge's exact
-// leave-one-out value is that sum less the edge's own entry -- -inf when another entry
-// or the evidence is -inf -- formed in float-float from the four numbers and the entry,
-// so that the pass writes nothing per edge. Returned as a (hi, lo) pair.
-__device__ __forceinline__ float2 hd_pair(const DevGraph &G, int vs, int x, float mo) {
-    const float4 t = __ldg(reinterpret_cast<const float4 *>(G.hd_b) + (vs & 0x7fffffff) + x);
-    const bool own = (mo == -CUDART_INF_F);
-    if (t.z > (own ? 1.f : 0.f)) return make_float2(-CUDART_INF_F, 0.f);
-    if (own) return make_float2(t.x, t.y);
-    const float sh = t.x - mo;
-    if (!isfinite(sh)) return make_float2(sh, 0.f);
-    // two-sum of the high parts, then the low part, renormalised
-    const float bb = sh - t.x;
-    const float err = (t.x - (sh - bb)) + (-mo - bb);
-    const float lo = err + t.y;
-    const float hi = sh + lo;
-    return make_float2(hi, lo - (hi - sh));
-}
-
-__device__ __forceinline__ float hd_rel(float2 a, float2 mx) {
-    if (!isfinite(a.x) || !isfinite(mx.x)) return a.x - mx.x;
-    return (a.x - mx.x) + (a.y - mx.y);
-}
-
-__device__ __forceinline__ bool hd_gt(float2 a, float2 b) {
-    if (a.x == -CUDART_INF_F) return false;
-    if (b.x == -CUDART_INF_F) return true;
-    return hd_rel(a, b) > 0.f;
-}
-
-// The variable-to-factor values of an edge of a high-degree variable (vs: its edge_vs,
-// mo: the edge's stored entries), relative to the edge's largest state.
-template <int K>
-__device__ __forceinline__ void hd_v2f(const DevGraph &G, int vs, const float (&mo)[K], float (&v)[K]) {
-    float2 d[K];
-    int arg = 0;
-#pragma unroll
-    for (int x = 0; x < K; ++x) {
-        d[x] = hd_pair(G, vs, x, mo[x]);
-        if (x > 0 && hd_gt(d[x], d[arg])) arg = x;
-    }
-    float2 mx = d[0];
-#pragma unroll
-    for (int x = 1; x < K; ++x)
-        if (x == arg) mx = d[x];
-    if (mx.x == -CUDART_INF_F) {
-#pragma unroll
-        for (int x = 0; x < K; ++x) v[x] = -CUDART_INF_F;
-        return;
-    }
-#pragma unroll
-    for (int x = 0; x < K; ++x) v[x] = hd_rel(d[x], mx);
-}
-
-// Variable-to-factor values of one K-state edge. Edges of high-degree variables
-// (edge_vs < 0) take the exact leave-one-out values from the variable's totals (hd_pair);
-// all others use b - m, or the explicit sum when an entry needs it.
-template <int K>
-__device__ __forceinline__ void gather_v2f(const DevGraph &G, const float *__restrict__ b,
-                                           const float *__restrict__ ev, const float *__restrict__ m_old,
-                                           int vs, int es, const float (&mo)[K], float (&v)[K]) {
-    if (vs < 0) {
-        hd_v2f<K>(G, vs, mo, v);
-        return;
-    }
-    bool exact = false;
-#pragma unroll
-    for (int x = 0; x < K; ++x) exact |= needs_exact(mo[x]);
-    if (exact) {
-        v2f_slow_edge(G, ev, m_old, vs, es, K, v);
-        return;
-    }
-    load_n<K>(v, b + vs);
-#pragma unroll
-    for (int x = 0; x < K; ++x) v[x] -= mo[x];
-}
-
-// ---- log-sum-exp helpers -------------------------------------------------------------
-
-
-// T > 0 logical factors: the closed forms chain several exp / log evaluations per edge;
-// in FP32 their rounding errors are biased, which long runs on logical-factor graphs
-// amplify. They are therefore evaluated in FP64 from the FP32 inputs (the outputs are
-// rounded once to FP32). Sums of softplus terms s(x_j / T) are kept as logarithms,
-// log A = LSE_j log s(x_j / T), so that very negative log-odds do not underflow.
-
-// log(s(u)), s(u) = log(1 + e^u)
-__device__ __forceinline__ double log_softplus_d(double u) {
-    if (u < -30.0) return u + log1p(-0.5 * exp(u));
-    if (u > 0.0) return log(u + log1p(exp(-u)));
-    return log(log1p(exp(u)));
-}
-
-__device__ __forceinline__ double lse2_d(double a, double b) {
-    const double mx = fmax(a, b);
-    if (mx == -CUDART_INF || mx == CUDART_INF) return mx;
-    return mx + log1p(exp(fmin(a, b) - mx));
-}
-
-// log(e^a - 1) from la = log a
-__device__ __forceinline__ double log_expm1_from_log_d(double la) {
-    if (la == -CUDART_INF) return -CUDART_INF;
-    if (la == CUDART_INF) return CUDART_INF;
-    if (la > 0.0) {
-        const double a = exp(la);
-        return a + log(-expm1(-a));
-    }
-    if (la > -700.0) {
-        const double a = exp(la);
-        return la + log(expm1(a) / a);
-    }
-    return la;
-}
-
-// -log(1 - e^{-a}) from la = log a
-__device__ __forceinline__ double neg_log_1mexp_from_log_d(double la) {
-    if (la == CUDART_INF) return 0.0;
-    if (la > 0.0) return -log(-expm1(-exp(la)));
-    if (la > -700.0) {
-        const double a = exp(la);
-        return -la - log(-expm1(-a) / a);
-    }
-    return -la;
-}
-
-// OR update to parent i (T > 0): la = log of the leave-one-out softplus sum (units of
-// T), xc = child log-odds.
-__device__ __forceinline__ float or_parent_soft(double la, float xc_f, double T) {
-    const double xc = xc_f;
-    if (la == -CUDART_INF) return xc_f;
-    const double y = xc + T * log_expm1_from_log_d(la);
-    if (y >= 0.0) return (float)(T * neg_log_1mexp_from_log_d(la) - T * log1p(exp(-y / T)));
-    return (float)(xc + T * exp(la) - T * log1p(exp(y / T)));
-}
-
-// OR update to parent i (T = 0): S = leave-one-out sum of max(x_j, 0), M = leave-one-out max.
-__device__ __forceinline__ float or_parent_max(float S, float M, float xc) {
-    float mn = M < 0.f ? M : 0.f;
-    float z = xc + S + mn;
-    return (z >= 0.f) ? -mn : xc + S;
-}
-
-// XOR (parity) factors: the parents and the child have even parity, and a member's
-// message depends on all the others alike. With log-odds a_j = x_j / T of the others,
-// the product rule of parity checks gives D = prod tanh(-a_j / 2) and the log-odds
-// T log((1 - D) / (1 + D)). The magnitude is carried as l_j = log u_j,
-// u_j = -log tanh(|a_j| / 2) = log1p(2 / expm1(|a_j|)) (log 2 - |a_j| beyond 30), and the
-// others' LSE lambda of the l_j gives log((1 - |D|) / (1 + |D|)) =
-// log(-expm1(-e^lambda)) - log1p(e^-e^lambda) (lambda - log 2 once e^lambda < 1e-9); the
-// sign is the parity of the others' positive log-odds. T = 0: the others' smallest |x|,
-// positive when an odd number of them is positive. FP64 at T > 0, as the OR / AND forms.
-__device__ __forceinline__ double xor_log_u(double a) {
-    a = fabs(a);
-    if (a == 0.0) return CUDART_INF;
-    if (isinf(a)) return -CUDART_INF;
-    if (a > 30.0) return 0.6931471805599453 - a;
-    return log(log1p(2.0 / expm1(a)));
-}
-
-// XOR output (T > 0) from the others' LSE lambda and their parity.
-__device__ __forceinline__ float xor_out_soft(double lam, bool odd, double T) {
-    double r;
-    if (lam == CUDART_INF) r = 0.0;
-    else if (lam == -CUDART_INF) r = -CUDART_INF;
-    else if (lam < -20.7) r = lam - 0.6931471805599453;
-    else {
-        const double u = exp(lam);
-        r = log(-expm1(-u)) - log1p(exp(-u));
-    }
-    return (float)(T * (odd ? -r : r));
-}
-
-__device__ __forceinline__ float xor_out_max(float mn, bool odd) { return odd ? mn : -mn; }
-
-__device__ __forceinline__ float log_odds(float a0, float a1) {
-    return (a0 == kNegInf && a1 == kNegInf) ? 0.f : a1 - a0;
-}
-
-// ---- message epilogue: normalise, damp, normalise ------------------------------------
-
-template <int K>
-__device__ __forceinline__ void normalise_k(float (&t)[K], uint32_t *flags) {
-    float mx = kNegInf;
-#pragma unroll
-    for (int x = 0; x < K; ++x)
-        if (t[x] > mx) mx = t[x];
-    if (mx == kNegInf) {
-#pragma unroll
-        for (int x = 0; x < K; ++x) t[x] = 0.f;
-        atomicOr(flags, kFlagContradiction);
-        return;
-    }
-#pragma unroll
-    for (int x = 0; x < K; ++x) t[x] -= mx;
-}
-
-template <int K>
-__device__ __forceinline__ void finish_k(float (&t)[K], const float (&mo)[K], float damping,
-                                         uint32_t *flags) {
-    normalise_k<K>(t, flags);
-    if (damping != 0.f) {
-        const float w = 1.f - damping;
-#pragma unroll
-        for (int x = 0; x < K; ++x) t[x] = damping * mo[x] + w * t[x];
-    }
-    normalise_k<K>(t, flags);
-}
-
-__device__ __forceinline__ void normalise_rt(float *t, int K, uint32_t *flags) {
-    float mx = kNegInf;
-    for (int x = 0; x < K; ++x)
-        if (t[x] > mx) mx = t[x];
-    if (mx == kNegInf) {
-        for (int x = 0; x < K; ++x) t[x] = 0.f;
-        atomicOr(flags, kFlagContradiction);
-        return;
-    }
-    for (int x = 0; x < K; ++x) t[x] -= mx;
-}
-
-// ---- LSE_T over a row of K values ---------------------------------------------------
-
-template <int K, bool MAXP>
-__device__ __forceinline__ float lse_row(const float (&z)[K], float T, float invT) {
-    float mx = kNegInf;
-#pragma unroll
-    for (int y = 0; y < K; ++y) mx = fmaxf(mx, z[y]);
-    if (MAXP || mx == kNegInf) return mx;
-    if constexpr (K == 2) {
-        // log(1 + e^-d), d >= 0, with the SFU exp2 / log2 (absolute error below 3e-7)
-        return mx + T * __logf(1.f + __expf((fminf(z[0], z[1]) - mx) * invT));
-    } else {
-        float s = 0.f;
-#pragma unroll
-        for (int y = 0; y < K; ++y) s += expf((z[y] - mx) * invT);
-        return mx + T * logf(s);
-    }
-}
-
 // =====================================================================================
 // Variable pass
 // =====================================================================================
-
-// Multi-sample launches (pgm_run_bp_multi on graphs without the joint log-ratio path;
-// the kernels' MS instantiations): gridDim.y samples share the index arrays; a block
-// works on sample blockIdx.y, whose
-// messages, beliefs, evidence and log-potentials lie at the DevGraph strides (0 for an
-// ordinary launch) and whose scratch (exact leave-one-out sums, belief residuals) is the
-// sample's slice.
-__device__ __forceinline__ int64_t sample_select(DevGraph &G) {
-    const int64_t smp = blockIdx.y;
-    if (smp != 0) {
-        if (G.hd_b) G.hd_b += smp * 4 * G.s_vs;
-        if (G.b_lo) G.b_lo += smp * G.s_vs;
-    }
-    return smp;
-}
 
 // Thread per variable (degree <= kVarBlockDegree). Sums are compensated (float-float)
 // in ascending edge order. KFIX = 2: every variable binary (states at 2v, edge-states
@@ -1078,28 +679,6 @@ __global__ void __launch_bounds__(kVarBlockThreads) k_var_hd(DevGraph G, const i
 // Factor pass: dense pairwise tables (Ising, RBM, Potts), thread per factor
 // =====================================================================================
 
-// A batch member whose early exit has frozen it: the factor pass leaves its messages
-// alone (a block, or a chunk of the persistent kernel, lies in one member's group).
-__device__ __forceinline__ bool member_frozen(const DevGraph &G, int member) {
-    return G.frozen != nullptr && __ldg(G.frozen + member) != 0;
-}
-
-// A batch run with parameters per member (pgm_run_bp_batch): the member's T, 1 / T and
-// damping replace the launch's, and the launch of the other kind (max-product or not)
-// skips it. Also true for a frozen member.
-template <bool MAXP>
-__device__ __forceinline__ bool member_skip(const DevGraph &G, int member, float &T, float &invT, float &damping) {
-    if (member_frozen(G, member)) return true;
-    if (G.mem_prm != nullptr) {
-        const float4 p = __ldg(reinterpret_cast<const float4 *>(G.mem_prm) + member);
-        if ((p.x == 0.f) != MAXP) return true;
-        T = p.x;
-        invT = p.y;
-        damping = p.z;
-    }
-    return false;
-}
-
 // The factor-to-variable update of one dense pairwise factor from its two
 // variable-to-factor vectors v0, v1 and stored messages mo0, mo1; writes the damped,
 // normalised messages.
@@ -1559,60 +1138,12 @@ k_pair_group(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, int n_vblo
 
 // ---- K-state pairwise tables, thread per factor ------------------------------------
 
-// One direction of a K-state pairwise factor, thread-local: o(x) = LSE_T (or max) over y
-// of phi(x, y) + v(y) for the message to variable 0 (TR = false, rows of phi), or of
-// phi(y, x) + v(y) for the message to variable 1 (TR = true, columns). Linear form for a
-// shared table with E = exp((phi - tmax) / T) (tabE row-major E, tabET row-major E^T):
-// o(x) = T log(sum_y E(x, y) w(y)) + vmax + tmax with w(y) = exp((v(y) - vmax) / T), the
-// rows read as float4 (every thread of the block reads the same row: a broadcast).
-template <int K, bool MAXP, bool TR>
-__device__ __forceinline__ void pair_dir_thr(float (&v)[K], float (&o)[K], bool linear, const float *tabE,
-                                             const float *phi, bool phi_shared, float tmax, float T,
-                                             float invT) {
-    if (!MAXP && linear) {
-        float vmax = kNegInf;
-#pragma unroll
-        for (int y = 0; y < K; ++y) vmax = fmaxf(vmax, v[y]);
-        if (vmax == kNegInf) {
-#pragma unroll
-            for (int x = 0; x < K; ++x) o[x] = kNegInf;
-            return;
-        }
-#pragma unroll
-        for (int y = 0; y < K; ++y) v[y] = __expf((v[y] - vmax) * invT);  // w(y), in (0, 1]
-#pragma unroll
-        for (int x = 0; x < K; ++x) {
-            const float4 *row = reinterpret_cast<const float4 *>(tabE + x * K);
-            float s = 0.f;
-#pragma unroll
-            for (int j = 0; j < K / 4; ++j) {
-                const float4 a = row[j];
-                s = fmaf(a.x, v[4 * j], fmaf(a.y, v[4 * j + 1], fmaf(a.z, v[4 * j + 2], fmaf(a.w, v[4 * j + 3], s))));
-            }
-            o[x] = T * logf(s) + vmax + tmax;
-        }
-    } else {
-#pragma unroll
-        for (int x = 0; x < K; ++x) {
-            float z[K];
-#pragma unroll
-            for (int y = 0; y < K; ++y) {
-                const int i = TR ? y * K + x : x * K + y;
-                z[y] = (phi_shared ? phi[i] : __ldg(phi + i)) + v[y];
-            }
-            o[x] = lse_row<K, MAXP>(z, T, invT);
-        }
-    }
-}
-
-// Dense K-state pairwise tables (Potts, K = 4, 8, 16), thread per factor: the thread
-// keeps the factor's two stored messages and one variable-to-factor vector in registers
-// and forms the K x K table product itself, one direction at a time (no cross-lane
-// traffic, so the per-factor work is the product's K^2 multiply-adds plus 2K
-// exponentials and logarithms per direction). Shared tables are staged per block in
-// shared memory (with E and E^T for the linear form); per-factor tables are read from
-// the factor's own K*K entries. The rare cases (an edge of a high-degree variable, a
-// stored entry that is -inf or large) go to pair_factor_rare.
+// Dense K-state pairwise tables (Potts, K = 4, 8, 16), thread per factor, one direction at a
+// time (pair_math.cuh), for graphs that the fused form (pair_fused.cu) does not take: variables
+// with more than 4 factors or factors of several groups. Shared tables are staged per block in
+// shared memory; per-factor tables are read from the factor's own K*K entries. A source edge
+// that is a high-degree variable's or has a stored entry that is -inf or large goes to
+// pair_dir_rare.
 template <int K, bool MAXP, bool MS = false>
 __global__ void __launch_bounds__(K >= 16 ? 128 : 256)
 k_pair_thr(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float *__restrict__ pot,
@@ -1629,55 +1160,37 @@ k_pair_thr(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float 
         m_new += smp * G.s_es;
     }
     __shared__ float tab[K * K];
-    __shared__ __align__(16) float tabE[MAXP ? 4 : K * K];
-    __shared__ __align__(16) float tabET[MAXP ? 4 : K * K];
-    __shared__ float tinfo[2];
+    __shared__ __align__(16) float S0[K * K], S1[K * K];
+    __shared__ float red[16];
     const EnumSeg *S = segs + find_seg(segs, n_seg, blockIdx.x);
     if (member_skip<MAXP>(G, S->member, T, invT, damping)) return;  // the whole block
     const int n_fac = __ldg(&S->n_fac), shared = __ldg(&S->shared), pot_base = __ldg(&S->pot_base);
-    bool linear = false;
-    if (shared) {  // uniform over the block (a block lies in one segment)
-        for (int i = threadIdx.x; i < K * K; i += blockDim.x) tab[i] = __ldg(pot + pot_base + i);
-        __syncthreads();
-        linear = prepare_linear_table<K, MAXP>(tab, tabE, tinfo, invT);
-        if (linear) {
-            for (int i = threadIdx.x; i < K * K; i += blockDim.x) tabET[(i % K) * K + i / K] = tabE[i];
-            __syncthreads();
-        }
-    }
+    const bool linear = shared && pair_tables<K, MAXP>(pot + pot_base, tab, S0, S1, red, invT);  // uniform over the block
     const int f = (blockIdx.x - __ldg(&S->block_begin)) * blockDim.x + threadIdx.x;
     if (f >= n_fac) return;
     const int e = __ldg(&S->edge_base) + 2 * f;
     const int es0 = __ldg(&S->es_base) + 2 * K * f, es1 = es0 + K;
     const int vs0 = __ldg(G.edge_vs + e), vs1 = __ldg(G.edge_vs + e + 1);
     const float *phi = shared ? tab : pot + pot_base + (size_t)f * (K * K);
-    const float tmax = linear ? tinfo[0] : 0.f;
-    float mo0[K], mo1[K];
-    load_n_stream<K>(mo0, m_old + es0);
-    load_n_stream<K>(mo1, m_old + es1);
-    bool rare = (vs0 < 0) | (vs1 < 0);
+#pragma unroll 1
+    for (int side = 1; side >= 0; --side) {  // the source edge: variable 1's, then variable 0's
+        const int vs = side ? vs1 : vs0, es = side ? es1 : es0, es_t = side ? es0 : es1;
+        const int step_s = side ? 1 : K, step_t = side ? K : 1;
+        F2 v[K / 2], b2[K / 2];
+        f2_load<K>(v, m_old + es);
+        if (vs < 0 || f2_needs_exact<K>(v)) {
+            pair_dir_rare<K, MAXP>(G, phi, step_s, step_t, b, ev, m_old, m_new, vs, es, es_t, T, invT, damping);
+            continue;
+        }
+        f2_load<K>(b2, b + vs);
 #pragma unroll
-    for (int x = 0; x < K; ++x) rare |= needs_exact(mo0[x]) | needs_exact(mo1[x]);
-    if (rare) {
-        pair_factor_rare<K, MAXP>(G, shared ? tab : nullptr, pot + pot_base + (size_t)f * (K * K), b, ev, m_old,
-                                  m_new, vs0, vs1, es0, es1, T, invT, damping);
-        return;
+        for (int i = 0; i < K / 2; ++i) {
+            const float2 m = f2_get(v[i]);
+            v[i] = f2_add(b2[i], f2(-m.x, -m.y));
+        }
+        pair_direction<K, MAXP>(v, linear, shared, side ? S1 : S0, phi, step_s, step_t, m_old, m_new, es_t, T, invT,
+                                damping, G.flags);
     }
-    float v[K], o[K];
-    // to variable 0: rows of phi against v1 = b1 - m1
-    load_n<K>(v, b + vs1);
-#pragma unroll
-    for (int y = 0; y < K; ++y) v[y] -= mo1[y];
-    pair_dir_thr<K, MAXP, false>(v, o, linear, tabE, phi, shared, tmax, T, invT);
-    finish_k<K>(o, mo0, damping, G.flags);
-    store_n<K>(m_new + es0, o);
-    // to variable 1: columns of phi against v0 = b0 - m0
-    load_n<K>(v, b + vs0);
-#pragma unroll
-    for (int y = 0; y < K; ++y) v[y] -= mo0[y];
-    pair_dir_thr<K, MAXP, true>(v, o, linear, tabET, phi, shared, tmax, T, invT);
-    finish_k<K>(o, mo1, damping, G.flags);
-    store_n<K>(m_new + es1, o);
 }
 
 // ---- K-state pairwise tables, a thread per factor and direction ------------------------
@@ -1689,9 +1202,7 @@ k_pair_thr(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float 
 // one input vector, one output and one old message (3K values instead of the thread
 // form's 4K plus a second output) and twice as many factors are in flight per SM at the
 // same arithmetic per factor. Each thread runs the thread form's direction code on the
-// same inputs, so both forms give the same bits; a factor with a rare case (an edge of a
-// high-degree variable, a stored entry that is -inf or large) is finished whole by the
-// even warp's thread through pair_factor_rare, as in the thread form.
+// same inputs, so both forms give the same bits.
 template <int K, bool MAXP, bool MS = false>
 __global__ void __launch_bounds__(256, K >= 16 ? 3 : 5)
 k_pair_dir(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float *__restrict__ pot,
@@ -1708,54 +1219,34 @@ k_pair_dir(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float 
         m_new += smp * G.s_es;
     }
     __shared__ float tab[K * K];
-    __shared__ __align__(16) float tabE[MAXP ? 4 : K * K];
-    __shared__ __align__(16) float tabET[MAXP ? 4 : K * K];
-    __shared__ float tinfo[2];
+    __shared__ __align__(16) float S0[K * K], S1[K * K];
+    __shared__ float red[16];
     const EnumSeg *S = segs + find_seg(segs, n_seg, blockIdx.x);
     if (member_skip<MAXP>(G, S->member, T, invT, damping)) return;  // the whole block
     const int n_fac = __ldg(&S->n_fac), shared = __ldg(&S->shared), pot_base = __ldg(&S->pot_base);
-    bool linear = false;
-    if (shared) {  // uniform over the block (a block lies in one segment)
-        for (int i = threadIdx.x; i < K * K; i += blockDim.x) tab[i] = __ldg(pot + pot_base + i);
-        __syncthreads();
-        linear = prepare_linear_table<K, MAXP>(tab, tabE, tinfo, invT);
-        if (linear) {
-            for (int i = threadIdx.x; i < K * K; i += blockDim.x) tabET[(i % K) * K + i / K] = tabE[i];
-            __syncthreads();
-        }
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d = warp & 1;  // d: warp-uniform
+    const bool linear = shared && pair_tables<K, MAXP>(pot + pot_base, tab, S0, S1, red, invT);  // uniform over the block
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, side = 1 - (warp & 1);  // the source edge's, warp-uniform
     const int f = (blockIdx.x - __ldg(&S->block_begin)) * (blockDim.x >> 1) + (warp >> 1) * 32 + lane;
     if (f >= n_fac) return;
     const int e = __ldg(&S->edge_base) + 2 * f;
-    const int es0 = __ldg(&S->es_base) + 2 * K * f, es1 = es0 + K;
-    const int vs0 = __ldg(G.edge_vs + e), vs1 = __ldg(G.edge_vs + e + 1);
+    const int es0 = __ldg(&S->es_base) + 2 * K * f;
+    const int vs = __ldg(G.edge_vs + e + side), es = es0 + side * K, es_t = es0 + (1 - side) * K;
     const float *phi = shared ? tab : pot + pot_base + (size_t)f * (K * K);
-    // this thread's output edge (target) and input edge (source)
-    const int es_t = d ? es1 : es0, es_s = d ? es0 : es1, vs_s = d ? vs0 : vs1;
-    float mo_t[K], v[K];
-    load_n<K>(mo_t, m_old + es_t);
-    load_n<K>(v, m_old + es_s);
-    bool rare = (vs0 < 0) | (vs1 < 0);
-#pragma unroll
-    for (int x = 0; x < K; ++x) rare |= needs_exact(mo_t[x]) | needs_exact(v[x]);
-    if (rare) {  // both warps see the same rare flag; the even one finishes the factor
-        if (d == 0)
-            pair_factor_rare<K, MAXP>(G, shared ? tab : nullptr, pot + pot_base + (size_t)f * (K * K), b, ev, m_old,
-                                      m_new, vs0, vs1, es0, es1, T, invT, damping);
+    const int step_s = side ? 1 : K, step_t = side ? K : 1;
+    F2 v[K / 2], b2[K / 2];
+    f2_load<K>(v, m_old + es);
+    if (vs < 0 || f2_needs_exact<K>(v)) {
+        pair_dir_rare<K, MAXP>(G, phi, step_s, step_t, b, ev, m_old, m_new, vs, es, es_t, T, invT, damping);
         return;
     }
-    const float tmax = linear ? tinfo[0] : 0.f;
-    float bs[K], o[K];
-    load_n<K>(bs, b + vs_s);
+    f2_load<K>(b2, b + vs);
 #pragma unroll
-    for (int y = 0; y < K; ++y) v[y] = bs[y] - v[y];
-    if (d == 0)  // to variable 0: rows of phi against v1
-        pair_dir_thr<K, MAXP, false>(v, o, linear, tabE, phi, shared, tmax, T, invT);
-    else  // to variable 1: columns of phi against v0
-        pair_dir_thr<K, MAXP, true>(v, o, linear, tabET, phi, shared, tmax, T, invT);
-    finish_k<K>(o, mo_t, damping, G.flags);
-    store_n<K>(m_new + es_t, o);
+    for (int i = 0; i < K / 2; ++i) {
+        const float2 m = f2_get(v[i]);
+        v[i] = f2_add(b2[i], f2(-m.x, -m.y));
+    }
+    pair_direction<K, MAXP>(v, linear, shared, side ? S1 : S0, phi, step_s, step_t, m_old, m_new, es_t, T, invT, damping,
+                            G.flags);
 }
 
 // ---- K / 4 lanes per factor, four consecutive states each (K = 8, 16, shared tables) ----
@@ -1769,8 +1260,8 @@ k_pair_dir(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float 
 // lanes with a quarter of its registers, so four times as many factors are in flight per
 // SM. The arithmetic is the thread form's, term for term and in the same order (the
 // table rows in the same float4 chunks, the maxima exact), so both forms give the same
-// bits. The rare cases (an edge of a high-degree variable, a stored entry that is -inf
-// or large) go to pair_factor_rare on the group's first lane.
+// bits. A message whose source edge is rare (a high-degree variable's, or with a stored entry
+// that is -inf or large) goes to pair_dir_rare on the group's first lane.
 
 // Shared tables of the K / 4-lane form: row x of a K x K table holds its 16-byte chunk j
 // at chunk slot j ^ ((x >> 2) & (K / 4 - 1)), so that the group's lanes, reading rows
@@ -1840,20 +1331,21 @@ __device__ __forceinline__ void quad_normalise(float4 &t, uint32_t *flags, bool 
 // four states) against the rows of `rows` (a padded K x K table: E or E^T for the linear
 // form, phi or phi^T otherwise). xs is the group's exchange slot (K floats).
 template <int K, bool MAXP>
-__device__ __forceinline__ float4 quad_dir(float4 v, bool linear, const float *rows, float *xs, int q, float tmax,
-                                          float T, float invT) {
+__device__ __forceinline__ float4 quad_dir(float4 v, bool linear, const float *rows, float *xs, int q, float T,
+                                          float invT) {
     constexpr int L = K / 4;
     float4 o;
     if (!MAXP && linear) {
         const float vm = quad_max<L>(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
-        // all -inf: w = 0 and every output -inf, as in the thread form
+        // all -inf: w = 0 and every output -inf, as in the thread form (pair_weights)
         const float vmax = vm;
         float4 w;
         if (vmax == kNegInf) {
             w = make_float4(0.f, 0.f, 0.f, 0.f);
         } else {
-            w = make_float4(__expf((v.x - vmax) * invT), __expf((v.y - vmax) * invT), __expf((v.z - vmax) * invT),
-                            __expf((v.w - vmax) * invT));
+            const float c = invT * 1.4426950408889634f, n = -vmax * c;
+            w = make_float4(ex2_ftz(fmaf(v.x, c, n)), ex2_ftz(fmaf(v.y, c, n)), ex2_ftz(fmaf(v.z, c, n)),
+                            ex2_ftz(fmaf(v.w, c, n)));
         }
         reinterpret_cast<float4 *>(xs)[q] = w;
         __syncwarp();
@@ -1869,15 +1361,18 @@ __device__ __forceinline__ float4 quad_dir(float4 v, bool linear, const float *r
         for (int i = 0; i < 4; ++i) {
             const int x = 4 * q + i, sw = (x >> 2) & (K / 4 - 1);
             const float4 *row = reinterpret_cast<const float4 *>(rows + x * K);
-            float s = 0.f;
+            float se = 0.f, so = 0.f;  // even and odd sources, as pair_linear
 #pragma unroll
             for (int j = 0; j < K / 4; ++j) {
                 const float4 a = row[j ^ sw];  // chunk j of the row
-                s = fmaf(a.x, wa[4 * j], fmaf(a.y, wa[4 * j + 1], fmaf(a.z, wa[4 * j + 2], fmaf(a.w, wa[4 * j + 3], s))));
+                se = fmaf(a.z, wa[4 * j + 2], fmaf(a.x, wa[4 * j], se));
+                so = fmaf(a.w, wa[4 * j + 3], fmaf(a.y, wa[4 * j + 1], so));
             }
-            out[i] = vmax == kNegInf ? kNegInf : T * logf(s) + vmax + tmax;
+            out[i] = se + so;
         }
-        o = make_float4(out[0], out[1], out[2], out[3]);
+        const F2 T2 = f2(T, T);
+        const float2 oa = f2_get(f2_mul(T2, f2_log(f2(out[0], out[1])))), ob = f2_get(f2_mul(T2, f2_log(f2(out[2], out[3]))));
+        o = vmax == kNegInf ? make_float4(kNegInf, kNegInf, kNegInf, kNegInf) : make_float4(oa.x, oa.y, ob.x, ob.y);
     } else {
         reinterpret_cast<float4 *>(xs)[q] = v;
         __syncwarp();
@@ -1952,7 +1447,6 @@ k_pair_quad(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float
         }
         __syncthreads();
     }
-    const float tmax = linear ? tinfo[0] : 0.f;
     const int q = threadIdx.x & (L - 1);
     const int fi = (blockIdx.x - __ldg(&S->block_begin)) * (blockDim.x / L) + (threadIdx.x / L);
     const bool valid = fi < n_fac;
@@ -1962,39 +1456,44 @@ k_pair_quad(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float
     const int vs0 = __ldg(G.edge_vs + e), vs1 = __ldg(G.edge_vs + e + 1);
     const float4 mo0 = ld4(m_old + es0 + 4 * q, true);
     const float4 mo1 = ld4(m_old + es1 + 4 * q, true);
-    const bool rare_lane = (vs0 < 0) | (vs1 < 0) | needs_exact(mo0.x) | needs_exact(mo0.y) | needs_exact(mo0.z) |
-                           needs_exact(mo0.w) | needs_exact(mo1.x) | needs_exact(mo1.y) | needs_exact(mo1.z) |
-                           needs_exact(mo1.w);
+    // whether each message's source edge is rare (pair_dir_rare)
+    const bool rare_lane0 = (vs1 < 0) | needs_exact(mo1.x) | needs_exact(mo1.y) | needs_exact(mo1.z) | needs_exact(mo1.w);
+    const bool rare_lane1 = (vs0 < 0) | needs_exact(mo0.x) | needs_exact(mo0.y) | needs_exact(mo0.z) | needs_exact(mo0.w);
     const unsigned lane = threadIdx.x & 31;
     const unsigned gbits = ((1u << L) - 1u) << (lane & ~(unsigned)(L - 1));
-    const bool rare = (__ballot_sync(0xffffffffu, rare_lane) & gbits) != 0u;
+    const bool rare0 = (__ballot_sync(0xffffffffu, rare_lane0) & gbits) != 0u;
+    const bool rare1 = (__ballot_sync(0xffffffffu, rare_lane1) & gbits) != 0u;
     float *xs = xchg + (threadIdx.x & ~(L - 1)) * 4;
     // the common path runs on every lane (the exchanges are warp-synchronous); a rare
     // group's results are discarded
     const float4 b1 = ld4(b + max(vs1, 0) + 4 * q, false);
     float4 v = make_float4(b1.x - mo1.x, b1.y - mo1.y, b1.z - mo1.z, b1.w - mo1.w);
-    float4 o0 = quad_dir<K, MAXP>(v, linear, rows0, xs, q, tmax, T, invT);
+    float4 o0 = quad_dir<K, MAXP>(v, linear, rows0, xs, q, T, invT);
     const float4 b0 = ld4(b + max(vs0, 0) + 4 * q, false);
     v = make_float4(b0.x - mo0.x, b0.y - mo0.y, b0.z - mo0.z, b0.w - mo0.w);
-    float4 o1 = quad_dir<K, MAXP>(v, linear, rows1, xs, q, tmax, T, invT);
-    const bool lead = q == 0 && valid && !rare;
-    quad_normalise<L>(o0, G.flags, lead);
-    quad_normalise<L>(o1, G.flags, lead);
+    float4 o1 = quad_dir<K, MAXP>(v, linear, rows1, xs, q, T, invT);
+    const bool lead0 = q == 0 && valid && !rare0, lead1 = q == 0 && valid && !rare1;
+    if (MAXP || !linear) {  // (as pair_finish)
+        quad_normalise<L>(o0, G.flags, lead0);
+        quad_normalise<L>(o1, G.flags, lead1);
+    }
     if (damping != 0.f) {
         const float w = 1.f - damping;
-        o0 = make_float4(damping * mo0.x + w * o0.x, damping * mo0.y + w * o0.y, damping * mo0.z + w * o0.z,
-                         damping * mo0.w + w * o0.w);
-        o1 = make_float4(damping * mo1.x + w * o1.x, damping * mo1.y + w * o1.y, damping * mo1.z + w * o1.z,
-                         damping * mo1.w + w * o1.w);
+        o0 = make_float4(fmaf(damping, mo0.x, w * o0.x), fmaf(damping, mo0.y, w * o0.y), fmaf(damping, mo0.z, w * o0.z),
+                         fmaf(damping, mo0.w, w * o0.w));
+        o1 = make_float4(fmaf(damping, mo1.x, w * o1.x), fmaf(damping, mo1.y, w * o1.y), fmaf(damping, mo1.z, w * o1.z),
+                         fmaf(damping, mo1.w, w * o1.w));
     }
-    quad_normalise<L>(o0, G.flags, lead);
-    quad_normalise<L>(o1, G.flags, lead);
-    if (valid && !rare) {
-        st4(m_new + es0 + 4 * q, o0);
-        st4(m_new + es1 + 4 * q, o1);
+    quad_normalise<L>(o0, G.flags, lead0);
+    quad_normalise<L>(o1, G.flags, lead1);
+    if (valid && !rare0) st4(m_new + es0 + 4 * q, o0);
+    if (valid && !rare1) st4(m_new + es1 + 4 * q, o1);
+    if (valid && q == 0) {
+        if (rare0)
+            pair_dir_rare<K, MAXP>(G, tab, 1, K, b, ev, m_old, m_new, vs1, es1, es0, T, invT, damping);
+        if (rare1)
+            pair_dir_rare<K, MAXP>(G, tab, K, 1, b, ev, m_old, m_new, vs0, es0, es1, T, invT, damping);
     }
-    if (valid && rare && q == 0)
-        pair_factor_rare<K, MAXP>(G, tab, pot + pot_base, b, ev, m_old, m_new, vs0, vs1, es0, es1, T, invT, damping);
 }
 
 // =====================================================================================
@@ -4231,7 +3730,7 @@ static void launch_dep(void (*kernel)(KArgs...), dim3 grid, int threads, size_t 
 
 template <int MODE, bool MS>
 static void var_pass_mode(const DevGraph &G, const Plan &P, const float *ev, const float *m,
-                          float *out, int32_t *dec, cudaStream_t s, int S, const LaunchHook *hook) {
+                          float *out, int32_t *dec, cudaStream_t s, int S, const LaunchHook *hook, bool full) {
     if (G.vin_tab4 != nullptr) {
         const int n = G.V;
         k_var_tab4<MODE, MS><<<dim3((n + 255) / 256, S), 256, 0, s>>>(G, n, ev, m, out, dec);
@@ -4240,6 +3739,12 @@ static void var_pass_mode(const DevGraph &G, const Plan &P, const float *ev, con
     }
     for (const VarLaunch &L : P.var) {
         if (L.n == 0) continue;
+        const bool fused = MODE == kVarIter && !full && L.fused_by >= 0 && L.fused_by < (int)P.factor.size() &&
+                           is_fused(P.factor[L.fused_by].variant);
+        if (fused) {  // done by the factor launch (its place in the launch times stays, empty)
+            if (hook) hook->after(hook->ctx);
+            continue;
+        }
         switch (L.kind) {
             case kVarBlock:  // single-sample launches: a block per tile; else a block per variable
                 if (!MS && S == 1 && L.tiles != nullptr && G.hd_tot != nullptr && G.hd_cnt != nullptr)
@@ -4271,12 +3776,13 @@ static void var_pass_mode(const DevGraph &G, const Plan &P, const float *ev, con
 }
 
 cudaError_t launch_var_pass(const DevGraph &G, const Plan &P, const float *ev, const float *m,
-                            float *b, int mode, int32_t *decode, cudaStream_t s, int S, const LaunchHook *hook) {
-    if (mode == kVarIter && S > 1) var_pass_mode<kVarIter, true>(G, P, ev, m, b, decode, s, S, hook);
-    else if (mode == kVarIter) var_pass_mode<kVarIter, false>(G, P, ev, m, b, decode, s, 1, hook);
-    else if (mode == kVarBeliefs) var_pass_mode<kVarBeliefs, false>(G, P, ev, m, b, decode, s, 1, hook);
-    else if (mode == kVarNormalised) var_pass_mode<kVarNormalised, false>(G, P, ev, m, b, decode, s, 1, hook);
-    else var_pass_mode<kVarDecode, false>(G, P, ev, m, b, decode, s, 1, hook);
+                            float *b, int mode, int32_t *decode, cudaStream_t s, int S, const LaunchHook *hook,
+                            bool full) {
+    if (mode == kVarIter && S > 1) var_pass_mode<kVarIter, true>(G, P, ev, m, b, decode, s, S, hook, full);
+    else if (mode == kVarIter) var_pass_mode<kVarIter, false>(G, P, ev, m, b, decode, s, 1, hook, full);
+    else if (mode == kVarBeliefs) var_pass_mode<kVarBeliefs, false>(G, P, ev, m, b, decode, s, 1, hook, full);
+    else if (mode == kVarNormalised) var_pass_mode<kVarNormalised, false>(G, P, ev, m, b, decode, s, 1, hook, full);
+    else var_pass_mode<kVarDecode, false>(G, P, ev, m, b, decode, s, 1, hook, full);
     return cudaGetLastError();
 }
 
@@ -4319,6 +3825,11 @@ static void factor_pass_t(const DevGraph &G, const Plan &P, const float *pot, co
                 break;
             case kPairD16:
                 launch_dep(k_pair_dir<16, MAXP, MS>, dim3(dim3(L.n_blocks, S)), L.threads, 0, s, G, es, L.n_seg, pot, b, ev, m_old, m_new, T, invT, damping);
+                break;
+            case kPairF4:
+            case kPairF8:
+            case kPairF16:
+                launch_pair_fused(G, L, pot, ev, m_old, m_new, T, damping, S, s);
                 break;
             case kPairQ8:
                 launch_dep(k_pair_quad<8, MAXP, MS>, dim3(dim3(L.n_blocks, S)), L.threads, 0, s, G, es, L.n_seg, pot, b, ev, m_old, m_new, T, invT, damping);

@@ -1,0 +1,423 @@
+// Variable pass and factor pass of dense K-state pairwise groups (K = 4, 8, 16) in one kernel,
+// for variables with at most 4 factors, all of one group (grids, chains, lattices).
+//
+// Method: one flooding iteration of PGMax's damped updates (arXiv 2202.04110, Sec. 3; dense
+// pairwise enumeration factors, Sec. 5.2). A message from factor to variable depends on one
+// variable-to-factor value, so an iteration can be computed source by source: the lanes of a
+// variable sum its beliefs (the arithmetic of k_var_group) and then form the message that
+// leaves each of its edges (the arithmetic of pair_direction, lane by lane), so the messages
+// are bitwise those of the two passes.
+//
+// Why: the two passes moved 18 K floats per variable and iteration, 13 K here (the beliefs stay
+// in registers), and paid two launch boundaries. What bounded the factor pass was not its
+// arithmetic but the L1: a thread that loads its own 4 K-byte rows touches 32 lines with every
+// 16-byte load of a warp, one line per cycle, and reads the whole table for every message.
+// Here K / 4 lanes share a variable, four states each: a warp's load covers whole rows, and a
+// lane reads the four targets' part of the table, once for two edges of the same side. The next
+// launch's blocks load their indices and table while this one ends (programmatic launch).
+// Measured against the two passes it replaces (GB300, T = 1): a 181 x 181 grid of K = 16, whole
+// calls of 100 iterations 1.79 -> 0.88 ms (8.8 us per iteration); per launch on 128 uneven
+// grids K = 16 (662,000 variables) 60 + 222 -> 168 us, K = 8 (800,000) 43 + 88 -> 100, K = 4
+// (672,000) 28 + 46 -> 48. What bounds it now: issue slots (half of them) and the chain index ->
+// messages -> weights -> targets of a round; more resident blocks win against fewer spills
+// (K = 16: 2, 3, 4 blocks per SM 232, 183, 171 us), more rounds per block lose.
+#include <cstdint>
+
+#include "pair_math.cuh"
+
+namespace pgm {
+namespace {
+
+constexpr int kThreads = 256;
+
+template <int L>
+__device__ __forceinline__ float team_max(float v) {
+#pragma unroll
+    for (int d = L / 2; d > 0; d >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, d, L));
+    return v;
+}
+// Subtracts the team's maximum and returns it.
+template <int L>
+__device__ __forceinline__ float team_normalise(F2 (&t)[2]) {
+    const float mx = team_max<L>(f2_max<4>(t));
+    const F2 n = f2(-mx, -mx);
+    t[0] = f2_add(t[0], n);
+    t[1] = f2_add(t[1], n);
+    return mx;
+}
+// Four floats; AL: 16-byte aligned.
+template <bool AL>
+__device__ __forceinline__ void row_load(float (&d)[4], const float *p) {
+    if constexpr (AL) {
+        const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
+        d[0] = q.x, d[1] = q.y, d[2] = q.z, d[3] = q.w;
+    } else {
+        load_n<4>(d, p);
+    }
+}
+
+// One outgoing edge by one thread, with the beliefs formed here: a sum-product table of range
+// above 60 T, entry by entry, and the guarded arithmetic (pair_dir_rare). tab: the table.
+template <int K, bool MAXP>
+__device__ __noinline__ void fused_edge(const DevGraph &G, const float *tab, const float *ev, const float *m_old,
+                                        float *m_new, int v, int i, int es_base, float T, float invT, float damping) {
+    const int k0 = G.vin_off[v], k1 = G.vin_off[v + 1], vs = G.vs_off[v];
+    const int es = G.vin_es[k0 + i], side = ((es - es_base) / K) & 1, es_t = side ? es - K : es + K;
+    float m[K], x[K], o[K];
+    load_n<K>(m, m_old + es);
+    bool odd = false;
+    for (int y = 0; y < K; ++y) odd |= needs_exact(m[y]);
+    if (odd) {
+        pair_dir_rare<K, MAXP>(G, tab, side ? 1 : K, side ? K : 1, nullptr, ev, m_old, m_new, vs, es, es_t, T, invT, damping);
+        return;
+    }
+    FF s[K];
+    float mx = kNegInf;
+    int arg = 0;
+    for (int y = 0; y < K; ++y) {
+        s[y] = ff_make(ev[vs + y]);
+        for (int k = k0; k < k1; ++k) s[y] = ff_add(s[y], m_old[G.vin_es[k] + y]);
+        if (s[y].hi + s[y].lo > mx) {
+            mx = s[y].hi + s[y].lo;
+            arg = y;
+        }
+    }
+    const FF best = s[arg];
+    for (int y = 0; y < K; ++y)
+        x[y] = (best.hi == kNegInf ? kNegInf : y == arg ? 0.f : ff_diff(s[y], best)) - m[y];
+    pair_entries<K, MAXP>(x, o, tab, side ? 1 : K, side ? K : 1, T, invT);
+    F2 o2[K / 2], m2[K / 2];
+#pragma unroll
+    for (int y = 0; y < K / 2; ++y) o2[y] = f2(o[2 * y], o[2 * y + 1]);
+    f2_load<K>(m2, m_old + es_t);
+    pair_finish<K>(o2, m2, damping, G.flags);
+    f2_store<K>(m_new + es_t, o2);
+}
+
+// A team's variable: its incoming edges (es_base where there is none) and their number.
+struct TeamVar {
+    int v, deg, es[4];
+};
+__device__ __forceinline__ TeamVar team_var(const DevGraph &G, const int32_t *list, int pos, bool valid, int es_base) {
+    TeamVar t;
+    t.v = list ? __ldg(list + pos) : pos;
+    const int k0 = __ldg(G.vin_off + t.v);
+    t.deg = valid ? __ldg(G.vin_off + t.v + 1) - k0 : 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t.es[i] = i < t.deg ? __ldg(G.vin_es + k0 + i) : es_base;
+    return t;
+}
+
+// The four states of lane l (of a team of K / 4): the beliefs' sums s + evidence and the stored
+// messages q, then the message that leaves each edge. Returns the edges (bit i, the same for
+// the whole team) that fused_edge has to take: stored entries that are -inf, large or NaN, or
+// a maximum of -inf on the way (contradictions and their flags are left to it).
+template <int K, bool MAXP, bool AL>
+__device__ __forceinline__ unsigned team_edges(const TeamVar &t, const float (&e4)[4], const float (&q)[4][4], int l,
+                                               int es_base, const float *S0, const float *S1, float *xs, int xs_step,
+                                               const float *m_old, float *m_new, float T, float invT, float damping) {
+    constexpr int L = K / 4;
+    const F2 minus1 = f2(-1.f, -1.f);
+    F2 qa[4], qb[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        qa[i] = f2(q[i][0], q[i][1]);
+        qb[i] = f2(q[i][2], q[i][3]);
+    }
+    // beliefs relative to the variable's best state (k_var_group, kVarIter): ff_add on two
+    // states at a time; a sum that is not finite has lo = 0, set once at the end
+    F2 b[2];
+    {
+        F2 hi[2] = {f2(e4[0], e4[1]), f2(e4[2], e4[3])}, lo[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const F2 v = h ? qb[i] : qa[i];
+                const F2 s = f2_add(hi[h], v), bp = f2_fma(hi[h], minus1, s);
+                const F2 ea = f2_fma(f2_fma(bp, minus1, s), minus1, hi[h]), eb = f2_fma(bp, minus1, v);
+                lo[h] = f2_add(lo[h], f2_add(ea, eb));
+                hi[h] = s;
+            }
+        float sh[4], sl[4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 x = f2_get(hi[h]), y = f2_get(lo[h]);
+            sh[2 * h] = x.x;
+            sh[2 * h + 1] = x.y;
+            sl[2 * h] = isfinite(x.x) ? y.x : 0.f;
+            sl[2 * h + 1] = isfinite(x.y) ? y.y : 0.f;
+        }
+        // the best state: the largest rounded sum, lowest state on ties; its sum comes along
+        float lmx = kNegInf, bh = sh[0], bl = sl[0];
+        int larg = 4 * l;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const float rs = sh[x] + sl[x];
+            if (rs > lmx) {
+                lmx = rs;
+                larg = 4 * l + x;
+                bh = sh[x];
+                bl = sl[x];
+            }
+        }
+#pragma unroll
+        for (int d = L / 2; d > 0; d >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, lmx, d, L);
+            const int oi = __shfl_xor_sync(0xffffffffu, larg, d, L);
+            const float oh = __shfl_xor_sync(0xffffffffu, bh, d, L), ol = __shfl_xor_sync(0xffffffffu, bl, d, L);
+            if (ov > lmx || (ov == lmx && oi < larg)) {
+                lmx = ov;
+                larg = oi;
+                bh = oh;
+                bl = ol;
+            }
+        }
+        float r[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) r[x] = 4 * l + x == larg ? 0.f : (sh[x] - bh) + (sl[x] - bl);  // ff_diff
+        if (bh == kNegInf) r[0] = r[1] = r[2] = r[3] = kNegInf;
+        b[0] = f2(r[0], r[1]);
+        b[1] = f2(r[2], r[3]);
+    }
+    unsigned rare = 0;
+    {
+        float big = 0.f, sum = 0.f;  // sum: NaN if an entry is
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            big = fmaxf(big, fmaxf(fmaxf(fabsf(q[i][0]), fabsf(q[i][1])), fmaxf(fabsf(q[i][2]), fabsf(q[i][3]))));
+            sum += (q[i][0] + q[i][1]) + (q[i][2] + q[i][3]);
+        }
+        if (!(big <= kExactThreshold) | (sum != sum))  // seldom: which edges
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (needs_exact(q[i][0]) | needs_exact(q[i][1]) | needs_exact(q[i][2]) | needs_exact(q[i][3])) rare |= 1u << i;
+    }
+#pragma unroll
+    for (int d = L / 2; d > 0; d >>= 1) rare |= __shfl_xor_sync(0xffffffffu, rare, d, L);
+    // two edges at a time
+#pragma unroll
+    for (int p = 0; p < 4; p += 2) {
+        if (!__any_sync(0xffffffffu, t.deg > p)) break;
+        const int side0 = ((t.es[p] - es_base) / K) & 1, side1 = ((t.es[p + 1] - es_base) / K) & 1;  // the sources' places
+        const float c = invT * 1.4426950408889634f;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const F2 v[2] = {f2_fma(qa[p + h], minus1, b[0]), f2_fma(qb[p + h], minus1, b[1])};
+            F2 wa = v[0], wb = v[1];
+            if constexpr (!MAXP) {  // pair_weights
+                const float vmax = team_max<L>(f2_max<4>(v)), n = -vmax * c;
+                if (vmax == kNegInf) rare |= 1u << (p + h);
+                const float2 xa = f2_get(f2_fma(v[0], f2(c, c), f2(n, n))), xb = f2_get(f2_fma(v[1], f2(c, c), f2(n, n)));
+                wa = f2(ex2_ftz(xa.x), ex2_ftz(xa.y));
+                wb = f2(ex2_ftz(xb.x), ex2_ftz(xb.y));
+            }
+            ulonglong2 w;
+            w.x = wa;
+            w.y = wb;
+            *reinterpret_cast<ulonglong2 *>(xs + h * xs_step + 4 * l) = w;
+        }
+        __syncwarp();
+        F2 acc[2][4];
+        float mxp[2][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            acc[0][i] = acc[1][i] = f2(0.f, 0.f);
+            mxp[0][i] = mxp[1][i] = kNegInf;
+        }
+        auto step = [&](int h, int i, const ulonglong2 a, const ulonglong2 w) {
+            if constexpr (MAXP) {  // pair_max
+                const float2 x = f2_get(f2_add(a.x, w.x)), y = f2_get(f2_add(a.y, w.y));
+                mxp[h][i] = fmaxf(fmaxf(mxp[h][i], x.x), x.y);
+                mxp[h][i] = fmaxf(fmaxf(mxp[h][i], y.x), y.y);
+            } else {  // pair_linear
+                acc[h][i] = f2_fma(a.y, w.y, f2_fma(a.x, w.x, acc[h][i]));
+            }
+        };
+        const ulonglong2 *S4 = reinterpret_cast<const ulonglong2 *>(side0 ? S1 : S0) + l;
+        if (__all_sync(0xffffffffu, side0 == side1 || p + 1 >= t.deg)) {  // one reading of the table for both
+#pragma unroll
+            for (int cc = 0; cc < K / 4; ++cc) {
+                const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(xs + 4 * cc);
+                const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(xs + xs_step + 4 * cc);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const ulonglong2 a = S4[(4 * cc + i) * L];
+                    step(0, i, a, w0);
+                    step(1, i, a, w1);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h == 1) S4 = reinterpret_cast<const ulonglong2 *>(side1 ? S1 : S0) + l;
+#pragma unroll
+                for (int cc = 0; cc < K / 4; ++cc) {
+                    const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(xs + h * xs_step + 4 * cc);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) step(h, i, S4[(4 * cc + i) * L], w);
+                }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int es_t = (h ? side1 : side0) ? t.es[p + h] - K : t.es[p + h] + K;
+            const bool have = p + h < t.deg;
+            float mo4[4] = {0.f, 0.f, 0.f, 0.f};
+            if (have) row_load<AL>(mo4, m_old + es_t + 4 * l);
+            const F2 mo[2] = {f2(mo4[0], mo4[1]), f2(mo4[2], mo4[3])};
+            F2 o[2];
+            bool none = false;
+            if constexpr (MAXP) {
+                o[0] = f2(mxp[h][0], mxp[h][1]);
+                o[1] = f2(mxp[h][2], mxp[h][3]);
+                none = team_normalise<L>(o) == kNegInf;
+            } else {
+                float r[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 a = f2_get(acc[h][i]);
+                    r[i] = a.x + a.y;
+                }
+                o[0] = f2_mul(f2(T, T), f2_log(f2(r[0], r[1])));
+                o[1] = f2_mul(f2(T, T), f2_log(f2(r[2], r[3])));
+            }
+            // pair_finish
+            if (damping != 0.f) {
+                const float w = 1.f - damping;
+                o[0] = f2_fma(f2(damping, damping), mo[0], f2_mul(f2(w, w), o[0]));
+                o[1] = f2_fma(f2(damping, damping), mo[1], f2_mul(f2(w, w), o[1]));
+            }
+            none |= team_normalise<L>(o) == kNegInf;
+            if (none) rare |= 1u << (p + h);
+            if (have && !((rare >> (p + h)) & 1)) {
+                if constexpr (AL) {
+                    ulonglong2 x;
+                    x.x = o[0];
+                    x.y = o[1];
+                    *reinterpret_cast<ulonglong2 *>(m_new + es_t + 4 * l) = x;
+                } else {
+                    f2_store<4>(m_new + es_t + 4 * l, o);
+                }
+            }
+        }
+    }
+    return rare;
+}
+
+template <int K, bool MAXP, bool MS>
+__global__ void __launch_bounds__(kThreads, K == 16 ? 4 : 5)
+k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ blocks, const int32_t *__restrict__ list,
+             const float *__restrict__ pot, const float *__restrict__ ev, const float *__restrict__ m_old,
+             float *__restrict__ m_new, float T, float invT, float damping) {
+    constexpr int L = K / 4;                  // lanes per variable
+    constexpr int kStep = kThreads / L;       // variables per round of the block
+    constexpr int kRow = K == 4 ? 4 : K + 4;  // a team's exchange row: no bank conflicts between teams
+    __shared__ __align__(16) float S0[K * K], S1[K * K];
+    __shared__ __align__(16) float xch[2 * kStep * kRow];
+    __shared__ float tab[K * K];
+    __shared__ float red[2 * kThreads / 32];
+    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    if constexpr (MS) {  // multi-sample launches: this block's sample
+        const int64_t smp = blockIdx.y;
+        pot += smp * G.s_pot;
+        ev += smp * G.s_vs;
+        m_old += smp * G.s_es;
+        m_new += smp * G.s_es;
+    }
+    // before the previous launch has finished: what is fixed for the run (indices, the table)
+    const int4 B = __ldg(reinterpret_cast<const int4 *>(blocks + blockIdx.x));  // pos, n, es_base, pot_base
+    const int es_base = B.z, n = B.y;
+    const int l = threadIdx.x & (L - 1), team = threadIdx.x / L;
+    float *xs = xch + team * kRow;
+    TeamVar t = team_var(G, list, B.x + (team < n ? team : 0), team < n, es_base);
+    int vs = __ldg(G.vs_off + t.v);
+    pair_tables_load<K, kThreads>(pot + B.w, tab);
+    pdl_wait();  // messages of the previous launch
+    __syncthreads();
+    if (member_skip<MAXP>(G, __ldg(&blocks[blockIdx.x].member), T, invT, damping)) return;  // the whole block
+    const bool lin = pair_tables_make<K, MAXP, kThreads>(tab, S0, S1, red, invT);
+    if (!MAXP && !lin) {
+        for (int k = threadIdx.x; k < 4 * n; k += kThreads) {
+            const int pos = B.x + (k >> 2), v = list ? __ldg(list + pos) : pos;
+            if ((k & 3) < __ldg(G.vin_off + v + 1) - __ldg(G.vin_off + v))
+                fused_edge<K, MAXP>(G, tab, ev, m_old, m_new, v, k & 3, es_base, T, invT, damping);
+        }
+        return;
+    }
+    // rows are 16-byte aligned or not for the whole run (K is a multiple of 4)
+    const bool al = ((reinterpret_cast<uintptr_t>(m_old + es_base) | reinterpret_cast<uintptr_t>(m_new + es_base) |
+                      reinterpret_cast<uintptr_t>(ev + vs)) & 15u) == 0;
+    const bool all_al = __syncthreads_and(al);
+    for (int j = team; j - team < n; j += kStep) {
+        float e4[4], q[4][4];
+        unsigned rare;
+        if (all_al) {
+            row_load<true>(e4, ev + vs + 4 * l);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i < t.deg) row_load<true>(q[i], m_old + t.es[i] + 4 * l);
+                else q[i][0] = q[i][1] = q[i][2] = q[i][3] = 0.f;  // adds exactly nothing
+            }
+            rare = team_edges<K, MAXP, true>(t, e4, q, l, es_base, S0, S1, xs, kStep * kRow, m_old, m_new, T, invT, damping);
+        } else {
+            row_load<false>(e4, ev + vs + 4 * l);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i < t.deg) row_load<false>(q[i], m_old + t.es[i] + 4 * l);
+                else q[i][0] = q[i][1] = q[i][2] = q[i][3] = 0.f;
+            }
+            rare = team_edges<K, MAXP, false>(t, e4, q, l, es_base, S0, S1, xs, kStep * kRow, m_old, m_new, T, invT, damping);
+        }
+        if (rare != 0 && l == 0)
+#pragma unroll 1
+            for (int i = 0; i < t.deg; ++i)
+                if ((rare >> i) & 1) fused_edge<K, MAXP>(G, tab, ev, m_old, m_new, t.v, i, es_base, T, invT, damping);
+        if (j - team + kStep < n) {  // the next round's variable
+            const int jn = j + kStep;
+            t = team_var(G, list, B.x + (jn < n ? jn : 0), jn < n, es_base);
+            vs = __ldg(G.vs_off + t.v);
+        }
+    }
+}
+
+template <int K, bool MAXP, bool MS>
+cudaError_t launch_k(const DevGraph &G, const FactorLaunch &L, const float *pot, const float *ev, const float *m_old,
+                     float *m_new, float T, float damping, int S, cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)L.fuse_blocks, (unsigned)S);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_pair_fused<K, MAXP, MS>, G, L.fuse, L.fuse_list, pot, ev, m_old, m_new, T,
+                              MAXP ? 0.f : 1.f / T, damping);
+}
+
+template <int K>
+cudaError_t launch_pick(const DevGraph &G, const FactorLaunch &L, const float *pot, const float *ev, const float *m_old,
+                        float *m_new, float T, float damping, int S, cudaStream_t s) {
+    if (S > 1)
+        return T == 0.f ? launch_k<K, true, true>(G, L, pot, ev, m_old, m_new, T, damping, S, s)
+                        : launch_k<K, false, true>(G, L, pot, ev, m_old, m_new, T, damping, S, s);
+    return T == 0.f ? launch_k<K, true, false>(G, L, pot, ev, m_old, m_new, T, damping, 1, s)
+                    : launch_k<K, false, false>(G, L, pot, ev, m_old, m_new, T, damping, 1, s);
+}
+
+}  // namespace
+
+cudaError_t launch_pair_fused(const DevGraph &G, const FactorLaunch &L, const float *pot, const float *ev,
+                              const float *m_old, float *m_new, float T, float damping, int S, cudaStream_t s) {
+    switch (L.variant) {
+        case kPairF4: return launch_pick<4>(G, L, pot, ev, m_old, m_new, T, damping, S, s);
+        case kPairF8: return launch_pick<8>(G, L, pot, ev, m_old, m_new, T, damping, S, s);
+        case kPairF16: return launch_pick<16>(G, L, pot, ev, m_old, m_new, T, damping, S, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace pgm

@@ -51,7 +51,16 @@ enum FactorVariant : int32_t {
     kPairD4 = 13,      // dense pairwise table, K = 4, 8, 16: a thread per factor and
     kPairD8 = 14,      // direction (a warp pair per 32 factors; an alternative the autotuner
     kPairD16 = 15,     // may pick)
-    kNumFactorVariants = 16
+    kPairF4 = 16,      // dense pairwise table, K = 4, 8, 16, variable and factor pass in one
+    kPairF8 = 17,      // kernel (pair_fused.cu): members whose only group this is, with at
+    kPairF16 = 18,     // most 4 factors per variable
+    kNumFactorVariants = 19
+};
+
+// One block of the fused pairwise form: the variables at positions pos .. pos + n - 1 of their
+// bucket, and their group's first edge-state, first log-potential and member.
+struct FuseBlock {
+    int32_t pos, n, es_base, pot_base, member, pad[3];
 };
 
 // One enumeration group as seen by a launch. Edges of factor f are
@@ -151,7 +160,16 @@ struct FactorLaunch {
     int32_t max_blocks;  // K-lane pairwise launches: physical blocks (each walks a range
                          // of the n_blocks chunks)
     int32_t base_variant;  // the variant the compiler chose (before options and autotuning)
+    // fused form of a dense pairwise launch
+    const FuseBlock *fuse;      // device
+    const int32_t *fuse_list;   // the variables' bucket (device; null: identity)
+    int32_t fuse_blocks;        // 0: not eligible
 };
+
+inline bool is_fused(int variant) { return variant == kPairF4 || variant == kPairF8 || variant == kPairF16; }
+inline int fused_variant(int base) {
+    return base == kPairT4 ? kPairF4 : base == kPairT8 ? kPairF8 : base == kPairT16 ? kPairF16 : -1;
+}
 
 // Variable-pass kernel variants (buckets of variables).
 enum VarKind : int32_t {
@@ -176,6 +194,8 @@ struct VarLaunch {
     // the list, tile, first DevGraph::hd_tot entry of the variable, its tile count)
     const int4 *tiles;
     int32_t n_tiles;
+    int32_t fused_by;        // index of the factor launch that replaces this one in an
+                             // iteration while it has its fused form; -1: none
 };
 
 // The grid form of a one-launch run of this graph (lr_run.cu): nb blocks of Vc variables,
@@ -247,9 +267,13 @@ struct LaunchHook {
 
 // Kernel launchers (kernels.cu). Each returns cudaGetLastError() of its launches.
 // (n_samples > 1: samples as the launches' y dimension, at the strides of G)
+// An iteration's variable pass (kVarIter) leaves out the launches that a fused factor launch
+// of the plan replaces, unless `full`.
 cudaError_t launch_var_pass(const DevGraph &G, const Plan &P, const float *ev, const float *m,
                             float *b, int mode, int32_t *decode, cudaStream_t s, int n_samples = 1,
-                            const LaunchHook *hook = nullptr);
+                            const LaunchHook *hook = nullptr, bool full = false);
+cudaError_t launch_pair_fused(const DevGraph &G, const FactorLaunch &L, const float *pot, const float *ev,
+                              const float *m_old, float *m_new, float T, float damping, int n_samples, cudaStream_t s);
 cudaError_t launch_factor_pass(const DevGraph &G, const Plan &P, const float *log_pot,
                                const float *b, const float *ev, const float *m_old,
                                float *m_new, float T, float damping, cudaStream_t s, int n_samples = 1,
