@@ -20,6 +20,15 @@ namespace {
 // writes are visible (at once for a kernel launched without the attribute);
 // pdl_launch_dependents() lets the next kernel be scheduled before this one ends.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
+// The same for a grid of at most kPdlBlocks blocks. The next launch's blocks wait on the SMs for
+// this one to end: that hides a launch when the grid is small (4 blocks per SM), but where blocks
+// of this grid still queue, the waiting ones take their places (a 256 x 256 grid of K = 8: 8.7 us
+// per iteration without, 11.2 with; deconvolution of 100 images 118 without, 125 with).
+constexpr unsigned kPdlBlocks = 640;
+__device__ __forceinline__ bool pdl_small() { return gridDim.x * gridDim.y <= kPdlBlocks; }
+__device__ __forceinline__ void pdl_launch_if_small() {
+    if (pdl_small()) pdl_launch_dependents();
+}
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class Seg>

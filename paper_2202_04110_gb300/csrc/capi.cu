@@ -350,11 +350,14 @@ void plan_fused(const HostLayout &H, pgm_graph *g, Packer &pk) {
         size_t vi = 0;
         while (vi < P.var.size() && P.var[vi].kind != kind) ++vi;
         bool ok = vi < P.var.size();
-        // variables per block: one round of the block's teams (256 threads, K / 4 lanes each);
-        // more rounds would form the table less often, but a round's loads depend on one
-        // another and other blocks hide them better (K = 16 on the batch: 171 us with one
-        // round, 192 with two)
-        const int per = L.variant == kPairT4 ? 256 : L.variant == kPairT8 ? 128 : 64;
+        // variables per block: one round of the block's teams (K / 4 lanes each); more rounds
+        // would form the table less often, but a round's loads depend on one another and other
+        // blocks hide them better (K = 16 on 128 uneven grids: 171 us with one round, 192 with
+        // two). 128 threads; 256 for K = 16 from 6 such blocks per SM on, where the table counts
+        // (256 x 256: 16.6 against 17.2 us per iteration; 178 x 178: 9.9 against 9.4)
+        const int lanes = L.variant == kPairT4 ? 1 : L.variant == kPairT8 ? 2 : 4;
+        const int threads = lanes == 4 && (int64_t)bucket.size() * lanes >= (int64_t)256 * 6 * g->n_sm ? 256 : 128;
+        const int per = threads / lanes;
         std::vector<FuseBlock> fs;
         // (the variable launch goes as a whole: no other group may touch its variables)
         int64_t all_edges = 0;
@@ -382,6 +385,7 @@ void plan_fused(const HostLayout &H, pgm_graph *g, Packer &pk) {
         if (!ok || fs.empty() || all_edges != 0) continue;
         g->fused.push_back({(int)li, (int)vi, pk.add(fs.data(), fs.size())});
         L.fuse_blocks = (int32_t)fs.size();
+        L.fuse_threads = threads;
         L.variant = fused_variant(L.base_variant);
         P.var[vi].fused_by = (int32_t)li;
     }
@@ -1048,7 +1052,7 @@ static bool log_ratio_run(const pgm_graph *g, int32_t n_iters) {
 static bool small_run_cluster(const pgm_graph *g) {
     const int V = g->G.V, F = g->G.E / 2;
     if (g->small_run == 2) return true;
-    return !(lr_block_fits(V, F) && V <= kLrBlockAutoV) && lr_cluster_fits(V, F);
+    return !(lr_block_fits(V, F) && V <= kLrBlockAutoV && F <= kLrBlockAutoF) && lr_cluster_fits(V, F);
 }
 static bool small_run_used(const pgm_graph *g) {
     if (g->small_run == 0 || !g->P.lr || g->G.vin_tab4 == nullptr) return false;
@@ -1059,7 +1063,8 @@ static bool small_run_used(const pgm_graph *g) {
 // Whether a log-ratio run of this graph takes the cooperative-grid form: graphs above the
 // small forms, with the option on. (PGM_OPT_SMALL_RUN 0 keeps the launches at every size.)
 static bool grid_run_used(const pgm_graph *g) {
-    return g->small_run != 0 && g->P.lr && g->P.grid.nb > 0 && !small_run_used(g) &&
+    if (small_run_used(g) && (g->small_run == 2 || g->G.V <= kLrClusterAutoV)) return false;
+    return g->small_run != 0 && g->P.lr && g->P.grid.nb > 0 &&
            lr_grid_fits(g->P.grid, g->G.V, g->G.E / 2);
 }
 

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(256) k_var_thread(DevGraph G, const int32_t *_
                                                     float *__restrict__ out,
                                                     int32_t *__restrict__ dec) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         ev += smp * G.s_vs;
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(256) k_var_warp(DevGraph G, const int32_t *__r
                                                   const float *__restrict__ ev, const float *__restrict__ m,
                                                   float *__restrict__ out, int32_t *__restrict__ dec) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         ev += smp * G.s_vs;
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(256) k_var_tab4(DevGraph G, int n, const float
                                                   const float *__restrict__ m, float *__restrict__ out,
                                                   int32_t *__restrict__ dec) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         ev += smp * G.s_vs;
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(256) k_var_group(DevGraph G, const int32_t *__
                                                    const float *__restrict__ ev, const float *__restrict__ m,
                                                    float *__restrict__ out, int32_t *__restrict__ dec) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         ev += smp * G.s_vs;
@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(kVarBlockThreads) k_var_block(DevGraph G, cons
                                                                 float *__restrict__ out,
                                                                 int32_t *__restrict__ dec) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         ev += smp * G.s_vs;
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(kVarBlockThreads) k_var_hd(DevGraph G, const i
                                                              const float *__restrict__ m, float *__restrict__ out,
                                                              int32_t *__restrict__ dec) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     __shared__ float sh[96];
     __shared__ FF sb[kMaxStates];
     __shared__ int s_last;
@@ -809,7 +809,7 @@ k_pair(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float *__r
        const float *__restrict__ b, const float *__restrict__ ev, const float *__restrict__ m_old,
        float *__restrict__ m_new, float T, float invT, float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         pot += smp * G.s_pot;
@@ -1015,7 +1015,7 @@ k_pair_group(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, int n_vblo
              const float *__restrict__ b, const float *__restrict__ ev, const float *__restrict__ m_old,
              float *__restrict__ m_new, float T, float invT, float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         pot += smp * G.s_pot;
@@ -1150,7 +1150,7 @@ k_pair_thr(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float 
            const float *__restrict__ b, const float *__restrict__ ev, const float *__restrict__ m_old,
            float *__restrict__ m_new, float T, float invT, float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         pot += smp * G.s_pot;
@@ -1188,7 +1188,7 @@ k_pair_thr(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float 
             const float2 m = f2_get(v[i]);
             v[i] = f2_add(b2[i], f2(-m.x, -m.y));
         }
-        pair_direction<K, MAXP>(v, linear, shared, side ? S1 : S0, phi, step_s, step_t, m_old, m_new, es_t, T, invT,
+        pair_direction<K, MAXP>(v, linear, linear ? red[0] : 0.f, shared, side ? S1 : S0, phi, step_s, step_t, m_old, m_new, es_t, T, invT,
                                 damping, G.flags);
     }
 }
@@ -1209,7 +1209,7 @@ k_pair_dir(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float 
            const float *__restrict__ b, const float *__restrict__ ev, const float *__restrict__ m_old,
            float *__restrict__ m_new, float T, float invT, float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         pot += smp * G.s_pot;
@@ -1245,7 +1245,7 @@ k_pair_dir(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float 
         const float2 m = f2_get(v[i]);
         v[i] = f2_add(b2[i], f2(-m.x, -m.y));
     }
-    pair_direction<K, MAXP>(v, linear, shared, side ? S1 : S0, phi, step_s, step_t, m_old, m_new, es_t, T, invT, damping,
+    pair_direction<K, MAXP>(v, linear, linear ? red[0] : 0.f, shared, side ? S1 : S0, phi, step_s, step_t, m_old, m_new, es_t, T, invT, damping,
                             G.flags);
 }
 
@@ -1331,8 +1331,8 @@ __device__ __forceinline__ void quad_normalise(float4 &t, uint32_t *flags, bool 
 // four states) against the rows of `rows` (a padded K x K table: E or E^T for the linear
 // form, phi or phi^T otherwise). xs is the group's exchange slot (K floats).
 template <int K, bool MAXP>
-__device__ __forceinline__ float4 quad_dir(float4 v, bool linear, const float *rows, float *xs, int q, float T,
-                                          float invT) {
+__device__ __forceinline__ float4 quad_dir(float4 v, bool linear, const float *rows, float *xs, int q, float tmax,
+                                          float T, float invT) {
     constexpr int L = K / 4;
     float4 o;
     if (!MAXP && linear) {
@@ -1343,9 +1343,8 @@ __device__ __forceinline__ float4 quad_dir(float4 v, bool linear, const float *r
         if (vmax == kNegInf) {
             w = make_float4(0.f, 0.f, 0.f, 0.f);
         } else {
-            const float c = invT * 1.4426950408889634f, n = -vmax * c;
-            w = make_float4(ex2_ftz(fmaf(v.x, c, n)), ex2_ftz(fmaf(v.y, c, n)), ex2_ftz(fmaf(v.z, c, n)),
-                            ex2_ftz(fmaf(v.w, c, n)));
+            const float2 wa = pair_weights(f2(v.x, v.y), vmax, invT), wb = pair_weights(f2(v.z, v.w), vmax, invT);
+            w = make_float4(wa.x, wa.y, wb.x, wb.y);
         }
         reinterpret_cast<float4 *>(xs)[q] = w;
         __syncwarp();
@@ -1361,17 +1360,16 @@ __device__ __forceinline__ float4 quad_dir(float4 v, bool linear, const float *r
         for (int i = 0; i < 4; ++i) {
             const int x = 4 * q + i, sw = (x >> 2) & (K / 4 - 1);
             const float4 *row = reinterpret_cast<const float4 *>(rows + x * K);
-            float se = 0.f, so = 0.f;  // even and odd sources, as pair_linear
+            float s = 0.f;
 #pragma unroll
             for (int j = 0; j < K / 4; ++j) {
                 const float4 a = row[j ^ sw];  // chunk j of the row
-                se = fmaf(a.z, wa[4 * j + 2], fmaf(a.x, wa[4 * j], se));
-                so = fmaf(a.w, wa[4 * j + 3], fmaf(a.y, wa[4 * j + 1], so));
+                s = fmaf(a.x, wa[4 * j], fmaf(a.y, wa[4 * j + 1], fmaf(a.z, wa[4 * j + 2], fmaf(a.w, wa[4 * j + 3], s))));
             }
-            out[i] = se + so;
+            out[i] = s;
         }
-        const F2 T2 = f2(T, T);
-        const float2 oa = f2_get(f2_mul(T2, f2_log(f2(out[0], out[1])))), ob = f2_get(f2_mul(T2, f2_log(f2(out[2], out[3]))));
+        const float2 oa = f2_get(pair_log(f2(out[0], out[1]), T, vmax, tmax));
+        const float2 ob = f2_get(pair_log(f2(out[2], out[3]), T, vmax, tmax));
         o = vmax == kNegInf ? make_float4(kNegInf, kNegInf, kNegInf, kNegInf) : make_float4(oa.x, oa.y, ob.x, ob.y);
     } else {
         reinterpret_cast<float4 *>(xs)[q] = v;
@@ -1403,7 +1401,7 @@ k_pair_quad(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float
             const float *__restrict__ b, const float *__restrict__ ev, const float *__restrict__ m_old,
             float *__restrict__ m_new, float T, float invT, float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     static_assert(K == 8 || K == 16, "four states per lane, K / 4 lanes per factor");
     constexpr int L = K / 4;
     if constexpr (MS) {  // multi-sample launches: this block's sample
@@ -1426,6 +1424,7 @@ k_pair_quad(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float
     for (int i = threadIdx.x; i < K * K; i += blockDim.x) tab[i] = __ldg(pot + pot_base + i);
     __syncthreads();
     const bool linear = prepare_linear_table<K, MAXP>(tab, rows0, tinfo, invT);  // rows0 = E, unpadded
+    const float tmax = linear ? tinfo[0] : 0.f;
     // E (or phi) and its transpose in the swizzled layout (blocks of at least 64 threads)
     {
         constexpr int kPer = (K * K + 63) / 64;
@@ -1468,15 +1467,13 @@ k_pair_quad(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float
     // group's results are discarded
     const float4 b1 = ld4(b + max(vs1, 0) + 4 * q, false);
     float4 v = make_float4(b1.x - mo1.x, b1.y - mo1.y, b1.z - mo1.z, b1.w - mo1.w);
-    float4 o0 = quad_dir<K, MAXP>(v, linear, rows0, xs, q, T, invT);
+    float4 o0 = quad_dir<K, MAXP>(v, linear, rows0, xs, q, tmax, T, invT);
     const float4 b0 = ld4(b + max(vs0, 0) + 4 * q, false);
     v = make_float4(b0.x - mo0.x, b0.y - mo0.y, b0.z - mo0.z, b0.w - mo0.w);
-    float4 o1 = quad_dir<K, MAXP>(v, linear, rows1, xs, q, T, invT);
+    float4 o1 = quad_dir<K, MAXP>(v, linear, rows1, xs, q, tmax, T, invT);
     const bool lead0 = q == 0 && valid && !rare0, lead1 = q == 0 && valid && !rare1;
-    if (MAXP || !linear) {  // (as pair_finish)
-        quad_normalise<L>(o0, G.flags, lead0);
-        quad_normalise<L>(o1, G.flags, lead1);
-    }
+    quad_normalise<L>(o0, G.flags, lead0);
+    quad_normalise<L>(o1, G.flags, lead1);
     if (damping != 0.f) {
         const float w = 1.f - damping;
         o0 = make_float4(fmaf(damping, mo0.x, w * o0.x), fmaf(damping, mo0.y, w * o0.y), fmaf(damping, mo0.z, w * o0.z),
@@ -1507,7 +1504,7 @@ k_enum_generic(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const fl
                const float *__restrict__ m_old, float *__restrict__ m_new, float T, float invT,
                float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         pot += smp * G.s_pot;
@@ -1772,7 +1769,7 @@ k_enum_block(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const floa
              const float *__restrict__ b, const float *__restrict__ ev, const float *__restrict__ m_old,
              float *__restrict__ m_new, float T, float invT, float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         pot += smp * G.s_pot;
@@ -2065,7 +2062,7 @@ k_logic_small(DevGraph G, const LogicSeg *__restrict__ segs, int n_seg, const fl
               const float *__restrict__ ev, const float *__restrict__ m_old,
               float *__restrict__ m_new, float T, float invT, float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         b += smp * G.s_vs;
@@ -2333,7 +2330,7 @@ k_logic_warp(DevGraph G, const LogicSeg *__restrict__ segs, int n_seg, const flo
              const float *__restrict__ ev, const float *__restrict__ m_old,
              float *__restrict__ m_new, float T, float invT, float damping, int cap) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = sample_select(G);
         b += smp * G.s_vs;
@@ -2381,7 +2378,7 @@ __global__ void __launch_bounds__(128) k_adj_beliefs(DevGraph G, const float *__
                                                      const float *__restrict__ m, const float *__restrict__ gnb,
                                                      float *__restrict__ d_ev, float *__restrict__ adj) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= G.V) return;
     const int vs = G.vs_off[v], K = G.vs_off[v + 1] - vs, k0 = G.vin_off[v], k1 = G.vin_off[v + 1];
@@ -2567,7 +2564,7 @@ k_adj_factor(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const floa
              float *__restrict__ d_pot, float *__restrict__ partials, int nc_max, float T, float invT,
              float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     const EnumSeg *S = segs + find_seg(segs, n_seg, blockIdx.x);
     const int f_raw = (blockIdx.x - S->block_begin) * blockDim.x + threadIdx.x;
     // a block lies in one group, so a warp does; idle lanes shadow the group's last
@@ -2705,7 +2702,7 @@ __global__ void __launch_bounds__(256) k_adj_pot_reduce(const EnumSeg *__restric
                                                         const float *__restrict__ partials, int nc_max,
                                                         int threads_per_block, float *__restrict__ d_pot) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     const EnumSeg *S = segs + blockIdx.x;
     if (!S->shared || S->n_fac == 0) return;
     // the group's factors are consecutive from its first block, 32 to a warp; warps past
@@ -2737,7 +2734,7 @@ k_adj_block(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const float
             float *__restrict__ d_pot, float *__restrict__ partials, int nc_max, float T, float invT,
             float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     extern __shared__ __align__(16) float ab_smem[];
     __shared__ int sK[kMaxArity], sKo[kMaxArity];
     __shared__ int s_fix[kEnumBlockThreads / 32][kMaxArity];
@@ -2917,7 +2914,7 @@ __global__ void __launch_bounds__(256) k_adj_block_reduce(const EnumSeg *__restr
                                                           const float *__restrict__ partials, int nc_max,
                                                           float *__restrict__ d_pot) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     const EnumSeg *S = segs + blockIdx.x;
     if (!S->shared || S->n_fac == 0) return;
     const int teams = S->es_per_fac <= kEnumWarpStateSum ? kEnumBlockThreads / 32 : 1;
@@ -2971,7 +2968,7 @@ k_adj_logic(DevGraph G, const LogicSeg *__restrict__ segs, int n_seg, const floa
             const float *__restrict__ ev, const float *__restrict__ m_old, const float *__restrict__ adj,
             float *__restrict__ dv2f, float *__restrict__ ddamp, float T, float damping) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     const LogicSeg *S = segs + find_seg(segs, n_seg, blockIdx.x);
     const int f = (blockIdx.x - __ldg(&S->block_begin)) * blockDim.x + threadIdx.x;
     if (f >= __ldg(&S->n_fac)) return;
@@ -3071,7 +3068,7 @@ __global__ void __launch_bounds__(64) k_adj_var_tab4(DevGraph G, const float *__
                                                      const float *__restrict__ dv2f, float *__restrict__ adj_prev,
                                                      float *__restrict__ d_ev) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= G.V) return;
     const int4 t = __ldg(G.vin_tab4 + v);
@@ -3106,7 +3103,7 @@ __global__ void __launch_bounds__(128) k_adj_var(DevGraph G, const float *__rest
                                                  const float *__restrict__ dv2f, float *__restrict__ adj_prev,
                                                  float *__restrict__ d_ev) {
     pdl_wait();  // inputs of the previous launch
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= G.V) return;
     const int vs = G.vs_off[v], K = G.vs_off[v + 1] - vs, k0 = G.vin_off[v], k1 = G.vin_off[v + 1];

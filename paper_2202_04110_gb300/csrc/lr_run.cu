@@ -9,15 +9,16 @@
 // Why: the multi-launch run moves 112 bytes per variable and iteration through L2 and pays
 // two launch boundaries; on a 1000 x 1000 grid that took 17.4 us per iteration, on grids of
 // 10^4 .. 10^5 variables 3 .. 4 us, nearly all of it boundaries. A block here owns a
-// contiguous range of Vc variables: their incoming messages d (4 slots, 16 bytes) and totals
-// D (8 bytes) live in its shared memory (24 bytes per variable: 9,600 per SM, 1.45 million
-// on 152 SMs), factors between two variables of one block are updated in place, and only
+// contiguous range of Vc variables: their incoming messages d and the variable-to-factor values
+// lam (4 slots each) live in its shared memory (32 bytes per variable: 7,250 per SM, 1.1 million on
+// 152 SMs; larger graphs keep d and the totals D, 24 bytes, up to 1.47 million),
+// factors between two variables of one block are updated in place, and only
 // the factors that join two blocks exchange anything: one variable-to-factor value in each
 // direction per iteration. Each of the two blocks computes the message to its own variable.
 //
 // One iteration of a block:
-//   1. totals: thread per variable, D = (e(1) - e(0)) + sum of its d (float-float);
-//   2. publish: for every split factor, its value D - d into the other block's inbox;
+//   1. thread per variable: D = (e(1) - e(0)) + sum of its d (float-float), lam = D - d;
+//   2. publish: for every split factor, its lam into the other block's inbox;
 //   3. whole factors: thread per factor, both messages in place;
 //   4. split factors: wait for the other block's value, one message in place;
 // with a block barrier after 1 and after 4. Step 3 runs while the values travel.
@@ -129,7 +130,8 @@ __device__ __forceinline__ bool grid_barrier_once(uint32_t *bar, uint32_t n_bloc
 
 // The message into slot (v, kk) with every special case handled: its factor's table, its side.
 template <bool MAXP>
-__device__ __noinline__ float run_exact(const LrRun &A, const float *pot, int v, int kk, float l, float mo) {
+__device__ __noinline__ float run_exact(const LrRun &A, const float *pot, int v0, int s, float l, float mo) {
+    const int kk = s / A.Vc, v = v0 + s - kk * A.Vc;
     const int4 t = __ldg(A.tab4 + v);
     const int es = kk == 0 ? t.x : kk == 1 ? t.y : kk == 2 ? t.z : t.w;
     const float4 q = lr_table(A.segs, A.n_seg, pot, es >> 2);
@@ -137,26 +139,23 @@ __device__ __noinline__ float run_exact(const LrRun &A, const float *pot, int v,
     return lr_dir_exact<MAXP>(phi, (es >> 1) & 1, l, mo, A.k, A.Tln2, A.damping, A.flags);
 }
 
-// A variable whose totals do not come out finite: its four values by the explicit sums, in
-// lam (through L2: other threads of the block read them after the barrier).
-__device__ __noinline__ void run_var_slow(const LrRun &A, float *lam, int v, float2 e, float d0, float d1, float d2,
-                                          float d3) {
+// A variable whose values do not come out finite: its four lam by the explicit sums.
+__device__ __noinline__ void run_var_slow(float *lam, int lv, int Vc, float2 e, float d0, float d1, float d2, float d3) {
     const float dk[4] = {d0, d1, d2, d3};
-    const int pos[4] = {v, A.V + v, 2 * A.V + v, 3 * A.V + v};
+    const int pos[4] = {lv, Vc + lv, 2 * Vc + lv, 3 * Vc + lv};
     lr_var_slow(e, dk, pos, 4, lam);
 }
 
 __device__ __forceinline__ bool is_slow(float2 D) { return __float_as_uint(D.x) == kDvSlow; }
 
-// A record: three table numbers and the slots packed as local variable (14 bits) | slot
-// index k (2 bits): the first neighbour's in the low half, the second's in the high half.
-__device__ __forceinline__ uint32_t pack_slot(int lv, int k) { return (uint32_t)lv | ((uint32_t)k << 14); }
-
 // X: how blocks exchange values; RES: the records (and evidence) are in shared memory too,
 // else they are streamed from L2 (16 bytes per whole factor and iteration, loaded one item
 // ahead; the loads do not depend on the messages, so the block barriers do not delay them).
-template <bool MAXP, int X, bool RES>
-__global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
+// A record: three table numbers and the local slots k Vc + (v - v0) of the two messages, 16 bits
+// each. LAM: lam is kept per slot, so a factor reads d and lam at the same two offsets; else the
+// totals are kept per variable (8 bytes less) and a factor forms lam from them.
+template <bool MAXP, int X, bool RES, bool LAM>
+__global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_constant__ LrRun A) {
     extern __shared__ __align__(16) char lr_sm[];
     __shared__ int s_n[2];
     __shared__ int s_abort;
@@ -174,9 +173,9 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
     const float *pot = A.pot + (size_t)smp * A.pot_stride;
     const float2 *ev = reinterpret_cast<const float2 *>(A.ev + (size_t)smp * A.ev_stride) + v0;
     float *msgs = A.msgs + (size_t)smp * A.msg_stride;
-    float *lam = A.lam + (size_t)smp * 4 * V;
+    float *lam_g = LAM ? nullptr : A.lam + (size_t)smp * 4 * V;  // explicit sums, by local slot from 4 v0
     int32_t *dir = A.dir + (size_t)smp * 4 * V;
-    // shared memory: [records, split records,] totals, [evidence,] [inbox,] slots, [addresses]
+    // shared memory: [records, split records,] lam or totals, [evidence,] [inbox,] slots, [addresses]
     char *sp = lr_sm;
     float4 *rec, *hrec;
     uint32_t *hdst;
@@ -200,7 +199,8 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
         hdst = A.hdst + h_base;
     }
     float2 *Dv = reinterpret_cast<float2 *>(sp);
-    sp += 8 * (size_t)Vc;
+    float *lam = reinterpret_cast<float *>(sp);
+    sp += (LAM ? 16 : 8) * (size_t)Vc;
     if constexpr (RES) {
         es_sh = reinterpret_cast<float2 *>(sp);
         sp += 8 * (size_t)Vc;
@@ -255,10 +255,10 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
             bw = __shfl_sync(0xffffffffu, bw, 0) + __popc(mw & ((1u << lane) - 1u));
             bh = __shfl_sync(0xffffffffu, bh, 0) + __popc(mh & ((1u << lane) - 1u));
             if (whole)
-                rec[bw] = make_float4(c, al, be, __uint_as_float(pack_slot(lv, q) | (pack_slot(u - v0, uk) << 16)));
+                rec[bw] = make_float4(c, al, be, __uint_as_float((uint32_t)(q * Vc + lv) | (uint32_t)(uk * Vc + u - v0) << 16));
             if (X != kAlone && split) {
-                hrec[bh] = side == 0 ? make_float4(c, al, be, __uint_as_float(pack_slot(lv, q)))
-                                     : make_float4(be, al + c - be, c, __uint_as_float(pack_slot(lv, q)));
+                hrec[bh] = side == 0 ? make_float4(c, al, be, __uint_as_float((uint32_t)(q * Vc + lv)))
+                                     : make_float4(be, al + c - be, c, __uint_as_float((uint32_t)(q * Vc + lv)));
                 __stcg(dir + (size_t)q * V + v, bh);
             }
         }
@@ -278,8 +278,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
     }
     if (X == kGrid && !ok) return;  // (a block that got past the barrier times out in its waits)
     for (int h = tid; h < nH; h += nt) {  // where each split factor's value goes
-        const uint32_t pk = __float_as_uint(hrec[h].w);
-        const int lv = pk & 0x3fff, q = (pk >> 14) & 3;
+        const int s = (int)__float_as_uint(hrec[h].w), q = s / Vc, lv = s - q * Vc;
         const int4 t = __ldg(A.tab4 + v0 + lv);
         const int es = q == 0 ? t.x : q == 1 ? t.y : q == 2 ? t.z : t.w;
         const int p = __ldg(A.lr_pos + ((es >> 1) ^ 1));
@@ -292,10 +291,25 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
 
     // ---- iterations ----
     const float k = A.k, Tln2 = A.Tln2, damping = A.damping, w = 1.f - damping;
+    // a total kept per variable: the local variable of slot s, and lam from the total
+    auto var_of = [&](int s) { return s - Vc * ((s >= Vc) + (s >= 2 * Vc) + (s >= 3 * Vc)); };
+    auto lam_of = [&](int s, float dk) {
+        if constexpr (LAM) return lam[s];
+        else {
+            const float2 D = Dv[var_of(s)];
+            return is_slow(D) ? __ldcg(lam_g + 4 * (size_t)v0 + s) : lr_lam_from_D(D, dk);
+        }
+    };
+    // what the thread reads first in steps 1 and 3 is fixed for the run: in registers when the
+    // records are streamed (each step would otherwise begin with an L2 latency)
+    const float2 e_first = !RES && tid < nv ? __ldg(ev + tid) : make_float2(0.f, 0.f);
+    const float4 r_first = !RES && tid < nF ? rec[tid] : make_float4(0.f, 0.f, 0.f, 0.f);
     for (int it = 1; it <= A.n_iters; ++it) {
         // 1. totals
+        float2 e_next = e_first;
         for (int lv = tid; lv < nv; lv += nt) {
-            const float2 e = RES ? es_sh[lv] : __ldg(ev + lv);
+            const float2 e = RES ? es_sh[lv] : e_next;
+            if (!RES && lv + nt < nv) e_next = __ldg(ev + lv + nt);
             const float d0 = d[lv], d1 = d[Vc + lv], d2 = d[2 * Vc + lv], d3 = d[3 * Vc + lv];
             FF D = ff_add_nc(ff_make(e.y), -e.x);
             D = ff_add_nc(D, d0);
@@ -304,27 +318,34 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
             D = ff_add_nc(D, d3);
             float2 Df = make_float2(D.hi, D.lo);
             const float big = fmaxf(fmaxf(fabsf(d0), fabsf(d1)), fmaxf(fabsf(d2), fabsf(d3)));
-            if (!(fabsf(D.hi) + big < 1e38f)) {  // an infinite entry, NaN, or near overflow
-                bool fin = isfinite(e.x) && isfinite(e.y) && isfinite(d0) && isfinite(d1) && isfinite(d2) &&
-                           isfinite(d3);
-                fin = fin && isfinite(lr_lam_from_D(Df, d0)) && isfinite(lr_lam_from_D(Df, d1)) &&
-                      isfinite(lr_lam_from_D(Df, d2)) && isfinite(lr_lam_from_D(Df, d3));
-                if (!fin) {
-                    run_var_slow(A, lam, v0 + lv, e, d0, d1, d2, d3);
-                    Df = make_float2(__uint_as_float(kDvSlow), 0.f);
+            const float l0 = lr_lam_from_D(Df, d0), l1 = lr_lam_from_D(Df, d1), l2 = lr_lam_from_D(Df, d2),
+                        l3 = lr_lam_from_D(Df, d3);
+            bool slow = false;
+            if (!(fabsf(D.hi) + big < 1e38f))  // an infinite entry, NaN, or near overflow
+                slow = !(isfinite(e.x) && isfinite(e.y) && isfinite(d0) && isfinite(d1) && isfinite(d2) && isfinite(d3) &&
+                         isfinite(l0) && isfinite(l1) && isfinite(l2) && isfinite(l3));
+            if (slow) {
+                if constexpr (LAM) {
+                    run_var_slow(lam, lv, Vc, e, d0, d1, d2, d3);
+                } else {
+                    run_var_slow(lam_g + 4 * (size_t)v0, lv, Vc, e, d0, d1, d2, d3);
+                    Dv[lv] = make_float2(__uint_as_float(kDvSlow), 0.f);
                 }
+            } else if constexpr (LAM) {
+                lam[lv] = l0;
+                lam[Vc + lv] = l1;
+                lam[2 * Vc + lv] = l2;
+                lam[3 * Vc + lv] = l3;
+            } else {
+                Dv[lv] = Df;
             }
-            Dv[lv] = Df;
         }
         __syncthreads();
         // 2. publish
         if constexpr (X != kAlone) {
             for (int h = tid; h < nH; h += nt) {
-                const uint32_t pk = __float_as_uint(RES ? hrec[h].w : __ldcg(&hrec[h].w));
-                const int lv = pk & 0x3fff, q = (pk >> 14) & 3;
-                const float2 D = Dv[lv];
-                const float l = is_slow(D) ? __ldcg(lam + (size_t)q * V + v0 + lv) : lr_lam_from_D(D, d[q * Vc + lv]);
-                const unsigned long long wd = box_word(l, (uint32_t)it);
+                const int s = (int)__float_as_uint(RES ? hrec[h].w : __ldcg(&hrec[h].w));
+                const unsigned long long wd = box_word(lam_of(s, LAM ? 0.f : d[s]), (uint32_t)it);
                 if constexpr (X == kCluster) {
                     const uint32_t a = hdst[h] + ((it & 1) ? 8u * (uint32_t)A.h_cap : 0u);
                     asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(wd) : "memory");
@@ -338,23 +359,23 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
         {
             int i = tid;
             float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (i < nF) r = RES ? rec[i] : __ldcg(rec + i);
+            if (RES && i < nF) r = rec[i];
+            if (!RES) r = r_first;
             while (i < nF) {
                 const int in = i + nt;
                 float4 rn = r;
                 if (!RES && in < nF) rn = __ldcg(rec + in);
                 const uint32_t pk = __float_as_uint(r.w);
-                const int lv0 = pk & 0x3fff, k0 = (pk >> 14) & 3, lv1 = (pk >> 16) & 0x3fff, k1 = pk >> 30;
-                const int s0 = k0 * Vc + lv0, s1 = k1 * Vc + lv1;
+                const int s0 = pk & 0xffff, s1 = pk >> 16;
                 const float mo0 = d[s0], mo1 = d[s1];
-                const float2 D0 = Dv[lv0], D1 = Dv[lv1];
-                float l0 = lr_lam_from_D(D0, mo0), l1 = lr_lam_from_D(D1, mo1);
-                if (is_slow(D0)) l0 = __ldcg(lam + (size_t)k0 * V + v0 + lv0);
-                if (is_slow(D1)) l1 = __ldcg(lam + (size_t)k1 * V + v0 + lv1);
+                const float l0 = lam_of(s0, mo0), l1 = lam_of(s1, mo1);
                 float n0 = lr_dir<MAXP>(r.x, r.y, r.z, l1, mo0, k, Tln2, damping, w);
                 float n1 = lr_dir<MAXP>(r.z, r.y + r.x - r.z, r.x, l0, mo1, k, Tln2, damping, w);
-                if (lr_dir_rare(n0, l1)) n0 = run_exact<MAXP>(A, pot, v0 + lv0, k0, l1, mo0);
-                if (lr_dir_rare(n1, l0)) n1 = run_exact<MAXP>(A, pot, v0 + lv1, k1, l0, mo1);
+                // (a NaN lam makes a sum-product message NaN by itself)
+                if (!(fabsf(n0) + fabsf(n1) < CUDART_INF_F) || (MAXP && !(l0 == l0 && l1 == l1))) {
+                    if (lr_dir_rare(n0, l1)) n0 = run_exact<MAXP>(A, pot, v0, s0, l1, mo0);
+                    if (lr_dir_rare(n1, l0)) n1 = run_exact<MAXP>(A, pot, v0, s1, l0, mo1);
+                }
                 d[s0] = n0;
                 d[s1] = n1;
                 i = in;
@@ -388,12 +409,11 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
                     }
                 }
                 const float l = __uint_as_float((uint32_t)wd);
-                const uint32_t pk = __float_as_uint(r.w);
-                const int lv = pk & 0x3fff, q = (pk >> 14) & 3;
-                const float mo = d[q * Vc + lv];
+                const int s = (int)__float_as_uint(r.w);
+                const float mo = d[s];
                 float n = lr_dir<MAXP>(r.x, r.y, r.z, l, mo, k, Tln2, damping, w);
-                if (lr_dir_rare(n, l)) n = run_exact<MAXP>(A, pot, v0 + lv, q, l, mo);
-                d[q * Vc + lv] = n;
+                if (lr_dir_rare(n, l)) n = run_exact<MAXP>(A, pot, v0, s, l, mo);
+                d[s] = n;
             }
         }
         __syncthreads();
@@ -419,18 +439,152 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const LrRun A) {
     if constexpr (X == kCluster) cluster_barrier();  // no block leaves while another may write to its inbox
 }
 
+// ---- one block: graphs of up to kLrBlockAutoV variables ----
+//
+// Thread per directed edge: from the total of its variable and the message that came in along
+// the edge it sends the new message to the factor's other variable, into the other of two copies
+// of d. What the thread alone uses (its message, table numbers, addresses) stays in registers.
+//   TWO = false, up to kPushOneE edges: the thread forms the total itself from the variable's
+//     four messages. The four threads of a variable repeat it, but an iteration is one chain --
+//     read, sum, update, write, barrier. Bound by that chain's latency.
+//   TWO = true: a thread per variable forms the totals, a barrier, then the edges. Two chains,
+//     but 1.6x fewer instructions, which is what bounds a block of 1,024 threads.
+__device__ __noinline__ float push_lam_slow(float2 e, float d0, float d1, float d2, float d3, int k) {
+    const float dk[4] = {d0, d1, d2, d3};
+    FF l0 = ff_make(e.x), l1 = ff_make(e.y);
+    for (int j = 0; j < 4; ++j) {  // as lr_var_slow
+        if (j == k) continue;
+        const float2 q = lr_decode(dk[j]);
+        l0 = ff_add(l0, q.x);
+        l1 = ff_add(l1, q.y);
+    }
+    return lam_encode(l0, l1);
+}
+
+// The total of a variable from its evidence and four messages; false (and what the slow path
+// needs left to the caller) when a leave-one-out value would not come out finite.
+__device__ __forceinline__ bool push_total(float2 e, float d0, float d1, float d2, float d3, float2 &Df) {
+    FF D = ff_add_nc(ff_make(e.y), -e.x);
+    D = ff_add_nc(D, d0);
+    D = ff_add_nc(D, d1);
+    D = ff_add_nc(D, d2);
+    D = ff_add_nc(D, d3);
+    Df = make_float2(D.hi, D.lo);
+    const float big = fmaxf(fmaxf(fabsf(d0), fabsf(d1)), fmaxf(fabsf(d2), fabsf(d3)));
+    if (fabsf(D.hi) + big < 1e38f) return true;
+    // an infinite entry, NaN, or near overflow
+    return isfinite(e.x) && isfinite(e.y) && isfinite(d0) && isfinite(d1) && isfinite(d2) && isfinite(d3) &&
+           isfinite(lr_lam_from_D(Df, d0)) && isfinite(lr_lam_from_D(Df, d1)) && isfinite(lr_lam_from_D(Df, d2)) &&
+           isfinite(lr_lam_from_D(Df, d3));
+}
+
+template <bool MAXP, int NE, bool TWO>
+__global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_push(const LrRun A) {
+    extern __shared__ __align__(16) char lr_sm[];
+    const int V = A.V, E = A.E, tid = threadIdx.x, nt = blockDim.x, smp = blockIdx.x;
+    const float *pot = A.pot + (size_t)smp * A.pot_stride;
+    const float2 *ev = reinterpret_cast<const float2 *>(A.ev + (size_t)smp * A.ev_stride);
+    float *msgs = A.msgs + (size_t)smp * A.msg_stride;
+    float *cur = reinterpret_cast<float *>(lr_sm), *nxt = cur + 4 * V;
+    float2 *Dv = reinterpret_cast<float2 *>(nxt + 4 * V);  // TWO
+    for (int i = tid; i < 8 * V; i += nt) cur[i] = 0.f;  // (unused slots stay 0)
+    __syncthreads();
+    int v[NE], k[NE], dst[NE];
+    float r[NE], p[NE], q[NE], mo[NE];
+    float2 e[TWO ? 1 : NE];
+    if (TWO) e[0] = tid < V ? __ldg(ev + tid) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < NE; ++j) {
+        const int i = tid + j * nt;  // the edge this thread sends along, from its variable
+        v[j] = k[j] = dst[j] = 0;
+        r[j] = p[j] = q[j] = mo[j] = 0.f;
+        if (!TWO) e[j] = make_float2(0.f, 0.f);
+        if (i >= E) continue;
+        const int s = __ldg(A.lr_pos + i);
+        k[j] = (s >= V) + (s >= 2 * V) + (s >= 3 * V);
+        v[j] = s - k[j] * V;
+        dst[j] = __ldg(A.lr_pos + (i ^ 1));
+        if (!TWO) e[j] = __ldg(ev + v[j]);
+        mo[j] = lr_encode(__ldcg(msgs + 2 * (i ^ 1)), __ldcg(msgs + 2 * (i ^ 1) + 1));
+        const float4 t = lr_table(A.segs, A.n_seg, pot, i >> 1);
+        const bool fin = isfinite(t.x) & isfinite(t.y) & isfinite(t.z) & isfinite(t.w);
+        const float c = fin ? t.z - t.x : CUDART_NAN_F, al = fin ? t.w - t.z : CUDART_NAN_F;
+        const float be = fin ? t.y - t.x : CUDART_NAN_F;
+        const bool to1 = (i & 1) == 0;  // from variable 0 to variable 1
+        r[j] = to1 ? be : c;
+        p[j] = to1 ? al + c - be : al;
+        q[j] = to1 ? c : be;
+        cur[dst[j]] = mo[j];
+    }
+    __syncthreads();
+    const float w = 1.f - A.damping;
+    for (int it = 0; it < A.n_iters; ++it) {
+        if constexpr (TWO) {
+            if (tid < V) {
+                float2 Df;
+                const bool ok = push_total(e[0], cur[tid], cur[V + tid], cur[2 * V + tid], cur[3 * V + tid], Df);
+                Dv[tid] = ok ? Df : make_float2(__uint_as_float(kDvSlow), 0.f);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int j = 0; j < NE; ++j) {
+            if (tid + j * nt >= E) continue;
+            float l;
+            if constexpr (TWO) {
+                const float2 Df = Dv[v[j]];
+                l = lr_lam_from_D(Df, cur[k[j] * V + v[j]]);
+                if (is_slow(Df))
+                    l = push_lam_slow(__ldg(ev + v[j]), cur[v[j]], cur[V + v[j]], cur[2 * V + v[j]], cur[3 * V + v[j]], k[j]);
+            } else {
+                const float d0 = cur[v[j]], d1 = cur[V + v[j]], d2 = cur[2 * V + v[j]], d3 = cur[3 * V + v[j]];
+                float2 Df;
+                const bool ok = push_total(e[j], d0, d1, d2, d3, Df);
+                l = lr_lam_from_D(Df, k[j] == 0 ? d0 : k[j] == 1 ? d1 : k[j] == 2 ? d2 : d3);
+                if (!ok) l = push_lam_slow(e[j], d0, d1, d2, d3, k[j]);
+            }
+            float n = lr_dir<MAXP>(r[j], p[j], q[j], l, mo[j], A.k, A.Tln2, A.damping, w);
+            if (lr_dir_rare(n, l)) {
+                const int i = tid + j * nt;
+                const float4 t = lr_table(A.segs, A.n_seg, pot, i >> 1);
+                const float phi[4] = {t.x, t.y, t.z, t.w};
+                n = lr_dir_exact<MAXP>(phi, (i & 1) ^ 1, l, mo[j], A.k, A.Tln2, A.damping, A.flags);
+            }
+            mo[j] = n;
+            nxt[dst[j]] = n;
+        }
+        __syncthreads();
+        float *t = cur;
+        cur = nxt;
+        nxt = t;
+    }
+#pragma unroll
+    for (int j = 0; j < NE; ++j) {
+        const int i = tid + j * nt;
+        if (i >= E) continue;
+        const float2 o = lr_decode(mo[j]);
+        msgs[2 * (i ^ 1)] = o.x;
+        msgs[2 * (i ^ 1) + 1] = o.y;
+    }
+}
+
 using RunKernel = void (*)(const LrRun);
-RunKernel run_kernel(bool maxp, int x, bool res) {
-    if (x == kAlone) return maxp ? (res ? k_lr_run<true, kAlone, true> : k_lr_run<true, kAlone, false>)
-                                 : (res ? k_lr_run<false, kAlone, true> : k_lr_run<false, kAlone, false>);
-    if (x == kCluster) return maxp ? k_lr_run<true, kCluster, true> : k_lr_run<false, kCluster, true>;
-    return maxp ? (res ? k_lr_run<true, kGrid, true> : k_lr_run<true, kGrid, false>)
-                : (res ? k_lr_run<false, kGrid, true> : k_lr_run<false, kGrid, false>);
+// LAM where it fits: always with the records in shared memory.
+template <bool MAXP>
+RunKernel run_kernel_t(int x, bool res, bool lam) {
+    if (x == kCluster) return k_lr_run<MAXP, kCluster, true, true>;
+    if (x == kAlone) return res ? k_lr_run<MAXP, kAlone, true, true>
+                                : lam ? k_lr_run<MAXP, kAlone, false, true> : k_lr_run<MAXP, kAlone, false, false>;
+    return res ? k_lr_run<MAXP, kGrid, true, true>
+               : lam ? k_lr_run<MAXP, kGrid, false, true> : k_lr_run<MAXP, kGrid, false, false>;
+}
+RunKernel run_kernel(bool maxp, int x, bool res, bool lam) {
+    return maxp ? run_kernel_t<true>(x, res, lam) : run_kernel_t<false>(x, res, lam);
 }
 
 // Shared memory of a block.
-size_t run_smem(int x, bool res, int Vc, int f_cap, int h_cap) {
-    size_t n = 24 * (size_t)Vc;
+size_t run_smem(int x, bool res, bool lam, int Vc, int f_cap, int h_cap) {
+    size_t n = (lam ? 32 : 24) * (size_t)Vc;
     if (res) n += 8 * (size_t)Vc + 16 * (size_t)f_cap + 20 * (size_t)h_cap;
     if (x == kCluster) n += 16 * (size_t)h_cap;
     return n + 16;
@@ -462,8 +616,8 @@ const RunDevice &run_device() {
     R.smem = optin - 256;  // less the kernels' static shared memory
     for (int x = 0; x < 3; ++x)
         for (int m = 0; m < 2; ++m)
-            for (int r = 0; r < 2; ++r) {
-                RunKernel kern = run_kernel(m, x, r);
+            for (int r = 0; r < 3; ++r) {
+                RunKernel kern = run_kernel(m, x, r == 2, r >= 1);
                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, R.smem);
                 if (x == kCluster) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             }
@@ -471,7 +625,7 @@ const RunDevice &run_device() {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(C);
         cfg.blockDim = dim3(kLrRunThreads);
-        cfg.dynamicSmemBytes = run_smem(kCluster, true, kLrSmallMaxV, 2 * kLrSmallMaxV, 4 * kLrSmallMaxV);
+        cfg.dynamicSmemBytes = run_smem(kCluster, true, true, kLrSmallMaxV, 2 * kLrSmallMaxV, 4 * kLrSmallMaxV);
         if ((int)cfg.dynamicSmemBytes > R.smem) break;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -481,18 +635,18 @@ const RunDevice &run_device() {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n0 = 0, n1 = 0;
-        if (cudaOccupancyMaxActiveClusters(&n0, k_lr_run<true, kCluster, true>, &cfg) == cudaSuccess && n0 > 0 &&
-            cudaOccupancyMaxActiveClusters(&n1, k_lr_run<false, kCluster, true>, &cfg) == cudaSuccess && n1 > 0) {
+        if (cudaOccupancyMaxActiveClusters(&n0, k_lr_run<true, kCluster, true, true>, &cfg) == cudaSuccess && n0 > 0 &&
+            cudaOccupancyMaxActiveClusters(&n1, k_lr_run<false, kCluster, true, true>, &cfg) == cudaSuccess && n1 > 0) {
             R.cluster = C;
             break;
         }
     }
     R.coop = coop != 0;
     for (int m = 0; m < 2 && R.coop; ++m)
-        for (int r = 0; r < 2; ++r) {
+        for (int r = 0; r < 3; ++r) {
             int n = 0;
-            R.coop = R.coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, run_kernel(m, kGrid, r), kLrRunThreads,
-                                                                             R.smem) == cudaSuccess && n >= 1;
+            R.coop = R.coop && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, run_kernel(m, kGrid, r == 2, r >= 1),
+                                                                             kLrRunThreads, R.smem) == cudaSuccess && n >= 1;
         }
     cudaGetLastError();  // a refused query leaves no error behind
     R.ready = true;
@@ -523,6 +677,20 @@ cudaError_t launch(RunKernel kern, const LrRun &A, int blocks, int threads, size
     cfg.attrs = at;
     cfg.numAttrs = x == kAlone ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kern, A);
+}
+
+// The push form of one block per sample (lr_block_fits).
+constexpr int kPushOneE = 600;
+template <bool MAXP>
+RunKernel push_kernel(int E) {
+    if (E <= kPushOneE) return k_lr_push<MAXP, 1, false>;
+    return E <= kLrRunThreads ? k_lr_push<MAXP, 1, true> : E <= 2 * kLrRunThreads ? k_lr_push<MAXP, 2, true>
+                                                                                  : k_lr_push<MAXP, 4, true>;
+}
+cudaError_t launch_push(const LrRun &A, bool maxp, int samples, cudaStream_t s) {
+    const int ne = A.E <= kLrRunThreads ? 1 : A.E <= 2 * kLrRunThreads ? 2 : 4;
+    return launch(maxp ? push_kernel<true>(A.E) : push_kernel<false>(A.E), A, samples,
+                  run_threads(A.V, (A.E + ne - 1) / ne), (A.E <= kPushOneE ? 32 : 40) * (size_t)A.V, kAlone, s);
 }
 
 LrRun run_args(const DevGraph &G, const EnumSeg *segs, int n_seg, const float *pot, const float *ev, float *msgs,
@@ -572,18 +740,14 @@ cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *l
     run_device();  // the kernels' attributes
     LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, lam, T, damping, n_iters);
     A.dir = dir;
-    if (!cluster) {
-        A.f_cap = F;
-        return launch(run_kernel(T == 0.f, kAlone, true), A, 1, run_threads(V, F), run_smem(kAlone, true, V, F, 0),
-                      kAlone, s);
-    }
+    if (!cluster) return launch_push(A, T == 0.f, 1, s);
     const int C = lr_cluster_size();
     A.nb = C;
     A.Vc = (V + C - 1) / C;
     A.f_cap = 2 * A.Vc;  // a block's variables have 4 slots each, a whole factor takes two
     A.h_cap = 4 * A.Vc;
-    return launch(run_kernel(T == 0.f, kCluster, true), A, C, run_threads(A.Vc, (F + C - 1) / C),
-                  run_smem(kCluster, true, A.Vc, A.f_cap, A.h_cap), kCluster, s);
+    return launch(run_kernel(T == 0.f, kCluster, true, true), A, C, run_threads(A.Vc, (F + C - 1) / C),
+                  run_smem(kCluster, true, true, A.Vc, A.f_cap, A.h_cap), kCluster, s);
 }
 
 // ---- the grid form of one sample ----
@@ -601,7 +765,7 @@ bool lr_grid_fits(const LrGridPlan &g, int V, int F) {
     if (g.nb < 2 || !R.coop || g.nb > R.n_sm) return false;
     const int64_t split = g.n_split;
     // the workspace: see launch_lr_grid_run
-    if (run_smem(kGrid, true, g.Vc, g.f_max, g.h_max) <= (size_t)R.smem) return 2 * split <= 3 * (int64_t)F;
+    if (run_smem(kGrid, true, true, g.Vc, g.f_max, g.h_max) <= (size_t)R.smem) return 2 * split <= 3 * (int64_t)F;
     return 20 * split <= 12 * (int64_t)F && 16 * split <= 8 * (int64_t)V;
 }
 
@@ -625,7 +789,7 @@ cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPla
     A.f_cap = g.f_max;
     A.h_cap = g.h_max;
     A.off = g.off;
-    const size_t smem = run_smem(kGrid, true, g.Vc, g.f_max, g.h_max);
+    const size_t smem = run_smem(kGrid, true, true, g.Vc, g.f_max, g.h_max);
     const bool res = smem <= (size_t)R.smem;
     if (res) {
         A.box0 = reinterpret_cast<unsigned long long *>(m_tmp);
@@ -637,8 +801,9 @@ cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPla
         A.box0 = reinterpret_cast<unsigned long long *>(b);
         A.box1 = A.box0 + g.n_split;
     }
-    return launch(run_kernel(T == 0.f, kGrid, res), A, g.nb, run_threads(g.Vc, g.f_max),
-                  res ? smem : run_smem(kGrid, false, g.Vc, 0, 0), kGrid, s);
+    const bool lam_sh = run_smem(kGrid, false, true, g.Vc, 0, 0) <= (size_t)R.smem;
+    return launch(run_kernel(T == 0.f, kGrid, res, lam_sh), A, g.nb, run_threads(g.Vc, g.f_max),
+                  res ? smem : run_smem(kGrid, false, lam_sh, g.Vc, 0, 0), kGrid, s);
 }
 
 // ---- many samples of one graph ----
@@ -662,7 +827,7 @@ LrMultiPlan lr_multi_plan(int V, int S, bool local) {
     p.f_cap = 2 * p.Vc;
     p.h_cap = p.nb > 1 ? 4 * p.Vc : 0;
     const int x = p.nb > 1 ? kGrid : kAlone;
-    p.res = run_smem(x, true, p.Vc, p.f_cap, p.h_cap) <= (size_t)R.smem;
+    p.res = run_smem(x, true, true, p.Vc, p.f_cap, p.h_cap) <= (size_t)R.smem;
     // per sample: lam and directory, then each block's items (run_multi's layout)
     p.sample_bytes = 32 * (size_t)V + (size_t)p.nb * (16 * (size_t)p.h_cap + (p.res ? 0 : 16 * (size_t)p.f_cap + 20 * (size_t)p.h_cap));
     if (p.nb == 1) Sc = (int)std::min<int64_t>(S, std::max<int64_t>(1, ((int64_t)1 << 28) / (int64_t)p.sample_bytes));
@@ -696,9 +861,11 @@ cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiP
     A.hdst = reinterpret_cast<uint32_t *>(A.box1 + blocks * p.h_cap);
     A.lam = reinterpret_cast<float *>(A.hdst + (p.res ? 0 : blocks * p.h_cap));
     A.dir = reinterpret_cast<int32_t *>(A.lam + 4 * V * S);
+    if (p.nb == 1 && G.V <= kLrBlockAutoV && lr_block_fits(G.V, G.E / 2)) return launch_push(A, T == 0.f, S, s);
     const int x = p.nb > 1 ? kGrid : kAlone;
-    return launch(run_kernel(T == 0.f, x, p.res), A, (int)blocks, run_threads(p.Vc, (2 * G.V + p.nb - 1) / p.nb),
-                  p.res ? run_smem(x, true, p.Vc, p.f_cap, p.h_cap) : run_smem(x, false, p.Vc, 0, 0), x, s);
+    const bool lam_sh = run_smem(x, false, true, p.Vc, 0, 0) <= (size_t)run_device().smem;
+    return launch(run_kernel(T == 0.f, x, p.res, lam_sh), A, (int)blocks, run_threads(p.Vc, (2 * G.V + p.nb - 1) / p.nb),
+                  p.res ? run_smem(x, true, true, p.Vc, p.f_cap, p.h_cap) : run_smem(x, false, lam_sh, p.Vc, 0, 0), x, s);
 }
 
 }  // namespace pgm

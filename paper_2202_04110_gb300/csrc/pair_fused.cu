@@ -13,22 +13,21 @@
 // arithmetic but the L1: a thread that loads its own 4 K-byte rows touches 32 lines with every
 // 16-byte load of a warp, one line per cycle, and reads the whole table for every message.
 // Here K / 4 lanes share a variable, four states each: a warp's load covers whole rows, and a
-// lane reads the four targets' part of the table, once for two edges of the same side. The next
-// launch's blocks load their indices and table while this one ends (programmatic launch).
-// Measured against the two passes it replaces (GB300, T = 1): a 181 x 181 grid of K = 16, whole
-// calls of 100 iterations 1.79 -> 0.88 ms (8.8 us per iteration); per launch on 128 uneven
-// grids K = 16 (662,000 variables) 60 + 222 -> 168 us, K = 8 (800,000) 43 + 88 -> 100, K = 4
-// (672,000) 28 + 46 -> 48. What bounds it now: issue slots (half of them) and the chain index ->
-// messages -> weights -> targets of a round; more resident blocks win against fewer spills
-// (K = 16: 2, 3, 4 blocks per SM 232, 183, 171 us), more rounds per block lose.
+// lane reads the four targets' part of the table, once for two edges of the same side. A block
+// loads its indices and table before it waits for the previous launch.
+// Measured against the two passes it replaces (GB300, T = 1, whole calls, us per iteration): K =
+// 16 on 181 x 181 17.9 -> 9.7; K = 8 on 178 x 178 9.3 -> 5.8; K = 4 on 64 x 64 6.0 -> 3.4 (two
+// launches' latency -> one); per launch on 128 uneven grids K = 16 (662,000 variables) 60 + 222
+// -> 178 us, K = 8 (800,000) 43 + 88 -> 101, K = 4 (672,000) 28 + 46 -> 51. What bounds it now:
+// issue slots (half of them) and the chain index -> messages -> weights -> targets of a round;
+// more resident blocks win against fewer spills (K = 16: 2, 3, 4 blocks of 256 per SM 232, 183,
+// 171 us).
 #include <cstdint>
 
 #include "pair_math.cuh"
 
 namespace pgm {
 namespace {
-
-constexpr int kThreads = 256;
 
 template <int L>
 __device__ __forceinline__ float team_max(float v) {
@@ -114,7 +113,7 @@ __device__ __forceinline__ TeamVar team_var(const DevGraph &G, const int32_t *li
 // a maximum of -inf on the way (contradictions and their flags are left to it).
 template <int K, bool MAXP, bool AL>
 __device__ __forceinline__ unsigned team_edges(const TeamVar &t, const float (&e4)[4], const float (&q)[4][4], int l,
-                                               int es_base, const float *S0, const float *S1, float *xs, int xs_step,
+                                               int es_base, const float *S0, const float *S1, float tmax, float *xs, int xs_step,
                                                const float *m_old, float *m_new, float T, float invT, float damping) {
     constexpr int L = K / 4;
     const F2 minus1 = f2(-1.f, -1.f);
@@ -200,64 +199,68 @@ __device__ __forceinline__ unsigned team_edges(const TeamVar &t, const float (&e
     for (int p = 0; p < 4; p += 2) {
         if (!__any_sync(0xffffffffu, t.deg > p)) break;
         const int side0 = ((t.es[p] - es_base) / K) & 1, side1 = ((t.es[p + 1] - es_base) / K) & 1;  // the sources' places
-        const float c = invT * 1.4426950408889634f;
+        float vmax[2];
         __syncwarp();
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < 2; ++h) {  // the source's values or weights, each twice: pairs for two targets
             const F2 v[2] = {f2_fma(qa[p + h], minus1, b[0]), f2_fma(qb[p + h], minus1, b[1])};
-            F2 wa = v[0], wb = v[1];
-            if constexpr (!MAXP) {  // pair_weights
-                const float vmax = team_max<L>(f2_max<4>(v)), n = -vmax * c;
-                if (vmax == kNegInf) rare |= 1u << (p + h);
-                const float2 xa = f2_get(f2_fma(v[0], f2(c, c), f2(n, n))), xb = f2_get(f2_fma(v[1], f2(c, c), f2(n, n)));
-                wa = f2(ex2_ftz(xa.x), ex2_ftz(xa.y));
-                wb = f2(ex2_ftz(xb.x), ex2_ftz(xb.y));
+            float2 wa = f2_get(v[0]), wb = f2_get(v[1]);
+            if constexpr (!MAXP) {
+                vmax[h] = team_max<L>(f2_max<4>(v));
+                if (vmax[h] == kNegInf) rare |= 1u << (p + h);
+                wa = pair_weights(v[0], vmax[h], invT);
+                wb = pair_weights(v[1], vmax[h], invT);
             }
-            ulonglong2 w;
-            w.x = wa;
-            w.y = wb;
-            *reinterpret_cast<ulonglong2 *>(xs + h * xs_step + 4 * l) = w;
+            float4 *x = reinterpret_cast<float4 *>(xs + h * xs_step + 8 * l);
+            x[0] = make_float4(wa.x, wa.x, wa.y, wa.y);
+            x[1] = make_float4(wb.x, wb.x, wb.y, wb.y);
         }
         __syncwarp();
-        F2 acc[2][4];
+        F2 acc[2][2];
         float mxp[2][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            acc[0][i] = acc[1][i] = f2(0.f, 0.f);
-            mxp[0][i] = mxp[1][i] = kNegInf;
+        for (int h = 0; h < 2; ++h) {
+            acc[h][0] = acc[h][1] = f2(0.f, 0.f);
+            mxp[h][0] = mxp[h][1] = mxp[h][2] = mxp[h][3] = kNegInf;
         }
-        auto step = [&](int h, int i, const ulonglong2 a, const ulonglong2 w) {
+        auto step = [&](int h, const ulonglong2 a, const F2 w) {
             if constexpr (MAXP) {  // pair_max
-                const float2 x = f2_get(f2_add(a.x, w.x)), y = f2_get(f2_add(a.y, w.y));
-                mxp[h][i] = fmaxf(fmaxf(mxp[h][i], x.x), x.y);
-                mxp[h][i] = fmaxf(fmaxf(mxp[h][i], y.x), y.y);
+                const float2 x = f2_get(f2_add(a.x, w)), y = f2_get(f2_add(a.y, w));
+                mxp[h][0] = fmaxf(mxp[h][0], x.x);
+                mxp[h][1] = fmaxf(mxp[h][1], x.y);
+                mxp[h][2] = fmaxf(mxp[h][2], y.x);
+                mxp[h][3] = fmaxf(mxp[h][3], y.y);
             } else {  // pair_linear
-                acc[h][i] = f2_fma(a.y, w.y, f2_fma(a.x, w.x, acc[h][i]));
+                acc[h][0] = f2_fma(a.x, w, acc[h][0]);
+                acc[h][1] = f2_fma(a.y, w, acc[h][1]);
             }
         };
-        const ulonglong2 *S4 = reinterpret_cast<const ulonglong2 *>(side0 ? S1 : S0) + l;
+        const ulonglong2 *S4 = reinterpret_cast<const ulonglong2 *>(side0 ? S1 : S0) + l;  // row s: S4[s L]
         if (__all_sync(0xffffffffu, side0 == side1 || p + 1 >= t.deg)) {  // one reading of the table for both
 #pragma unroll
-            for (int cc = 0; cc < K / 4; ++cc) {
-                const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(xs + 4 * cc);
-                const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(xs + xs_step + 4 * cc);
+            for (int c = 0; c < K / 4; ++c)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const ulonglong2 a = S4[(4 * cc + i) * L];
-                    step(0, i, a, w0);
-                    step(1, i, a, w1);
+                for (int i = 2; i >= 0; i -= 2) {  // sources 4 c + 3, 4 c + 2, then 4 c + 1, 4 c
+                    const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(xs + 2 * (4 * c + i));
+                    const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(xs + xs_step + 2 * (4 * c + i));
+                    const ulonglong2 hi = S4[(4 * c + i + 1) * L], lo = S4[(4 * c + i) * L];
+                    step(0, hi, w0.y);
+                    step(1, hi, w1.y);
+                    step(0, lo, w0.x);
+                    step(1, lo, w1.x);
                 }
-            }
         } else {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if (h == 1) S4 = reinterpret_cast<const ulonglong2 *>(side1 ? S1 : S0) + l;
 #pragma unroll
-                for (int cc = 0; cc < K / 4; ++cc) {
-                    const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(xs + h * xs_step + 4 * cc);
+                for (int c = 0; c < K / 4; ++c)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) step(h, i, S4[(4 * cc + i) * L], w);
-                }
+                    for (int i = 2; i >= 0; i -= 2) {
+                        const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(xs + h * xs_step + 2 * (4 * c + i));
+                        step(h, S4[(4 * c + i + 1) * L], w.y);
+                        step(h, S4[(4 * c + i) * L], w.x);
+                    }
             }
         }
 #pragma unroll
@@ -272,18 +275,12 @@ __device__ __forceinline__ unsigned team_edges(const TeamVar &t, const float (&e
             if constexpr (MAXP) {
                 o[0] = f2(mxp[h][0], mxp[h][1]);
                 o[1] = f2(mxp[h][2], mxp[h][3]);
-                none = team_normalise<L>(o) == kNegInf;
             } else {
-                float r[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float2 a = f2_get(acc[h][i]);
-                    r[i] = a.x + a.y;
-                }
-                o[0] = f2_mul(f2(T, T), f2_log(f2(r[0], r[1])));
-                o[1] = f2_mul(f2(T, T), f2_log(f2(r[2], r[3])));
+                o[0] = pair_log(acc[h][0], T, vmax[h], tmax);
+                o[1] = pair_log(acc[h][1], T, vmax[h], tmax);
             }
             // pair_finish
+            none = team_normalise<L>(o) == kNegInf;
             if (damping != 0.f) {
                 const float w = 1.f - damping;
                 o[0] = f2_fma(f2(damping, damping), mo[0], f2_mul(f2(w, w), o[0]));
@@ -306,19 +303,19 @@ __device__ __forceinline__ unsigned team_edges(const TeamVar &t, const float (&e
     return rare;
 }
 
-template <int K, bool MAXP, bool MS>
-__global__ void __launch_bounds__(kThreads, K == 16 ? 4 : 5)
+// NT: threads of a block.
+template <int K, bool MAXP, bool MS, int NT>
+__global__ void __launch_bounds__(NT, (K == 16 ? 1024 : 1280) / NT)
 k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ blocks, const int32_t *__restrict__ list,
              const float *__restrict__ pot, const float *__restrict__ ev, const float *__restrict__ m_old,
              float *__restrict__ m_new, float T, float invT, float damping) {
     constexpr int L = K / 4;                  // lanes per variable
-    constexpr int kStep = kThreads / L;       // variables per round of the block
-    constexpr int kRow = K == 4 ? 4 : K + 4;  // a team's exchange row: no bank conflicts between teams
+    constexpr int kStep = NT / L;       // variables per round of the block
+    constexpr int kRow = K == 4 ? 8 : 2 * K + 4;  // a team's exchange row: few bank conflicts between teams
     __shared__ __align__(16) float S0[K * K], S1[K * K];
     __shared__ __align__(16) float xch[2 * kStep * kRow];
     __shared__ float tab[K * K];
-    __shared__ float red[2 * kThreads / 32];
-    pdl_launch_dependents();  // the next launch may be scheduled (it waits likewise)
+    __shared__ float red[2 * NT / 32];
     if constexpr (MS) {  // multi-sample launches: this block's sample
         const int64_t smp = blockIdx.y;
         pot += smp * G.s_pot;
@@ -333,19 +330,20 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
     float *xs = xch + team * kRow;
     TeamVar t = team_var(G, list, B.x + (team < n ? team : 0), team < n, es_base);
     int vs = __ldg(G.vs_off + t.v);
-    pair_tables_load<K, kThreads>(pot + B.w, tab);
+    pair_tables_load<K, NT>(pot + B.w, tab);
     pdl_wait();  // messages of the previous launch
     __syncthreads();
     if (member_skip<MAXP>(G, __ldg(&blocks[blockIdx.x].member), T, invT, damping)) return;  // the whole block
-    const bool lin = pair_tables_make<K, MAXP, kThreads>(tab, S0, S1, red, invT);
+    const bool lin = pair_tables_make<K, MAXP, NT>(tab, S0, S1, red, invT);
     if (!MAXP && !lin) {
-        for (int k = threadIdx.x; k < 4 * n; k += kThreads) {
+        for (int k = threadIdx.x; k < 4 * n; k += NT) {
             const int pos = B.x + (k >> 2), v = list ? __ldg(list + pos) : pos;
             if ((k & 3) < __ldg(G.vin_off + v + 1) - __ldg(G.vin_off + v))
                 fused_edge<K, MAXP>(G, tab, ev, m_old, m_new, v, k & 3, es_base, T, invT, damping);
         }
         return;
     }
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
     // rows are 16-byte aligned or not for the whole run (K is a multiple of 4)
     const bool al = ((reinterpret_cast<uintptr_t>(m_old + es_base) | reinterpret_cast<uintptr_t>(m_new + es_base) |
                       reinterpret_cast<uintptr_t>(ev + vs)) & 15u) == 0;
@@ -360,7 +358,8 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
                 if (i < t.deg) row_load<true>(q[i], m_old + t.es[i] + 4 * l);
                 else q[i][0] = q[i][1] = q[i][2] = q[i][3] = 0.f;  // adds exactly nothing
             }
-            rare = team_edges<K, MAXP, true>(t, e4, q, l, es_base, S0, S1, xs, kStep * kRow, m_old, m_new, T, invT, damping);
+            rare = team_edges<K, MAXP, true>(t, e4, q, l, es_base, S0, S1, red[0], xs, kStep * kRow, m_old, m_new, T, invT,
+                                             damping);
         } else {
             row_load<false>(e4, ev + vs + 4 * l);
 #pragma unroll
@@ -368,12 +367,14 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
                 if (i < t.deg) row_load<false>(q[i], m_old + t.es[i] + 4 * l);
                 else q[i][0] = q[i][1] = q[i][2] = q[i][3] = 0.f;
             }
-            rare = team_edges<K, MAXP, false>(t, e4, q, l, es_base, S0, S1, xs, kStep * kRow, m_old, m_new, T, invT, damping);
+            rare = team_edges<K, MAXP, false>(t, e4, q, l, es_base, S0, S1, red[0], xs, kStep * kRow, m_old, m_new, T, invT,
+                                             damping);
         }
         if (rare != 0 && l == 0)
 #pragma unroll 1
             for (int i = 0; i < t.deg; ++i)
                 if ((rare >> i) & 1) fused_edge<K, MAXP>(G, tab, ev, m_old, m_new, t.v, i, es_base, T, invT, damping);
+        if (j - team + kStep >= n && !pdl_small()) pdl_launch_dependents();
         if (j - team + kStep < n) {  // the next round's variable
             const int jn = j + kStep;
             t = team_var(G, list, B.x + (jn < n ? jn : 0), jn < n, es_base);
@@ -387,15 +388,16 @@ cudaError_t launch_k(const DevGraph &G, const FactorLaunch &L, const float *pot,
                      float *m_new, float T, float damping, int S, cudaStream_t s) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)L.fuse_blocks, (unsigned)S);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned)L.fuse_threads);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_pair_fused<K, MAXP, MS>, G, L.fuse, L.fuse_list, pot, ev, m_old, m_new, T,
-                              MAXP ? 0.f : 1.f / T, damping);
+    auto kern = L.fuse_threads == 128 ? k_pair_fused<K, MAXP, MS, 128> : k_pair_fused<K, MAXP, MS, 256>;
+    return cudaLaunchKernelEx(&cfg, kern, G, L.fuse, L.fuse_list, pot, ev, m_old, m_new, T, MAXP ? 0.f : 1.f / T,
+                              damping);
 }
 
 template <int K>

@@ -6,14 +6,12 @@
 //
 // What bounds it: the bytes a warp takes from shared memory (the return path gives 128 a
 // cycle, broadcast or not) and issue slots. At K = 16 the direction is 256 multiply-adds, 16
-// exponentials and 16 logarithms; with scalar FMAs, logf and the guarded exponential a factor took 2,760
-// instructions. Here:
-//   - two sources share an instruction (fma.rn.f32x2 and its add and mul, Blackwell's packed
-//     FP32, rounding each half as the scalar does): the sums over even and odd sources side by
-//     side, added at the end; weights and table entries pair up as they lie in memory;
-//   - the weights are one FMA and one ex2.approx each; the constant -vmax c is rounded once for
-//     all of a message's weights, a common factor that the normalisation removes;
-//   - log is a degree-8 polynomial (below), packed, without logf's range checks.
+// exponentials and 16 logarithms. Here two targets share an instruction (fma.rn.f32x2 and its add
+// and mul, Blackwell's packed FP32, rounding each half as the scalar does), and the tables are
+// stored source-major so that a 16-byte load brings four targets of one source. The operations
+// and their order are the scalar form's (w = __expf, sources 3, 2, 1, 0, 7, 6, ..., T logf(s) + max
+// v + max phi, two normalisations): grids with strong couplings amplify any change of rounding by
+// 10^4 over 100 iterations. (A polynomial logarithm and one normalisation measured 1.2x faster.)
 #pragma once
 
 #include "bp_common.cuh"
@@ -60,106 +58,82 @@ __device__ __forceinline__ float f2_max(const F2 (&a)[K / 2]) {
     return mx;
 }
 
-// Natural logarithm of two positive normal numbers (NaN stays NaN): s = 2^e m with m in
-// [2/3, 4/3), log s = e ln 2 + f + f^2 Q(f), f = m - 1. Q (degree 8) is a fit of
-// (log1p(f) - f) / f^2 on [-1/3, 1/3] made for this file by iteratively reweighted least
-// squares of the relative error (4.5e-9). Error against FP64 over s = e^-60 .. e^3: at most
-// 0.94 ulp, mean 0.26 ulp, mean signed -7e-4 ulp (no bias to accumulate over iterations, which
-// lg2.approx has).
-__device__ __forceinline__ F2 f2_log(F2 s) {
-    const float2 sv = f2_get(s);
-    const int ia = __float_as_int(sv.x), ib = __float_as_int(sv.y);
-    const int ea = (ia - 0x3f2aaaab) & (int)0xff800000, eb = (ib - 0x3f2aaaab) & (int)0xff800000;
-    const F2 m = f2(__int_as_float(ia - ea), __int_as_float(ib - eb));
-    const F2 e = f2((float)ea, (float)eb);  // 2^23 e
-    const F2 f = f2_add(m, f2(-1.f, -1.f));
-    F2 q = f2(-0.12948694825172424f, -0.12948694825172424f);
-    q = f2_fma(q, f, f2(0.14004768431186676f, 0.14004768431186676f));
-    q = f2_fma(q, f, f2(-0.12167218327522278f, -0.12167218327522278f));
-    q = f2_fma(q, f, f2(0.14001157879829407f, 0.14001157879829407f));
-    q = f2_fma(q, f, f2(-0.16682301461696625f, -0.16682301461696625f));
-    q = f2_fma(q, f, f2(0.20010748505592346f, 0.20010748505592346f));
-    q = f2_fma(q, f, f2(-0.24999716877937317f, -0.24999716877937317f));
-    q = f2_fma(q, f, f2(0.3333320915699005f, 0.3333320915699005f));
-    q = f2_fma(q, f, f2(-0.5f, -0.5f));
-    F2 r = f2_fma(f2_mul(f, f), q, f);
-    r = f2_fma(e, f2(8.262958294867817e-08f, 8.262958294867817e-08f), r);  // 2^-23 ln 2
-    return f2_fma(s, f2(0.f, 0.f), r);  // NaN through
-}
-
 __device__ __forceinline__ float ex2_ftz(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 
-// The weights exp((v - max v) / T); false when every v is -inf.
+// Two weights exp((v - vmax) / T) (__expf, but a result below the normal numbers is 0: beside the
+// largest weight, 1, it adds nothing).
+__device__ __forceinline__ float2 pair_weights(F2 v, float vmax, float invT) {
+    const F2 x = f2_mul(f2_mul(f2_add(v, f2(-vmax, -vmax)), f2(invT, invT)), f2(1.4426950408889634f, 1.4426950408889634f));
+    const float2 q = f2_get(x);
+    return make_float2(ex2_ftz(q.x), ex2_ftz(q.y));
+}
+
+// Two outputs of the linear form from their sums.
+__device__ __forceinline__ F2 pair_log(F2 s, float T, float vmax, float tmax) {
+    const float2 q = f2_get(s);
+    return f2_add(f2_fma(f2(T, T), f2(logf(q.x), logf(q.y)), f2(vmax, vmax)), f2(tmax, tmax));
+}
+
+// Linear form (sum-product, a shared table of range at most 60 T): S[s K + t] = exp((phi(s, t) -
+// tmax) / T) in shared memory, 16-byte aligned, tmax = max phi; o = T log(sum_s S(s, t) w(s)) + vmax +
+// tmax. The sum is at least exp(-range / T), a normal number.
 template <int K>
-__device__ __forceinline__ bool pair_weights(const F2 (&v)[K / 2], float (&w)[K], float invT) {
+__device__ __forceinline__ void pair_linear(const F2 (&v)[K / 2], F2 (&o)[K / 2], const float *S, float tmax, float T,
+                                            float invT) {
     const float vmax = f2_max<K>(v);
-    if (vmax == kNegInf) return false;
-    const float c = invT * 1.4426950408889634f, n = -vmax * c;
-    const F2 c2 = f2(c, c), n2 = f2(n, n);
-#pragma unroll
-    for (int i = 0; i < K / 2; ++i) {
-        const float2 q = f2_get(f2_fma(v[i], c2, n2));
-        w[2 * i] = ex2_ftz(q.x);
-        w[2 * i + 1] = ex2_ftz(q.y);
-    }
-    return true;
-}
-
-// Tables in shared memory: 16-byte chunks of four sources for one target, target t = 4 l + i and
-// sources 4 c .. 4 c + 3 at chunk (4 c + i) (K / 4) + l, so that lanes l = 0 .. K / 4 - 1 that own
-// four targets each read neighbouring chunks.
-template <int K>
-__device__ __forceinline__ int table_chunk(int t, int c) {
-    return (4 * c + (t & 3)) * (K / 4) + (t >> 2);
-}
-
-// Linear form (sum-product, a shared table of range at most 60 T): S holds exp((phi(s, t) - max
-// phi) / T); o = T log(sum_s S(s, t) w(s)). The sum is at least exp(-range / T), a normal number.
-template <int K>
-__device__ __forceinline__ void pair_linear(const F2 (&v)[K / 2], F2 (&o)[K / 2], const float *S, float T, float invT) {
-    float w[K];
-    if (!pair_weights<K>(v, w, invT)) {
+    if (vmax == kNegInf) {
 #pragma unroll
         for (int i = 0; i < K / 2; ++i) o[i] = f2(kNegInf, kNegInf);
         return;
     }
-    const ulonglong2 *S4 = reinterpret_cast<const ulonglong2 *>(S);
-    float r[K];
+    float w[K];
 #pragma unroll
-    for (int t = 0; t < K; ++t) {
-        F2 acc = f2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < K / 4; ++c) {
-            const ulonglong2 a = S4[table_chunk<K>(t, c)];
-            acc = f2_fma(a.x, f2(w[4 * c], w[4 * c + 1]), acc);
-            acc = f2_fma(a.y, f2(w[4 * c + 2], w[4 * c + 3]), acc);
-        }
-        const float2 q = f2_get(acc);
-        r[t] = q.x + q.y;
+    for (int i = 0; i < K / 2; ++i) {
+        const float2 q = pair_weights(v[i], vmax, invT);
+        w[2 * i] = q.x;
+        w[2 * i + 1] = q.y;
+        o[i] = f2(0.f, 0.f);
     }
-    const F2 T2 = f2(T, T);
 #pragma unroll
-    for (int i = 0; i < K / 2; ++i) o[i] = f2_mul(T2, f2_log(f2(r[2 * i], r[2 * i + 1])));
+    for (int j = 0; j < K / 4; ++j)
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+            const ulonglong2 *row = reinterpret_cast<const ulonglong2 *>(S + (4 * j + i) * K);
+            const F2 ws = f2(w[4 * j + i], w[4 * j + i]);
+#pragma unroll
+            for (int q = 0; q < K / 4; ++q) {
+                const ulonglong2 a = row[q];
+                o[2 * q] = f2_fma(a.x, ws, o[2 * q]);
+                o[2 * q + 1] = f2_fma(a.y, ws, o[2 * q + 1]);
+            }
+        }
+#pragma unroll
+    for (int i = 0; i < K / 2; ++i) o[i] = pair_log(o[i], T, vmax, tmax);
 }
 
-// Max-product with a shared table, S holding phi(s, t).
+// Max-product with a shared table, S[s K + t] = phi(s, t) in shared memory.
 template <int K>
 __device__ __forceinline__ void pair_max(const F2 (&v)[K / 2], F2 (&o)[K / 2], const float *S) {
-    const ulonglong2 *S4 = reinterpret_cast<const ulonglong2 *>(S);
     float m[K];
 #pragma unroll
-    for (int t = 0; t < K; ++t) {
-        m[t] = kNegInf;
+    for (int t = 0; t < K; ++t) m[t] = kNegInf;
 #pragma unroll
-        for (int c = 0; c < K / 4; ++c) {
-            const ulonglong2 a = S4[table_chunk<K>(t, c)];
-            const float2 x = f2_get(f2_add(a.x, v[2 * c])), y = f2_get(f2_add(a.y, v[2 * c + 1]));
-            m[t] = fmaxf(fmaxf(m[t], x.x), x.y);
-            m[t] = fmaxf(fmaxf(m[t], y.x), y.y);
+    for (int s = 0; s < K; ++s) {
+        const ulonglong2 *row = reinterpret_cast<const ulonglong2 *>(S + s * K);
+        const float2 p = f2_get(v[s / 2]);
+        const F2 vs = (s & 1) ? f2(p.y, p.y) : f2(p.x, p.x);
+#pragma unroll
+        for (int q = 0; q < K / 4; ++q) {
+            const ulonglong2 a = row[q];
+            const float2 x = f2_get(f2_add(a.x, vs)), y = f2_get(f2_add(a.y, vs));
+            m[4 * q] = fmaxf(m[4 * q], x.x);
+            m[4 * q + 1] = fmaxf(m[4 * q + 1], x.y);
+            m[4 * q + 2] = fmaxf(m[4 * q + 2], y.x);
+            m[4 * q + 3] = fmaxf(m[4 * q + 3], y.y);
         }
     }
 #pragma unroll
@@ -193,11 +167,9 @@ __device__ __forceinline__ void f2_normalise(F2 (&t)[K / 2], uint32_t *flags) {
 #pragma unroll
     for (int i = 0; i < K / 2; ++i) t[i] = f2_add(t[i], n);
 }
-// The linear form's outputs (in [-60 - T log K, T log K]) need no first normalisation: it would add
-// a constant that the second removes.
-template <int K, bool TWICE = true>
+template <int K>
 __device__ __forceinline__ void pair_finish(F2 (&o)[K / 2], const F2 (&mo)[K / 2], float damping, uint32_t *flags) {
-    if (TWICE) f2_normalise<K>(o, flags);
+    f2_normalise<K>(o, flags);
     if (damping != 0.f) {
         const float w = 1.f - damping;
         const F2 d2 = f2(damping, damping), w2 = f2(w, w);
@@ -260,19 +232,15 @@ __device__ __noinline__ void pair_dir_rare(const DevGraph &G, const float *phi, 
 // the new message goes to m_new + es_t. lin: S holds the linear table; else, for max-product
 // with a shared table, phi itself; else phi entry by entry.
 template <int K, bool MAXP>
-__device__ __forceinline__ void pair_direction(const F2 (&v)[K / 2], bool lin, bool shared, const float *S,
+__device__ __forceinline__ void pair_direction(const F2 (&v)[K / 2], bool lin, float tmax, bool shared, const float *S,
                                                const float *phi, int step_s, int step_t, const float *m_old,
                                                float *m_new, int es_t, float T, float invT, float damping,
                                                uint32_t *flags) {
     F2 o[K / 2], mo[K / 2];
     f2_load<K>(mo, m_old + es_t);
     if (!MAXP && lin) {
-        pair_linear<K>(v, o, S, T, invT);
-        pair_finish<K, false>(o, mo, damping, flags);
-        f2_store<K>(m_new + es_t, o);
-        return;
-    }
-    if (MAXP && shared) {
+        pair_linear<K>(v, o, S, tmax, T, invT);
+    } else if (MAXP && shared) {
         pair_max<K>(v, o, S);
     } else {
         float vv[K], oo[K];
@@ -291,14 +259,13 @@ __device__ __forceinline__ void pair_direction(const F2 (&v)[K / 2], bool lin, b
 }
 
 // A group's shared table for a block (all threads): the raw entries in tab (row-major) and, for
-// the fast forms, the chunked tables S0 (source: variable 0) and S1 (source: variable 1):
-// exp((phi - max) / T) when lin (returned: sum-product and a range of at most 60 T), phi for
-// max-product. red: 2 floats per warp.
+// the fast forms, source-major tables S0 (source: variable 0) and S1 (source: variable 1):
+// exp((phi - max) / T) when lin (returned: sum-product and a range of at most 60 T, red[0] = max),
+// phi for max-product. red: 2 floats per warp.
 template <int K>
 __device__ __forceinline__ void table_store(float *S0, float *S1, int i, float e) {
-    const int x = i / K, y = i % K;  // states of variable 0 and 1
-    S0[4 * table_chunk<K>(y, x >> 2) + (x & 3)] = e;
-    S1[4 * table_chunk<K>(x, y >> 2) + (y & 3)] = e;
+    S0[i] = e;
+    S1[(i % K) * K + i / K] = e;
 }
 // The raw entries (pair_tables_load), then, after a barrier, the fast forms' (pair_tables_make).
 // NT: threads of the block, 0 if known at run time only.
@@ -336,6 +303,8 @@ __device__ __forceinline__ bool pair_tables_make(const float *tab, float *S0, fl
         lin = isfinite(mx) && isfinite(mn) && (mx - mn) * invT <= 60.f;
         if (lin)
             for (int i = threadIdx.x; i < K * K; i += nt) table_store<K>(S0, S1, i, expf((tab[i] - mx) * invT));
+        __syncthreads();
+        if (threadIdx.x == 0) red[0] = mx;
     }
     __syncthreads();
     return lin;

@@ -163,7 +163,7 @@ struct FactorLaunch {
     // fused form of a dense pairwise launch
     const FuseBlock *fuse;      // device
     const int32_t *fuse_list;   // the variables' bucket (device; null: identity)
-    int32_t fuse_blocks;        // 0: not eligible
+    int32_t fuse_blocks, fuse_threads;  // blocks (0: not eligible), threads of each (128 or 256)
 };
 
 inline bool is_fused(int variant) { return variant == kPairF4 || variant == kPairF8 || variant == kPairF16; }
@@ -340,8 +340,11 @@ cudaError_t launch_lr_unpack(const DevGraph &G, const float *d, float *m, cudaSt
 constexpr int kLrRunThreads = 1024, kLrSmallMaxV = 1024, kLrSmallMaxF = 2048;
 constexpr int kLrClusterMax = 16;
 int lr_cluster_size();
-// Setting 1 of PGM_OPT_SMALL_RUN: one block up to this many variables, the cluster above.
-constexpr int kLrBlockAutoV = 700;
+// Setting 1 of PGM_OPT_SMALL_RUN: one block up to this many variables and factors, the cluster
+// up to kLrClusterAutoV variables, the grid form above (us per iteration, T = 1, square grids:
+// 22 x 22 block 0.65, cluster 0.82; 24 x 24 1.03, 0.81; 90 x 90 cluster 1.17; 128 x 128 cluster
+// 1.75, grid 1.22).
+constexpr int kLrBlockAutoV = 700, kLrBlockAutoF = 1024, kLrClusterAutoV = 9000;
 inline bool lr_block_fits(int V, int F) { return V > 0 && V <= kLrSmallMaxV && F <= kLrSmallMaxF; }
 inline bool lr_cluster_fits(int V, int F) {
     const int C = lr_cluster_size();
