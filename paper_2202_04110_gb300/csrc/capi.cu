@@ -391,6 +391,27 @@ void plan_fused(const HostLayout &H, pgm_graph *g, Packer &pk) {
     }
 }
 
+// The max-product pairs form (k_enum_pairs) of a block-form launch: every group a packed pairwise
+// list with one shared table and a state sum up to kEnumWarpStateSum, and enough factors that
+// four per warp leave every SM a block (fewer are faster one per warp).
+static void plan_enum_pairs(FactorLaunch &L, const EnumSeg *segs, int n_seg, int n_sm) {
+    L.pairs_blocks = L.pairs_smem = L.pairs_rows = 0;
+    int64_t blocks = 0, smem = 0;
+    int32_t rows = 0;
+    for (int i = 0; i < n_seg; ++i) {
+        const EnumSeg &sg = segs[i];
+        if (!sg.packed || !sg.shared || sg.arity != 2 || sg.es_per_fac > kEnumWarpStateSum) return;
+        blocks += (sg.n_fac + kEnumPairsBlock - 1) / kEnumPairsBlock;
+        const int64_t k4 = (sg.es_per_fac + 3) & ~3, ob = (sg.es_per_fac + 1 + 3) & ~3;
+        smem = std::max(smem, (kEnumBlockThreads / 32) * 20 * k4 + 4 * ob + 16 * (int64_t)sg.n_cfg);
+        rows = std::max(rows, (sg.es_per_fac + 31) / 32);
+    }
+    if (blocks < n_sm || smem > kEnumTableSmem) return;
+    L.pairs_blocks = (int32_t)blocks;
+    L.pairs_smem = (int32_t)smem;
+    L.pairs_rows = rows;
+}
+
 pgm_status build_plan(const HostLayout &H, pgm_graph *g, Packer &pk, std::vector<size_t> &seg_off,
                       std::vector<int> &seg_kind) {
     // variable pass: one launch per non-empty bucket of variables
@@ -401,6 +422,8 @@ pgm_status build_plan(const HostLayout &H, pgm_graph *g, Packer &pk, std::vector
         VarLaunch L{};
         L.kind = kind;
         L.fused_by = -1;
+        if (kind == kVarWarp)
+            for (int32_t v : bucket) L.max_k = std::max(L.max_k, H.vs_off[v + 1] - H.vs_off[v]);
         L.n = (int32_t)bucket.size();
         L.threads = 256;
         L.n_blocks = (kind == kVarBlock) ? L.n : (int32_t)(((int64_t)L.n * var_lanes(kind) + 255) / 256);
@@ -542,8 +565,10 @@ pgm_status build_plan(const HostLayout &H, pgm_graph *g, Packer &pk, std::vector
                 segs.push_back(s);
             }
             if (segs.empty()) continue;
-            if (variant == kEnumBlock)
+            if (variant == kEnumBlock) {
                 blk = plan_enum_block(segs.data(), (int)segs.size(), threads, g->n_sm, false, &L.smem);
+                plan_enum_pairs(L, segs.data(), (int)segs.size(), g->n_sm);
+            }
             L.n_seg = (int32_t)segs.size();
             L.n_blocks = blk;
             L.threads = threads;
@@ -861,7 +886,7 @@ static pgm_status build_from_layout(const HostLayout &H, pgm_graph **out, cudaSt
         } else {
             FactorLaunch &L = g->P.factor[fi++];
             L.segs = dmem + seg_off[k];
-            max_smem = std::max(max_smem, L.smem);
+            max_smem = std::max({max_smem, L.smem, L.pairs_smem});
         }
     }
     for (const auto &f : g->fused) {
@@ -1971,7 +1996,8 @@ static bool replan_factor_launch(pgm_graph *g, size_t li, int threads, cudaStrea
         blk = plan_enum_block(reinterpret_cast<EnumSeg *>(host.data()), L.n_seg, threads, g->n_sm,
                               L.base_variant == kEnumGeneric, &sm);
         smem = (size_t)sm;
-        if (prepare_kernels(sm) != cudaSuccess) return false;
+        plan_enum_pairs(L, reinterpret_cast<const EnumSeg *>(host.data()), L.n_seg, g->n_sm);
+        if (prepare_kernels(std::max(sm, L.pairs_smem)) != cudaSuccess) return false;
     } else {
         EnumSeg *segs = reinterpret_cast<EnumSeg *>(host.data());
         for (int i = 0; i < L.n_seg; ++i) {

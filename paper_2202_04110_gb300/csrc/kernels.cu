@@ -173,7 +173,11 @@ __global__ void __launch_bounds__(256) k_var_thread(DevGraph G, const int32_t *_
 // bits (normalised beliefs sum e^r in another order). The iteration also writes b_lo,
 // the rounding residual of each value, so that a factor can form b - m without the
 // cancellation a large message would cause.
-template <int MODE, bool MS = false>
+// R: rounds of 32 states (2, 4 or 8, by the launch's largest variable). The incoming edges are
+// read by the lanes at once and four edges' messages are in flight: one edge after the other,
+// index then message, made the pass a chain of eight L2 latencies (16,384 variables of 49
+// states: 26.6 -> 14.6 us).
+template <int MODE, bool MS, int R>
 __global__ void __launch_bounds__(256) k_var_warp(DevGraph G, const int32_t *__restrict__ list, int n,
                                                   const float *__restrict__ ev, const float *__restrict__ m,
                                                   float *__restrict__ out, int32_t *__restrict__ dec) {
@@ -191,19 +195,32 @@ __global__ void __launch_bounds__(256) k_var_warp(DevGraph G, const int32_t *__r
     const int v = list ? __ldg(list + w) : w;
     const int k0 = __ldg(G.vin_off + v), k1 = __ldg(G.vin_off + v + 1);
     const int vs = __ldg(G.vs_off + v), K = __ldg(G.vs_off + v + 1) - vs;
-    constexpr int R = kMaxStates / 32;
     FF s[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int x = lane + 32 * r;
         s[r] = ff_make(x < K ? __ldg(ev + vs + x) : kNegInf);
     }
-    for (int k = k0; k < k1; ++k) {
-        const int es = __ldg(G.vin_es + k);
+    for (int kb = k0; kb < k1; kb += 32) {
+        const int mine = kb + lane < k1 ? __ldg(G.vin_es + kb + lane) : 0, nk = min(32, k1 - kb);
+        for (int k = 0; k < nk; k += 4) {
+            float q[4][R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int x = lane + 32 * r;
-            if (x < K) s[r] = ff_add(s[r], __ldg(m + es + x));
+            for (int i = 0; i < 4; ++i) {
+                const int es = __shfl_sync(0xffffffffu, mine, k + i);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int x = lane + 32 * r;
+                    q[i][r] = k + i < nk && x < K ? __ldg(m + es + x) : 0.f;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (k + i < nk) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        if (lane + 32 * r < K) s[r] = ff_add(s[r], q[i][r]);
+                }
         }
     }
     FF best = ff_make(kNegInf);
@@ -1620,7 +1637,7 @@ k_enum_generic(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const fl
 // does, and the two give the same bits; otherwise T > 0 differs by rounding.
 // v2f_slow_edge for the edge of variable v, the states spread over the lanes of a warp
 // (same sums, same bits).
-__device__ __noinline__ void v2f_slow_edge_warp(const DevGraph G, const float *__restrict__ ev,
+__device__ __noinline__ void v2f_slow_edge_warp(const DevGraph &G, const float *__restrict__ ev,
                                                 const float *__restrict__ m, int v, int vs, int es, int K,
                                                 float *out, int lane) {
     const int k0 = G.vin_off[v], k1 = G.vin_off[v + 1];
@@ -1981,6 +1998,187 @@ k_enum_block(DevGraph G, const EnumSeg *__restrict__ segs, int n_seg, const floa
             for (int r = 0; r < kMaxStates / 32; ++r) {
                 const int x = lane + 32 * r;
                 if (x < K) m_new[es + x] = mx2 == kNegInf ? 0.f : v[r] - mx2;
+            }
+        }
+    }
+}
+
+// ---- max-product over shared pairwise lists, four factors per warp ----------------------
+//
+// The block form above walks a factor's lists one factor at a time: every entry costs an
+// 8-byte read of the list and a 4-byte gather of the other state's value, and that shared
+// memory traffic bounds it (250 wavefronts per factor of 2 x 49 states and 361
+// configurations). Here a warp takes four consecutive factors of a group at once, their values
+// side by side in 16-byte rows, so that an entry is read once for four of them: lane l owns
+// the outputs l, l + 32, .. of all four. The values' loads are independent for four factors, and
+// the maxima of the normalisations are one redux.sync each. Maxima do not depend on their order,
+// so the messages are bitwise those of the block form. Measured on a 128 x 128 grid of 49 states
+// (32,512 factors): 59.7 -> 35.6 us per launch; below one block per SM the block form stays.
+__device__ __forceinline__ float warp_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+template <int R, bool MS>
+__global__ void __launch_bounds__(kEnumBlockThreads, R <= 4 ? 3 : 2)
+k_enum_pairs(const __grid_constant__ DevGraph Gc, const EnumSeg *__restrict__ segs, int n_seg,
+             const float *__restrict__ pot, const float *__restrict__ b, const float *__restrict__ ev,
+             const float *__restrict__ m_old, float *__restrict__ m_new, float T, float invT, float damping) {
+    pdl_wait();  // inputs of the previous launch
+    pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
+    DevGraph Gm;
+    if constexpr (MS) {  // multi-sample launches: this block's sample
+        Gm = Gc;
+        sample_select(Gm);
+    }
+    const DevGraph &G = MS ? Gm : Gc;
+    if constexpr (MS) {
+        const int64_t smp = blockIdx.y;
+        pot += smp * G.s_pot;
+        b += smp * G.s_vs;
+        ev += smp * G.s_vs;
+        m_old += smp * G.s_es;
+        m_new += smp * G.s_es;
+    }
+    extern __shared__ __align__(16) unsigned char eb_smem[];
+    __shared__ int sK[2], sKo[2];
+    __shared__ int s_fix[kEnumBlockThreads / 32][kMaxArity];
+    int si = 0, blk = blockIdx.x;  // kEnumPairsBlock factors per block, segment by segment
+    for (; si < n_seg - 1; ++si) {
+        const int nb = (__ldg(&segs[si].n_fac) + kEnumPairsBlock - 1) / kEnumPairsBlock;
+        if (blk < nb) break;
+        blk -= nb;
+    }
+    const EnumSeg *S = segs + si;
+    if (member_skip<true>(G, S->member, T, invT, damping)) return;  // the whole block
+    const int nc = __ldg(&S->n_cfg), ksum = __ldg(&S->es_per_fac), n_fac = __ldg(&S->n_fac);
+    const int K0 = __ldg(&S->K[0]);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x < 2) {
+        sK[threadIdx.x] = __ldg(&S->K[threadIdx.x]);
+        sKo[threadIdx.x] = __ldg(&S->Koff[threadIdx.x]);
+    }
+    // shared memory: per warp the four factors' values [ksum] (float4) and a spare [ksum]; the
+    // offsets of the lists; the entries (byte offset of the other state's row, log-potential)
+    const size_t per_warp = 20 * (size_t)((ksum + 3) & ~3);
+    float4 *v4 = reinterpret_cast<float4 *>(eb_smem + warp * per_warp);
+    float *spare = reinterpret_cast<float *>(v4 + ((ksum + 3) & ~3));
+    const int ob = (ksum + 1 + 3) & ~3;
+    int32_t *tbs = reinterpret_cast<int32_t *>(eb_smem + (kEnumBlockThreads / 32) * per_warp);
+    int2 *fl = reinterpret_cast<int2 *>(tbs + ob);
+    {
+        const int32_t *bs = G.bs_pool + __ldg(&S->bs_base);
+        const float *phi = pot + __ldg(&S->pot_base);
+        for (int i = threadIdx.x; i < ob; i += kEnumBlockThreads) tbs[i] = __ldg(bs + i);
+        for (int i = threadIdx.x; i < 2 * nc; i += kEnumBlockThreads) {
+            const int e = __ldg(bs + ob + i);
+            fl[i] = make_int2((e & 2047) * 16, __float_as_int(__ldg(phi + (e >> 11))));
+        }
+    }
+    const int f = blk * kEnumPairsBlock + 4 * warp;
+    const int es_f = __ldg(&S->es_base) + f * ksum, e_f = __ldg(&S->edge_base) + 2 * f;
+    const int nf = min(4, n_fac - f);  // (<= 0: a warp past the end)
+    float mo[4][R];
+    // (1) variable-to-factor values, as enum_team_v2f
+    if (nf > 0) {
+        bool rare = false;
+        int vs[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int e = e_f + 2 * min(i, nf - 1);
+            vs[i][0] = __ldg(G.edge_vs + e);
+            vs[i][1] = __ldg(G.edge_vs + e + 1);
+            rare |= (vs[i][0] < 0) | (vs[i][1] < 0);
+        }
+        const bool lo0 = G.b_lo != nullptr && K0 > 16, lo1 = G.b_lo != nullptr && ksum - K0 > 16;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int t = lane + 32 * r;
+            float v[4];
+            const bool one = t >= K0, lo = one ? lo1 : lo0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                mo[i][r] = 0.f;
+                v[i] = 0.f;
+                if (t < ksum) {
+                    mo[i][r] = __ldg(m_old + es_f + min(i, nf - 1) * ksum + t);
+                    const int at = one ? (vs[i][1] & 0x7fffffff) + t - K0 : (vs[i][0] & 0x7fffffff) + t;
+                    rare |= lo ? !isfinite(mo[i][r]) : needs_exact(mo[i][r]);
+                    v[i] = __ldg(b + at) - mo[i][r];
+                    if (lo) v[i] += __ldg(G.b_lo + at);
+                }
+            }
+            if (t < ksum) v4[t] = make_float4(v[0], v[1], v[2], v[3]);
+        }
+        rare = __any_sync(0xffffffffu, rare);
+        if (rare)  // explicit sums or totals of high-degree variables: one factor at a time
+            for (int i = 0; i < nf; ++i) {
+                __syncwarp();
+                enum_team_v2f(G, b, ev, m_old, e_f + 2 * i, es_f + i * ksum, 2, ksum, sK, sKo, spare, nullptr, s_fix[warp],
+                              true, lane, 32, 0, 1, lane);
+                for (int t = lane; t < ksum; t += 32) reinterpret_cast<float *>(v4 + t)[i] = spare[t];
+            }
+    }
+    __syncthreads();
+    if (nf <= 0) return;
+    // (2) every output over its list, for four factors
+    float out[4][R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int o = lane + 32 * r;
+        float4 mx = make_float4(kNegInf, kNegInf, kNegInf, kNegInf);
+        if (o < ksum) {
+            const int i1 = tbs[o + 1];
+#pragma unroll 4
+            for (int i = tbs[o]; i < i1; ++i) {
+                const int2 e = fl[i];
+                const float4 v = *reinterpret_cast<const float4 *>(reinterpret_cast<const unsigned char *>(v4) + e.x);
+                const float phi = __int_as_float(e.y);
+                mx.x = fmaxf(mx.x, phi + v.x);
+                mx.y = fmaxf(mx.y, phi + v.y);
+                mx.z = fmaxf(mx.z, phi + v.z);
+                mx.w = fmaxf(mx.w, phi + v.w);
+            }
+        }
+        out[0][r] = mx.x;
+        out[1][r] = mx.y;
+        out[2][r] = mx.z;
+        out[3][r] = mx.w;
+    }
+    // (3) normalise, damp, normalise
+    const float w = 1.f - damping;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (i >= nf) break;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float mx = kNegInf;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int o = lane + 32 * r;
+                if (o < ksum && (o >= K0) == (j == 1)) mx = fmaxf(mx, out[i][r]);
+            }
+            mx = warp_max(mx);
+            if (mx == kNegInf && lane == 0) atomicOr(G.flags, kFlagContradiction);
+            float mx2 = kNegInf;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int o = lane + 32 * r;
+                if (o < ksum && (o >= K0) == (j == 1)) {
+                    float y = mx == kNegInf ? 0.f : out[i][r] - mx;
+                    if (damping != 0.f) y = fmaf(damping, mo[i][r], w * y);
+                    out[i][r] = y;
+                    mx2 = fmaxf(mx2, y);
+                }
+            }
+            mx2 = warp_max(mx2);
+            if (mx2 == kNegInf && lane == 0) atomicOr(G.flags, kFlagContradiction);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int o = lane + 32 * r;
+                if (o < ksum && (o >= K0) == (j == 1))
+                    m_new[es_f + i * ksum + o] = mx2 == kNegInf ? 0.f : out[i][r] - mx2;
             }
         }
     }
@@ -3700,6 +3898,10 @@ cudaError_t prepare_kernels(int max_smem_bytes) {
     if ((e = allow((const void *)k_enum_block<false>)) != cudaSuccess) return e;
     if ((e = allow((const void *)k_logic_warp<true, true>)) != cudaSuccess) return e;
     if ((e = allow((const void *)k_logic_warp<false, true>)) != cudaSuccess) return e;
+    if ((e = allow((const void *)k_enum_pairs<4, false>)) != cudaSuccess) return e;
+    if ((e = allow((const void *)k_enum_pairs<8, false>)) != cudaSuccess) return e;
+    if ((e = allow((const void *)k_enum_pairs<4, true>)) != cudaSuccess) return e;
+    if ((e = allow((const void *)k_enum_pairs<8, true>)) != cudaSuccess) return e;
     if ((e = allow((const void *)k_enum_block<true, true>)) != cudaSuccess) return e;
     if ((e = allow((const void *)k_enum_block<false, true>)) != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) done[dev] = 1;
@@ -3761,9 +3963,11 @@ static void var_pass_mode(const DevGraph &G, const Plan &P, const float *ev, con
             case kVarGroup16:
                 launch_dep(k_var_group<16, MODE, MS>, dim3(dim3(L.n_blocks, S)), L.threads, 0, s, G, L.list, L.n, ev, m, out, dec);
                 break;
-            case kVarWarp:
-                launch_dep(k_var_warp<MODE, MS>, dim3(dim3(L.n_blocks, S)), L.threads, 0, s, G, L.list, L.n, ev, m, out, dec);
+            case kVarWarp: {
+                auto kern = L.max_k <= 64 ? k_var_warp<MODE, MS, 2> : L.max_k <= 128 ? k_var_warp<MODE, MS, 4> : k_var_warp<MODE, MS, 8>;
+                launch_dep(kern, dim3(dim3(L.n_blocks, S)), L.threads, 0, s, G, L.list, L.n, ev, m, out, dec);
                 break;
+            }
             default:
                 launch_dep(k_var_thread<0, MODE, MS>, dim3(dim3(L.n_blocks, S)), L.threads, 0, s, G, L.list, L.n, 0, ev, m, out, dec);
                 break;
@@ -3838,6 +4042,11 @@ static void factor_pass_t(const DevGraph &G, const Plan &P, const float *pot, co
                 launch_dep(k_enum_generic<MAXP, MS>, dim3(dim3(L.n_blocks, S)), L.threads, 0, s, G, es, L.n_seg, pot, b, ev, m_old, m_new, T, invT, damping);
                 break;
             case kEnumBlock:
+                if (MAXP && L.pairs_blocks > 0) {
+                    auto kern = L.pairs_rows <= 4 ? k_enum_pairs<4, MS> : k_enum_pairs<8, MS>;
+                    launch_dep(kern, dim3(L.pairs_blocks, S), kEnumBlockThreads, L.pairs_smem, s, G, es, L.n_seg, pot, b, ev, m_old, m_new, T, invT, damping);
+                    break;
+                }
                 launch_dep(k_enum_block<MAXP, MS>, dim3(dim3(L.n_blocks, S)), L.threads, L.smem, s, G, es, L.n_seg, pot, b, ev, m_old, m_new, T, invT, damping);
                 break;
             case kLogicSmall:

@@ -23,6 +23,7 @@ constexpr int kEnumBlockStateSum = 2048;  // block-per-factor form (kMaxArity x 
 constexpr int kEnumGenericMaxCfg = 256;   // longer configuration lists use the block form
 constexpr int kEnumBlockThreads = 256;
 constexpr int kEnumWarpStateSum = 256;  // block form: a warp per factor up to this state sum
+constexpr int kEnumPairsBlock = 32;         // factors per block of the max-product pairs form
 constexpr int kEnumTableSmem = 160 * 1024;  // largest configuration table staged per block
 constexpr int kMaxStates = 256;
 constexpr int kVarBlockDegree = 64;  // variables with more factors use a block each
@@ -160,6 +161,9 @@ struct FactorLaunch {
     int32_t max_blocks;  // K-lane pairwise launches: physical blocks (each walks a range
                          // of the n_blocks chunks)
     int32_t base_variant;  // the variant the compiler chose (before options and autotuning)
+    // max-product form of a block-form launch over shared pairwise lists (k_enum_pairs): blocks
+    // (0: not eligible), shared memory, rounds of 32 output states of the largest factor
+    int32_t pairs_blocks, pairs_smem, pairs_rows;
     // fused form of a dense pairwise launch
     const FuseBlock *fuse;      // device
     const int32_t *fuse_list;   // the variables' bucket (device; null: identity)
@@ -194,6 +198,7 @@ struct VarLaunch {
     // the list, tile, first DevGraph::hd_tot entry of the variable, its tile count)
     const int4 *tiles;
     int32_t n_tiles;
+    int32_t max_k;           // kVarWarp: the largest state count of the variables
     int32_t fused_by;        // index of the factor launch that replaces this one in an
                              // iteration while it has its fused form; -1: none
 };
