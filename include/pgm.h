@@ -282,6 +282,12 @@ pgm_status pgm_launch_times(pgm_graph *g, int32_t n, double *ms, int64_t *count,
  * call is recorded as a CUDA graph on first use of an argument tuple (up to 4 kept) and
  * replayed on the caller's stream; with it off, the scratch is a stream-ordered
  * allocation freed before the call's work ends.
+ * A binary pairwise graph whose variables have at most 4 factors each, every factor with its
+ * own table, runs the call as one kernel launch where PGM_OPT_SMALL_RUN and PGM_OPT_CUDA_GRAPH
+ * are on and the blocks of that option's forms hold it: each iteration's variable-to-factor
+ * log-ratios are kept instead of checkpoints (16 bytes per variable and iteration beside the
+ * scratch above, up to 1 GiB, else the launches). A table with a non-finite entry or an
+ * infinite message makes the same recorded call run the launches after all.
  * Every sum is taken in a fixed order, so repeated calls give the same bits: gradients of
  * log-potentials shared by a group of factors with a state sum up to 64 through warp
  * partials (each warp of 32 factors adds its contributions by a fixed shuffle tree, then

@@ -2276,6 +2276,75 @@ static pgm_status enqueue_grad(pgm_graph *g, const float *log_pot, const float *
     return st;
 }
 
+// The recorded gradient of a graph that takes the one-launch form: that launch, and the ordinary
+// launches in a conditional node that runs when the kernel has set its bail word. Work: the
+// launches' buffers, the word, the kernel's history.
+static pgm_status one_launch_grad(pgm_graph *g, const LrGradPlan &one, const float *log_pot, const float *evidence, float T,
+                                  float damping, int32_t n_iters, int32_t ckpt_every, const float *d_beliefs,
+                                  float *d_log_pot, float *d_evidence, size_t launches, cudaGraphExec_t *exec) {
+    cudaStream_t cs = g->capture_stream;
+    char *mem = static_cast<char *>(g->grad_mem);
+    int *bail = reinterpret_cast<int *>(mem + align_up(launches, 256));
+    float *hist = reinterpret_cast<float *>(mem + align_up(launches, 256) + 256);
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaGraphCreate(&graph, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphCreate");
+    auto failed = [&](cudaError_t err, const char *what) {
+        cudaGraphDestroy(graph);
+        return cuda_fail(err, what);
+    };
+    cudaGraphConditionalHandle h;
+    e = cudaGraphConditionalHandleCreate(&h, graph, 0, cudaGraphCondAssignDefault);
+    if (e != cudaSuccess) return failed(e, "cudaGraphConditionalHandleCreate");
+    e = cudaStreamBeginCaptureToGraph(cs, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return failed(e, "cudaStreamBeginCaptureToGraph");
+    cudaGraph_t captured = nullptr;
+    e = cudaMemsetAsync(bail, 0, sizeof(int), cs);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_log_pot, 0, (size_t)g->info.n_potentials * sizeof(float), cs);
+    if (e == cudaSuccess)
+        e = launch_lr_grad(g->G, g->P, one, log_pot, evidence, d_beliefs, d_log_pot, d_evidence, hist, bail, g->m_tmp,
+                           g->lr_d, g->lr_prm, T, damping, n_iters, cs);
+    if (e == cudaSuccess) e = launch_set_condition(h, bail, cs);
+    cudaError_t e2 = cudaStreamEndCapture(cs, &captured);
+    if (e == cudaSuccess) e = e2;
+    if (e != cudaSuccess) return failed(e, "one-launch gradient");
+    // the captured chain's last node
+    size_t n = 0;
+    e = cudaGraphGetNodes(graph, nullptr, &n);
+    std::vector<cudaGraphNode_t> nodes(n);
+    if (e == cudaSuccess) e = cudaGraphGetNodes(graph, nodes.data(), &n);
+    cudaGraphNode_t last = nullptr;
+    for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+        size_t out = 0;
+        e = cudaGraphNodeGetDependentNodes(nodes[i], nullptr, nullptr, &out);
+        if (out == 0) last = nodes[i];
+    }
+    if (e != cudaSuccess || last == nullptr) return failed(e, "cudaGraphNodeGetDependentNodes");
+    cudaGraphNodeParams cp{};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = h;
+    cp.conditional.type = cudaGraphCondTypeIf;
+    cp.conditional.size = 1;
+    cudaGraphNode_t cond = nullptr;
+    e = cudaGraphAddNode(&cond, graph, &last, nullptr, 1, &cp);
+    if (e != cudaSuccess) return failed(e, "cudaGraphAddNode(if)");
+    e = cudaStreamBeginCaptureToGraph(cs, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return failed(e, "cudaStreamBeginCaptureToGraph");
+    pgm_status st = enqueue_grad(g, log_pot, evidence, T, damping, n_iters, ckpt_every, d_beliefs, d_log_pot, d_evidence, mem,
+                                 cs);
+    e = cudaStreamEndCapture(cs, &captured);
+    if (st != PGM_OK) {
+        cudaGraphDestroy(graph);
+        return st;
+    }
+    if (e != cudaSuccess) return failed(e, "cudaStreamEndCapture");
+    e = cudaGraphInstantiate(exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate(gradient)");
+    return PGM_OK;
+}
+
 static void drop_cached_grads(pgm_graph *g) {
     for (auto &c : g->grads) cudaGraphExecDestroy(c.exec);
     g->grads.clear();
@@ -2295,7 +2364,7 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
     if (pgm_status st = checked_gate(g, stream); st != PGM_OK) return st;
     DeviceGuard dg(g->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const size_t total = grad_work_bytes(g, n_iters, ckpt_every);
+    size_t total = grad_work_bytes(g, n_iters, ckpt_every);
     if (!g->use_cuda_graph || g->ordered) {  // stream-ordered work buffers, direct launches
         char *mem = nullptr;
         cudaError_t e = cudaMallocAsync(&mem, total, s);
@@ -2306,6 +2375,13 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
         return st;
     }
     // CUDA graph of the whole call on persistent work buffers (grown when needed)
+    const size_t launches = total;  // the launches' part
+    LrGradPlan one;
+    if (g->small_run != 0 && g->P.lr && g->G.vin_tab4 != nullptr && n_iters >= 1 && g->adj_nc_max == 0)
+        one = lr_grad_plan(g->P.grid, g->G.V, g->G.E / 2, n_iters);
+    // (its lam of every iteration: up to 1 GiB; a longer run keeps the checkpoints' bound)
+    if (one.form != 0 && one.hist_bytes <= (size_t)1 << 30) total = align_up(launches, 256) + 256 + one.hist_bytes;
+    else one = LrGradPlan{};
     if (g->grad_bytes < total) {
         cudaError_t e = cudaDeviceSynchronize();  // the old buffers may be in use by a replay
         if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
@@ -2313,7 +2389,14 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
         if (g->grad_mem) cudaFree(g->grad_mem);
         g->grad_mem = nullptr;
         g->grad_bytes = 0;
-        if (cudaMalloc(&g->grad_mem, total) != cudaSuccess) {
+        e = cudaMalloc(&g->grad_mem, total);
+        if (e != cudaSuccess && one.form != 0) {  // no room for the one-launch form
+            cudaGetLastError();
+            one = LrGradPlan{};
+            total = launches;
+            e = cudaMalloc(&g->grad_mem, total);
+        }
+        if (e != cudaSuccess) {
             g->grad_mem = nullptr;
             return fail(PGM_ENOMEM, "cudaMalloc(grad)");
         }
@@ -2333,20 +2416,26 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
             cudaError_t e = cudaStreamCreateWithFlags(&g->capture_stream, cudaStreamNonBlocking);
             if (e != cudaSuccess) return cuda_fail(e, "cudaStreamCreate");
         }
-        cudaError_t e = cudaStreamBeginCapture(g->capture_stream, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
-        pgm_status st = enqueue_grad(g, log_pot, evidence, T, damping, n_iters, ckpt_every, d_beliefs, d_log_pot,
-                                     d_evidence, static_cast<char *>(g->grad_mem), g->capture_stream);
-        cudaGraph_t graph = nullptr;
-        e = cudaStreamEndCapture(g->capture_stream, &graph);
-        if (st != PGM_OK) {
-            if (graph) cudaGraphDestroy(graph);
-            return st;
+        if (one.form != 0) {
+            pgm_status st = one_launch_grad(g, one, log_pot, evidence, T, damping, n_iters, ckpt_every, d_beliefs, d_log_pot,
+                                            d_evidence, launches, &exec);
+            if (st != PGM_OK) return st;
+        } else {
+            cudaError_t e = cudaStreamBeginCapture(g->capture_stream, cudaStreamCaptureModeThreadLocal);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
+            pgm_status st = enqueue_grad(g, log_pot, evidence, T, damping, n_iters, ckpt_every, d_beliefs, d_log_pot,
+                                         d_evidence, static_cast<char *>(g->grad_mem), g->capture_stream);
+            cudaGraph_t graph = nullptr;
+            e = cudaStreamEndCapture(g->capture_stream, &graph);
+            if (st != PGM_OK) {
+                if (graph) cudaGraphDestroy(graph);
+                return st;
+            }
+            if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
+            e = cudaGraphInstantiate(&exec, graph, 0);
+            cudaGraphDestroy(graph);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
         }
-        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&exec, graph, 0);
-        cudaGraphDestroy(graph);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
         if (g->grads.size() >= 4) {
             cudaGraphExecDestroy(g->grads.front().exec);
             g->grads.erase(g->grads.begin());

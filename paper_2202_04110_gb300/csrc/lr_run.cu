@@ -568,6 +568,376 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_push(const LrRun A) {
     }
 }
 
+// ---- gradient in one launch ----
+//
+// pgm_grad of a graph with a table per factor: the forward iterations of k_lr_run from zero
+// messages, with each iteration's lam also kept in global memory (16 bytes per variable and
+// iteration), the read-out, and the reverse steps, in the same blocks with the same exchange.
+// The launches it replaces (a 64 x 64 grid, 100 iterations: 590 of 2.4 us, half of them to
+// recompute the forward from checkpoints) were bound by their latency; here a step forward or
+// back costs one exchange between blocks, and nothing is recomputed.
+//
+// In log-ratios one step is d' = damping d + w (r + sp_T(p + lam) - sp_T(q + lam)) per message, lam =
+// D - d, so with the adjoint a of the new message into a slot and the lam of the slot it came
+// from, s_p = sigma((p + lam) / T), s_q likewise:
+//   g = w a (s_p - s_q) is lam's adjoint, and w a s_p, w a (1 - s_p), -w a s_q, -w a (1 - s_q) those
+//   of the table entries that p and q are differences of;
+//   the stored message of slot k gets damping a_k + the g of the variable's other slots, the
+//   evidence difference the sum of all four.
+// A whole factor's two messages are done by one thread; of a split factor each block does the
+// message that left it, for which the blocks exchange a instead of lam. The table's gradient is
+// kept per factor and written once; the two blocks of a split factor add theirs to zeros (a sum of
+// two terms: the same bits in either order), so repeated calls give the same bits.
+// Tables with non-finite entries, contradictions and infinite messages (a lam of +-inf is
+// fine: its sigmas are 0 or 1) set *bail, and the caller's launches take over.
+// Measured (GB300, whole calls): 64 x 64, 100 iterations, checkpoints every 10: 1.59 ms as ~590
+// dependent launches of 2.4 us, 0.31 in one; with lr_dir's SFU forms 0.28, but the table
+// gradients' error against 64 bits rose from 2.3e-7 to 2.7e-7 (mean of 15 grids). What bounds it:
+// two barriers and an exchange per step of 200.
+struct LrGrad {
+    LrRun A;                // msgs unused
+    const float *gnb;       // [2 V] cotangent of the normalised log-beliefs
+    float *d_pot, *d_ev;
+    float *hist;            // [n_iters][blocks][4 Vc]
+    int *bail;
+    float T;
+};
+
+// sigma(x / T) and 1 - sigma(x / T), each to a few ulp of itself.
+struct Sigma {
+    float s, c;
+};
+__device__ __forceinline__ Sigma sigma_t(float x, float invT) {
+    const float t = expf(-fabsf(x) * invT), big = __fdividef(1.f, 1.f + t), small = t * big;
+    return x >= 0.f ? Sigma{big, small} : Sigma{small, big};
+}
+
+// lr_dir (T > 0) with the accurate exponential and logarithm: its 3e-7 T would be the largest
+// error of the gradient's forward messages.
+__device__ __forceinline__ float grad_dir(float r, float p, float q, float l, float mo, float T, float invT,
+                                          float damping, float w) {
+    const float x = p + l, y = q + l;
+    const float sx = fmaf(T, log1pf(expf(-fabsf(x) * invT)), fmaxf(x, 0.f));
+    const float sy = fmaf(T, log1pf(expf(-fabsf(y) * invT)), fmaxf(y, 0.f));
+    return fmaf(damping, mo, w * (r + sx - sy));
+}
+
+// The gradients of one direction's four table entries -- the two that p and the two that q are
+// differences of, each weight formed as itself, since the differences of sums over the
+// iterations would lose to cancellation -- and of the lam it came from.
+struct DirGrad {
+    float p1, p0, q1, q0, lam;
+};
+__device__ __forceinline__ DirGrad dir_grad(float p, float q, float l, float wa, float invT) {
+    const Sigma P = sigma_t(p + l, invT), Q = sigma_t(q + l, invT);
+    return DirGrad{wa * P.s, wa * P.c, -wa * Q.s, -wa * Q.c, wa * (P.s * Q.c - Q.s * P.c)};
+}
+
+// One value per split slot: out in step st, and in from the other block.
+template <int X>
+__device__ __forceinline__ void grad_publish(const LrRun &A, const float *val, const float4 *hrec, const uint32_t *hdst,
+                                             int nH, int st) {
+    if (X == kAlone) return;
+    for (int h = threadIdx.x; h < nH; h += blockDim.x) {
+        const unsigned long long wd = box_word(val[__float_as_uint(hrec[h].w) & 0xffff], (uint32_t)st);
+        if (X == kCluster) {
+            const uint32_t a = hdst[h] + ((st & 1) ? 8u * (uint32_t)A.h_cap : 0u);
+            asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(wd) : "memory");
+        } else {
+            unsigned long long *p = ((st & 1) ? A.box1 : A.box0) + hdst[h];
+            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(wd) : "memory");
+        }
+    }
+}
+template <int X>
+__device__ __forceinline__ float grad_receive(const LrRun &A, const unsigned long long *box, size_t h_base, int h, int st,
+                                              int *s_abort) {
+    unsigned long long wd = 0;
+    int polls = 0;
+    while (true) {
+        if (X == kCluster) {
+            const uint32_t a = smem_addr(box + h) + ((st & 1) ? 8u * (uint32_t)A.h_cap : 0u);
+            asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(wd) : "r"(a) : "memory");
+        } else {
+            const unsigned long long *p = ((st & 1) ? A.box1 : A.box0) + h_base + h;
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(wd) : "l"(p) : "memory");
+        }
+        if ((uint32_t)(wd >> 32) == (uint32_t)st) break;
+        if (*(volatile int *)s_abort) break;
+        if (++polls >= kWaitLimit) {
+            atomicOr(A.flags, kFlagTimeout);
+            *(volatile int *)s_abort = 1;
+            break;
+        }
+    }
+    return __uint_as_float((uint32_t)wd);
+}
+
+template <int X>
+__global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_constant__ LrGrad P) {
+    extern __shared__ __align__(16) char lr_sm[];
+    __shared__ int s_n[2];
+    __shared__ int s_abort;
+    const LrRun &A = P.A;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    const int V = A.V, Vc = A.Vc;
+    const int b = X == kCluster ? (int)cluster_rank() : (int)blockIdx.x;
+    const int v0 = b * Vc, nv = max(0, min(Vc, V - v0));
+    const size_t h_base = X == kGrid ? (size_t)A.off[b].y : 0;
+    float *hist = P.hist + (size_t)b * 4 * Vc;
+    const size_t hist_step = (size_t)A.nb * 4 * Vc;
+    // shared memory
+    char *sp = lr_sm;
+    float4 *rec = reinterpret_cast<float4 *>(sp);  // c, al, be, slots
+    sp += 16 * (size_t)A.f_cap;
+    float4 *hrec = reinterpret_cast<float4 *>(sp);  // c, al, be, slot | side << 16
+    sp += 16 * (size_t)A.h_cap;
+    float4 *racc = reinterpret_cast<float4 *>(sp);  // gradients of a table's entries
+    sp += 16 * (size_t)A.f_cap;
+    float4 *hacc = reinterpret_cast<float4 *>(sp);
+    sp += 16 * (size_t)A.h_cap;
+    float2 *es_sh = reinterpret_cast<float2 *>(sp);
+    sp += 8 * (size_t)Vc;
+    unsigned long long *box = reinterpret_cast<unsigned long long *>(sp);
+    if (X == kCluster) sp += 16 * (size_t)A.h_cap;
+    float *lam = reinterpret_cast<float *>(sp);  // reverse: g
+    sp += 16 * (size_t)Vc;
+    float *d = reinterpret_cast<float *>(sp);    // reverse: a
+    sp += 16 * (size_t)Vc;
+    float *dD = reinterpret_cast<float *>(sp);   // the evidence difference's gradient
+    sp += 4 * (size_t)Vc;
+    uint32_t *hdst = reinterpret_cast<uint32_t *>(sp);
+
+    if (tid < 2) s_n[tid] = 0;
+    if (tid == 0) s_abort = 0;
+    for (int i = tid; i < A.f_cap; i += nt) racc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = tid; i < A.h_cap; i += nt) hacc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    bool bad = false;
+    for (int l0 = 0; l0 < nv; l0 += nt) {  // as k_lr_run's prologue
+        const int lv = l0 + tid, v = v0 + lv;
+        const int4 t = lv < nv ? __ldg(A.tab4 + v) : make_int4(-1, -1, -1, -1);
+        if (lv < nv) es_sh[lv] = __ldg(reinterpret_cast<const float2 *>(A.ev) + v);
+        const int es[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool have = es[q] >= 0;
+            int u = 0, uk = 0;
+            if (have) {
+                const int p = __ldg(A.lr_pos + ((es[q] >> 1) ^ 1));  // the factor's other slot
+                uk = (p >= V) + (p >= 2 * V) + (p >= 3 * V);
+                u = p - uk * V;
+            }
+            if (lv < nv) d[q * Vc + lv] = 0.f;
+            const bool local = X == kAlone || (u >= v0 && u < v0 + nv);
+            const int side = (es[q] >> 1) & 1;
+            const bool whole = have && local && side == 0, split = have && !local;
+            float c = 0.f, al = 0.f, be = 0.f;
+            if (whole || split) {
+                const float4 tb = lr_table(A.segs, A.n_seg, A.pot, es[q] >> 2);
+                c = tb.z - tb.x;
+                al = tb.w - tb.z;
+                be = tb.y - tb.x;
+                bad |= !(isfinite(tb.x) & isfinite(tb.y) & isfinite(tb.z) & isfinite(tb.w));
+            }
+            const unsigned mw = __ballot_sync(0xffffffffu, whole), mh = __ballot_sync(0xffffffffu, split);
+            int bw = 0, bh = 0;
+            if (lane == 0) {
+                if (mw) bw = atomicAdd(&s_n[0], __popc(mw));
+                if (mh) bh = atomicAdd(&s_n[1], __popc(mh));
+            }
+            bw = __shfl_sync(0xffffffffu, bw, 0) + __popc(mw & ((1u << lane) - 1u));
+            bh = __shfl_sync(0xffffffffu, bh, 0) + __popc(mh & ((1u << lane) - 1u));
+            if (whole)
+                rec[bw] = make_float4(c, al, be, __uint_as_float((uint32_t)(q * Vc + lv) | (uint32_t)(uk * Vc + u - v0) << 16));
+            if (X != kAlone && split) {
+                hrec[bh] = make_float4(c, al, be, __uint_as_float((uint32_t)(q * Vc + lv) | (uint32_t)side << 16));
+                __stcg(A.dir + (size_t)q * V + v, bh);
+            }
+        }
+    }
+    __syncthreads();
+    const int nF = s_n[0], nH = X == kAlone ? 0 : s_n[1];
+    bool ok = true;
+    if constexpr (X == kCluster) {
+        for (int h = tid; h < 2 * A.h_cap; h += nt) box[h] = 0;
+        cluster_barrier();
+    } else if constexpr (X == kGrid) {
+        for (int h = tid; h < nH; h += nt) {
+            __stcg(A.box0 + h_base + h, 0ull);
+            __stcg(A.box1 + h_base + h, 0ull);
+        }
+        ok = grid_barrier_once(A.bar, gridDim.x, A.flags);
+    }
+    if (X == kGrid && !ok) return;
+    for (int h = tid; h < nH; h += nt) {
+        const int s = (int)(__float_as_uint(hrec[h].w) & 0xffff), q = s / Vc, lv = s - q * Vc;
+        const int4 t = __ldg(A.tab4 + v0 + lv);
+        const int es = q == 0 ? t.x : q == 1 ? t.y : q == 2 ? t.z : t.w;
+        const int p = __ldg(A.lr_pos + ((es >> 1) ^ 1));
+        const int u = p - V * ((p >= V) + (p >= 2 * V) + (p >= 3 * V));
+        const int ub = u / Vc, at = __ldcg(A.dir + p);
+        if constexpr (X == kCluster) hdst[h] = rank_addr(smem_addr(box + at), (uint32_t)ub);
+        else hdst[h] = (uint32_t)(A.off[ub].y + at);
+    }
+    __syncthreads();
+
+    const float T = P.T, invT = 1.f / P.T, damping = A.damping, w = 1.f - damping;
+    // a message that lr_dir could not form
+    auto rare = [&](int s, float l, float mo) {
+        const float n = l == l ? run_exact<false>(A, A.pot, v0, s, l, mo) : 0.f;
+        bad |= !(l == l) | !isfinite(n);
+        return n;
+    };
+
+    // ---- forward ----
+    for (int it = 1; it <= A.n_iters; ++it) {
+        float *H = hist + (size_t)(it - 1) * hist_step;
+        for (int lv = tid; lv < nv; lv += nt) {
+            const float2 e = es_sh[lv];
+            const float d0 = d[lv], d1 = d[Vc + lv], d2 = d[2 * Vc + lv], d3 = d[3 * Vc + lv];
+            float2 Df;
+            if (push_total(e, d0, d1, d2, d3, Df)) {
+                lam[lv] = lr_lam_from_D(Df, d0);
+                lam[Vc + lv] = lr_lam_from_D(Df, d1);
+                lam[2 * Vc + lv] = lr_lam_from_D(Df, d2);
+                lam[3 * Vc + lv] = lr_lam_from_D(Df, d3);
+            } else {
+                run_var_slow(lam, lv, Vc, e, d0, d1, d2, d3);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) __stcg(H + q * Vc + lv, lam[q * Vc + lv]);
+        }
+        __syncthreads();
+        grad_publish<X>(A, lam, hrec, hdst, nH, it);
+        for (int i = tid; i < nF; i += nt) {
+            const float4 r = rec[i];
+            const uint32_t pk = __float_as_uint(r.w);
+            const int s0 = pk & 0xffff, s1 = pk >> 16;
+            const float mo0 = d[s0], mo1 = d[s1], l0 = lam[s0], l1 = lam[s1];
+            float n0 = grad_dir(r.x, r.y, r.z, l1, mo0, T, invT, damping, w);
+            float n1 = grad_dir(r.z, r.y + r.x - r.z, r.x, l0, mo1, T, invT, damping, w);
+            if (!(fabsf(n0) + fabsf(n1) < CUDART_INF_F)) {
+                if (lr_dir_rare(n0, l1)) n0 = rare(s0, l1, mo0);
+                if (lr_dir_rare(n1, l0)) n1 = rare(s1, l0, mo1);
+            }
+            d[s0] = n0;
+            d[s1] = n1;
+        }
+        for (int h = tid; h < nH; h += nt) {
+            const float4 r = hrec[h];
+            const uint32_t pk = __float_as_uint(r.w);
+            const int s = pk & 0xffff;
+            const bool one = (pk >> 16) != 0;  // the message into the factor's variable 1
+            const float mo = d[s], l = grad_receive<X>(A, box, h_base, h, it, &s_abort);
+            float n = one ? grad_dir(r.z, r.y + r.x - r.z, r.x, l, mo, T, invT, damping, w)
+                          : grad_dir(r.x, r.y, r.z, l, mo, T, invT, damping, w);
+            if (lr_dir_rare(n, l)) n = rare(s, l, mo);
+            d[s] = n;
+        }
+        __syncthreads();
+    }
+    // ---- the read-out: L = sum g (b - LSE(b)), dL/dD = g1 - (g0 + g1) sigma(D) ----
+    for (int lv = tid; lv < nv; lv += nt) {
+        float2 D;
+        if (!push_total(es_sh[lv], d[lv], d[Vc + lv], d[2 * Vc + lv], d[3 * Vc + lv], D)) {
+            const float2 e = es_sh[lv];  // (finite messages: an infinite evidence entry, or none)
+            D = make_float2(e.y - e.x, 0.f);
+            bad |= !(D.x == D.x) | !(fabsf(d[lv]) + fabsf(d[Vc + lv]) + fabsf(d[2 * Vc + lv]) + fabsf(d[3 * Vc + lv]) < CUDART_INF_F);
+        }
+        const float2 g = __ldg(reinterpret_cast<const float2 *>(P.gnb) + v0 + lv);
+        const float x = D.x + D.y, a = g.y * sigma_t(x, 1.f).c - g.x * sigma_t(x, 1.f).s;
+        dD[lv] = a;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            d[q * Vc + lv] = a;
+            lam[q * Vc + lv] = 0.f;  // unused slots have no g
+        }
+    }
+    __syncthreads();
+    // ---- reverse ----
+    for (int it = A.n_iters; it >= 1; --it) {
+        const float *H = hist + (size_t)(it - 1) * hist_step;
+        const int st = 2 * A.n_iters + 1 - it;
+        grad_publish<X>(A, d, hrec, hdst, nH, st);
+        for (int i = tid; i < nF; i += nt) {
+            const float4 r = rec[i];
+            const uint32_t pk = __float_as_uint(r.w);
+            const int s0 = pk & 0xffff, s1 = pk >> 16;
+            const float l0 = __ldcg(H + s0), l1 = __ldcg(H + s1);
+            const DirGrad a = dir_grad(r.y, r.z, l1, w * d[s0], invT), c = dir_grad(r.y + r.x - r.z, r.x, l0, w * d[s1], invT);
+            lam[s1] = a.lam;
+            lam[s0] = c.lam;
+            float4 t = racc[i];  // to variable 0: p = phi11 - phi10, q = phi01 - phi00; to 1: phi11 - phi01, phi10 - phi00
+            t.x += a.q0 + c.q0;
+            t.y += a.q1 + c.p0;
+            t.z += a.p0 + c.q1;
+            t.w += a.p1 + c.p1;
+            racc[i] = t;
+        }
+        for (int h = tid; h < nH; h += nt) {  // the message that left slot s, towards the other block
+            const float4 r = hrec[h];
+            const uint32_t pk = __float_as_uint(r.w);
+            const int s = pk & 0xffff;
+            const bool one = (pk >> 16) != 0;  // the source is variable 1: the message to variable 0
+            const float l = __ldcg(H + s), a = w * grad_receive<X>(A, box, h_base, h, st, &s_abort);
+            const DirGrad g = one ? dir_grad(r.y, r.z, l, a, invT) : dir_grad(r.y + r.x - r.z, r.x, l, a, invT);
+            lam[s] = g.lam;
+            float4 t = hacc[h];
+            t.x += g.q0;
+            t.y += one ? g.q1 : g.p0;
+            t.z += one ? g.p0 : g.q1;
+            t.w += g.p1;
+            hacc[h] = t;
+        }
+        __syncthreads();
+        for (int lv = tid; lv < nv; lv += nt) {
+            const float g0 = lam[lv], g1 = lam[Vc + lv], g2 = lam[2 * Vc + lv], g3 = lam[3 * Vc + lv];
+            const float g01 = g0 + g1, g23 = g2 + g3;
+            d[lv] = fmaf(damping, d[lv], g1 + g23);
+            d[Vc + lv] = fmaf(damping, d[Vc + lv], g0 + g23);
+            d[2 * Vc + lv] = fmaf(damping, d[2 * Vc + lv], g01 + g3);
+            d[3 * Vc + lv] = fmaf(damping, d[3 * Vc + lv], g01 + g2);
+            dD[lv] += g01 + g23;
+        }
+        __syncthreads();
+    }
+    // ---- out ----
+    for (int lv = tid; lv < nv; lv += nt) {
+        P.d_ev[2 * (size_t)(v0 + lv)] = -dD[lv];
+        P.d_ev[2 * (size_t)(v0 + lv) + 1] = dD[lv];
+    }
+    auto table_of = [&](int s) {  // the table of slot s's factor in d_pot
+        const int q = s / Vc, v = v0 + s - q * Vc;
+        const int4 t = __ldg(A.tab4 + v);
+        const int g = (q == 0 ? t.x : q == 1 ? t.y : q == 2 ? t.z : t.w) >> 2;
+        const EnumSeg *S = A.segs + lr_seg_of(A.segs, A.n_seg, g);
+        return P.d_pot + __ldg(&S->pot_base) + 4 * (size_t)(g - (__ldg(&S->edge_base) >> 1));
+    };
+    for (int i = tid; i < nF; i += nt) {
+        float *t = table_of((int)(__float_as_uint(rec[i].w) & 0xffff));
+        const float4 a = racc[i];
+        t[0] = a.x;
+        t[1] = a.y;
+        t[2] = a.z;
+        t[3] = a.w;
+    }
+    for (int h = tid; h < nH; h += nt) {
+        float *t = table_of((int)(__float_as_uint(hrec[h].w) & 0xffff));
+        const float4 a = hacc[h];
+        atomicAdd(t, a.x);
+        atomicAdd(t + 1, a.y);
+        atomicAdd(t + 2, a.z);
+        atomicAdd(t + 3, a.w);
+    }
+    if (bad) *P.bail = 1;
+    if constexpr (X == kCluster) cluster_barrier();
+}
+
+__global__ void k_set_condition(cudaGraphConditionalHandle h, const int *__restrict__ word) {
+    cudaGraphSetConditional(h, *word != 0 ? 1u : 0u);
+}
+
 using RunKernel = void (*)(const LrRun);
 // LAM where it fits: always with the records in shared memory.
 template <bool MAXP>
@@ -621,6 +991,9 @@ const RunDevice &run_device() {
                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, R.smem);
                 if (x == kCluster) cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             }
+    for (auto kern : {k_lr_grad<kAlone>, k_lr_grad<kCluster>, k_lr_grad<kGrid>})
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, R.smem);
+    cudaFuncSetAttribute(k_lr_grad<kCluster>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     for (int C : {kLrClusterMax, 8}) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(C);
@@ -653,12 +1026,18 @@ const RunDevice &run_device() {
     return R;
 }
 
+// Shared memory of a gradient block.
+size_t grad_smem(int x, int Vc, int f_cap, int h_cap) {
+    return 44 * (size_t)Vc + 32 * (size_t)f_cap + (x == kCluster ? 52 : 36) * (size_t)h_cap + 16;
+}
+
 int run_threads(int Vc, int items) {
     const int per = std::max(Vc, items);
     return std::min(kLrRunThreads, std::max(32, (per + 31) / 32 * 32));
 }
 
-cudaError_t launch(RunKernel kern, const LrRun &A, int blocks, int threads, size_t smem, int x, cudaStream_t s) {
+template <class Args>
+cudaError_t launch(void (*kern)(const Args), const Args &A, int blocks, int threads, size_t smem, int x, cudaStream_t s) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3((unsigned)threads);
@@ -866,6 +1245,72 @@ cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiP
     const bool lam_sh = run_smem(x, false, true, p.Vc, 0, 0) <= (size_t)run_device().smem;
     return launch(run_kernel(T == 0.f, x, p.res, lam_sh), A, (int)blocks, run_threads(p.Vc, (2 * G.V + p.nb - 1) / p.nb),
                   p.res ? run_smem(x, true, true, p.Vc, p.f_cap, p.h_cap) : run_smem(x, false, lam_sh, p.Vc, 0, 0), x, s);
+}
+
+// ---- gradient ----
+
+LrGradPlan lr_grad_plan(const LrGridPlan &g, int V, int F, int n_iters) {
+    const RunDevice &R = run_device();
+    LrGradPlan p;
+    if (V < 1 || F < 1 || n_iters < 1 || n_iters > (1 << 28)) return p;
+    const int C = R.cluster;
+    if (V <= kLrBlockAutoV && F <= kLrBlockAutoF && grad_smem(kAlone, V, F, 0) <= (size_t)R.smem) {
+        p.form = 1;
+        p.nb = 1;
+        p.Vc = V;
+        p.f_cap = F;
+    } else if (C > 0 && V <= kLrClusterAutoV && grad_smem(kCluster, (V + C - 1) / C, 2 * ((V + C - 1) / C), 4 * ((V + C - 1) / C)) <= (size_t)R.smem) {
+        p.form = 2;
+        p.nb = C;
+        p.Vc = (V + C - 1) / C;
+        p.f_cap = 2 * p.Vc;
+        p.h_cap = 4 * p.Vc;
+    } else if (g.nb >= 2 && R.coop && g.nb <= R.n_sm && grad_smem(kGrid, g.Vc, g.f_max, g.h_max) <= (size_t)R.smem &&
+               2 * g.n_split <= 3 * (int64_t)F) {  // (the inboxes, as launch_lr_grid_run)
+        p.form = 3;
+        p.nb = g.nb;
+        p.Vc = g.Vc;
+        p.f_cap = g.f_max;
+        p.h_cap = g.h_max;
+    } else {
+        return p;
+    }
+    p.hist_bytes = (size_t)n_iters * p.nb * 16 * (size_t)p.Vc;
+    if (p.hist_bytes > ((size_t)512 << 20)) p.form = 0;
+    return p;
+}
+
+cudaError_t launch_lr_grad(const DevGraph &G, const Plan &P, const LrGradPlan &p, const float *log_pot, const float *ev,
+                           const float *gnb, float *d_pot, float *d_ev, float *hist, int *bail, float *m_tmp, float *d,
+                           float *prm, float T, float damping, int n_iters, cudaStream_t s) {
+    const FactorLaunch *L = only_launch(P);
+    if (L == nullptr || p.form == 0) return cudaErrorInvalidValue;
+    const EnumSeg *segs = static_cast<const EnumSeg *>(L->segs);
+    LrGrad a{};
+    a.A = run_args(G, segs, L->n_seg, log_pot, ev, nullptr, nullptr, T, damping, n_iters);
+    a.A.nb = p.nb;
+    a.A.Vc = p.Vc;
+    a.A.f_cap = p.f_cap;
+    a.A.h_cap = p.h_cap;
+    a.A.off = P.grid.off;
+    a.A.dir = reinterpret_cast<int32_t *>(d);
+    a.A.box0 = reinterpret_cast<unsigned long long *>(m_tmp);
+    a.A.box1 = reinterpret_cast<unsigned long long *>(prm);
+    a.gnb = gnb;
+    a.d_pot = d_pot;
+    a.d_ev = d_ev;
+    a.hist = hist;
+    a.bail = bail;
+    a.T = T;
+    const int x = p.form == 1 ? kAlone : p.form == 2 ? kCluster : kGrid;
+    auto kern = p.form == 1 ? k_lr_grad<kAlone> : p.form == 2 ? k_lr_grad<kCluster> : k_lr_grad<kGrid>;
+    const int items = p.form == 3 ? p.f_cap : (G.E / 2 + p.nb - 1) / p.nb;
+    return launch(kern, a, p.nb, run_threads(p.Vc, items), grad_smem(x, p.Vc, p.f_cap, p.h_cap), x, s);
+}
+
+cudaError_t launch_set_condition(cudaGraphConditionalHandle h, const int *word, cudaStream_t s) {
+    k_set_condition<<<1, 1, 0, s>>>(h, word);
+    return cudaGetLastError();
 }
 
 }  // namespace pgm

@@ -381,6 +381,19 @@ LrMultiPlan lr_multi_plan(int V, int S, bool local);
 cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiPlan &p, int S, int64_t pot_stride,
                                 const float *log_pot, const float *ev, float *msgs, char *work, float T, float damping,
                                 int n_iters, cudaStream_t s);
+// pgm_grad in one launch (lr_run.cu; every group with a table per factor): form 1 one block, 2 a
+// cluster, 3 the grid; 0: not taken. hist: hist_bytes of work; *bail (zeroed by the caller)
+// is set when the launches have to do it after all. d_pot zeroed by the caller.
+struct LrGradPlan {
+    int form = 0, nb = 0, Vc = 0, f_cap = 0, h_cap = 0;
+    size_t hist_bytes = 0;
+};
+LrGradPlan lr_grad_plan(const LrGridPlan &g, int V, int F, int n_iters);
+cudaError_t launch_lr_grad(const DevGraph &G, const Plan &P, const LrGradPlan &p, const float *log_pot, const float *ev,
+                           const float *gnb, float *d_pot, float *d_ev, float *hist, int *bail, float *m_tmp, float *d,
+                           float *prm, float T, float damping, int n_iters, cudaStream_t s);
+// In a graph: the conditional h = (*word != 0).
+cudaError_t launch_set_condition(cudaGraphConditionalHandle h, const int *word, cudaStream_t s);
 // Adjoint launchers (kernels.cu).
 cudaError_t launch_adj_beliefs(const DevGraph &G, const float *ev, const float *m, const float *gnb, float *d_ev,
                                float *adj, cudaStream_t s);
