@@ -224,6 +224,31 @@ __device__ __forceinline__ void hd_v2f(const DevGraph &G, int vs, const float (&
     for (int x = 0; x < K; ++x) v[x] = hd_rel(d[x], mx);
 }
 
+// Block-wide float-float sum of v and plain sum of c (a count) in a fixed order; sh holds
+// 3 floats per warp.
+__device__ __forceinline__ FF block_sum_count(FF v, float &c, float *sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        v = ff_add(v, ff_shfl_down(v, d));
+        c += __shfl_down_sync(0xffffffffu, c, d);
+    }
+    if (lane == 0) {
+        sh[3 * warp] = v.hi;
+        sh[3 * warp + 1] = v.lo;
+        sh[3 * warp + 2] = c;
+    }
+    __syncthreads();
+    FF tot = ff_make(0.f);
+    c = 0.f;
+    for (int w = 0; w < nw; ++w) {
+        tot = ff_add(tot, FF{sh[3 * w], sh[3 * w + 1]});
+        c += sh[3 * w + 2];
+    }
+    __syncthreads();
+    return tot;
+}
+
 // Variable-to-factor values of one K-state edge. Edges of high-degree variables
 // (edge_vs < 0) take the exact leave-one-out values from the variable's totals (hd_pair);
 // all others use b - m, or the explicit sum when an entry needs it.

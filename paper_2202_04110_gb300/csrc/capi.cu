@@ -243,6 +243,18 @@ bool lr_eligible(const HostLayout &H) {
     return lr && (H.vin_tab4.empty() ? H.E : 4 * H.V) <= INT32_MAX;
 }
 
+// Whether the graph's runs can use the edge-order log-ratio form (Plan::lr_edge): as
+// lr_eligible, with high-degree variables, none of more than kLrEdgeMaxDegree factors.
+bool lr_edge_eligible(const HostLayout &H) {
+    bool ok = H.all_binary && H.logic_groups.empty() && !H.enum_groups.empty() && H.ES == 2 * H.E && H.VS == 2 * H.V &&
+              H.E % 2 == 0 && !H.var_bucket[kVarBlock].empty();
+    for (const HostEnumGroup &hg : H.enum_groups) ok = ok && hg.variant == kPair2;
+    for (int kind = 0; kind < kNumVarKinds; ++kind)
+        if (kind != kVarBinary && kind != kVarBlock) ok = ok && H.var_bucket[kind].empty();
+    for (int32_t v : H.var_bucket[kVarBlock]) ok = ok && H.vin_off[v + 1] - H.vin_off[v] <= kLrEdgeMaxDegree;
+    return ok;
+}
+
 // Slots of each log-ratio array: 4 per variable with the 4-slot table, else one per edge.
 int64_t lr_slot_count(const HostLayout &H) { return H.vin_tab4.empty() ? H.E : 4 * H.V; }
 
@@ -583,6 +595,7 @@ pgm_status build_plan(const HostLayout &H, pgm_graph *g, Packer &pk, std::vector
     }
     plan_fused(H, g, pk);
     P.lr = lr_eligible(H);
+    P.lr_edge = lr_edge_eligible(H);
     P.lr_blocks = std::max(1, g->n_sm * 8);
     return PGM_OK;
 }
@@ -1070,6 +1083,13 @@ static bool log_ratio_run(const pgm_graph *g, int32_t n_iters) {
     return g->P.lr && !g->force_es && g->log_ratio_min_iters > 0 && n_iters >= g->log_ratio_min_iters;
 }
 
+// Whether such a run takes the edge-order form: graphs with high-degree variables, from the same
+// number of iterations. Per iteration it replaces the edge-state launches one for one, and the
+// first and last read and write msgs themselves, so no run length loses by it.
+static bool edge_ratio_run(const pgm_graph *g, int32_t n_iters) {
+    return g->P.lr_edge && !g->force_es && g->log_ratio_min_iters > 0 && n_iters >= g->log_ratio_min_iters;
+}
+
 // Whether a log-ratio run of this graph is one launch, and whether that launch is the
 // cluster form: the option is on, the graph has the 4-slot layout and fits the form's limits.
 // Setting 1 takes one block up to kLrBlockAutoV variables, the cluster above; 2 the
@@ -1093,9 +1113,11 @@ static bool grid_run_used(const pgm_graph *g) {
            lr_grid_fits(g->P.grid, g->G.V, g->G.E / 2);
 }
 
+// edge_form: a run of its own, which may take the edge-order log-ratio form (the parts of other
+// runs keep their ping-pong buffers).
 static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const float *evidence, float T,
                                      float damping, int32_t n_iters, float *msgs, cudaStream_t s,
-                                     bool profile) {
+                                     bool profile, bool edge_form = false) {
     float *cur = msgs, *nxt = g->m_tmp;
     const bool lr = log_ratio_run(g, n_iters);
     // per-variable totals of the 4-slot layout in the belief buffer (VS = 2V floats on a
@@ -1109,6 +1131,7 @@ static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const f
         if (e != cudaSuccess) return cuda_fail(e, "small-graph run launch");
         return PGM_OK;
     }
+    const bool edge = edge_form && edge_ratio_run(g, n_iters);
     if (lr) {
         cudaError_t e = launch_lr_pack(g->G, msgs, d, s);
         if (e == cudaSuccess) e = launch_lr_params(g->G, g->P, log_pot, g->lr_prm, s);
@@ -1145,20 +1168,23 @@ static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const f
             cudaEventRecordWithFlags(e0, s, ctx.flags);
         }
         const LaunchHook *h = prof ? &hook : nullptr;
-        cudaError_t e = lr ? launch_lr_var_pass(g->G, g->P, evidence, d, Dv, lam, s, h)
-                           : launch_var_pass(g->G, g->P, evidence, cur, g->b, kVarIter, nullptr, s, 1, h);
+        float *m_in = edge && it == 0 ? msgs : nullptr, *m_out = edge && it == n_iters - 1 ? msgs : nullptr;
+        cudaError_t e = lr     ? launch_lr_var_pass(g->G, g->P, evidence, d, Dv, lam, s, h)
+                        : edge ? launch_edge_var_pass(g->G, g->P, evidence, g->m_tmp, m_in, Dv, s, 1, h)
+                               : launch_var_pass(g->G, g->P, evidence, cur, g->b, kVarIter, nullptr, s, 1, h);
         if (e != cudaSuccess) return cuda_fail(e, "variable pass launch");
         grp.nv = (uint16_t)ctx.count;
         ctx.count = 0;
-        e = lr ? launch_lr_factor_pass(g->G, g->P, log_pot, g->lr_prm, Dv, lam, d, T, damping, s, h)
-               : launch_factor_pass(g->G, g->P, log_pot, g->b, evidence, cur, nxt, T, damping, s, 1, h);
+        e = lr     ? launch_lr_factor_pass(g->G, g->P, log_pot, g->lr_prm, Dv, lam, d, T, damping, s, h)
+            : edge ? launch_edge_factor_pass(g->G, g->P, log_pot, Dv, g->m_tmp, m_in, m_out, T, damping, s, 1, h)
+                   : launch_factor_pass(g->G, g->P, log_pot, g->b, evidence, cur, nxt, T, damping, s, 1, h);
         if (e != cudaSuccess) return cuda_fail(e, "factor pass launch");
         grp.nf = (uint16_t)ctx.count;
         if (prof) {
             if (ctx.st != PGM_OK) return ctx.st;
             (g->capture_groups ? *g->capture_groups : g->prof_groups).push_back(grp);
         }
-        if (!lr) std::swap(cur, nxt);
+        if (!lr && !edge) std::swap(cur, nxt);
     }
     if (lr) {
         cudaError_t e = launch_lr_unpack(g->G, d, msgs, s);
@@ -1216,7 +1242,7 @@ static pgm_status cached_run(pgm_graph *g, const float *log_pot, const float *ev
     g->capture_events = &events;
     g->capture_groups = &groups;
     pgm_status st = enqueue_iterations(g, log_pot, evidence, T, damping, n_iters, msgs, g->capture_stream,
-                                       g->profiling > 0);
+                                       g->profiling > 0, true);
     g->capture_events = nullptr;
     g->capture_groups = nullptr;
     cudaGraph_t graph = nullptr;
@@ -1337,6 +1363,7 @@ static pgm_status run_multi_es(pgm_graph *g, int32_t n_samples, const float *log
         if (cudaMalloc(&g->mse_mem, need) != cudaSuccess) return fail(PGM_ENOMEM, "cudaMalloc(multi-sample scratch)");
         g->mse_bytes = need;
     }
+    const bool edge = edge_ratio_run(g, n_iters);
     float *mt = reinterpret_cast<float *>(g->mse_mem), *bb = reinterpret_cast<float *>(g->mse_mem + r_mt);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     for (int64_t s0 = 0; s0 < n_samples; s0 += chunk) {
@@ -1350,7 +1377,15 @@ static pgm_status run_multi_es(pgm_graph *g, int32_t n_samples, const float *log
         const float *lp = log_pot + (pot_per_sample ? (size_t)s0 * P : 0);
         const float *ev = evidence + (size_t)s0 * VS;
         float *m0 = msgs + (size_t)s0 * ES, *cur = m0, *nxt = mt;
-        for (int it = 0; it < n_iters; ++it) {
+        for (int it = 0; edge && it < n_iters; ++it) {  // (as the samples' own runs)
+            float2 *Dv = reinterpret_cast<float2 *>(bb);
+            float *m_in = it == 0 ? m0 : nullptr, *m_out = it == n_iters - 1 ? m0 : nullptr;
+            cudaError_t e = launch_edge_var_pass(Gs, g->P, ev, mt, m_in, Dv, s, S, nullptr);
+            if (e == cudaSuccess)
+                e = launch_edge_factor_pass(Gs, g->P, lp, Dv, mt, m_in, m_out, T, damping, s, S, nullptr);
+            if (e != cudaSuccess) return cuda_fail(e, "multi-sample pass launch");
+        }
+        for (int it = 0; !edge && it < n_iters; ++it) {
             cudaError_t e = launch_var_pass(Gs, g->P, ev, cur, bb, kVarIter, nullptr, s, S);
             if (e == cudaSuccess) e = launch_factor_pass(Gs, g->P, lp, bb, ev, cur, nxt, T, damping, s, S);
             if (e != cudaSuccess) return cuda_fail(e, "multi-sample pass launch");
@@ -1937,7 +1972,7 @@ pgm_status pgm_run_bp(pgm_graph *g, const float *log_pot, const float *evidence,
         run->pending = !run->groups.empty();
         return PGM_OK;
     }
-    return enqueue_iterations(g, log_pot, evidence, T, damping, n_iters, msgs, s, true);
+    return enqueue_iterations(g, log_pot, evidence, T, damping, n_iters, msgs, s, true, true);
 }
 
 // The other kernel forms for the same factors: dense K-state pairwise tables run with K

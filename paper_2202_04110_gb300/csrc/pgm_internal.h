@@ -27,6 +27,7 @@ constexpr int kEnumPairsBlock = 32;         // factors per block of the max-prod
 constexpr int kEnumTableSmem = 160 * 1024;  // largest configuration table staged per block
 constexpr int kMaxStates = 256;
 constexpr int kVarBlockDegree = 64;  // variables with more factors use a block each
+constexpr int kLrEdgeMaxDegree = 4096;  // Plan::lr_edge: a variable's sum is one block's work
 constexpr int kVarBlockThreads = 256;
 constexpr int kVarItems = 8;                               // contiguous edges per thread
 constexpr int kVarTile = kVarBlockThreads * kVarItems;     // edges per tile
@@ -218,6 +219,9 @@ struct Plan {
     // Binary pairwise graph (every variable binary, every factor a kPair2 factor, no
     // high-degree variable): iterations may keep one log-ratio per edge.
     bool lr = false;
+    // The same with high-degree variables of at most kLrEdgeMaxDegree factors: runs may
+    // iterate on log-ratios in edge order (lr_edge.cu).
+    bool lr_edge = false;
     int32_t lr_blocks = 1;  // persistent log-ratio factor pass: blocks of 256 (8 per SM)
     LrGridPlan grid;        // nb = 0: none
 };
@@ -355,6 +359,14 @@ inline bool lr_cluster_fits(int V, int F) {
     const int C = lr_cluster_size();
     return C > 0 && V > 0 && V <= C * kLrSmallMaxV && F <= C * kLrSmallMaxF;
 }
+// One iteration's passes of the edge-order log-ratio form (Plan::lr_edge): d one number per edge,
+// m_in / m_out the run's messages in its first / last iteration (else nullptr), S samples (d, m and
+// Dv of sample i at i s_es, i s_es and i s_vs floats, DevGraph).
+cudaError_t launch_edge_var_pass(const DevGraph &G, const Plan &P, const float *ev, const float *d, const float *m_in,
+                                 float2 *Dv, cudaStream_t s, int S, const LaunchHook *hook);
+cudaError_t launch_edge_factor_pass(const DevGraph &G, const Plan &P, const float *log_pot, const float2 *Dv, float *d,
+                                    const float *m_in, float *m_out, float T, float damping, cudaStream_t s,
+                                    int S, const LaunchHook *hook);
 cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *log_pot, const float *ev,
                                 float *msgs, float *lam, int32_t *dir, float T, float damping, int n_iters,
                                 bool cluster, cudaStream_t s);
