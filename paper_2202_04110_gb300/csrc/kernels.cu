@@ -3468,11 +3468,8 @@ __global__ void __launch_bounds__(256) k_pair2_lr(const EnumSeg *__restrict__ se
         }
         float2 dn = make_float2(lr_dir<MAXP>(c, al, be, l1, mo0, k, Tln2, damping, w),
                                 lr_dir<MAXP>(be, al + c - be, c, l0, mo1, k, Tln2, damping, w));
-        if (lr_dir_rare(dn.x, l1) || lr_dir_rare(dn.y, l0)) {
-            const float4 t = lr_table(segs, n_seg, pot, g);
-            const float t4[4] = {t.x, t.y, t.z, t.w};
-            if (lr_dir_rare(dn.x, l1)) dn.x = lr_dir_exact<MAXP>(t4, 0, l1, mo0, k, Tln2, damping, flags);
-            if (lr_dir_rare(dn.y, l0)) dn.y = lr_dir_exact<MAXP>(t4, 1, l0, mo1, k, Tln2, damping, flags);
+        if (lr_dir_rare(dn.x, l1) | lr_dir_rare(dn.y, l0)) {
+            dn = lr_pair_exact<MAXP>(lr_table(segs, n_seg, pot, g), l0, l1, mo0, mo1, dn, k, Tln2, damping, flags);
         }
         d[p.x] = dn.x;
         d[p.y] = dn.y;
@@ -3655,11 +3652,9 @@ __global__ void __launch_bounds__(256) k_ms_pair(const EnumSeg *__restrict__ seg
         const float l1 = __float_as_uint(D1.x) == kDvSlow ? __ldcg(lam + py) : lr_lam_from_D(D1, mo1);
         float2 dn = make_float2(lr_dir<MAXP>(c, al, be, l1, mo0, k, Tln2, damping, w),
                                 lr_dir<MAXP>(be, al + c - be, c, l0, mo1, k, Tln2, damping, w));
-        if (lr_dir_rare(dn.x, l1) || lr_dir_rare(dn.y, l0)) {
-            const float4 tq = lr_table(segs, n_seg, pot + (Sp > 1 ? (size_t)s * P : 0), g);
-            const float t4[4] = {tq.x, tq.y, tq.z, tq.w};
-            if (lr_dir_rare(dn.x, l1)) dn.x = lr_dir_exact<MAXP>(t4, 0, l1, mo0, k, Tln2, damping, flags);
-            if (lr_dir_rare(dn.y, l0)) dn.y = lr_dir_exact<MAXP>(t4, 1, l0, mo1, k, Tln2, damping, flags);
+        if (lr_dir_rare(dn.x, l1) | lr_dir_rare(dn.y, l0)) {
+            dn = lr_pair_exact<MAXP>(lr_table(segs, n_seg, pot + (Sp > 1 ? (size_t)s * P : 0), g), l0, l1, mo0, mo1, dn,
+                                     k, Tln2, damping, flags);
         }
         d[px] = dn.x;
         d[py] = dn.y;

@@ -233,5 +233,16 @@ __device__ __forceinline__ float lr_dir(float r, float p, float q, float l, floa
 }
 __device__ __forceinline__ bool lr_dir_rare(float dn, float l) { return !(isfinite(dn) && l == l); }
 
+// Both messages of a factor of which at least one is rare: one call, so that the callers' common
+// path keeps nothing across two.
+template <bool MAXP>
+__device__ __noinline__ float2 lr_pair_exact(float4 t, float l0, float l1, float mo0, float mo1, float2 dn, float k,
+                                             float Tln2, float damping, uint32_t *flags) {
+    const float t4[4] = {t.x, t.y, t.z, t.w};
+    if (lr_dir_rare(dn.x, l1)) dn.x = lr_dir_exact<MAXP>(t4, 0, l1, mo0, k, Tln2, damping, flags);
+    if (lr_dir_rare(dn.y, l0)) dn.y = lr_dir_exact<MAXP>(t4, 1, l0, mo1, k, Tln2, damping, flags);
+    return dn;
+}
+
 }  // namespace
 }  // namespace pgm
