@@ -484,7 +484,8 @@ pgm_status pgm_run_bp_until_members(pgm_graph *g, const float *log_pot, const fl
  * A binary pairwise graph with variables of 65 to 4,096 factors keeps one number per edge
  * as well in pgm_run_bp and pgm_run_bp_multi from the same n_iters (in edge order, the
  * variables' totals in double-float; early-exit and per-member runs keep the edge-state
- * iteration), and pgm_get_option stays 0 for it.
+ * iteration), and so do max-product runs of binary graphs of OR and AND factors only (fan-in
+ * up to 256) with variables of 65 to 16,384 factors; pgm_get_option stays 0 for both.
  * Negative values: PGM_EINVAL. pgm_launch_info / launches_per_iter do not count the 3
  * launches per run around the iterations (pack, table differences, unpack).
  */

@@ -243,16 +243,23 @@ bool lr_eligible(const HostLayout &H) {
     return lr && (H.vin_tab4.empty() ? H.E : 4 * H.V) <= INT32_MAX;
 }
 
-// Whether the graph's runs can use the edge-order log-ratio form (Plan::lr_edge): as
-// lr_eligible, with high-degree variables, none of more than kLrEdgeMaxDegree factors.
-bool lr_edge_eligible(const HostLayout &H) {
-    bool ok = H.all_binary && H.logic_groups.empty() && !H.enum_groups.empty() && H.ES == 2 * H.E && H.VS == 2 * H.V &&
-              H.E % 2 == 0 && !H.var_bucket[kVarBlock].empty();
-    for (const HostEnumGroup &hg : H.enum_groups) ok = ok && hg.variant == kPair2;
+// Whether the graph's runs can use the edge-order log-ratio form: binary variables, some of high
+// degree (G.hd_b), and either pairwise factors only (Plan::lr_edge) or OR and AND factors only
+// (Plan::lr_edge_logic), within the limits that one block and one warp sum.
+void plan_edge(const HostLayout &H, Plan *P) {
+    bool ok = H.all_binary && H.ES == 2 * H.E && H.VS == 2 * H.V && !H.var_bucket[kVarBlock].empty();
     for (int kind = 0; kind < kNumVarKinds; ++kind)
         if (kind != kVarBinary && kind != kVarBlock) ok = ok && H.var_bucket[kind].empty();
-    for (int32_t v : H.var_bucket[kVarBlock]) ok = ok && H.vin_off[v + 1] - H.vin_off[v] <= kLrEdgeMaxDegree;
-    return ok;
+    int32_t deg = 0;
+    for (int32_t v : H.var_bucket[kVarBlock]) deg = std::max(deg, H.vin_off[v + 1] - H.vin_off[v]);
+    bool pair = ok && H.logic_groups.empty() && !H.enum_groups.empty() && H.E % 2 == 0 && deg <= kLrEdgeMaxDegree;
+    for (const HostEnumGroup &hg : H.enum_groups) pair = pair && hg.variant == kPair2;
+    bool logic = ok && H.enum_groups.empty() && !H.logic_groups.empty() && deg <= kLrEdgeLogicDegree;
+    for (const HostLogicGroup &hg : H.logic_groups)
+        logic = logic && hg.seg.kind != PGM_LOGIC_XOR && hg.seg.max_fan <= kLrEdgeLogicFan;
+    P->lr_edge = pair;
+    P->lr_edge_logic = logic;
+    P->edge_var_threads = deg <= kLrEdgeMaxDegree ? 128 : 1024;
 }
 
 // Slots of each log-ratio array: 4 per variable with the 4-slot table, else one per edge.
@@ -595,7 +602,7 @@ pgm_status build_plan(const HostLayout &H, pgm_graph *g, Packer &pk, std::vector
     }
     plan_fused(H, g, pk);
     P.lr = lr_eligible(H);
-    P.lr_edge = lr_edge_eligible(H);
+    plan_edge(H, &P);
     P.lr_blocks = std::max(1, g->n_sm * 8);
     return PGM_OK;
 }
@@ -1086,8 +1093,8 @@ static bool log_ratio_run(const pgm_graph *g, int32_t n_iters) {
 // Whether such a run takes the edge-order form: graphs with high-degree variables, from the same
 // number of iterations. Per iteration it replaces the edge-state launches one for one, and the
 // first and last read and write msgs themselves, so no run length loses by it.
-static bool edge_ratio_run(const pgm_graph *g, int32_t n_iters) {
-    return g->P.lr_edge && !g->force_es && g->log_ratio_min_iters > 0 && n_iters >= g->log_ratio_min_iters;
+static bool edge_ratio_run(const pgm_graph *g, int32_t n_iters, float T) {
+    return (g->P.lr_edge || (g->P.lr_edge_logic && T == 0.f)) && !g->force_es && g->log_ratio_min_iters > 0 && n_iters >= g->log_ratio_min_iters;
 }
 
 // Whether a log-ratio run of this graph is one launch, and whether that launch is the
@@ -1131,7 +1138,7 @@ static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const f
         if (e != cudaSuccess) return cuda_fail(e, "small-graph run launch");
         return PGM_OK;
     }
-    const bool edge = edge_form && edge_ratio_run(g, n_iters);
+    const bool edge = edge_form && edge_ratio_run(g, n_iters, T);
     if (lr) {
         cudaError_t e = launch_lr_pack(g->G, msgs, d, s);
         if (e == cudaSuccess) e = launch_lr_params(g->G, g->P, log_pot, g->lr_prm, s);
@@ -1363,7 +1370,7 @@ static pgm_status run_multi_es(pgm_graph *g, int32_t n_samples, const float *log
         if (cudaMalloc(&g->mse_mem, need) != cudaSuccess) return fail(PGM_ENOMEM, "cudaMalloc(multi-sample scratch)");
         g->mse_bytes = need;
     }
-    const bool edge = edge_ratio_run(g, n_iters);
+    const bool edge = edge_ratio_run(g, n_iters, T);
     float *mt = reinterpret_cast<float *>(g->mse_mem), *bb = reinterpret_cast<float *>(g->mse_mem + r_mt);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     for (int64_t s0 = 0; s0 < n_samples; s0 += chunk) {

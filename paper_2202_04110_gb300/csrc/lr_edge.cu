@@ -1,5 +1,5 @@
-// Log-ratio iterations of binary pairwise graphs with high-degree variables (an RBM's layers):
-// one number per edge, d = m(1) - m(0), in edge order. The variable pass sums a variable's d into
+// Log-ratio iterations of binary graphs with high-degree variables -- pairwise factors (an RBM's
+// layers), or OR and AND factors in max-product (deconvolution): one number per edge, d = m(1) - m(0), in edge order. The variable pass sums a variable's d into
 // its total D (float-float); the factor pass forms both variable-to-factor log-ratios as D - d,
 // updates both messages and stores them in place.
 //
@@ -7,12 +7,16 @@
 // 64 bytes of state totals per factor; this one reads 4 and writes 4 bytes per edge, gathers 16
 // bytes of totals per factor and reads the tables as they are. The first iteration reads the
 // caller's messages and the last one writes them, so a run has no conversion passes and needs
-// no memory beyond the edge-state form's (d in its second message buffer, D in its beliefs).
+// no memory beyond the edge-state form's (d, and explicit sums where a term is infinite, in its
+// second message buffer, D in its beliefs).
 //
-// Measured against the edge-state launches (GB300, T = 1, whole calls, us per iteration): 784 x 500
-// (392,000 factors) 22.7 -> 11.1, 1000 x 1000 35.4 -> 17.5, 2000 x 128 22.9 -> 12.5, 100 x 150 10.7 ->
-// 4.0, 70 x 80 10.6 -> 3.6 (two launches' latency). Error of the messages against 64 bits, relative:
-// 7.7e-7 -> 9.4e-8.
+// Measured against the edge-state launches (GB300, whole calls, us per iteration), T = 1: 784 x 500
+// (392,000 factors) 22.7 -> 9.7, 1000 x 1000 35.4 -> 17.5, 2000 x 128 22.9 -> 12.5, 100 x 150 10.7 ->
+// 4.0, 70 x 80 10.6 -> 3.6 (two launches' latency); deconvolution of 100 images (T = 0, 1.8 million
+// AND factors, 22,500 ORs of up to 180 parents) 125 -> 91: per launch, events included, AND 42.8 ->
+// 27.1, OR 36.2 -> 24.9, the two variable launches 24.8 -> 22.1 and 32 -> 28.7, which are bound by
+// gathers of 4 bytes a sector. Error against 64 bits, relative: RBM messages 7.7e-7 -> 9.4e-8,
+// deconvolution 1.7e-7 -> 9.7e-8.
 #include <algorithm>
 
 #include "bp_common.cuh"
@@ -39,6 +43,13 @@ __device__ __forceinline__ float edge_ratio(const float *__restrict__ d, const f
 
 __device__ __forceinline__ bool aligned16(const float *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// The next launch may be scheduled once every block of this one has its inputs: where they are
+// all resident (784 x 500: 164,000 and 196,000 threads). Blocks that still queue need the places
+// (pdl_launch_if_small).
+__device__ __forceinline__ void pdl_launch_if_one_wave() {
+    if ((int64_t)gridDim.x * gridDim.y * blockDim.x <= 300000) pdl_launch_dependents();
+}
+
 // A state's total as hd_pair takes it: the float-float sum of the finite terms and the count
 // of the -inf ones.
 __device__ __forceinline__ void add_term(FF &s, float &c, float q) {
@@ -46,23 +57,24 @@ __device__ __forceinline__ void add_term(FF &s, float &c, float q) {
     else s = ff_add(s, q);
 }
 
-// Block per variable of more than kVarBlockDegree factors, 128 threads with 8 edges each in
-// flight. The gathers' latency bounds it: every block is resident at once (1284 blocks for 784 x
+// Block per variable of more than kVarBlockDegree factors, 128 threads (1024 on graphs with
+// variables of more than kLrEdgeMaxDegree) with 8 edges each in flight. The gathers' latency bounds it: every block is resident at once (1284 blocks for 784 x
 // 500), the edge list is read before the previous pass ends, and each thread adds its edges in
 // float-float before two levels of block sums.
-constexpr int kEdgeVarThreads = 128, kEdgeVarItems = 8;
-__global__ void __launch_bounds__(kEdgeVarThreads) k_edge_var_block(DevGraph G, const int32_t *__restrict__ list,
+constexpr int kEdgeVarItems = 8;
+template <int B>
+__global__ void __launch_bounds__(B) k_edge_var_block(DevGraph G, const int32_t *__restrict__ list,
                                                                     const float *__restrict__ ev,
                                                                     const float *__restrict__ d,
                                                                     const float *__restrict__ m,
                                                                     float2 *__restrict__ Dv) {
-    __shared__ float sh[3 * kEdgeVarThreads / 32];
+    __shared__ float sh[3 * B / 32];
     const int64_t smp = sample_select(G);  // multi-sample launches: this block's sample
     ev += smp * G.s_vs;
     d += smp * G.s_es;
     if (m) m += smp * G.s_es;
     Dv += smp * (G.s_vs / 2);
-    constexpr int N = kEdgeVarItems, B = kEdgeVarThreads;
+    constexpr int N = kEdgeVarItems;
     const int v = list ? __ldg(list + blockIdx.x) : (int)blockIdx.x;
     const int k0 = __ldg(G.vin_off + v), k1 = __ldg(G.vin_off + v + 1);
     int es[N];
@@ -75,7 +87,7 @@ __global__ void __launch_bounds__(kEdgeVarThreads) k_edge_var_block(DevGraph G, 
     };
     load_es(k0);
     pdl_wait();  // the previous pass's messages
-    pdl_launch_dependents();
+    pdl_launch_if_one_wave();
     const float2 e = make_float2(__ldg(ev + 2 * (size_t)v), __ldg(ev + 2 * (size_t)v + 1));
     FF s = ff_make(0.f);
     bool fin = isfinite(e.x) & isfinite(e.y);
@@ -129,7 +141,7 @@ __global__ void __launch_bounds__(256) k_edge_var_thread(DevGraph G, const int32
     const int v = i < n ? (list ? __ldg(list + i) : i) : 0;
     const int k0 = __ldg(G.vin_off + v), k1 = __ldg(G.vin_off + v + 1);
     pdl_wait();  // the previous pass's messages
-    pdl_launch_dependents();
+    pdl_launch_if_one_wave();
     if (i >= n) return;
     const float2 e = make_float2(__ldg(ev + 2 * (size_t)v), __ldg(ev + 2 * (size_t)v + 1));
     FF D = ff_add_nc(ff_make(e.y), -e.x);
@@ -148,30 +160,34 @@ __global__ void __launch_bounds__(256) k_edge_var_thread(DevGraph G, const int32
         Dv[v] = make_float2(D.hi, D.lo);
         return;
     }
-    FF s0 = ff_make(0.f), s1 = ff_make(0.f);
-    float c0 = 0.f, c1 = 0.f;
+    // an infinite (or NaN) term: each edge's explicit sums without its own message
+    float *lam = const_cast<float *>(d) + G.E;
     for (int k = k0; k < k1; ++k) {
-        const float2 q = lam_decode(edge_ratio(d, m, __ldg(G.vin_es + k)));
-        add_term(s0, c0, q.x);
-        add_term(s1, c1, q.y);
+        FF l0 = ff_make(e.x), l1 = ff_make(e.y);
+        for (int o = k0; o < k1; ++o) {
+            if (o == k) continue;
+            const float2 q = lam_decode(edge_ratio(d, m, __ldg(G.vin_es + o)));
+            l0 = ff_add(l0, q.x);
+            l1 = ff_add(l1, q.y);
+        }
+        lam[__ldg(G.vin_es + k) >> 1] = lam_encode(l0, l1);
     }
-    add_term(s0, c0, e.x);
-    add_term(s1, c1, e.y);
-    float4 *t = reinterpret_cast<float4 *>(G.hd_b) + 2 * (size_t)v;
-    t[0] = make_float4(s0.hi, s0.lo, c0, 0.f);
-    t[1] = make_float4(s1.hi, s1.lo, c1, 0.f);
     Dv[v] = make_float2(__uint_as_float(kDvSlow), 0.f);
 }
 
-// The leave-one-out log-ratio of an edge from its variable's two state totals.
-__device__ __noinline__ float edge_lam_slow(const DevGraph &G, int v, float mo) {
+// The leave-one-out log-ratio of edge e (vs: its edge_vs, mo its d) of a variable with an infinite
+// term: a high-degree variable's from its two state totals, another's from the explicit sums.
+__device__ __noinline__ float edge_lam_slow(const DevGraph &G, const float *d, int e, int vs, float mo) {
+    if (vs >= 0) return __ldcg(d + G.E + e);
     const float2 q = lam_decode(mo);
-    const float2 a = hd_pair(G, 2 * v, 0, q.x), b = hd_pair(G, 2 * v, 1, q.y);
-    return lam_encode(FF{a.x, a.y}, FF{b.x, b.y});
+    const float m2[2] = {q.x, q.y};
+    float l[2];
+    hd_v2f<2>(G, vs, m2, l);
+    return lam_encode(ff_make(l[0]), ff_make(l[1]));
 }
 
-__device__ __forceinline__ float edge_lam(const DevGraph &G, float2 D, int v, float mo) {
-    if (__float_as_uint(D.x) == kDvSlow) return edge_lam_slow(G, v, mo);
+__device__ __forceinline__ float edge_lam(const DevGraph &G, float2 D, const float *d, int e, int vs, float mo) {
+    if (__float_as_uint(D.x) == kDvSlow) return edge_lam_slow(G, d, e, vs, mo);
     const FF l = ff_add(FF{D.x, D.y}, -mo);
     return l.hi + l.lo;
 }
@@ -239,7 +255,7 @@ __global__ void __launch_bounds__(256) k_edge_pair(DevGraph G, const EnumSeg *__
     if (n > 0) tab[0] = lr_table(segs, n_seg, pot, g);
     if (n < 2) tab[1] = tab[0];
     pdl_wait();  // the variable pass's totals
-    pdl_launch_dependents();
+    pdl_launch_if_one_wave();
     if (n <= 0) return;
     float mo[4];
     if (m_in != nullptr) {
@@ -253,11 +269,10 @@ __global__ void __launch_bounds__(256) k_edge_pair(DevGraph G, const EnumSeg *__
         const float2 q = __ldcg(reinterpret_cast<const float2 *>(d + 2 * (size_t)g));
         mo[0] = q.x, mo[1] = q.y, mo[2] = 0.f, mo[3] = 0.f;
     }
-    const int v[4] = {(vs.x & 0x7fffffff) >> 1, (vs.y & 0x7fffffff) >> 1, (vs.z & 0x7fffffff) >> 1,
-                      (vs.w & 0x7fffffff) >> 1};
+    const int v[4] = {vs.x, vs.y, vs.z, vs.w};
     float2 D[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) D[i] = __ldcg(Dv + v[i]);
+    for (int i = 0; i < 4; ++i) D[i] = __ldca(Dv + ((v[i] & 0x7fffffff) >> 1));
     const float w = 1.f - damping;
     float o[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -269,7 +284,8 @@ __global__ void __launch_bounds__(256) k_edge_pair(DevGraph G, const EnumSeg *__
         const float al = fin ? t.w - t.z : CUDART_NAN_F;
         const float be = fin ? t.y - t.x : CUDART_NAN_F;
         const float m0 = mo[2 * f], m1 = mo[2 * f + 1];
-        const float l0 = edge_lam(G, D[2 * f], v[2 * f], m0), l1 = edge_lam(G, D[2 * f + 1], v[2 * f + 1], m1);
+        const int e = 2 * (g + f);
+        const float l0 = edge_lam(G, D[2 * f], d, e, v[2 * f], m0), l1 = edge_lam(G, D[2 * f + 1], d, e + 1, v[2 * f + 1], m1);
         const float dpq = al - be, E = MAXP ? 0.f : expm1f(-fabsf(dpq) * invT);
         float a = edge_dir<MAXP>(c, al, be, dpq, E, l1, m0, T, invT, damping, w);
         float b = edge_dir<MAXP>(be, c + dpq, c, dpq, E, l0, m1, T, invT, damping, w);
@@ -298,6 +314,167 @@ __global__ void __launch_bounds__(256) k_edge_pair(DevGraph G, const EnumSeg *__
     }
 }
 
+// ---- OR / AND factors, max-product ------------------------------------------------------
+//
+// The closed forms of k_logic_small and k_logic_warp on log-odds x = +-lam, which the log-ratio
+// form has at hand: no states to gather and subtract.
+
+__device__ __forceinline__ float edge_odds(const DevGraph &G, const float2 *Dv, const float *d, int e, int vs, float mo,
+                                           float sgn) {
+    const float l = edge_lam(G, __ldca(Dv + ((vs & 0x7fffffff) >> 1)), d, e, vs, mo);
+    return __float_as_uint(l) == kLamBothNegInf ? 0.f : sgn * l;  // (log_odds of a contradiction)
+}
+// The stored d of edge e, and the new one written.
+__device__ __forceinline__ float edge_load(const float *d, const float *m_in, int e) {
+    return m_in != nullptr ? edge_encode(load_pair(m_in + 2 * (size_t)e)) : __ldcg(d + e);
+}
+__device__ __noinline__ float edge_finish(float o, float mo, float damping, uint32_t *flags) {
+    const float2 q = lam_decode(mo);
+    const float old[2] = {q.x, q.y};
+    float t[2] = {o >= 0.f ? -o : 0.f, o >= 0.f ? 0.f : o};  // as write_logic_edge
+    finish_k<2>(t, old, damping, flags);
+    return t[1] - t[0];
+}
+__device__ __forceinline__ void edge_store(float *d, float *m_out, int e, float o, float mo, float damping,
+                                           uint32_t *flags) {
+    float n = fmaf(damping, mo, (1.f - damping) * o);
+    if (!isfinite(n)) n = edge_finish(o, mo, damping, flags);
+    if (m_out != nullptr) reinterpret_cast<float2 *>(m_out)[e] = lr_decode(n);
+    else d[e] = n;
+}
+
+// Thread per factor of at most F parents. A factor's edges and those of the next thread are
+// neighbours in d, and so are most of their variables' totals (L1).
+template <int F>
+__global__ void __launch_bounds__(256) k_edge_logic_small(DevGraph G, const LogicSeg *__restrict__ segs, int n_seg,
+                                                          const float2 *Dv, float *d, const float *m_in, float *m_out,
+                                                          float damping) {
+    const int64_t smp = sample_select(G);  // multi-sample launches: this block's sample
+    d += smp * G.s_es;
+    if (m_in) m_in += smp * G.s_es;
+    if (m_out) m_out += smp * G.s_es;
+    Dv += smp * (G.s_vs / 2);
+    const LogicSeg *S = segs + find_seg(segs, n_seg, blockIdx.x);
+    const int f = (blockIdx.x - __ldg(&S->block_begin)) * blockDim.x + threadIdx.x;
+    const bool have = f < __ldg(&S->n_fac);
+    const float sgn = __ldg(&S->kind) == PGM_LOGIC_AND ? -1.f : 1.f;
+    int n = 0, e0 = 0, vs[F], vc = 0;
+    if (have) {
+        const int *po = G.paroff_pool + __ldg(&S->paroff_base);
+        const int p0 = __ldg(po + f);
+        n = __ldg(po + f + 1) - p0;
+        e0 = __ldg(&S->edge_base) + p0 + f;
+#pragma unroll
+        for (int k = 0; k < F; ++k) vs[k] = k < n ? __ldg(G.edge_vs + e0 + k) : 0;
+        vc = __ldg(G.edge_vs + e0 + n);
+    }
+    pdl_wait();  // the variable pass's totals
+    pdl_launch_if_one_wave();
+    if (!have) return;
+    float x[F], mo[F];
+#pragma unroll
+    for (int k = 0; k < F; ++k) mo[k] = k < n ? edge_load(d, m_in, e0 + k) : 0.f;
+    const float moc = edge_load(d, m_in, e0 + n);
+#pragma unroll
+    for (int k = 0; k < F; ++k) x[k] = k < n ? edge_odds(G, Dv, d, e0 + k, vs[k], mo[k], sgn) : 0.f;
+    const float xc = edge_odds(G, Dv, d, e0 + n, vc, moc, sgn);
+    float A = 0.f, M = kNegInf;
+#pragma unroll
+    for (int j = 0; j < F; ++j)
+        if (j < n) {
+            A += fmaxf(x[j], 0.f);
+            M = fmaxf(M, x[j]);
+        }
+    edge_store(d, m_out, e0 + n, sgn * (A + (M < 0.f ? M : 0.f)), moc, damping, G.flags);
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+        if (i >= n) break;
+        float Si = 0.f, Mi = kNegInf;
+#pragma unroll
+        for (int j = 0; j < F; ++j)
+            if (j < n && j != i) {
+                Si += fmaxf(x[j], 0.f);
+                Mi = fmaxf(Mi, x[j]);
+            }
+        edge_store(d, m_out, e0 + i, sgn * or_parent_max(Si, Mi, xc), mo[i], damping, G.flags);
+    }
+}
+
+// Warp per factor of at most 32 R parents, R a lane. Every edge of the factor is in flight at
+// once and its indices are read before the variable pass ends; the parents' leave-one-out terms
+// come from the total (float-float, +inf terms counted) less their own and from the two largest
+// log-odds, instead of a scan in each direction.
+template <int R>
+__global__ void __launch_bounds__(128) k_edge_logic_warp(DevGraph G, const LogicSeg *__restrict__ segs, int n_seg,
+                                                         const float2 *Dv, float *d, const float *m_in, float *m_out,
+                                                         float damping) {
+    const int64_t smp = sample_select(G);  // multi-sample launches: this block's sample
+    d += smp * G.s_es;
+    if (m_in) m_in += smp * G.s_es;
+    if (m_out) m_out += smp * G.s_es;
+    Dv += smp * (G.s_vs / 2);
+    const int lane = threadIdx.x & 31;
+    const LogicSeg *S = segs + find_seg(segs, n_seg, blockIdx.x);
+    const int f = (blockIdx.x - __ldg(&S->block_begin)) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const bool have = f < __ldg(&S->n_fac);  // the whole warp
+    const float sgn = __ldg(&S->kind) == PGM_LOGIC_AND ? -1.f : 1.f;
+    int n = 0, e0 = 0, vs[R], vc = 0;
+    if (have) {
+        const int *po = G.paroff_pool + __ldg(&S->paroff_base);
+        const int p0 = __ldg(po + f);
+        n = __ldg(po + f + 1) - p0;
+        e0 = __ldg(&S->edge_base) + p0 + f;
+#pragma unroll
+        for (int r = 0; r < R; ++r) vs[r] = lane + 32 * r < n ? __ldg(G.edge_vs + e0 + lane + 32 * r) : 0;
+        vc = __ldg(G.edge_vs + e0 + n);
+    }
+    pdl_wait();  // the variable pass's totals
+    pdl_launch_if_one_wave();
+    if (!have) return;
+    float x[R], mo[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) mo[r] = lane + 32 * r < n ? edge_load(d, m_in, e0 + lane + 32 * r) : 0.f;
+    const float moc = edge_load(d, m_in, e0 + n);
+    const float xc = edge_odds(G, Dv, d, e0 + n, vc, moc, sgn);
+    FF A = ff_make(0.f);
+    float c = 0.f, M1 = kNegInf, M2 = kNegInf;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        x[r] = kNegInf;
+        if (lane + 32 * r < n) {
+            x[r] = edge_odds(G, Dv, d, e0 + lane + 32 * r, vs[r], mo[r], sgn);
+            if (x[r] == CUDART_INF_F) c += 1.f;
+            else A = ff_add(A, fmaxf(x[r], 0.f));
+            if (x[r] == x[r]) M2 = fmaxf(M2, fminf(M1, x[r]));  // (a NaN counts as nothing)
+            M1 = fmaxf(M1, x[r]);
+        }
+    }
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        A = ff_add(A, FF{__shfl_xor_sync(0xffffffffu, A.hi, s), __shfl_xor_sync(0xffffffffu, A.lo, s)});
+        c += __shfl_xor_sync(0xffffffffu, c, s);
+        const float o1 = __shfl_xor_sync(0xffffffffu, M1, s), o2 = __shfl_xor_sync(0xffffffffu, M2, s);
+        M2 = fmaxf(fminf(M1, o1), fmaxf(M2, o2));
+        M1 = fmaxf(M1, o1);
+    }
+    if (lane == 0) {
+        const float a = c > 0.f ? CUDART_INF_F : A.hi + A.lo;
+        edge_store(d, m_out, e0 + n, sgn * (a + (M1 < 0.f ? M1 : 0.f)), moc, damping, G.flags);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (lane + 32 * r >= n) break;
+        const bool inf = x[r] == CUDART_INF_F;
+        float Si = CUDART_INF_F;
+        if (c == (inf ? 1.f : 0.f)) {
+            const FF a = inf ? A : ff_add(A, -fmaxf(x[r], 0.f));
+            Si = fmaxf(a.hi + a.lo, 0.f);
+        }
+        edge_store(d, m_out, e0 + lane + 32 * r, sgn * or_parent_max(Si, x[r] == M1 ? M2 : M1, xc), mo[r], damping,
+                   G.flags);
+    }
+}
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_after(void (*kernel)(KArgs...), int blocks, int S, int threads, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg{};
@@ -320,7 +497,8 @@ cudaError_t launch_edge_var_pass(const DevGraph &G, const Plan &P, const float *
         if (L.n == 0) continue;
         const cudaError_t e =
             L.kind == kVarBlock
-                ? launch_after(k_edge_var_block, L.n, S, kEdgeVarThreads, s, G, L.list, ev, d, m_in, Dv)
+                ? (P.edge_var_threads == 128 ? launch_after(k_edge_var_block<128>, L.n, S, 128, s, G, L.list, ev, d, m_in, Dv)
+                                             : launch_after(k_edge_var_block<1024>, L.n, S, 1024, s, G, L.list, ev, d, m_in, Dv))
                 : launch_after(k_edge_var_thread, (L.n + 255) / 256, S, 256, s, G, L.list, L.n, ev, d, m_in, Dv);
         if (e != cudaSuccess) return e;
         if (hook) hook->after(hook->ctx);
@@ -335,11 +513,24 @@ cudaError_t launch_edge_factor_pass(const DevGraph &G, const Plan &P, const floa
     const float k = T > 0.f ? (float)(1.4426950408889634 / (double)T) : 0.f;
     const float Tln2 = (float)((double)T * 0.6931471805599453);
     const int F = G.E / 2;
-    for (const FactorLaunch &L : P.factor) {  // the one kPair2 launch: every factor
+    for (const FactorLaunch &L : P.factor) {
         if (L.n_blocks == 0) continue;
-        const cudaError_t e = launch_after(T == 0.f ? k_edge_pair<true> : k_edge_pair<false>, (F + 511) / 512, S, 256,
-                                           s, G, static_cast<const EnumSeg *>(L.segs), L.n_seg, F, log_pot, Dv, d, m_in,
-                                           m_out, T, T > 0.f ? 1.f / T : 0.f, k, Tln2, damping);
+        const LogicSeg *ls = static_cast<const LogicSeg *>(L.segs);
+        cudaError_t e;
+        if (L.variant == kPair2) {  // the one launch: every factor
+            e = launch_after(T == 0.f ? k_edge_pair<true> : k_edge_pair<false>, (F + 511) / 512, S, 256, s, G,
+                             static_cast<const EnumSeg *>(L.segs), L.n_seg, F, log_pot, Dv, d, m_in, m_out, T,
+                             T > 0.f ? 1.f / T : 0.f, k, Tln2, damping);
+        } else if (L.variant == kLogicSmall) {
+            e = launch_after(L.max_fan <= 2 ? k_edge_logic_small<2> : k_edge_logic_small<kLogicSmallFan>, L.n_blocks, S,
+                             L.threads, s, G, ls, L.n_seg, Dv, d, m_in, m_out, damping);
+        } else {
+            auto kern = L.max_fan <= 64    ? k_edge_logic_warp<2>
+                        : L.max_fan <= 128 ? k_edge_logic_warp<4>
+                        : L.max_fan <= 192 ? k_edge_logic_warp<6>
+                                           : k_edge_logic_warp<8>;
+            e = launch_after(kern, L.n_blocks, S, L.threads, s, G, ls, L.n_seg, Dv, d, m_in, m_out, damping);
+        }
         if (e != cudaSuccess) return e;
         if (hook) hook->after(hook->ctx);
     }

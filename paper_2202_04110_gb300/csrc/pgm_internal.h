@@ -28,6 +28,8 @@ constexpr int kEnumTableSmem = 160 * 1024;  // largest configuration table stage
 constexpr int kMaxStates = 256;
 constexpr int kVarBlockDegree = 64;  // variables with more factors use a block each
 constexpr int kLrEdgeMaxDegree = 4096;  // Plan::lr_edge: a variable's sum is one block's work
+constexpr int kLrEdgeLogicDegree = 16384;  // the same for lr_edge_logic, in blocks of 1024
+constexpr int kLrEdgeLogicFan = 256;       // and a factor is one warp's, 8 parents a lane
 constexpr int kVarBlockThreads = 256;
 constexpr int kVarItems = 8;                               // contiguous edges per thread
 constexpr int kVarTile = kVarBlockThreads * kVarItems;     // edges per tile
@@ -221,7 +223,9 @@ struct Plan {
     bool lr = false;
     // The same with high-degree variables of at most kLrEdgeMaxDegree factors: runs may
     // iterate on log-ratios in edge order (lr_edge.cu).
-    bool lr_edge = false;
+    // Likewise max-product runs of graphs of OR and AND factors only (lr_edge_logic).
+    bool lr_edge = false, lr_edge_logic = false;
+    int32_t edge_var_threads = 128;  // block of a high-degree variable (1024: some above kLrEdgeMaxDegree)
     int32_t lr_blocks = 1;  // persistent log-ratio factor pass: blocks of 256 (8 per SM)
     LrGridPlan grid;        // nb = 0: none
 };
