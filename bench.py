@@ -113,17 +113,24 @@ LR_KERNELS = ("k_pair2_lr", "k_var_slot4_lr", "k_var_csr_lr")
 
 def kernel_source_hash(kernel: str) -> str:
     """sha256 (16 hex digits) of the source a kernel is built from: for the log-ratio
-    kernels, kernels.cu's helper prelude (before the first section), its log-ratio
-    section and the log-ratio launchers; for the others, the whole of kernels.cu."""
-    with open(os.path.join(ROOT, "paper_2202_04110_gb300", "csrc", "kernels.cu")) as f:
-        src = f.read()
+    kernels, lr_math.cuh, bp_common.cuh, the log-ratio section of kernels.cu and the
+    log-ratio launchers; for the others, the whole of kernels.cu and the headers."""
+    csrc = os.path.join(ROOT, "paper_2202_04110_gb300", "csrc")
+
+    def read(name):
+        with open(os.path.join(csrc, name)) as f:
+            return f.read()
+
+    src = read("kernels.cu")
+    head = read("lr_math.cuh") + read("bp_common.cuh")
     if kernel in LR_KERNELS:
-        first = src.index("// =====")
         a = src.index("// Binary pairwise graphs: log-ratio messages (Plan::lr)")
         b = src.index("// Many evidence / potential sets on one binary pairwise graph")
         c = src.index("static cudaError_t launch_pdl(")
         d = src.index("cudaError_t launch_ms_prepare(")
-        src = src[:first] + src[a:b] + src[c:d]
+        src = head + src[a:b] + src[c:d]
+    else:
+        src += head + read("pair_math.cuh")
     return hashlib.sha256(src.encode()).hexdigest()[:16]
 
 
@@ -950,7 +957,7 @@ def run_ours(args):
     stream = torch.cuda.current_stream()
     temps = (1.0, 0.0)
 
-    run_events = []  # CUDA events around each run (one CUDA graph replay) of the timed steps
+    run_events = []  # CUDA events around each run of the timed steps
 
     def step(record=False):
         for T in temps:
@@ -969,20 +976,19 @@ def run_ours(args):
     # clocks: nvidia-smi samples from before the warm-up on, kept inside the timed window
     sampler = ClockSampler(torch.cuda.current_device())
     sampler.start()
-    # per-pass timing inside the timed runs: the captured CUDA graphs record events
-    # around the variable and factor passes of every PROFILE_PERIOD-th iteration
-    g.set_profiling(min(PROFILE_PERIOD, args.iters))
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
-    g.pass_times()  # reset
     ES = I["n_edge_states"]
     updates_per_step = len(temps) * args.iters * ES
     # log-ratio iterations (binary pairwise graph): one number per edge during the run;
     # per run one pack, one table-differences and one unpack launch
     lr_min = g.get_option(binding.OPT_LOG_RATIO)
     lr = lr_min > 0 and args.iters >= lr_min
-    launches_per_step = len(temps) * (args.iters * I["launches_per_iter"] + 2 + (3 if lr else 0))
+    # (a grid above the small forms whose 24 bytes per variable fit the SMs' shared
+    # memories is one cooperative launch per run; beliefs and decode follow either way)
+    one_launch = lr and I["max_degree"] <= 4 and (g.get_option(binding.OPT_SMALL_RUN) != 0 or I["n_vars"] <= 1_450_000)
+    launches_per_step = len(temps) * (2 + (1 if one_launch else args.iters * I["launches_per_iter"] + (3 if lr else 0)))
 
     if dist is not None:
         dist.barrier()
@@ -1002,6 +1008,16 @@ def run_ours(args):
     if dist is not None:
         dist.barrier()
     clocks = sampler.stop()
+    # per-pass times after the timed region: with profiling on a run keeps the launch per
+    # pass, and its CUDA graph records events around every PROFILE_PERIOD-th iteration's
+    g.set_profiling(min(PROFILE_PERIOD, args.iters))
+    step()
+    torch.cuda.synchronize()
+    g.pass_times()  # reset
+    for _ in range(min(args.steps, 3)):
+        flush.fill_(1.0)
+        step()
+    torch.cuda.synchronize()
     var_ms, fac_ms, n_var, n_fac = g.pass_times()
     g.set_profiling(0)
     ms = [a.elapsed_time(b) for a, b in step_ms]
@@ -1037,7 +1053,7 @@ def run_ours(args):
     var_gbs = var_bytes / var_avg_s / 1e9
     iter_bytes = fac_bytes + var_bytes
     run_ms = [a.elapsed_time(b) for a, b in run_events]
-    iter_run_s = statistics.mean(run_ms) / 1e3 / args.iters  # includes the run's pack / unpack
+    iter_run_s = statistics.mean(run_ms) / 1e3 / args.iters  # includes the run's conversions
     iter_s = (var_ms + fac_ms) / 1e3 / max(n_fac, 1)
     if lr:
         fac_name, var_name = "k_pair2_lr", ("k_var_slot4_lr" if I["max_degree"] <= 4 else "k_var_csr_lr")
@@ -1068,7 +1084,9 @@ def run_ours(args):
                         "mean_launch_us": round(1e6 * oth_s, 2),
                         "traffic": profiled_traffic(other, wl)}},
             "kernel_timing": "CUDA events on the launching stream around the passes of every "
-                             f"{min(PROFILE_PERIOD, args.iters)}th iteration of the timed runs (event nodes in their CUDA graphs)",
+                             f"{min(PROFILE_PERIOD, args.iters)}th iteration of runs after the timed ones, launch by "
+                             "launch (event nodes in their CUDA graphs); a timed run is one launch of both passes "
+                             "where the graph's size allows",
             "nominal_peak": NOMINAL_HBM_GBS, "frac_of_nominal": round(dom_gbs / NOMINAL_HBM_GBS, 4),
             "iteration": {"algorithmic_bytes": iter_bytes,
                           "implementation_bytes": impl_fac_bytes + impl_var_bytes,
@@ -1076,8 +1094,8 @@ def run_ours(args):
                           "achieved": round(iter_bytes / iter_run_s / 1e9, 1),
                           "frac": round(iter_bytes / iter_run_s / 1e9 / peak, 4),
                           "frac_of_nominal": round(iter_bytes / iter_run_s / 1e9 / NOMINAL_HBM_GBS, 4),
-                          "timing": "CUDA events around each pgm_run_bp call (one CUDA graph replay) "
-                                    "of the timed steps / iterations; both passes back to back",
+                          "timing": "CUDA events around each pgm_run_bp call of the timed steps / "
+                                    "iterations; both passes back to back",
                           "sum_of_pass_events_us": round(1e6 * iter_s, 2)}}
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -1210,9 +1228,9 @@ def deconv_probe(args):
 
 def small_probe(args):
     """`--small-probe N` runs of the 10x10 Ising workload (T=1, damping 0.5, 50
-    iterations: one k_lr_small launch each), or of a `--small-side` grid (one k_lr_small
-    or k_lr_cluster launch each), CUDA graphs off, for ncu captures of the one-launch
-    run. Prints one JSON line."""
+    iterations: one k_lr_push launch each), or of a `--small-side` grid (one k_lr_push or
+    k_lr_run launch each), CUDA graphs off, for ncu captures of the one-launch run. Prints
+    one JSON line."""
     import torch
     from paper_2202_04110_gb300 import binding, build
     from paper_2202_04110_gb300 import workloads as W
