@@ -662,24 +662,20 @@ def measure_deconv(args, binding, W, torch, dev):
         np.add.at(deg, lg_.parents, 1)
         np.add.at(deg, lg_.child, 1)
     hi = deg > 64
-    # implementation bytes per launch: the high-degree pass reads the variables' K d
-    # messages and their incoming-edge index, writes and re-reads the tile totals (16 bytes
-    # per tile and state) and writes each state's totals (16 bytes) and belief;
-    # a logical factor reads its old messages, the beliefs of its edges (the totals of a
-    # high-degree variable) and their index, and writes its messages
-    n_hi_es = int((ks[hi] * deg[hi]).sum())
+    # implementation bytes per launch of the edge-order log-ratio form: a variable reads 4
+    # bytes and an index per edge and its evidence, and writes its total (8 bytes); a logical
+    # factor reads and writes 4 bytes per edge and reads its edges' index and totals
     and_g, or_g = fg.logic_groups[0], fg.logic_groups[1]
     e_and = int(and_g.par_off[-1]) + and_g.n_fac
     e_or = int(or_g.par_off[-1]) + or_g.n_fac
-    d_hi = int(deg[hi].sum())
-    n_tiles_st = int((ks[hi] * ((deg[hi] + 2047) // 2048)).sum())
-    impl = {"k_var_hd": 4 * n_hi_es + 4 * d_hi + 32 * n_tiles_st + 20 * int(ks[hi].sum()),
-            "k_logic_small": 4 * (4 * e_and + 2 * e_and + e_and),
-            "k_logic_warp": 4 * (4 * e_or + 2 * e_or + e_or)}
-    s8d = {"k_logic_small": sec8d_bytes(fg, [0]), "k_logic_warp": sec8d_bytes(fg, [1]),
-           "k_var_hd": 4 * int(ks[hi].sum())}
-    names = {(0, 1): "k_var_hd", (0, 2): "k_var_thread<2>", (0, 0): "k_var_thread",
-             (1, 5): "k_logic_small", (1, 6): "k_logic_warp"}
+    impl = {"k_edge_var_block": 8 * int(deg[hi].sum()) + 16 * int(hi.sum()),
+            "k_edge_var_thread": 8 * int(deg[~hi].sum()) + 20 * int((~hi).sum()),
+            "k_edge_logic_small": (4 + 4 + 4 + 8) * e_and,
+            "k_edge_logic_warp": (4 + 4 + 4 + 8) * e_or}
+    s8d = {"k_edge_logic_small": sec8d_bytes(fg, [0]), "k_edge_logic_warp": sec8d_bytes(fg, [1]),
+           "k_edge_var_block": 4 * int(ks[hi].sum()), "k_edge_var_thread": 4 * int(ks[~hi].sum())}
+    names = {(0, 1): "k_edge_var_block", (0, 2): "k_edge_var_thread",
+             (1, 5): "k_edge_logic_small", (1, 6): "k_edge_logic_warp"}
     per = {}
     for (kind, variant, threads, blocks), (ms, cnt) in zip(launches, lt):
         name = names.get((kind, variant), f"kind{kind}_variant{variant}")
