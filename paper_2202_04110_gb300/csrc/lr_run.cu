@@ -23,8 +23,8 @@
 //   4. split factors: wait for the other block's value, one message in place;
 // with a block barrier after 1 and after 4. Step 3 runs while the values travel.
 // Measured against the multi-launch run (whole calls, GB300): 1000 x 1000, 200 iterations
-// 3.65 -> 2.16 ms (10.6 us per iteration), 317 x 241 max-product, 50 iterations 213 -> 93 us,
-// 32 evidence sets of 256 x 256, 100 iterations 4.22 -> 2.24 ms.
+// 3.65 -> 1.80 ms (8.9 us per iteration), 317 x 241 max-product, 50 iterations 213 -> 87 us,
+// 32 evidence sets of 256 x 256, 100 iterations 4.22 -> 2.14 ms.
 //
 // Inbox words carry their iteration: one 8-byte store holds (value, iteration), and the
 // reader polls its own word until the iteration is the one it is in; no fence, flag or
