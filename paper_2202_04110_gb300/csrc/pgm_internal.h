@@ -27,8 +27,12 @@ constexpr int kEnumPairsBlock = 32;         // factors per block of the max-prod
 constexpr int kEnumTableSmem = 160 * 1024;  // largest configuration table staged per block
 constexpr int kMaxStates = 256;
 constexpr int kVarBlockDegree = 64;  // variables with more factors use a block each
-constexpr int kLrEdgeMaxDegree = 4096;  // Plan::lr_edge: a variable's sum is one block's work
-constexpr int kLrEdgeLogicDegree = 16384;  // the same for lr_edge_logic, in blocks of 1024
+// Plan::lr_edge: a variable's sum is one block's work, where the edge-state form splits it over
+// tiles. Measured on both sides up to degree 2,000 (2000 x 128: 22.9 -> 12.5 us per iteration);
+// above, 128 threads take rounds of gathers in turn (4 at the limit).
+constexpr int kLrEdgeMaxDegree = 4096;
+// The same for lr_edge_logic in blocks of 1024: 180 variables of 10,000 factors 24.8 -> 22.1 us.
+constexpr int kLrEdgeLogicDegree = 16384;
 constexpr int kLrEdgeLogicFan = 256;       // and a factor is one warp's, 8 parents a lane
 constexpr int kVarBlockThreads = 256;
 constexpr int kVarItems = 8;                               // contiguous edges per thread
