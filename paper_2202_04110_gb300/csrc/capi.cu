@@ -1184,7 +1184,7 @@ static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const f
         ctx.count = 0;
         e = lr     ? launch_lr_factor_pass(g->G, g->P, log_pot, g->lr_prm, Dv, lam, d, T, damping, s, h)
             : edge ? launch_edge_factor_pass(g->G, g->P, log_pot, Dv, g->m_tmp, m_in, m_out, T, damping, s, 1, h)
-                   : launch_factor_pass(g->G, g->P, log_pot, g->b, evidence, cur, nxt, T, damping, s, 1, h);
+                   : launch_factor_pass(g->G, g->P, log_pot, g->b, evidence, cur, nxt, T, damping, s, 1, h, it > 0);
         if (e != cudaSuccess) return cuda_fail(e, "factor pass launch");
         grp.nf = (uint16_t)ctx.count;
         if (prof) {
@@ -1394,7 +1394,7 @@ static pgm_status run_multi_es(pgm_graph *g, int32_t n_samples, const float *log
         }
         for (int it = 0; !edge && it < n_iters; ++it) {
             cudaError_t e = launch_var_pass(Gs, g->P, ev, cur, bb, kVarIter, nullptr, s, S);
-            if (e == cudaSuccess) e = launch_factor_pass(Gs, g->P, lp, bb, ev, cur, nxt, T, damping, s, S);
+            if (e == cudaSuccess) e = launch_factor_pass(Gs, g->P, lp, bb, ev, cur, nxt, T, damping, s, S, nullptr, it > 0);
             if (e != cudaSuccess) return cuda_fail(e, "multi-sample pass launch");
             std::swap(cur, nxt);
         }
@@ -1896,8 +1896,10 @@ pgm_status pgm_run_bp_batch(pgm_graph *g, const float *log_pot, const float *evi
     for (int32_t it = 0; it < max_it && e == cudaSuccess; ++it) {
         e = launch_var_pass(G2, g->P, evidence, cur, g->b, kVarIter, nullptr, s);
         // one launch per kind of member: max-product (T = 0) and the others
-        if (e == cudaSuccess && any_max) e = launch_factor_pass(G2, g->P, log_pot, g->b, evidence, cur, nxt, 0.f, 0.f, s);
-        if (e == cudaSuccess && any_sum) e = launch_factor_pass(G2, g->P, log_pot, g->b, evidence, cur, nxt, 1.f, 0.f, s);
+        if (e == cudaSuccess && any_max)
+            e = launch_factor_pass(G2, g->P, log_pot, g->b, evidence, cur, nxt, 0.f, 0.f, s, 1, nullptr, it > 0);
+        if (e == cudaSuccess && any_sum)
+            e = launch_factor_pass(G2, g->P, log_pot, g->b, evidence, cur, nxt, 1.f, 0.f, s, 1, nullptr, it > 0);
         std::swap(cur, nxt);
         if (e == cudaSuccess && ends[it + 1] && it + 1 < max_it)
             e = launch_batch_freeze(g->bm_iters, it + 1, nm, g->mu_off, g->mu_frozen, cur, nxt, g->n_sm, s);
@@ -2171,11 +2173,11 @@ pgm_status pgm_launch_info(const pgm_graph *g, int32_t i, int32_t *kind, int32_t
     return PGM_OK;
 }
 
-// One iteration from `in` into `out` (out != in).
+// One iteration from `in` into `out` (out != in), behind other work of the call.
 static pgm_status one_iteration(pgm_graph *g, const float *log_pot, const float *evidence, float T, float damping,
                                 const float *in, float *out, cudaStream_t s) {
     cudaError_t e = launch_var_pass(g->G, g->P, evidence, in, g->b, kVarIter, nullptr, s);
-    if (e == cudaSuccess) e = launch_factor_pass(g->G, g->P, log_pot, g->b, evidence, in, out, T, damping, s);
+    if (e == cudaSuccess) e = launch_factor_pass(g->G, g->P, log_pot, g->b, evidence, in, out, T, damping, s, 1, nullptr, true);
     if (e != cudaSuccess) return cuda_fail(e, "iteration launch");
     return PGM_OK;
 }
@@ -2290,7 +2292,7 @@ static pgm_status enqueue_grad(pgm_graph *g, const float *log_pot, const float *
                 e = launch_var_pass(Gs, g->P, evidence, recp(i - 1), step_b(i - 1), kVarIter, nullptr, s, 1, nullptr, true);
                 if (e == cudaSuccess && i < t1 - t0)
                     e = launch_factor_pass(Gs, g->P, log_pot, step_b(i - 1), evidence, recp(i - 1), recp(i), T,
-                                           damping, s);
+                                           damping, s, 1, nullptr, true);
                 if (e != cudaSuccess) st = cuda_fail(e, "recompute launch");
             }
         } else {

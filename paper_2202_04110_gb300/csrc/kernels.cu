@@ -34,7 +34,8 @@
 // totals of finite entries and counts of -inf ones (hd_pair).
 //
 // Launches: the iteration's kernels go out with programmatic dependent launch (each
-// waits, pdl_wait, before touching memory), inside CUDA graphs when the graph allows.
+// waits, pdl_wait, before touching memory; pair_fused.cu reads its indices and table earlier,
+// except in a run's first launch), inside CUDA graphs when the graph allows.
 #include <algorithm>
 #include <cstdint>
 
@@ -3960,7 +3961,7 @@ cudaError_t launch_var_pass(const DevGraph &G, const Plan &P, const float *ev, c
 template <bool MAXP, bool MS>
 static void factor_pass_t(const DevGraph &G, const Plan &P, const float *pot, const float *b,
                           const float *ev, const float *m_old, float *m_new, float T, float damping,
-                          cudaStream_t s, int S, const LaunchHook *hook) {
+                          cudaStream_t s, int S, const LaunchHook *hook, bool later) {
     const float invT = MAXP ? 0.f : 1.f / T;
     for (const FactorLaunch &L : P.factor) {
         if (L.n_blocks == 0) continue;
@@ -4000,7 +4001,7 @@ static void factor_pass_t(const DevGraph &G, const Plan &P, const float *pot, co
             case kPairF4:
             case kPairF8:
             case kPairF16:
-                launch_pair_fused(G, L, pot, ev, m_old, m_new, T, damping, S, s);
+                launch_pair_fused(G, L, pot, ev, m_old, m_new, T, damping, S, later, s);
                 break;
             case kPairQ8:
                 launch_dep(k_pair_quad<8, MAXP, MS>, dim3(dim3(L.n_blocks, S)), L.threads, 0, s, G, es, L.n_seg, pot, b, ev, m_old, m_new, T, invT, damping);
@@ -4214,13 +4215,13 @@ cudaError_t launch_lr_unpack(const DevGraph &G, const float *d, float *m, cudaSt
 cudaError_t launch_factor_pass(const DevGraph &G, const Plan &P, const float *log_pot,
                                const float *b, const float *ev, const float *m_old,
                                float *m_new, float T, float damping, cudaStream_t s, int S,
-                               const LaunchHook *hook) {
+                               const LaunchHook *hook, bool later) {
     if (S > 1) {  // the multi-sample instantiations
-        if (T == 0.f) factor_pass_t<true, true>(G, P, log_pot, b, ev, m_old, m_new, T, damping, s, S, hook);
-        else factor_pass_t<false, true>(G, P, log_pot, b, ev, m_old, m_new, T, damping, s, S, hook);
+        if (T == 0.f) factor_pass_t<true, true>(G, P, log_pot, b, ev, m_old, m_new, T, damping, s, S, hook, later);
+        else factor_pass_t<false, true>(G, P, log_pot, b, ev, m_old, m_new, T, damping, s, S, hook, later);
     } else {
-        if (T == 0.f) factor_pass_t<true, false>(G, P, log_pot, b, ev, m_old, m_new, T, damping, s, 1, hook);
-        else factor_pass_t<false, false>(G, P, log_pot, b, ev, m_old, m_new, T, damping, s, 1, hook);
+        if (T == 0.f) factor_pass_t<true, false>(G, P, log_pot, b, ev, m_old, m_new, T, damping, s, 1, hook, later);
+        else factor_pass_t<false, false>(G, P, log_pot, b, ev, m_old, m_new, T, damping, s, 1, hook, later);
     }
     return cudaGetLastError();
 }

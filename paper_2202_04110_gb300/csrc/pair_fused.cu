@@ -323,7 +323,9 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
         m_old += smp * G.s_es;
         m_new += smp * G.s_es;
     }
-    // before the previous launch has finished: what is fixed for the run (indices, the table)
+    // before the previous launch has finished: what is fixed for the run (indices, the table). The
+    // table is the caller's, so a run's first launch is an ordinary one (launch_k): nothing of it
+    // runs before the caller's work on the stream is done
     const int4 B = __ldg(reinterpret_cast<const int4 *>(blocks + blockIdx.x));  // pos, n, es_base, pot_base
     const int es_base = B.z, n = B.y;
     const int l = threadIdx.x & (L - 1), team = threadIdx.x / L;
@@ -385,7 +387,7 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
 
 template <int K, bool MAXP, bool MS>
 cudaError_t launch_k(const DevGraph &G, const FactorLaunch &L, const float *pot, const float *ev, const float *m_old,
-                     float *m_new, float T, float damping, int S, cudaStream_t s) {
+                     float *m_new, float T, float damping, int S, bool later, cudaStream_t s) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)L.fuse_blocks, (unsigned)S);
     cfg.blockDim = dim3((unsigned)L.fuse_threads);
@@ -394,7 +396,7 @@ cudaError_t launch_k(const DevGraph &G, const FactorLaunch &L, const float *pot,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = later ? 1 : 0;  // a run's first launch starts after the caller's work, which may write pot
     auto kern = L.fuse_threads == 128 ? k_pair_fused<K, MAXP, MS, 128> : k_pair_fused<K, MAXP, MS, 256>;
     return cudaLaunchKernelEx(&cfg, kern, G, L.fuse, L.fuse_list, pot, ev, m_old, m_new, T, MAXP ? 0.f : 1.f / T,
                               damping);
@@ -402,22 +404,22 @@ cudaError_t launch_k(const DevGraph &G, const FactorLaunch &L, const float *pot,
 
 template <int K>
 cudaError_t launch_pick(const DevGraph &G, const FactorLaunch &L, const float *pot, const float *ev, const float *m_old,
-                        float *m_new, float T, float damping, int S, cudaStream_t s) {
+                        float *m_new, float T, float damping, int S, bool later, cudaStream_t s) {
     if (S > 1)
-        return T == 0.f ? launch_k<K, true, true>(G, L, pot, ev, m_old, m_new, T, damping, S, s)
-                        : launch_k<K, false, true>(G, L, pot, ev, m_old, m_new, T, damping, S, s);
-    return T == 0.f ? launch_k<K, true, false>(G, L, pot, ev, m_old, m_new, T, damping, 1, s)
-                    : launch_k<K, false, false>(G, L, pot, ev, m_old, m_new, T, damping, 1, s);
+        return T == 0.f ? launch_k<K, true, true>(G, L, pot, ev, m_old, m_new, T, damping, S, later, s)
+                        : launch_k<K, false, true>(G, L, pot, ev, m_old, m_new, T, damping, S, later, s);
+    return T == 0.f ? launch_k<K, true, false>(G, L, pot, ev, m_old, m_new, T, damping, 1, later, s)
+                    : launch_k<K, false, false>(G, L, pot, ev, m_old, m_new, T, damping, 1, later, s);
 }
 
 }  // namespace
 
 cudaError_t launch_pair_fused(const DevGraph &G, const FactorLaunch &L, const float *pot, const float *ev,
-                              const float *m_old, float *m_new, float T, float damping, int S, cudaStream_t s) {
+                              const float *m_old, float *m_new, float T, float damping, int S, bool later, cudaStream_t s) {
     switch (L.variant) {
-        case kPairF4: return launch_pick<4>(G, L, pot, ev, m_old, m_new, T, damping, S, s);
-        case kPairF8: return launch_pick<8>(G, L, pot, ev, m_old, m_new, T, damping, S, s);
-        case kPairF16: return launch_pick<16>(G, L, pot, ev, m_old, m_new, T, damping, S, s);
+        case kPairF4: return launch_pick<4>(G, L, pot, ev, m_old, m_new, T, damping, S, later, s);
+        case kPairF8: return launch_pick<8>(G, L, pot, ev, m_old, m_new, T, damping, S, later, s);
+        case kPairF16: return launch_pick<16>(G, L, pot, ev, m_old, m_new, T, damping, S, later, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -286,15 +286,18 @@ struct LaunchHook {
 // (n_samples > 1: samples as the launches' y dimension, at the strides of G)
 // An iteration's variable pass (kVarIter) leaves out the launches that a fused factor launch
 // of the plan replaces, unless `full`.
+// later: work of the same call precedes the factor pass on the stream (false: its first launch may
+// directly follow a kernel of the caller's, and no kernel of it starts before that has ended).
 cudaError_t launch_var_pass(const DevGraph &G, const Plan &P, const float *ev, const float *m,
                             float *b, int mode, int32_t *decode, cudaStream_t s, int n_samples = 1,
                             const LaunchHook *hook = nullptr, bool full = false);
 cudaError_t launch_pair_fused(const DevGraph &G, const FactorLaunch &L, const float *pot, const float *ev,
-                              const float *m_old, float *m_new, float T, float damping, int n_samples, cudaStream_t s);
+                              const float *m_old, float *m_new, float T, float damping, int n_samples, bool later,
+                              cudaStream_t s);
 cudaError_t launch_factor_pass(const DevGraph &G, const Plan &P, const float *log_pot,
                                const float *b, const float *ev, const float *m_old,
                                float *m_new, float T, float damping, cudaStream_t s, int n_samples = 1,
-                               const LaunchHook *hook = nullptr);
+                               const LaunchHook *hook = nullptr, bool later = false);
 // Log-ratio iteration of a Plan::lr graph (kernels.cu): d the factor-to-variable
 // messages, lam the variable-to-factor values, one log-ratio per edge in variable order
 // (slots DevGraph::lr_pos; 4V of them with vin_tab4, else E); the factor pass updates d
