@@ -845,7 +845,8 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
             D = make_float2(e.y - e.x, 0.f);
             bad |= !(D.x == D.x) | !(fabsf(d[lv]) + fabsf(d[Vc + lv]) + fabsf(d[2 * Vc + lv]) + fabsf(d[3 * Vc + lv]) < CUDART_INF_F);
         }
-        const float2 g = __ldg(reinterpret_cast<const float2 *>(P.gnb) + v0 + lv);
+        const float *gp = P.gnb + 2 * (size_t)(v0 + lv);  // (the caller's, at any 4-byte address)
+        const float2 g = make_float2(__ldg(gp), __ldg(gp + 1));
         const float x = D.x + D.y, a = g.y * sigma_t(x, 1.f).c - g.x * sigma_t(x, 1.f).s;
         dD[lv] = a;
 #pragma unroll
