@@ -1422,8 +1422,9 @@ pgm_status pgm_run_bp_multi(pgm_graph *g, int32_t n_samples, const float *log_po
     if (!ms)  // any other graph: edge-state iterations with the samples side by side
         return run_multi_es(g, n_samples, log_pot, pot_per_sample, evidence, T, damping, n_iters, msgs, stream);
     // One launch for a chunk of samples, every iteration inside it, where the device takes it
-    // (and, when a sample needs several blocks, few factors join two of them: at most half)
-    if (g->small_run != 0) {
+    // (and, when a sample needs several blocks, few factors join two of them: at most half). It reads
+    // evidence 8 bytes at a time; the passes below transpose it entry by entry, from any address.
+    if (g->small_run != 0 && (reinterpret_cast<uintptr_t>(evidence) & 7u) == 0) {
         const bool local = g->P.grid.nb > 0 && g->P.grid.n_split <= g->info.n_edges / 2;
         const LrMultiPlan p = lr_multi_plan((int)g->info.n_vars, n_samples, local);
         if (p.S > 1 && multi_reserve(g, p.sample_bytes * p.S) == PGM_OK) {

@@ -59,3 +59,21 @@ def test_backward_through_a_concatenation(gpu):
         grads.append(torch.autograd.grad(out, (lp, ev)))
     for a, b in zip(*grads):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("rows,cols,S", [(10, 10, 5), (20, 21, 9), (40, 41, 4), (90, 100, 3)])
+@pytest.mark.parametrize("per_sample", [False, True])
+def test_samples(gpu, rows, cols, S, per_sample):
+    """Evidence, log-potentials and messages of many samples."""
+    import torch
+    p = W.ising_grid(rows, cols, seed=7)
+    rng = np.random.default_rng(8)
+    ev = rng.standard_normal((S, p.evidence.size)).astype(np.float32)
+    lp = np.stack([p.log_pot * (1 + s) for s in range(S)]).astype(np.float32) if per_sample else p.log_pot
+    m0 = -np.abs(rng.standard_normal((S, p.graph.n_edge_states))).astype(np.float32)
+    g = gpu.Graph(p.graph)
+    on = [torch.as_tensor(a).cuda() for a in (lp, ev, m0)]
+    want = g.run_bp_multi(on[0], on[1], 1.0, 0.5, 9, on[2].clone())
+    for which in ((1,), (0, 2), (0, 1, 2)):
+        a = [_shifted(h) if i in which else torch.as_tensor(h).cuda() for i, h in enumerate((lp, ev, m0))]
+        assert torch.equal(g.run_bp_multi(a[0], a[1], 1.0, 0.5, 9, a[2]), want), which
