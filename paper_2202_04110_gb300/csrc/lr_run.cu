@@ -139,10 +139,10 @@ __device__ __noinline__ float run_exact(const LrRun &A, const float *pot, int v0
     return lr_dir_exact<MAXP>(phi, (es >> 1) & 1, l, mo, A.k, A.Tln2, A.damping, A.flags);
 }
 
-// A variable whose values do not come out finite: its four lam by the explicit sums.
-__device__ __noinline__ void run_var_slow(float *lam, int lv, int Vc, float2 e, float d0, float d1, float d2, float d3) {
+// A variable whose values do not come out finite: its four lam by the explicit sums, at lam[k step].
+__device__ __noinline__ void run_var_slow(float *lam, int step, float2 e, float d0, float d1, float d2, float d3) {
     const float dk[4] = {d0, d1, d2, d3};
-    const int pos[4] = {lv, Vc + lv, 2 * Vc + lv, 3 * Vc + lv};
+    const int pos[4] = {0, step, 2 * step, 3 * step};
     lr_var_slow(e, dk, pos, 4, lam);
 }
 
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
     const float *pot = A.pot + (size_t)smp * A.pot_stride;
     const float2 *ev = reinterpret_cast<const float2 *>(A.ev + (size_t)smp * A.ev_stride) + v0;
     float *msgs = A.msgs + (size_t)smp * A.msg_stride;
-    float *lam_g = LAM ? nullptr : A.lam + (size_t)smp * 4 * V;  // explicit sums, by local slot from 4 v0
+    float *lam_g = LAM ? nullptr : A.lam + (size_t)smp * 4 * V + 4 * (size_t)v0;  // explicit sums, 4 a variable
     int32_t *dir = A.dir + (size_t)smp * 4 * V;
     // shared memory: [records, split records,] lam or totals, [evidence,] [inbox,] slots, [addresses]
     char *sp = lr_sm;
@@ -296,8 +296,9 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
     auto lam_of = [&](int s, float dk) {
         if constexpr (LAM) return lam[s];
         else {
-            const float2 D = Dv[var_of(s)];
-            return is_slow(D) ? __ldcg(lam_g + 4 * (size_t)v0 + s) : lr_lam_from_D(D, dk);
+            const int lv = var_of(s);
+            const float2 D = Dv[lv];
+            return is_slow(D) ? __ldcg(lam_g + 4 * (size_t)lv + (s - lv) / Vc) : lr_lam_from_D(D, dk);
         }
     };
     // what the thread reads first in steps 1 and 3 is fixed for the run: in registers when the
@@ -326,9 +327,9 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
                          isfinite(l0) && isfinite(l1) && isfinite(l2) && isfinite(l3));
             if (slow) {
                 if constexpr (LAM) {
-                    run_var_slow(lam, lv, Vc, e, d0, d1, d2, d3);
+                    run_var_slow(lam + lv, Vc, e, d0, d1, d2, d3);
                 } else {
-                    run_var_slow(lam_g + 4 * (size_t)v0, lv, Vc, e, d0, d1, d2, d3);
+                    run_var_slow(lam_g + 4 * (size_t)lv, 1, e, d0, d1, d2, d3);
                     Dv[lv] = make_float2(__uint_as_float(kDvSlow), 0.f);
                 }
             } else if constexpr (LAM) {
@@ -803,7 +804,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
                 lam[2 * Vc + lv] = lr_lam_from_D(Df, d2);
                 lam[3 * Vc + lv] = lr_lam_from_D(Df, d3);
             } else {
-                run_var_slow(lam, lv, Vc, e, d0, d1, d2, d3);
+                run_var_slow(lam + lv, Vc, e, d0, d1, d2, d3);
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) __stcg(H + q * Vc + lv, lam[q * Vc + lv]);
