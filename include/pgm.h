@@ -62,7 +62,8 @@ typedef int32_t pgm_status;
 #define PGM_FLAG_CONTRADICTION 1u /* a message or belief had every state at -inf */
 #define PGM_FLAG_NAN 2u           /* a NaN reached a belief */
 #define PGM_FLAG_INDEX 4u         /* checked mode: an index array entry out of range (pgm_checked_report) */
-#define PGM_FLAG_TIMEOUT 8u       /* a one-launch run gave up waiting for another of its blocks (msgs undefined) */
+#define PGM_FLAG_TIMEOUT 8u       /* a one-launch run gave up waiting for another of its blocks (msgs undefined;
+                                     pgm_infer_host, pgm_run_bp_until and served requests then fail) */
 
 /* Limits of this build (checked by pgm_build). */
 #define PGM_MAX_STATES 256        /* states per variable */
@@ -549,14 +550,24 @@ pgm_status pgm_run_bp_until_members(pgm_graph *g, const float *log_pot, const fl
  * launches_per_iter and pgm_launch_info describe. Changing it drops the cached CUDA
  * graphs. pgm_get_option returns the setting where a log-ratio run of the graph takes
  * the one-block or cluster form, else 0 (it asks the device once whether the cluster fits).
- * A block's wait for another block is bounded; one that runs out raises PGM_FLAG_TIMEOUT.
+ * A block's wait for another block is bounded (PGM_OPT_WAIT_POLLS). One that runs out raises
+ * PGM_FLAG_TIMEOUT in the status word and ends the run with msgs undefined: pgm_run_bp and
+ * pgm_run_bp_multi have returned by then, calls that return results to the host (pgm_infer_host,
+ * pgm_run_bp_until, served requests) fail with PGM_ECUDA, and pgm_grad makes its launches instead.
  * Values outside 0..2: PGM_EINVAL.
  */
 #define PGM_OPT_SMALL_RUN 6
+/*
+ * PGM_OPT_WAIT_POLLS (default 4,194,304: some seconds): how often a block of a one-launch run looks
+ * for another block's value before it gives up (PGM_FLAG_TIMEOUT); with 0 every run of several blocks
+ * counts as given up (for tests). Changing it drops the recorded CUDA graphs. Values outside 0..2^30:
+ * PGM_EINVAL.
+ */
+#define PGM_OPT_WAIT_POLLS 7
 pgm_status pgm_set_option(pgm_graph *g, int32_t option, int64_t value);
 /*
  * The option's effective value in *value: for PGM_OPT_CUDA_GRAPH, PGM_OPT_ENUM_BLOCK,
- * PGM_OPT_PAIR_FORM and PGM_OPT_CHECKED the setting; for PGM_OPT_LOG_RATIO the setting
+ * PGM_OPT_PAIR_FORM, PGM_OPT_CHECKED and PGM_OPT_WAIT_POLLS the setting; for PGM_OPT_LOG_RATIO the setting
  * if the graph qualifies, else 0; for PGM_OPT_SMALL_RUN the setting if it is on and the
  * graph qualifies, else 0. PGM_EINVAL for a NULL argument or an unknown option. No
  * device work (beyond one occupancy query per device for PGM_OPT_SMALL_RUN).

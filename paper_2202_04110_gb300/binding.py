@@ -20,6 +20,7 @@ STATUS_NAMES = {-1: "PGM_EINVAL", -2: "PGM_ENOMEM", -3: "PGM_ECUDA", -4: "PGM_EN
 FLAG_CONTRADICTION = 1
 FLAG_NAN = 2
 FLAG_INDEX = 4
+FLAG_TIMEOUT = 8
 
 # Every symbol include/pgm.h declares.
 EXPORTED = ["pgm_build", "pgm_build_batch", "pgm_batch_member", "pgm_check_desc", "pgm_free", "pgm_graph_info", "pgm_run_bp", "pgm_beliefs",
@@ -33,6 +34,7 @@ OPT_ENUM_BLOCK = 3
 OPT_PAIR_FORM = 4
 OPT_CHECKED = 5
 OPT_SMALL_RUN = 6
+OPT_WAIT_POLLS = 7
 
 
 class PgmError(RuntimeError):

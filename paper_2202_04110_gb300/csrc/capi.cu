@@ -81,8 +81,9 @@ struct pgm_graph {
     // word (device), its host copy (pinned); allocated on first use
     float *until_prev = nullptr;
     unsigned *until_res = nullptr;       // residual bits; the next word counts iterations done
-    unsigned *until_res_host = nullptr;  // 2 words (pinned; stream-ordered graphs: until_words)
-    unsigned until_words[2] = {0, 0};
+    // their host copies and that of status word kTimeoutWord (pinned; stream-ordered graphs: until_words)
+    unsigned *until_res_host = nullptr;
+    unsigned until_words[3] = {0, 0, 0};
     // device-side early-exit runs (conditional while node), keyed by their arguments
     struct CachedUntil {
         const float *log_pot, *evidence;
@@ -174,6 +175,10 @@ struct pgm_graph {
     int32_t use_cuda_graph = 1;
     int32_t log_ratio_min_iters = 4;  // PGM_OPT_LOG_RATIO
     int32_t small_run = 1;            // PGM_OPT_SMALL_RUN
+    int32_t wait_polls = kLrWaitPolls;  // PGM_OPT_WAIT_POLLS
+    uint32_t run_id = 0;              // number of the last run whose blocks wait for one another
+    bool run_waits = false;           // the last pgm_run_bp was such a run
+    uint32_t *io_word = nullptr;      // pgm_infer_host: its kTimeoutWord (pinned)
     cudaStream_t capture_stream = nullptr;
     std::vector<CachedRun> runs;
     // pgm_grad as CUDA graphs (PGM_OPT_CUDA_GRAPH): persistent work buffers and the
@@ -961,6 +966,18 @@ pgm_status pgm::build_graph_on_stream(const pgm_graph_desc *desc, cudaStream_t s
     return st;
 }
 
+// Results of a run with waits are good if none ran out: checked by every call that hands results to
+// the host (pgm_run_bp, pgm_run_bp_multi leave it to the status word).
+cudaError_t pgm::fetch_wait_word(const pgm_graph *g, uint32_t *host, cudaStream_t s) {
+    if (!g->run_waits) return cudaSuccess;
+    return cudaMemcpyAsync(host, g->G.flags + kTimeoutWord, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+}
+
+pgm_status pgm::wait_status(pgm_graph *g, uint32_t word) {
+    if (!g->run_waits || word != g->run_id) return PGM_OK;
+    return fail(PGM_ECUDA, "a block's wait for another block of the run ran out (PGM_FLAG_TIMEOUT): no result");
+}
+
 int64_t pgm::layout_device_bytes(const HostLayout &H) {
     size_t nb = 0;
     for (int kk = 0; kk < kNumVarKinds; ++kk) nb += H.var_bucket_identity[kk] ? 0 : H.var_bucket[kk].size();
@@ -1065,6 +1082,7 @@ void pgm_free(pgm_graph *g) {
     if (g->pmp_ev) cudaFree(g->pmp_ev);
     if (g->until_prev) cudaFree(g->until_prev);
     if (g->until_res_host) cudaFreeHost(g->until_res_host);
+    if (g->io_word) cudaFreeHost(g->io_word);
     if (g->mu_mem) cudaFree(g->mu_mem);
     if (g->bm_mem) cudaFree(g->bm_mem);
     if (g->audit_mem) cudaFree(g->audit_mem);
@@ -1120,6 +1138,13 @@ static bool grid_run_used(const pgm_graph *g) {
            lr_grid_fits(g->P.grid, g->G.V, g->G.E / 2);
 }
 
+// The waits of the run that is about to be launched.
+static LrWait next_wait(pgm_graph *g) {
+    g->run_waits = true;
+    if (++g->run_id == 0) g->run_id = 1;
+    return LrWait{g->wait_polls, g->run_id};
+}
+
 // edge_form: a run of its own, which may take the edge-order log-ratio form (the parts of other
 // runs keep their ping-pong buffers).
 static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const float *evidence, float T,
@@ -1133,8 +1158,9 @@ static pgm_status enqueue_iterations(pgm_graph *g, const float *log_pot, const f
     float2 *Dv = reinterpret_cast<float2 *>(g->b);
     // a small graph: the whole run in one launch (per-pass profiling keeps the passes)
     if (lr && small_run_used(g) && !(profile && g->profiling > 0)) {
+        const bool cluster = small_run_cluster(g);
         cudaError_t e = launch_lr_small_run(g->G, g->P, log_pot, evidence, msgs, lam, reinterpret_cast<int32_t *>(d), T,
-                                            damping, n_iters, small_run_cluster(g), s);
+                                            damping, n_iters, cluster, cluster ? next_wait(g) : LrWait{}, s);
         if (e != cudaSuccess) return cuda_fail(e, "small-graph run launch");
         return PGM_OK;
     }
@@ -1432,7 +1458,7 @@ pgm_status pgm_run_bp_multi(pgm_graph *g, int32_t n_samples, const float *log_po
                 cudaError_t e = launch_lr_multi_run(
                     g->G, g->P, p, std::min(p.S, n_samples - s0), pot_per_sample ? P : 0,
                     log_pot + (pot_per_sample ? (size_t)s0 * P : 0), evidence + (size_t)s0 * VS, msgs + (size_t)s0 * ES,
-                    static_cast<char *>(g->ms_mem), T, damping, n_iters, static_cast<cudaStream_t>(stream));
+                    static_cast<char *>(g->ms_mem), T, damping, n_iters, next_wait(g), static_cast<cudaStream_t>(stream));
                 if (e != cudaSuccess) return cuda_fail(e, "multi-sample run launch");
             }
             return PGM_OK;
@@ -1609,7 +1635,7 @@ pgm_status pgm_run_bp_until(pgm_graph *g, const float *log_pot, const float *evi
             return fail(PGM_ENOMEM, "cudaMalloc(residual buffers)");
         g->until_prev = reinterpret_cast<float *>(mem);
         g->until_res = reinterpret_cast<unsigned *>(mem + align_up((size_t)ES * sizeof(float), 256));
-        if (cudaMallocHost(&g->until_res_host, 2 * sizeof(unsigned)) != cudaSuccess) {
+        if (cudaMallocHost(&g->until_res_host, 3 * sizeof(unsigned)) != cudaSuccess) {
             cudaFree(g->until_prev);
             g->until_prev = nullptr;
             g->until_res = nullptr;
@@ -1620,6 +1646,18 @@ pgm_status pgm_run_bp_until(pgm_graph *g, const float *log_pot, const float *evi
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int32_t done = 0;
     float res = CUDART_NAN_F_HOST;
+    // chunks of small graphs may be cluster runs: their waits must not have run out
+    const bool waits = g->P.lr && small_run_used(g) && small_run_cluster(g);
+    uint32_t *word = g->until_res_host + 2;
+    *word = 0;
+    if (waits && cudaMemsetAsync(g->G.flags + kTimeoutWord, 0, sizeof(uint32_t), s) != cudaSuccess)
+        return cuda_fail(cudaGetLastError(), "cudaMemsetAsync(status word)");
+    auto finish = [&]() {
+        cudaError_t e = cudaSuccess;
+        if (waits) e = cudaMemcpyAsync(word, g->G.flags + kTimeoutWord, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+        return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+    };
+    const char *gave_up = "a block's wait for another block of the run ran out (PGM_FLAG_TIMEOUT): msgs undefined";
     // With CUDA graphs on, the full chunks run as one graph whose conditional while node
     // repeats a chunk while its residual is above tol: no host round trip per chunk.
     const int32_t limit = (max_iters / check_every) * check_every;
@@ -1630,8 +1668,9 @@ pgm_status pgm_run_bp_until(pgm_graph *g, const float *log_pot, const float *evi
         cudaError_t e = cudaGraphLaunch(exec, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(g->until_res_host, g->until_res, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = finish();
         if (e != cudaSuccess) return cuda_fail(e, "early-exit graph");
+        if (*word != 0) return fail(PGM_ECUDA, gave_up);
         std::memcpy(&res, g->until_res_host, sizeof res);
         done = (int32_t)g->until_res_host[1];
         if (res <= tol || done >= max_iters) {
@@ -1649,8 +1688,9 @@ pgm_status pgm_run_bp_until(pgm_graph *g, const float *log_pot, const float *evi
         if (e == cudaSuccess) e = launch_residual(ES, msgs, prev, g->until_res, g->n_sm, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(g->until_res_host, g->until_res, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = finish();
         if (e != cudaSuccess) return cuda_fail(e, "residual");
+        if (*word != 0) return fail(PGM_ECUDA, gave_up);
         std::memcpy(&res, g->until_res_host, sizeof res);
         done += n;
         if (res <= tol) break;
@@ -1961,10 +2001,11 @@ pgm_status pgm_run_bp(pgm_graph *g, const float *log_pot, const float *evidence,
     DeviceGuard dg(g->device);
     if (!dg.ok) return fail(PGM_ECUDA, "cudaSetDevice failed");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    g->run_waits = false;
     if (g->profiling == 0 && log_ratio_run(g, n_iters)) {  // one launch: nothing to record
         if (grid_run_used(g)) {
             cudaError_t e = launch_lr_grid_run(g->G, g->P, g->P.grid, log_pot, evidence, msgs, g->lr_lam, g->m_tmp, g->b,
-                                               g->lr_d, g->lr_prm, T, damping, n_iters, s);
+                                               g->lr_d, g->lr_prm, T, damping, n_iters, next_wait(g), s);
             if (e != cudaSuccess) return cuda_fail(e, "grid run launch");
             return PGM_OK;
         }
@@ -2348,7 +2389,7 @@ static pgm_status one_launch_grad(pgm_graph *g, const LrGradPlan &one, const flo
     if (e == cudaSuccess) e = cudaMemsetAsync(d_log_pot, 0, (size_t)g->info.n_potentials * sizeof(float), cs);
     if (e == cudaSuccess)
         e = launch_lr_grad(g->G, g->P, one, log_pot, evidence, d_beliefs, d_log_pot, d_evidence, hist, bail, g->m_tmp,
-                           g->lr_d, g->lr_prm, T, damping, n_iters, cs);
+                           g->lr_d, g->lr_prm, T, damping, n_iters, LrWait{g->wait_polls, 0}, cs);
     if (e == cudaSuccess) e = launch_set_condition(h, bail, cs);
     cudaError_t e2 = cudaStreamEndCapture(cs, &captured);
     if (e == cudaSuccess) e = e2;
@@ -2509,6 +2550,11 @@ pgm_status pgm_set_option(pgm_graph *g, int32_t option, int64_t value) {
             if (value != g->small_run) drop_cached_runs(g);
             g->small_run = (int32_t)value;
             return PGM_OK;
+        case PGM_OPT_WAIT_POLLS:
+            if (value < 0 || value > (1 << 30)) return fail(PGM_EINVAL, "PGM_OPT_WAIT_POLLS must be in 0..2^30");
+            if (value != g->wait_polls) drop_cached_runs(g);  // (recorded calls carry it)
+            g->wait_polls = (int32_t)value;
+            return PGM_OK;
         case PGM_OPT_ENUM_BLOCK: {
             if (value != 0 && value != 1) return fail(PGM_EINVAL, "PGM_OPT_ENUM_BLOCK must be 0 or 1");
             DeviceGuard dg(g->device);
@@ -2596,6 +2642,9 @@ pgm_status pgm_get_option(const pgm_graph *g, int32_t option, int64_t *value) {
         case PGM_OPT_CHECKED:
             *value = g->checked;
             return PGM_OK;
+        case PGM_OPT_WAIT_POLLS:
+            *value = g->wait_polls;
+            return PGM_OK;
         case PGM_OPT_SMALL_RUN: {
             DeviceGuard dg(g->device);  // whether the device can place the cluster form
             *value = small_run_used(g) ? g->small_run : 0;
@@ -2649,6 +2698,10 @@ pgm_status pgm_infer_host(pgm_graph *g, const float *log_pot, const float *evide
         cudaError_t e = cudaMalloc(&m, b_pot + 2 * b_ev + b_msgs + b_dec);
         if (e != cudaSuccess) return fail(PGM_ENOMEM, std::string("cudaMalloc(io): ") + cudaGetErrorString(e));
         g->host_io_mem = m;
+        if (g->P.grid.nb > 0 && cudaMallocHost(&g->io_word, sizeof(uint32_t)) != cudaSuccess) {
+            g->io_word = nullptr;  // (a pageable word then)
+            cudaGetLastError();
+        }
         g->io_pot = reinterpret_cast<float *>(m);
         g->io_ev = reinterpret_cast<float *>(m + b_pot);
         g->io_bel = reinterpret_cast<float *>(m + b_pot + b_ev);
@@ -2677,9 +2730,11 @@ pgm_status pgm_infer_host(pgm_graph *g, const float *log_pot, const float *evide
         e = cudaMemcpyAsync(decode, g->io_dec, I.n_vars * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return cuda_fail(e, "pgm_infer_host download");
     }
-    e = cudaStreamSynchronize(s);
+    uint32_t pageable = 0, *word = g->io_word ? g->io_word : &pageable;
+    e = fetch_wait_word(g, word, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    return PGM_OK;
+    return wait_status(g, *word);
 }
 
 pgm_status pgm_set_profiling(pgm_graph *g, int32_t period) {

@@ -37,8 +37,10 @@
 //     local read;
 //   - a cooperative grid of up to one block per SM (above that): the inboxes are in global
 //     memory (L2).
-// Every wait is bounded: after kWaitLimit polls a block raises PGM_FLAG_TIMEOUT in the status
-// word, stops waiting and runs to its end.
+// Every wait is bounded: after LrWait::polls polls a block raises PGM_FLAG_TIMEOUT in the status
+// word, notes the run beside it, stops waiting and runs to its end. (The barrier's words are right
+// again by then: every block of a launch arrives, also one that gives up, and the last one to
+// arrive resets the count.)
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
@@ -52,7 +54,6 @@ namespace pgm {
 namespace {
 
 constexpr uint32_t kFlagTimeout = PGM_FLAG_TIMEOUT;
-constexpr int kWaitLimit = 1 << 22;  // polls: about a second on a device-memory word
 
 // Where a block's items and exchanged values live.
 enum Exchange : int { kAlone = 0, kCluster = 1, kGrid = 2 };
@@ -78,7 +79,14 @@ struct LrRun {
     float4 *hrec;           // split factors' records when not in shared memory
     uint32_t *hdst;         // and the other block's inbox word
     uint32_t *bar;          // launch-wide barrier: arrivals, generation
+    LrWait wait;
 };
+
+// A wait of this run has run out.
+__device__ __forceinline__ void wait_failed(const LrRun &A) {
+    atomicOr(A.flags, kFlagTimeout);
+    *(volatile uint32_t *)(A.flags + kTimeoutWord) = A.wait.run_id;
+}
 
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -104,7 +112,7 @@ __device__ __forceinline__ unsigned long long box_word(float v, uint32_t it) {
 // All blocks of the launch (co-resident: a cooperative launch), once. The last to arrive
 // resets the count and moves the generation on, so the words need no clearing between
 // launches.
-__device__ __forceinline__ bool grid_barrier_once(uint32_t *bar, uint32_t n_blocks, uint32_t *flags) {
+__device__ __forceinline__ bool grid_barrier_once(uint32_t *bar, uint32_t n_blocks, int limit) {
     bool ok = true;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -117,11 +125,8 @@ __device__ __forceinline__ bool grid_barrier_once(uint32_t *bar, uint32_t n_bloc
             atomicAdd(bar + 1, 1u);
         } else {
             int polls = 0;
-            while (*gen == g0 && ++polls < kWaitLimit) __nanosleep(64);
-            if (*gen == g0) {
-                atomicOr(flags, kFlagTimeout);
-                ok = false;
-            }
+            while (*gen == g0 && ++polls < limit) __nanosleep(64);
+            ok = *gen != g0;
         }
         __threadfence();
     }
@@ -215,7 +220,10 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
 
     // ---- prologue: slots from msgs, the block's items ----
     if (tid < 2) s_n[tid] = 0;
-    if (tid == 0) s_abort = 0;
+    if (tid == 0) {
+        s_abort = X != kAlone && A.wait.polls == 0;
+        if (s_abort) wait_failed(A);
+    }
     __syncthreads();
     for (int l0 = 0; l0 < nv; l0 += nt) {
         const int lv = l0 + tid, v = v0 + lv;
@@ -274,9 +282,12 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
             __stcg(A.box0 + h_base + h, 0ull);
             __stcg(A.box1 + h_base + h, 0ull);
         }
-        ok = grid_barrier_once(A.bar, gridDim.x, A.flags);
+        ok = grid_barrier_once(A.bar, gridDim.x, A.wait.polls);
     }
-    if (X == kGrid && !ok) return;  // (a block that got past the barrier times out in its waits)
+    if (X == kGrid && !ok) {  // (a block that got past the barrier times out in its waits)
+        if (tid == 0) wait_failed(A);
+        return;
+    }
     for (int h = tid; h < nH; h += nt) {  // where each split factor's value goes
         const int s = (int)__float_as_uint(hrec[h].w), q = s / Vc, lv = s - q * Vc;
         const int4 t = __ldg(A.tab4 + v0 + lv);
@@ -403,8 +414,8 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
                     }
                     if ((uint32_t)(wd >> 32) == (uint32_t)it) break;
                     if (*(volatile int *)&s_abort) break;
-                    if (++polls >= kWaitLimit) {
-                        atomicOr(A.flags, kFlagTimeout);
+                    if (++polls >= A.wait.polls) {
+                        wait_failed(A);
                         *(volatile int *)&s_abort = 1;
                         break;
                     }
@@ -590,7 +601,8 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_push(const LrRun A) {
 // kept per factor and written once; the two blocks of a split factor add theirs to zeros (a sum of
 // two terms: the same bits in either order), so repeated calls give the same bits.
 // Tables with non-finite entries, contradictions and infinite messages (a lam of +-inf is
-// fine: its sigmas are 0 or 1) set *bail, and the caller's launches take over.
+// fine: its sigmas are 0 or 1) set *bail, and so does a wait that runs out: the caller's launches
+// take over.
 // Measured (GB300, whole calls): 64 x 64, 100 iterations, checkpoints every 10: 1.59 ms as ~590
 // dependent launches of 2.4 us, 0.31 in one; with lr_dir's SFU forms 0.28, but the table
 // gradients' error against 64 bits rose from 2.3e-7 to 2.7e-7 (mean of 15 grids). What bounds it:
@@ -652,7 +664,7 @@ __device__ __forceinline__ void grad_publish(const LrRun &A, const float *val, c
 }
 template <int X>
 __device__ __forceinline__ float grad_receive(const LrRun &A, const unsigned long long *box, size_t h_base, int h, int st,
-                                              int *s_abort) {
+                                              int *s_abort, int *bail) {
     unsigned long long wd = 0;
     int polls = 0;
     while (true) {
@@ -663,15 +675,15 @@ __device__ __forceinline__ float grad_receive(const LrRun &A, const unsigned lon
             const unsigned long long *p = ((st & 1) ? A.box1 : A.box0) + h_base + h;
             asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(wd) : "l"(p) : "memory");
         }
-        if ((uint32_t)(wd >> 32) == (uint32_t)st) break;
+        if ((uint32_t)(wd >> 32) == (uint32_t)st) return __uint_as_float((uint32_t)wd);
         if (*(volatile int *)s_abort) break;
-        if (++polls >= kWaitLimit) {
-            atomicOr(A.flags, kFlagTimeout);
+        if (++polls >= A.wait.polls) {
+            *(volatile int *)bail = 1;
             *(volatile int *)s_abort = 1;
             break;
         }
     }
-    return __uint_as_float((uint32_t)wd);
+    return 0.f;
 }
 
 template <int X>
@@ -710,7 +722,10 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
     uint32_t *hdst = reinterpret_cast<uint32_t *>(sp);
 
     if (tid < 2) s_n[tid] = 0;
-    if (tid == 0) s_abort = 0;
+    if (tid == 0) {
+        s_abort = X != kAlone && A.wait.polls == 0;
+        if (s_abort) *(volatile int *)P.bail = 1;
+    }
     for (int i = tid; i < A.f_cap; i += nt) racc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i = tid; i < A.h_cap; i += nt) hacc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
@@ -768,9 +783,12 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
             __stcg(A.box0 + h_base + h, 0ull);
             __stcg(A.box1 + h_base + h, 0ull);
         }
-        ok = grid_barrier_once(A.bar, gridDim.x, A.flags);
+        ok = grid_barrier_once(A.bar, gridDim.x, A.wait.polls);
     }
-    if (X == kGrid && !ok) return;
+    if (X == kGrid && !ok) {
+        if (tid == 0) *(volatile int *)P.bail = 1;
+        return;
+    }
     for (int h = tid; h < nH; h += nt) {
         const int s = (int)(__float_as_uint(hrec[h].w) & 0xffff), q = s / Vc, lv = s - q * Vc;
         const int4 t = __ldg(A.tab4 + v0 + lv);
@@ -830,7 +848,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
             const uint32_t pk = __float_as_uint(r.w);
             const int s = pk & 0xffff;
             const bool one = (pk >> 16) != 0;  // the message into the factor's variable 1
-            const float mo = d[s], l = grad_receive<X>(A, box, h_base, h, it, &s_abort);
+            const float mo = d[s], l = grad_receive<X>(A, box, h_base, h, it, &s_abort, P.bail);
             float n = one ? grad_dir(r.z, r.y + r.x - r.z, r.x, l, mo, T, invT, damping, w)
                           : grad_dir(r.x, r.y, r.z, l, mo, T, invT, damping, w);
             if (lr_dir_rare(n, l)) n = rare(s, l, mo);
@@ -882,7 +900,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
             const uint32_t pk = __float_as_uint(r.w);
             const int s = pk & 0xffff;
             const bool one = (pk >> 16) != 0;  // the source is variable 1: the message to variable 0
-            const float l = __ldcg(H + s), a = w * grad_receive<X>(A, box, h_base, h, st, &s_abort);
+            const float l = __ldcg(H + s), a = w * grad_receive<X>(A, box, h_base, h, st, &s_abort, P.bail);
             const DirGrad g = one ? dir_grad(r.y, r.z, l, a, invT) : dir_grad(r.y + r.x - r.z, r.x, l, a, invT);
             lam[s] = g.lam;
             float4 t = hacc[h];
@@ -1075,8 +1093,9 @@ cudaError_t launch_push(const LrRun &A, bool maxp, int samples, cudaStream_t s) 
 }
 
 LrRun run_args(const DevGraph &G, const EnumSeg *segs, int n_seg, const float *pot, const float *ev, float *msgs,
-               float *lam, float T, float damping, int n_iters) {
+               float *lam, float T, float damping, int n_iters, const LrWait &wait) {
     LrRun A{};
+    A.wait = wait;
     A.V = G.V;
     A.E = G.E;
     A.tab4 = G.vin_tab4;
@@ -1112,14 +1131,14 @@ int lr_cluster_size() { return run_device().cluster; }
 
 cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *log_pot, const float *ev, float *msgs,
                                 float *lam, int32_t *dir, float T, float damping, int n_iters, bool cluster,
-                                cudaStream_t s) {
+                                const LrWait &wait, cudaStream_t s) {
     const int F = G.E / 2, V = G.V;
     if (!(cluster ? lr_cluster_fits(V, F) : lr_block_fits(V, F)) || G.vin_tab4 == nullptr || G.lr_pos == nullptr)
         return cudaErrorInvalidValue;
     const FactorLaunch *L = only_launch(P);
     if (L == nullptr || n_iters <= 0) return cudaSuccess;
     run_device();  // the kernels' attributes
-    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, lam, T, damping, n_iters);
+    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, lam, T, damping, n_iters, wait);
     A.dir = dir;
     if (!cluster) return launch_push(A, T == 0.f, 1, s);
     const int C = lr_cluster_size();
@@ -1157,13 +1176,13 @@ bool lr_grid_fits(const LrGridPlan &g, int V, int F) {
 // factors' (16 + 4) in prm, the inboxes in b. lr_grid_fits has checked that they fit.
 cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPlan &g, const float *log_pot,
                                const float *ev, float *msgs, float *lam, float *m_tmp, float *b, float *d, float *prm,
-                               float T, float damping, int n_iters, cudaStream_t s) {
+                               float T, float damping, int n_iters, const LrWait &wait, cudaStream_t s) {
     const int F = G.E / 2, V = G.V;
     if (!lr_grid_fits(g, V, F)) return cudaErrorInvalidValue;
     const FactorLaunch *L = only_launch(P);
     if (L == nullptr || n_iters <= 0) return cudaSuccess;
     const RunDevice &R = run_device();
-    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, lam, T, damping, n_iters);
+    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, lam, T, damping, n_iters, wait);
     A.dir = reinterpret_cast<int32_t *>(d);
     A.nb = g.nb;
     A.Vc = g.Vc;
@@ -1218,12 +1237,12 @@ LrMultiPlan lr_multi_plan(int V, int S, bool local) {
 
 cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiPlan &p, int S, int64_t pot_stride,
                                 const float *log_pot, const float *ev, float *msgs, char *work, float T, float damping,
-                                int n_iters, cudaStream_t s) {
+                                int n_iters, const LrWait &wait, cudaStream_t s) {
     const FactorLaunch *L = only_launch(P);
     if (S < 1 || S > p.S || G.vin_tab4 == nullptr) return cudaErrorInvalidValue;
     if (L == nullptr || n_iters <= 0) return cudaSuccess;
     const size_t V = (size_t)G.V, blocks = (size_t)S * p.nb;
-    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, nullptr, T, damping, n_iters);
+    LrRun A = run_args(G, static_cast<const EnumSeg *>(L->segs), L->n_seg, log_pot, ev, msgs, nullptr, T, damping, n_iters, wait);
     A.pot_stride = pot_stride;
     A.ev_stride = G.VS;
     A.msg_stride = G.ES;
@@ -1284,12 +1303,12 @@ LrGradPlan lr_grad_plan(const LrGridPlan &g, int V, int F, int n_iters) {
 
 cudaError_t launch_lr_grad(const DevGraph &G, const Plan &P, const LrGradPlan &p, const float *log_pot, const float *ev,
                            const float *gnb, float *d_pot, float *d_ev, float *hist, int *bail, float *m_tmp, float *d,
-                           float *prm, float T, float damping, int n_iters, cudaStream_t s) {
+                           float *prm, float T, float damping, int n_iters, const LrWait &wait, cudaStream_t s) {
     const FactorLaunch *L = only_launch(P);
     if (L == nullptr || p.form == 0) return cudaErrorInvalidValue;
     const EnumSeg *segs = static_cast<const EnumSeg *>(L->segs);
     LrGrad a{};
-    a.A = run_args(G, segs, L->n_seg, log_pot, ev, nullptr, nullptr, T, damping, n_iters);
+    a.A = run_args(G, segs, L->n_seg, log_pot, ev, nullptr, nullptr, T, damping, n_iters, wait);
     a.A.nb = p.nb;
     a.A.Vc = p.Vc;
     a.A.f_cap = p.f_cap;

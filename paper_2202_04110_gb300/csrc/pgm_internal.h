@@ -357,6 +357,14 @@ cudaError_t launch_lr_unpack(const DevGraph &G, const float *d, float *m, cudaSt
 // blocks up to C times that. C is 16 where the device places a cluster of 16 such blocks (a
 // non-portable size), else 8 where it places 8, else there is no cluster form
 // (lr_cluster_size, asked once per device). dir: 4 V words of scratch.
+// A block's wait for another: polls of the word before it gives up (PGM_OPT_WAIT_POLLS; the default
+// is some seconds on a device-memory word; 0: the run counts as given up from its start), and the number of the run, which a wait that has run
+// out leaves in word kTimeoutWord of the status words.
+struct LrWait {
+    int polls;
+    uint32_t run_id;
+};
+constexpr int kLrWaitPolls = 1 << 22, kTimeoutWord = 1;
 constexpr int kLrRunThreads = 1024, kLrSmallMaxV = 1024, kLrSmallMaxF = 2048;
 constexpr int kLrClusterMax = 16;
 int lr_cluster_size();
@@ -380,7 +388,7 @@ cudaError_t launch_edge_factor_pass(const DevGraph &G, const Plan &P, const floa
                                     int S, const LaunchHook *hook);
 cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *log_pot, const float *ev,
                                 float *msgs, float *lam, int32_t *dir, float T, float damping, int n_iters,
-                                bool cluster, cudaStream_t s);
+                                bool cluster, const LrWait &wait, cudaStream_t s);
 // Larger graphs: a cooperative grid of nb blocks, block b owning variables b Vc ..
 // (b + 1) Vc - 1. lr_grid_blocks: nb for V variables on this device (0: none); the plan's
 // other fields are counted from the graph (capi.cu). lr_grid_fits: the device takes it and
@@ -390,7 +398,7 @@ int lr_grid_blocks(int V);
 bool lr_grid_fits(const LrGridPlan &g, int V, int F);
 cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPlan &g, const float *log_pot,
                                const float *ev, float *msgs, float *lam, float *m_tmp, float *b, float *d, float *prm,
-                               float T, float damping, int n_iters, cudaStream_t s);
+                               float T, float damping, int n_iters, const LrWait &wait, cudaStream_t s);
 // S samples of one graph (pgm_run_bp_multi), nb blocks each, up to p.S samples a launch;
 // work: p.sample_bytes per sample. local: few factors join different blocks (LrGridPlan).
 constexpr int kLrAloneV = 1536;  // up to this many variables a sample takes one block
@@ -403,7 +411,7 @@ struct LrMultiPlan {
 LrMultiPlan lr_multi_plan(int V, int S, bool local);
 cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiPlan &p, int S, int64_t pot_stride,
                                 const float *log_pot, const float *ev, float *msgs, char *work, float T, float damping,
-                                int n_iters, cudaStream_t s);
+                                int n_iters, const LrWait &wait, cudaStream_t s);
 // pgm_grad in one launch (lr_run.cu; every group with a table per factor): form 1 one block, 2 a
 // cluster, 3 the grid; 0: not taken. hist: hist_bytes of work; *bail (zeroed by the caller)
 // is set when the launches have to do it after all. d_pot zeroed by the caller.
@@ -414,7 +422,7 @@ struct LrGradPlan {
 LrGradPlan lr_grad_plan(const LrGridPlan &g, int V, int F, int n_iters);
 cudaError_t launch_lr_grad(const DevGraph &G, const Plan &P, const LrGradPlan &p, const float *log_pot, const float *ev,
                            const float *gnb, float *d_pot, float *d_ev, float *hist, int *bail, float *m_tmp, float *d,
-                           float *prm, float T, float damping, int n_iters, cudaStream_t s);
+                           float *prm, float T, float damping, int n_iters, const LrWait &wait, cudaStream_t s);
 // In a graph: the conditional h = (*word != 0).
 cudaError_t launch_set_condition(cudaGraphConditionalHandle h, const int *word, cudaStream_t s);
 // Adjoint launchers (kernels.cu).
@@ -440,6 +448,10 @@ cudaError_t prepare_kernels(int max_smem_bytes);
 // `s`, with CUDA-graph replay off (used by the serving loop; capi.cu): from a description,
 // or from a layout compile_graph made (the serving loop compiles each request once).
 int32_t build_graph_on_stream(const pgm_graph_desc *desc, cudaStream_t s, pgm_graph **out);
+// After a run of its own: copies the word that tells whether one of its waits ran out to *host (0 for
+// a run without waits); wait_status, once s is synchronised: PGM_OK, or the error.
+cudaError_t fetch_wait_word(const pgm_graph *g, uint32_t *host, cudaStream_t s);
+int32_t wait_status(pgm_graph *g, uint32_t word);
 int32_t build_layout_on_stream(const HostLayout &H, cudaStream_t s, pgm_graph **out);
 // Device bytes a graph built from this layout holds (index arrays and scratch).
 int64_t layout_device_bytes(const HostLayout &H);

@@ -214,8 +214,11 @@ pgm_status run_request(Request &r, const pgm::HostLayout &H, cudaStream_t st, st
         e = cudaMemcpyAsync(r.beliefs.data(), bel, I.n_var_states * sizeof(float), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(r.decode.data(), dec, I.n_vars * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+        uint32_t word = 0;
+        if (e == cudaSuccess) e = pgm::fetch_wait_word(g, &word, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = PGM_ECUDA;
+        else rc = pgm::wait_status(g, word);
     }
     if (rc != PGM_OK && err.empty()) err = (e != cudaSuccess) ? cudaGetErrorString(e) : pgm_last_error();
     cudaFreeAsync(mem, st);
