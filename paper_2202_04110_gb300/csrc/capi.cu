@@ -1138,6 +1138,15 @@ static bool grid_run_used(const pgm_graph *g) {
            lr_grid_fits(g->P.grid, g->G.V, g->G.E / 2);
 }
 
+// Whether the stream's context has fewer SMs to give than a launch of blocks that must all be resident
+// needs (the device has them; a context may be confined to a part of it). Such a launch has done
+// nothing, and the call takes the form that needs no such thing.
+static bool launch_refused(cudaError_t e) {
+    if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorLaunchOutOfResources) return false;
+    cudaGetLastError();
+    return true;
+}
+
 // The waits of the run that is about to be launched.
 static LrWait next_wait(pgm_graph *g) {
     g->run_waits = true;
@@ -1454,14 +1463,16 @@ pgm_status pgm_run_bp_multi(pgm_graph *g, int32_t n_samples, const float *log_po
         const bool local = g->P.grid.nb > 0 && g->P.grid.n_split <= g->info.n_edges / 2;
         const LrMultiPlan p = lr_multi_plan((int)g->info.n_vars, n_samples, local);
         if (p.S > 1 && multi_reserve(g, p.sample_bytes * p.S) == PGM_OK) {
-            for (int32_t s0 = 0; s0 < n_samples; s0 += p.S) {
-                cudaError_t e = launch_lr_multi_run(
+            cudaError_t e = cudaSuccess;
+            for (int32_t s0 = 0; s0 < n_samples && e == cudaSuccess; s0 += p.S) {
+                e = launch_lr_multi_run(
                     g->G, g->P, p, std::min(p.S, n_samples - s0), pot_per_sample ? P : 0,
                     log_pot + (pot_per_sample ? (size_t)s0 * P : 0), evidence + (size_t)s0 * VS, msgs + (size_t)s0 * ES,
                     static_cast<char *>(g->ms_mem), T, damping, n_iters, next_wait(g), static_cast<cudaStream_t>(stream));
-                if (e != cudaSuccess) return cuda_fail(e, "multi-sample run launch");
+                // (the first launch is the largest: a later one is not refused)
+                if (e != cudaSuccess && (s0 > 0 || !launch_refused(e))) return cuda_fail(e, "multi-sample run launch");
             }
-            return PGM_OK;
+            if (e == cudaSuccess) return PGM_OK;
         }
     }
     // Samples run together in chunks whose per-iteration exchange arrays (messages and
@@ -2006,8 +2017,9 @@ pgm_status pgm_run_bp(pgm_graph *g, const float *log_pot, const float *evidence,
         if (grid_run_used(g)) {
             cudaError_t e = launch_lr_grid_run(g->G, g->P, g->P.grid, log_pot, evidence, msgs, g->lr_lam, g->m_tmp, g->b,
                                                g->lr_d, g->lr_prm, T, damping, n_iters, next_wait(g), s);
-            if (e != cudaSuccess) return cuda_fail(e, "grid run launch");
-            return PGM_OK;
+            if (e == cudaSuccess) return PGM_OK;
+            if (!launch_refused(e)) return cuda_fail(e, "grid run launch");
+            g->run_waits = false;
         }
         if (small_run_used(g)) return enqueue_iterations(g, log_pot, evidence, T, damping, n_iters, msgs, s, false);
     }
@@ -2367,7 +2379,8 @@ static pgm_status enqueue_grad(pgm_graph *g, const float *log_pot, const float *
 // launches' buffers, the word, the kernel's history.
 static pgm_status one_launch_grad(pgm_graph *g, const LrGradPlan &one, const float *log_pot, const float *evidence, float T,
                                   float damping, int32_t n_iters, int32_t ckpt_every, const float *d_beliefs,
-                                  float *d_log_pot, float *d_evidence, size_t launches, cudaGraphExec_t *exec) {
+                                  float *d_log_pot, float *d_evidence, size_t launches, cudaGraphExec_t *exec,
+                                  bool *refused) {
     cudaStream_t cs = g->capture_stream;
     char *mem = static_cast<char *>(g->grad_mem);
     int *bail = reinterpret_cast<int *>(mem + align_up(launches, 256));
@@ -2377,6 +2390,7 @@ static pgm_status one_launch_grad(pgm_graph *g, const LrGradPlan &one, const flo
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphCreate");
     auto failed = [&](cudaError_t err, const char *what) {
         cudaGraphDestroy(graph);
+        *refused = launch_refused(err);
         return cuda_fail(err, what);
     };
     cudaGraphConditionalHandle h;
@@ -2426,8 +2440,8 @@ static pgm_status one_launch_grad(pgm_graph *g, const LrGradPlan &one, const flo
     }
     if (e != cudaSuccess) return failed(e, "cudaStreamEndCapture");
     e = cudaGraphInstantiate(exec, graph, 0);
+    if (e != cudaSuccess) return failed(e, "cudaGraphInstantiate(gradient)");
     cudaGraphDestroy(graph);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate(gradient)");
     return PGM_OK;
 }
 
@@ -2502,11 +2516,13 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
             cudaError_t e = cudaStreamCreateWithFlags(&g->capture_stream, cudaStreamNonBlocking);
             if (e != cudaSuccess) return cuda_fail(e, "cudaStreamCreate");
         }
+        bool refused = false;
         if (one.form != 0) {
             pgm_status st = one_launch_grad(g, one, log_pot, evidence, T, damping, n_iters, ckpt_every, d_beliefs, d_log_pot,
-                                            d_evidence, launches, &exec);
-            if (st != PGM_OK) return st;
-        } else {
+                                            d_evidence, launches, &exec, &refused);
+            if (st != PGM_OK && !refused) return st;
+        }
+        if (one.form == 0 || refused) {
             cudaError_t e = cudaStreamBeginCapture(g->capture_stream, cudaStreamCaptureModeThreadLocal);
             if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
             pgm_status st = enqueue_grad(g, log_pot, evidence, T, damping, n_iters, ckpt_every, d_beliefs, d_log_pot,
@@ -2529,6 +2545,9 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
         g->grads.push_back({log_pot, evidence, d_beliefs, d_log_pot, d_evidence, tb, db, n_iters, ckpt_every, exec});
     }
     cudaError_t e = cudaGraphLaunch(exec, s);
+    if (launch_refused(e))  // the one launch needs more SMs than the stream has: the launches, directly
+        return enqueue_grad(g, log_pot, evidence, T, damping, n_iters, ckpt_every, d_beliefs, d_log_pot, d_evidence,
+                            static_cast<char *>(g->grad_mem), s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
     return PGM_OK;
 }
