@@ -185,6 +185,7 @@ struct pgm_graph {
     // recorded calls, keyed by their arguments
     void *grad_mem = nullptr;
     size_t grad_bytes = 0;
+    size_t grad_refused = SIZE_MAX;  // what the device had no room for when it was last asked
     struct CachedGrad {
         const float *log_pot, *evidence, *d_beliefs;
         float *d_log_pot, *d_evidence;
@@ -2482,6 +2483,14 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
     // (its lam of every iteration: up to 1 GiB; a longer run keeps the checkpoints' bound)
     if (one.form != 0 && one.hist_bytes <= (size_t)1 << 30) total = align_up(launches, 256) + 256 + one.hist_bytes;
     else one = LrGradPlan{};
+    if (one.form != 0 && total >= g->grad_refused && g->grad_bytes < total) {
+        // refused before: asking again would free the launches' buffers and drop the recorded calls
+        size_t free_bytes = 0, all = 0;
+        if (cudaMemGetInfo(&free_bytes, &all) != cudaSuccess || free_bytes + g->grad_bytes < total + ((size_t)64 << 20)) {
+            one = LrGradPlan{};
+            total = launches;
+        }
+    }
     if (g->grad_bytes < total) {
         cudaError_t e = cudaDeviceSynchronize();  // the old buffers may be in use by a replay
         if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
@@ -2492,6 +2501,7 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
         e = cudaMalloc(&g->grad_mem, total);
         if (e != cudaSuccess && one.form != 0) {  // no room for the one-launch form
             cudaGetLastError();
+            g->grad_refused = total;
             one = LrGradPlan{};
             total = launches;
             e = cudaMalloc(&g->grad_mem, total);
@@ -2501,6 +2511,7 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
             return fail(PGM_ENOMEM, "cudaMalloc(grad)");
         }
         g->grad_bytes = total;
+        if (total >= g->grad_refused) g->grad_refused = SIZE_MAX;
     }
     uint32_t tb, db;
     std::memcpy(&tb, &T, sizeof tb);
