@@ -604,8 +604,9 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_push(const LrRun A) {
 // fine: its sigmas are 0 or 1) set *bail, and so does a wait that runs out: the caller's launches
 // take over.
 // Measured (GB300, whole calls): 64 x 64, 100 iterations, checkpoints every 10: 1.59 ms as ~590
-// dependent launches of 2.4 us, 0.31 in one; with lr_dir's SFU forms 0.28, but the table
-// gradients' error against 64 bits rose from 2.3e-7 to 2.7e-7 (mean of 15 grids). What bounds it:
+// dependent launches of 2.4 us, 0.32 in one (0.31 with plain sums over a variable's factors, which
+// lose what cancelling adjoints leave); with lr_dir's SFU forms 0.28, but the table gradients' error
+// against 64 bits rose from 2.3e-7 to 2.7e-7 (mean of 15 grids). What bounds it:
 // two barriers and an exchange per step of 200.
 struct LrGrad {
     LrRun A;                // msgs unused
@@ -616,7 +617,9 @@ struct LrGrad {
     float T;
 };
 
-// sigma(x / T) and 1 - sigma(x / T), each to a few ulp of itself.
+// sigma(x / T) and 1 - sigma(x / T), each to a few ulp of itself (the launches' weights are exp of a
+// difference of log-sum-exps, off by as many ulp of the exponent; a correctly rounded quotient costs
+// 6 % of the call and leaves the gradients' error where it is).
 struct Sigma {
     float s, c;
 };
@@ -913,12 +916,15 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
         __syncthreads();
         for (int lv = tid; lv < nv; lv += nt) {
             const float g0 = lam[lv], g1 = lam[Vc + lv], g2 = lam[2 * Vc + lv], g3 = lam[3 * Vc + lv];
-            const float g01 = g0 + g1, g23 = g2 + g3;
-            d[lv] = fmaf(damping, d[lv], g1 + g23);
-            d[Vc + lv] = fmaf(damping, d[Vc + lv], g0 + g23);
-            d[2 * Vc + lv] = fmaf(damping, d[2 * Vc + lv], g01 + g3);
-            d[3 * Vc + lv] = fmaf(damping, d[3 * Vc + lv], g01 + g2);
-            dD[lv] += g01 + g23;
+            FF S = ff_add_nc(ff_make(g0), g1);  // float-float, as k_adj_var_tab4's sums
+            S = ff_add_nc(S, g2);
+            S = ff_add_nc(S, g3);
+            const float2 t = make_float2(S.hi, S.lo);
+            d[lv] = fmaf(damping, d[lv], lr_lam_from_D(t, g0));
+            d[Vc + lv] = fmaf(damping, d[Vc + lv], lr_lam_from_D(t, g1));
+            d[2 * Vc + lv] = fmaf(damping, d[2 * Vc + lv], lr_lam_from_D(t, g2));
+            d[3 * Vc + lv] = fmaf(damping, d[3 * Vc + lv], lr_lam_from_D(t, g3));
+            dD[lv] += S.hi + S.lo;
         }
         __syncthreads();
     }
