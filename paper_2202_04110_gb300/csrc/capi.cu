@@ -81,9 +81,8 @@ struct pgm_graph {
     // word (device), its host copy (pinned); allocated on first use
     float *until_prev = nullptr;
     unsigned *until_res = nullptr;       // residual bits; the next word counts iterations done
-    // their host copies and that of status word kTimeoutWord (pinned; stream-ordered graphs: until_words)
-    unsigned *until_res_host = nullptr;
-    unsigned until_words[3] = {0, 0, 0};
+    unsigned *until_res_host = nullptr;  // 2 words (pinned; stream-ordered graphs: until_words)
+    unsigned until_words[2] = {0, 0};
     // device-side early-exit runs (conditional while node), keyed by their arguments
     struct CachedUntil {
         const float *log_pot, *evidence;
@@ -176,9 +175,9 @@ struct pgm_graph {
     int32_t log_ratio_min_iters = 4;  // PGM_OPT_LOG_RATIO
     int32_t small_run = 1;            // PGM_OPT_SMALL_RUN
     int32_t wait_polls = kLrWaitPolls;  // PGM_OPT_WAIT_POLLS
-    uint32_t run_id = 0;              // number of the last run whose blocks wait for one another
-    bool run_waits = false;           // the last pgm_run_bp was such a run
-    uint32_t *io_word = nullptr;      // pgm_infer_host: its kTimeoutWord (pinned)
+    bool run_waits = false;           // the last run's blocks wait for one another
+    uint32_t *wait_word = nullptr;    // pinned: set by a wait that runs out, in calls that return results to
+    bool wait_report = false;         // the host (those set wait_report while they launch)
     cudaStream_t capture_stream = nullptr;
     std::vector<CachedRun> runs;
     // pgm_grad as CUDA graphs (PGM_OPT_CUDA_GRAPH): persistent work buffers and the
@@ -967,16 +966,9 @@ pgm_status pgm::build_graph_on_stream(const pgm_graph_desc *desc, cudaStream_t s
     return st;
 }
 
-// Results of a run with waits are good if none ran out: checked by every call that hands results to
-// the host (pgm_run_bp, pgm_run_bp_multi leave it to the status word).
-cudaError_t pgm::fetch_wait_word(const pgm_graph *g, uint32_t *host, cudaStream_t s) {
+cudaError_t pgm::fetch_status(const pgm_graph *g, uint32_t *host, cudaStream_t s) {
     if (!g->run_waits) return cudaSuccess;
-    return cudaMemcpyAsync(host, g->G.flags + kTimeoutWord, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-}
-
-pgm_status pgm::wait_status(pgm_graph *g, uint32_t word) {
-    if (!g->run_waits || word != g->run_id) return PGM_OK;
-    return fail(PGM_ECUDA, "a block's wait for another block of the run ran out (PGM_FLAG_TIMEOUT): no result");
+    return cudaMemcpyAsync(host, g->G.flags, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
 }
 
 int64_t pgm::layout_device_bytes(const HostLayout &H) {
@@ -1083,7 +1075,7 @@ void pgm_free(pgm_graph *g) {
     if (g->pmp_ev) cudaFree(g->pmp_ev);
     if (g->until_prev) cudaFree(g->until_prev);
     if (g->until_res_host) cudaFreeHost(g->until_res_host);
-    if (g->io_word) cudaFreeHost(g->io_word);
+    if (g->wait_word) cudaFreeHost(g->wait_word);
     if (g->mu_mem) cudaFree(g->mu_mem);
     if (g->bm_mem) cudaFree(g->bm_mem);
     if (g->audit_mem) cudaFree(g->audit_mem);
@@ -1151,9 +1143,30 @@ static bool launch_refused(cudaError_t e) {
 // The waits of the run that is about to be launched.
 static LrWait next_wait(pgm_graph *g) {
     g->run_waits = true;
-    if (++g->run_id == 0) g->run_id = 1;
-    return LrWait{g->wait_polls, g->run_id};
+    return LrWait{g->wait_polls, g->wait_report ? g->wait_word : nullptr};
 }
+
+// While it lives the graph's runs report waits that run out in the pinned word, cleared here (the
+// runs are this call's own: one that is still under way has no such word or has been waited for).
+struct WaitReport {
+    pgm_graph *g;
+    bool ok;
+    explicit WaitReport(pgm_graph *graph) : g(graph), ok(true) {
+        if (g->ordered || !g->P.lr) return;  // (the serving loop reads the status word)
+        if (!g->wait_word && cudaMallocHost(&g->wait_word, sizeof(uint32_t)) != cudaSuccess) {
+            cudaGetLastError();
+            g->wait_word = nullptr;
+            ok = false;
+            return;
+        }
+        *g->wait_word = 0;
+        g->wait_report = true;
+    }
+    ~WaitReport() { g->wait_report = false; }
+    // Once the runs are done.
+    bool ran_out() const { return g->wait_report && *(volatile uint32_t *)g->wait_word != 0; }
+};
+static const char *const kRanOut = "a block's wait for another block of the run ran out (PGM_FLAG_TIMEOUT): no result";
 
 // edge_form: a run of its own, which may take the edge-order log-ratio form (the parts of other
 // runs keep their ping-pong buffers).
@@ -1647,7 +1660,7 @@ pgm_status pgm_run_bp_until(pgm_graph *g, const float *log_pot, const float *evi
             return fail(PGM_ENOMEM, "cudaMalloc(residual buffers)");
         g->until_prev = reinterpret_cast<float *>(mem);
         g->until_res = reinterpret_cast<unsigned *>(mem + align_up((size_t)ES * sizeof(float), 256));
-        if (cudaMallocHost(&g->until_res_host, 3 * sizeof(unsigned)) != cudaSuccess) {
+        if (cudaMallocHost(&g->until_res_host, 2 * sizeof(unsigned)) != cudaSuccess) {
             cudaFree(g->until_prev);
             g->until_prev = nullptr;
             g->until_res = nullptr;
@@ -1658,18 +1671,8 @@ pgm_status pgm_run_bp_until(pgm_graph *g, const float *log_pot, const float *evi
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     int32_t done = 0;
     float res = CUDART_NAN_F_HOST;
-    // chunks of small graphs may be cluster runs: their waits must not have run out
-    const bool waits = g->P.lr && small_run_used(g) && small_run_cluster(g);
-    uint32_t *word = g->until_res_host + 2;
-    *word = 0;
-    if (waits && cudaMemsetAsync(g->G.flags + kTimeoutWord, 0, sizeof(uint32_t), s) != cudaSuccess)
-        return cuda_fail(cudaGetLastError(), "cudaMemsetAsync(status word)");
-    auto finish = [&]() {
-        cudaError_t e = cudaSuccess;
-        if (waits) e = cudaMemcpyAsync(word, g->G.flags + kTimeoutWord, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-        return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
-    };
-    const char *gave_up = "a block's wait for another block of the run ran out (PGM_FLAG_TIMEOUT): msgs undefined";
+    WaitReport report(g);  // chunks of small graphs may be cluster runs
+    if (!report.ok) return fail(PGM_ENOMEM, "cudaMallocHost(status word)");
     // With CUDA graphs on, the full chunks run as one graph whose conditional while node
     // repeats a chunk while its residual is above tol: no host round trip per chunk.
     const int32_t limit = (max_iters / check_every) * check_every;
@@ -1680,9 +1683,9 @@ pgm_status pgm_run_bp_until(pgm_graph *g, const float *log_pot, const float *evi
         cudaError_t e = cudaGraphLaunch(exec, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(g->until_res_host, g->until_res, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = finish();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(e, "early-exit graph");
-        if (*word != 0) return fail(PGM_ECUDA, gave_up);
+        if (report.ran_out()) return fail(PGM_ECUDA, kRanOut);
         std::memcpy(&res, g->until_res_host, sizeof res);
         done = (int32_t)g->until_res_host[1];
         if (res <= tol || done >= max_iters) {
@@ -1700,9 +1703,9 @@ pgm_status pgm_run_bp_until(pgm_graph *g, const float *log_pot, const float *evi
         if (e == cudaSuccess) e = launch_residual(ES, msgs, prev, g->until_res, g->n_sm, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(g->until_res_host, g->until_res, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = finish();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(e, "residual");
-        if (*word != 0) return fail(PGM_ECUDA, gave_up);
+        if (report.ran_out()) return fail(PGM_ECUDA, kRanOut);
         std::memcpy(&res, g->until_res_host, sizeof res);
         done += n;
         if (res <= tol) break;
@@ -2404,7 +2407,7 @@ static pgm_status one_launch_grad(pgm_graph *g, const LrGradPlan &one, const flo
     if (e == cudaSuccess) e = cudaMemsetAsync(d_log_pot, 0, (size_t)g->info.n_potentials * sizeof(float), cs);
     if (e == cudaSuccess)
         e = launch_lr_grad(g->G, g->P, one, log_pot, evidence, d_beliefs, d_log_pot, d_evidence, hist, bail, g->m_tmp,
-                           g->lr_d, g->lr_prm, T, damping, n_iters, LrWait{g->wait_polls, 0}, cs);
+                           g->lr_d, g->lr_prm, T, damping, n_iters, LrWait{g->wait_polls, nullptr}, cs);
     if (e == cudaSuccess) e = launch_set_condition(h, bail, cs);
     cudaError_t e2 = cudaStreamEndCapture(cs, &captured);
     if (e == cudaSuccess) e = e2;
@@ -2728,16 +2731,14 @@ pgm_status pgm_infer_host(pgm_graph *g, const float *log_pot, const float *evide
         cudaError_t e = cudaMalloc(&m, b_pot + 2 * b_ev + b_msgs + b_dec);
         if (e != cudaSuccess) return fail(PGM_ENOMEM, std::string("cudaMalloc(io): ") + cudaGetErrorString(e));
         g->host_io_mem = m;
-        if (g->P.grid.nb > 0 && cudaMallocHost(&g->io_word, sizeof(uint32_t)) != cudaSuccess) {
-            g->io_word = nullptr;  // (a pageable word then)
-            cudaGetLastError();
-        }
         g->io_pot = reinterpret_cast<float *>(m);
         g->io_ev = reinterpret_cast<float *>(m + b_pot);
         g->io_bel = reinterpret_cast<float *>(m + b_pot + b_ev);
         g->io_msgs = reinterpret_cast<float *>(m + b_pot + 2 * b_ev);
         g->io_dec = reinterpret_cast<int32_t *>(m + b_pot + 2 * b_ev + b_msgs);
     }
+    WaitReport report(g);
+    if (!report.ok) return fail(PGM_ENOMEM, "cudaMallocHost(status word)");
     cudaError_t e = cudaSuccess;
     if (I.n_potentials > 0)
         e = cudaMemcpyAsync(g->io_pot, log_pot, I.n_potentials * sizeof(float), cudaMemcpyHostToDevice, s);
@@ -2760,11 +2761,10 @@ pgm_status pgm_infer_host(pgm_graph *g, const float *log_pot, const float *evide
         e = cudaMemcpyAsync(decode, g->io_dec, I.n_vars * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return cuda_fail(e, "pgm_infer_host download");
     }
-    uint32_t pageable = 0, *word = g->io_word ? g->io_word : &pageable;
-    e = fetch_wait_word(g, word, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    return wait_status(g, *word);
+    if (report.ran_out()) return fail(PGM_ECUDA, kRanOut);
+    return PGM_OK;
 }
 
 pgm_status pgm_set_profiling(pgm_graph *g, int32_t period) {

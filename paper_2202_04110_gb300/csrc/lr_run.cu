@@ -38,7 +38,7 @@
 //   - a cooperative grid of up to one block per SM (above that): the inboxes are in global
 //     memory (L2).
 // Every wait is bounded: after LrWait::polls polls a block raises PGM_FLAG_TIMEOUT in the status
-// word, notes the run beside it, stops waiting and runs to its end. (The barrier's words are right
+// word and the caller's (LrWait::host), stops waiting and runs to its end. (The barrier's words are right
 // again by then: every block of a launch arrives, also one that gives up, and the last one to
 // arrive resets the count.)
 #include <algorithm>
@@ -85,7 +85,10 @@ struct LrRun {
 // A wait of this run has run out.
 __device__ __forceinline__ void wait_failed(const LrRun &A) {
     atomicOr(A.flags, kFlagTimeout);
-    *(volatile uint32_t *)(A.flags + kTimeoutWord) = A.wait.run_id;
+    if (A.wait.host) {
+        *(volatile uint32_t *)A.wait.host = 1u;
+        __threadfence_system();
+    }
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {

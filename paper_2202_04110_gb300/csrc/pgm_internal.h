@@ -358,13 +358,13 @@ cudaError_t launch_lr_unpack(const DevGraph &G, const float *d, float *m, cudaSt
 // non-portable size), else 8 where it places 8, else there is no cluster form
 // (lr_cluster_size, asked once per device). dir: 4 V words of scratch.
 // A block's wait for another: polls of the word before it gives up (PGM_OPT_WAIT_POLLS; the default
-// is some seconds on a device-memory word; 0: the run counts as given up from its start), and the number of the run, which a wait that has run
-// out leaves in word kTimeoutWord of the status words.
+// is some seconds on a device-memory word; 0: the run counts as given up from its start), and the
+// pinned host word that a wait which has run out sets (null: the status word alone).
 struct LrWait {
     int polls;
-    uint32_t run_id;
+    uint32_t *host;
 };
-constexpr int kLrWaitPolls = 1 << 22, kTimeoutWord = 1;
+constexpr int kLrWaitPolls = 1 << 22;
 constexpr int kLrRunThreads = 1024, kLrSmallMaxV = 1024, kLrSmallMaxF = 2048;
 constexpr int kLrClusterMax = 16;
 int lr_cluster_size();
@@ -448,10 +448,8 @@ cudaError_t prepare_kernels(int max_smem_bytes);
 // `s`, with CUDA-graph replay off (used by the serving loop; capi.cu): from a description,
 // or from a layout compile_graph made (the serving loop compiles each request once).
 int32_t build_graph_on_stream(const pgm_graph_desc *desc, cudaStream_t s, pgm_graph **out);
-// After a run of its own: copies the word that tells whether one of its waits ran out to *host (0 for
-// a run without waits); wait_status, once s is synchronised: PGM_OK, or the error.
-cudaError_t fetch_wait_word(const pgm_graph *g, uint32_t *host, cudaStream_t s);
-int32_t wait_status(pgm_graph *g, uint32_t word);
+// Copies the status word to *host if the graph's last run had waits that can run out.
+cudaError_t fetch_status(const pgm_graph *g, uint32_t *host, cudaStream_t s);
 int32_t build_layout_on_stream(const HostLayout &H, cudaStream_t s, pgm_graph **out);
 // Device bytes a graph built from this layout holds (index arrays and scratch).
 int64_t layout_device_bytes(const HostLayout &H);

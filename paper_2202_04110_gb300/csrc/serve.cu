@@ -215,10 +215,14 @@ pgm_status run_request(Request &r, const pgm::HostLayout &H, cudaStream_t st, st
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(r.decode.data(), dec, I.n_vars * sizeof(int32_t), cudaMemcpyDeviceToHost, st);
         uint32_t word = 0;
-        if (e == cudaSuccess) e = pgm::fetch_wait_word(g, &word, st);
+        if (e == cudaSuccess) e = pgm::fetch_status(g, &word, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = PGM_ECUDA;
-        else rc = pgm::wait_status(g, word);
+        if (e != cudaSuccess) {
+            rc = PGM_ECUDA;
+        } else if (word & PGM_FLAG_TIMEOUT) {
+            rc = PGM_ECUDA;
+            err = "a block's wait for another block of the run ran out";
+        }
     }
     if (rc != PGM_OK && err.empty()) err = (e != cudaSuccess) ? cudaGetErrorString(e) : pgm_last_error();
     cudaFreeAsync(mem, st);
