@@ -287,10 +287,13 @@ std::vector<int32_t> lr_slot_map(const HostLayout &H) {
 // The grid form of a one-launch run: blocks of Vc consecutive variables; each block's first
 // whole item (factors between two of its variables) and split item (edges whose factor's
 // other variable is another block's), ending with the totals.
-std::vector<int2> lr_grid_plan(const HostLayout &H, LrGridPlan *g) {
+int lr_grid_plan_blocks(int64_t V, int n_sm, int smem) {
+    return V <= kLrBlockAutoV || V >= (1 << 24) ? 0 : lr_grid_blocks((int)V, n_sm, smem);
+}
+std::vector<int2> lr_grid_plan(const HostLayout &H, int n_sm, int smem, LrGridPlan *g) {
     *g = LrGridPlan{};
     std::vector<int2> off;
-    const int nb = H.V <= kLrBlockAutoV || H.V >= (1 << 24) ? 0 : lr_grid_blocks((int)H.V);
+    const int nb = lr_grid_plan_blocks(H.V, n_sm, smem);
     if (nb == 0) return off;
     g->nb = nb;
     g->Vc = (int32_t)((H.V + nb - 1) / nb);
@@ -357,56 +360,65 @@ static int32_t plan_enum_block(EnumSeg *segs, int n_seg, int threads, int n_sm, 
     return blk;
 }
 
-// The fused form (pair_fused.cu) of each dense K-state pairwise launch, K = 4, 8, 16: taken
-// when every group of the launch shares one table and is its member's only group (so its
-// variables' factors are all its own) and none of its variables has more than 4 factors; its blocks go into the index
-// memory.
-void plan_fused(const HostLayout &H, pgm_graph *g, Packer &pk) {
-    Plan &P = g->P;
+// The fused form (pair_fused.cu) of the dense K-state pairwise launch of a variant, K = 4, 8, 16: its
+// blocks, none where it is not taken. It is taken when every group of the launch shares one table and
+// is its member's only group (so its variables' factors are all its own) and none of its variables has
+// more than 4 factors. `kind`: the variables' bucket.
+std::vector<FuseBlock> fuse_plan(const HostLayout &H, int variant, int n_sm, int *kind_out, int *threads_out) {
+    std::vector<FuseBlock> fs;
+    const int kind = variant == kPairT4 ? kVarGroup4 : variant == kPairT8 ? kVarGroup8 : kVarGroup16;
+    const std::vector<int32_t> &bucket = H.var_bucket[kind];
+    if (fused_variant(variant) < 0 || bucket.empty()) return fs;
     std::vector<int32_t> groups(H.members.size(), 0);
     for (const HostEnumGroup &hg : H.enum_groups) groups[hg.seg.member] += hg.seg.n_fac > 0;
     for (const HostLogicGroup &hg : H.logic_groups) groups[hg.seg.member] += hg.seg.n_fac > 0;
+    // variables per block: one round of the block's teams (K / 4 lanes each); more rounds
+    // would form the table less often, but a round's loads depend on one another and other
+    // blocks hide them better (K = 16 on 128 uneven grids: 171 us with one round, 192 with
+    // two). 128 threads; 256 for K = 16 from 6 such blocks per SM on, where the table counts
+    // (256 x 256: 16.6 against 17.2 us per iteration; 178 x 178: 9.9 against 9.4)
+    const int lanes = variant == kPairT4 ? 1 : variant == kPairT8 ? 2 : 4;
+    const int threads = lanes == 4 && (int64_t)bucket.size() * lanes >= (int64_t)256 * 6 * n_sm ? 256 : 128;
+    const int per = threads / lanes;
+    bool ok = true;
+    // (the variable launch goes as a whole: no other group may touch its variables)
+    int64_t all_edges = 0;
+    for (int32_t v : bucket) all_edges += H.vin_off[v + 1] - H.vin_off[v];
+    for (const HostEnumGroup &hg : H.enum_groups) {
+        if (hg.variant != variant || hg.seg.n_fac == 0 || !ok) continue;
+        const HostMember &m = H.members[hg.seg.member];
+        ok = groups[hg.seg.member] == 1 && hg.seg.shared != 0;
+        const auto b0 = std::lower_bound(bucket.begin(), bucket.end(), (int32_t)m.var_off);
+        const auto b1 = std::lower_bound(b0, bucket.end(), (int32_t)(m.var_off + m.n_vars));
+        // every edge of the group belongs to a variable of the bucket
+        int64_t edges = 0;
+        for (auto it = b0; it != b1; ++it) {
+            const int32_t deg = H.vin_off[*it + 1] - H.vin_off[*it];
+            ok = ok && deg <= 4;
+            edges += deg;
+        }
+        ok = ok && edges == 2 * (int64_t)hg.seg.n_fac;
+        all_edges -= edges;
+        for (auto it = b0; it < b1; it += std::min<int64_t>(per, b1 - it))
+            fs.push_back({(int32_t)(it - bucket.begin()), (int32_t)std::min<int64_t>(per, b1 - it), hg.seg.es_base,
+                          hg.seg.pot_base, hg.seg.member, {0, 0, 0}});
+    }
+    if (!ok || all_edges != 0) fs.clear();
+    *kind_out = kind;
+    *threads_out = threads;
+    return fs;
+}
+
+// The plan's launches that have a fused form take it; their blocks go into the index memory.
+void plan_fused(const HostLayout &H, pgm_graph *g, Packer &pk) {
+    Plan &P = g->P;
     for (size_t li = 0; li < P.factor.size(); ++li) {
         FactorLaunch &L = P.factor[li];
-        if (fused_variant(L.variant) < 0) continue;
-        const int kind = L.variant == kPairT4 ? kVarGroup4 : L.variant == kPairT8 ? kVarGroup8 : kVarGroup16;
-        const std::vector<int32_t> &bucket = H.var_bucket[kind];
+        int kind = 0, threads = 0;
+        const std::vector<FuseBlock> fs = fuse_plan(H, L.variant, g->n_sm, &kind, &threads);
         size_t vi = 0;
         while (vi < P.var.size() && P.var[vi].kind != kind) ++vi;
-        bool ok = vi < P.var.size();
-        // variables per block: one round of the block's teams (K / 4 lanes each); more rounds
-        // would form the table less often, but a round's loads depend on one another and other
-        // blocks hide them better (K = 16 on 128 uneven grids: 171 us with one round, 192 with
-        // two). 128 threads; 256 for K = 16 from 6 such blocks per SM on, where the table counts
-        // (256 x 256: 16.6 against 17.2 us per iteration; 178 x 178: 9.9 against 9.4)
-        const int lanes = L.variant == kPairT4 ? 1 : L.variant == kPairT8 ? 2 : 4;
-        const int threads = lanes == 4 && (int64_t)bucket.size() * lanes >= (int64_t)256 * 6 * g->n_sm ? 256 : 128;
-        const int per = threads / lanes;
-        std::vector<FuseBlock> fs;
-        // (the variable launch goes as a whole: no other group may touch its variables)
-        int64_t all_edges = 0;
-        for (int32_t v : bucket) all_edges += H.vin_off[v + 1] - H.vin_off[v];
-        for (const HostEnumGroup &hg : H.enum_groups) {
-            if (hg.variant != L.variant) continue;
-            if (hg.seg.n_fac == 0 || !ok) continue;
-            const HostMember &m = H.members[hg.seg.member];
-            ok = ok && groups[hg.seg.member] == 1 && hg.seg.shared != 0;
-            const auto b0 = std::lower_bound(bucket.begin(), bucket.end(), (int32_t)m.var_off);
-            const auto b1 = std::lower_bound(b0, bucket.end(), (int32_t)(m.var_off + m.n_vars));
-            // every edge of the group belongs to a variable of the bucket
-            int64_t edges = 0;
-            for (auto it = b0; it != b1; ++it) {
-                const int32_t deg = H.vin_off[*it + 1] - H.vin_off[*it];
-                ok = ok && deg <= 4;
-                edges += deg;
-            }
-            ok = ok && edges == 2 * (int64_t)hg.seg.n_fac;
-            all_edges -= edges;
-            for (auto it = b0; it < b1; it += std::min<int64_t>(per, b1 - it))
-                fs.push_back({(int32_t)(it - bucket.begin()), (int32_t)std::min<int64_t>(per, b1 - it), hg.seg.es_base,
-                              hg.seg.pot_base, hg.seg.member, {0, 0, 0}});
-        }
-        if (!ok || fs.empty() || all_edges != 0) continue;
+        if (fs.empty() || vi == P.var.size()) continue;
         g->fused.push_back({(int)li, (int)vi, pk.add(fs.data(), fs.size())});
         L.fuse_blocks = (int32_t)fs.size();
         L.fuse_threads = threads;
@@ -815,7 +827,7 @@ static pgm_status build_from_layout(const HostLayout &H, pgm_graph **out, cudaSt
     }
     size_t o_grid = 0;
     if (g->P.lr && !H.vin_tab4.empty()) {
-        const std::vector<int2> off = lr_grid_plan(H, &g->P.grid);
+        const std::vector<int2> off = lr_grid_plan(H, lr_grid_device(), lr_grid_smem(), &g->P.grid);
         if (g->P.grid.nb > 0) o_grid = pk.add(off.data(), off.size());
     }
     g->ordered = ordered;
@@ -979,10 +991,15 @@ int64_t pgm::layout_device_bytes(const HostLayout &H) {
                      sizeof(int32_t) +
                  H.cfg_pool.size();
     size_t es_bytes = align_up(std::max<int64_t>(H.ES, 1) * sizeof(float), 256);
-    if (lr_eligible(H))  // the slot map, the two log-ratio arrays and the table differences
+    const int nb_grid = lr_grid_plan_blocks(H.V, kPlanSms, kPlanSmem);
+    if (lr_eligible(H))  // the slot map, the two log-ratio arrays, the table differences, the grid plan
         idx += H.E * sizeof(int32_t) + 2 * align_up((size_t)lr_slot_count(H) * sizeof(float), 256) +
                align_up((size_t)3 * (H.E / 2) * sizeof(float), 256) +
-               (H.vin_tab4.empty() ? 0 : ((size_t)lr_grid_blocks((int)H.V) + 1) * sizeof(int2));
+               (H.vin_tab4.empty() || nb_grid == 0 ? 0 : ((size_t)nb_grid + 1) * sizeof(int2));
+    for (int variant : {kPairT4, kPairT8, kPairT16}) {
+        int kind = 0, threads = 0;
+        idx += fuse_plan(H, variant, kPlanSms, &kind, &threads).size() * sizeof(FuseBlock);
+    }
     const size_t vs_bytes = align_up(std::max<int64_t>(H.VS, 1) * sizeof(float), 256);
     // the high-degree variables' tile list (index memory), tile totals and tickets (scratch)
     int64_t n_tiles = 0, tot = 0;

@@ -1161,12 +1161,14 @@ cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *l
 
 // ---- the grid form of one sample ----
 
-int lr_grid_blocks(int V) {
-    const RunDevice &R = run_device();
-    if (!R.coop || V < 2) return 0;
-    const int Vc = std::max((V + R.n_sm - 1) / R.n_sm, kLrGridMinV);
+int lr_grid_device() { return run_device().coop ? run_device().n_sm : 0; }
+int lr_grid_smem() { return run_device().smem; }
+
+int lr_grid_blocks(int V, int n_sm, int smem) {
+    if (n_sm < 1 || V < 2) return 0;
+    const int Vc = std::max((V + n_sm - 1) / n_sm, kLrGridMinV);
     const int nb = (V + Vc - 1) / Vc;
-    return nb >= 2 && 24 * (int64_t)Vc + 16 <= R.smem && Vc < (1 << 14) ? nb : 0;
+    return nb >= 2 && run_smem(kGrid, false, false, Vc, 0, 0) <= (size_t)smem && Vc < (1 << 14) ? nb : 0;
 }
 
 bool lr_grid_fits(const LrGridPlan &g, int V, int F) {

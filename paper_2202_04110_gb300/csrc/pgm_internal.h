@@ -390,11 +390,16 @@ cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *l
                                 float *msgs, float *lam, int32_t *dir, float T, float damping, int n_iters,
                                 bool cluster, const LrWait &wait, cudaStream_t s);
 // Larger graphs: a cooperative grid of nb blocks, block b owning variables b Vc ..
-// (b + 1) Vc - 1. lr_grid_blocks: nb for V variables on this device (0: none); the plan's
-// other fields are counted from the graph (capi.cu). lr_grid_fits: the device takes it and
-// the graph's scratch holds its workspace.
+// (b + 1) Vc - 1. lr_grid_blocks: nb for V variables on n_sm SMs with smem bytes a block (0: none);
+// the plan's other fields are counted from the graph (capi.cu). lr_grid_device, lr_grid_smem: this
+// device's (0 SMs: no cooperative launches). lr_grid_fits: the device takes the plan and the
+// graph's scratch holds its workspace.
 constexpr int kLrGridMinV = 256;  // variables per block at least
-int lr_grid_blocks(int V);
+int lr_grid_blocks(int V, int n_sm, int smem);
+int lr_grid_device();
+int lr_grid_smem();
+// A GB300's, for sizes that are stated without asking a device (pgm_check_desc, serving budgets).
+constexpr int kPlanSms = 152, kPlanSmem = 232448 - 256;
 bool lr_grid_fits(const LrGridPlan &g, int V, int F);
 cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPlan &g, const float *log_pot,
                                const float *ev, float *msgs, float *lam, float *m_tmp, float *b, float *d, float *prm,
