@@ -317,8 +317,9 @@ pgm_status pgm_device_flags(pgm_graph *g, uint32_t *flags, int32_t clear, void *
  * Checked mode: the first index-array violation found on this graph (*array = -1 if
  * none): the array (0 vs_off, 1 vin_off, 2 vin_es, 3 edge_vs, 4 edge_var, 5 vin_tab4,
  * 6 lr_pos, 7 paroff_pool, 8 cfg_pool, 9 configuration lists, 10 enumeration group
- * records, 11 logical group records, 12 variable lists), the entry's position (the
- * record's index for 10 and 11) and its value (-1 where none is read back). Host only.
+ * records, 11 logical group records, 12 variable lists, 13 the one-launch run's items by block,
+ * 14 the fused form's block records), the entry's position (the record's index for 10, 11 and
+ * 14) and its value (-1 where none is read back). Host only.
  */
 pgm_status pgm_checked_report(const pgm_graph *g, int32_t *array, int64_t *position, int64_t *value);
 
@@ -327,8 +328,8 @@ pgm_status pgm_checked_report(const pgm_graph *g, int32_t *array, int64_t *posit
  * the host copies of its index arrays (the same rules as the device checks), after
  * writing corrupt_value into entry corrupt_pos of array corrupt_array (ids as in
  * pgm_checked_report; for the records 10 / 11 the value replaces the record's first
- * edge-state / parent-offset base; for 12 the first variable list) when corrupt_array
- * >= 0. *bad_array, *bad_pos = the first violation in array order, -1 if none. For tests
+ * edge-state / parent-offset base; for 12 the first variable list; for 14 a block's first
+ * position in its list) when corrupt_array >= 0. The plans (13, 14) are those on a GB300. *bad_array, *bad_pos = the first violation in array order, -1 if none. For tests
  * of the checks on hosts without a GPU. PGM_EINVAL for a bad description or a corrupt
  * position outside the array.
  */
@@ -521,7 +522,8 @@ pgm_status pgm_run_bp_until_members(pgm_graph *g, const float *log_pot, const fl
  * graph's index arrays -- the per-variable state offsets and incoming-edge lists, each
  * edge's variable state, the padded incoming-edge table, the log-ratio slot map, the
  * logical groups' parent offsets, the configuration tables and lists by output state,
- * the group records of every launch and the variable lists of the variable pass --
+ * the group records of every launch, the variable lists of the variable pass, the
+ * one-launch run's items by block and the fused form's block records --
  * against the range the kernels assume (these arrays are where every gathered index of
  * Sec. 4's flat layout comes from), and waits for the result. On a violation it raises
  * PGM_FLAG_INDEX in the status word (pgm_device_flags), keeps the array, position and

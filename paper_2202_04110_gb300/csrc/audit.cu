@@ -56,11 +56,18 @@ __global__ void __launch_bounds__(128) k_audit_logic(const LogicSeg *__restrict_
         atomicMin(first + kAuditLogicSeg, (unsigned long long)(seg_pos0 + i));
 }
 
+__global__ void __launch_bounds__(128) k_audit_fuse(AuditFuse a, int64_t pos0, AuditSizes z,
+                                                    unsigned long long *__restrict__ first) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < a.n && !audit_fuse_ok(a.p[i], a, z)) atomicMin(first + kAuditFuse, (unsigned long long)(pos0 + i));
+}
+
 __global__ void k_audit_flag(uint32_t *flags) { atomicOr(flags, (uint32_t)PGM_FLAG_INDEX); }
 
 const char *const kArrayNames[kAuditNumArrays] = {
     "vs_off", "vin_off", "vin_es", "edge_vs", "edge_var", "vin_tab4", "lr_pos", "paroff_pool",
-    "cfg_pool", "bs_pool", "enumeration group records", "logical group records", "variable lists"};
+    "cfg_pool", "bs_pool", "enumeration group records", "logical group records", "variable lists",
+    "one-launch run's items", "fused form's block records"};
 
 }  // namespace
 
@@ -69,7 +76,8 @@ const char *audit_array_name(int id) { return id >= 0 && id < kAuditNumArrays ? 
 // Host twin of the device audit: the first violation in array-id order (ids as
 // AuditArrayId), -1 if none.
 void audit_host(const std::vector<AuditArray> &flat, const std::vector<EnumSeg> &esegs,
-                const std::vector<LogicSeg> &lsegs, const AuditSizes &z, int32_t *bad_array, int64_t *bad_pos) {
+                const std::vector<LogicSeg> &lsegs, const std::vector<AuditFuse> &fused, const AuditSizes &z,
+                int32_t *bad_array, int64_t *bad_pos) {
     std::vector<int64_t> first(kAuditNumArrays, -1);
     auto note = [&](int id, int64_t pos) {
         if (first[id] < 0 || pos < first[id]) first[id] = pos;
@@ -92,6 +100,12 @@ void audit_host(const std::vector<AuditArray> &flat, const std::vector<EnumSeg> 
     }
     for (size_t k = 0; k < lsegs.size(); ++k)
         if (!audit_logic_seg_ok(lsegs[k], z)) note(kAuditLogicSeg, (int64_t)k);
+    int64_t pos0 = 0;
+    for (const AuditFuse &a : fused) {
+        for (int i = 0; i < a.n; ++i)
+            if (!audit_fuse_ok(a.p[i], a, z)) note(kAuditFuse, pos0 + i);
+        pos0 += a.n;
+    }
     *bad_array = -1;
     *bad_pos = -1;
     for (int id = 0; id < kAuditNumArrays; ++id)
@@ -108,8 +122,8 @@ void audit_host(const std::vector<AuditArray> &flat, const std::vector<EnumSeg> 
 size_t audit_work_bytes(size_t n_flat) { return 256 + ((n_flat * sizeof(AuditArray) + 255) / 256) * 256; }
 
 cudaError_t audit_device(const std::vector<AuditArray> &flat, const std::vector<std::pair<const void *, int>> &enum_launches,
-                         const std::vector<std::pair<const void *, int>> &logic_launches, const AuditSizes &z,
-                         uint32_t *flags, char *work, cudaStream_t s, int32_t *bad_array, int64_t *bad_pos) {
+                         const std::vector<std::pair<const void *, int>> &logic_launches,
+                         const std::vector<AuditFuse> &fused, const AuditSizes &z, uint32_t *flags, char *work, cudaStream_t s, int32_t *bad_array, int64_t *bad_pos) {
     unsigned long long *first = reinterpret_cast<unsigned long long *>(work);
     AuditArray *arrs = reinterpret_cast<AuditArray *>(work + 256);
     cudaError_t e = cudaMemsetAsync(first, 0xff, kAuditNumArrays * sizeof(unsigned long long), s);
@@ -133,6 +147,12 @@ cudaError_t audit_device(const std::vector<AuditArray> &flat, const std::vector<
         k_audit_logic<<<(L.second + 127) / 128, 128, 0, s>>>(static_cast<const LogicSeg *>(L.first), L.second, pos0, z,
                                                              first);
         pos0 += L.second;
+    }
+    pos0 = 0;
+    for (const AuditFuse &a : fused) {
+        if (e != cudaSuccess || a.n <= 0) continue;
+        k_audit_fuse<<<(a.n + 127) / 128, 128, 0, s>>>(a, pos0, z, first);
+        pos0 += a.n;
     }
     if (e == cudaSuccess) e = cudaGetLastError();
     unsigned long long host[kAuditNumArrays];

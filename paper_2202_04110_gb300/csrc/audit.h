@@ -34,7 +34,9 @@ enum AuditArrayId : int32_t {
     kAuditEnumSeg = 10,   // enumeration group records: every derived range inside its array
     kAuditLogicSeg = 11,  // logical group records
     kAuditVarList = 12,   // variable lists of the variable-pass launches: 0..V-1
-    kAuditNumArrays = 13
+    kAuditGridOff = 13,   // Plan::grid.off, two words per entry: 0..items
+    kAuditFuse = 14,      // fused form's block records: variables inside their bucket, bases inside
+    kAuditNumArrays = 15
 };
 
 // One flat int32 array and its entries' range [lo, hi). allow_neg: 0 nothing else; 1 -1
@@ -54,6 +56,14 @@ struct AuditSizes {
     int64_t cfg_size, bs_size, paroff_size;
     const uint8_t *cfg_pool;
     const int32_t *bs_pool, *paroff_pool;
+    int64_t members;
+};
+
+// The blocks of one fused launch: n of at most `per` variables of K states, from a bucket of n_list.
+struct AuditFuse {
+    const FuseBlock *p;
+    int32_t n, K, per;
+    int64_t n_list;
 };
 
 __host__ __device__ __forceinline__ bool audit_entry_ok(int64_t x, const AuditArray &a) {
@@ -101,6 +111,15 @@ __host__ __device__ inline bool audit_logic_seg_ok(const LogicSeg &s, const Audi
     return true;
 }
 
+// A fused launch's block: its variables in the bucket, the group's first factor and table in range
+// (its edges are vin_es entries).
+__host__ __device__ __forceinline__ bool audit_fuse_ok(const FuseBlock &b, const AuditFuse &a, const AuditSizes &z) {
+    if (b.pos < 0 || b.n < 1 || b.n > a.per || (int64_t)b.pos + b.n > a.n_list) return false;
+    if (b.es_base < 0 || (int64_t)b.es_base + 2 * a.K > z.ES) return false;
+    if (b.pot_base < 0 || (int64_t)b.pot_base + a.K * a.K > z.P) return false;
+    return b.member >= 0 && b.member < z.members;
+}
+
 // Entry i of an enumeration group's configuration table: a state of neighbour i % arity.
 __host__ __device__ __forceinline__ bool audit_cfg_ok(const EnumSeg &s, int64_t i, const AuditSizes &z) {
     return z.cfg_pool[s.cfg_base + i] < s.K[i % s.arity];
@@ -123,10 +142,12 @@ __host__ __device__ __forceinline__ bool audit_bs_ok(const EnumSeg &s, int64_t i
 // `work` is a device buffer of audit_work_bytes(flat.size()) bytes).
 const char *audit_array_name(int id);
 void audit_host(const std::vector<AuditArray> &flat, const std::vector<EnumSeg> &esegs,
-                const std::vector<LogicSeg> &lsegs, const AuditSizes &z, int32_t *bad_array, int64_t *bad_pos);
+                const std::vector<LogicSeg> &lsegs, const std::vector<AuditFuse> &fused, const AuditSizes &z,
+                int32_t *bad_array, int64_t *bad_pos);
 size_t audit_work_bytes(size_t n_flat);
 cudaError_t audit_device(const std::vector<AuditArray> &flat, const std::vector<std::pair<const void *, int>> &enum_launches,
-                         const std::vector<std::pair<const void *, int>> &logic_launches, const AuditSizes &z,
-                         uint32_t *flags, char *work, cudaStream_t s, int32_t *bad_array, int64_t *bad_pos);
+                         const std::vector<std::pair<const void *, int>> &logic_launches,
+                         const std::vector<AuditFuse> &fused, const AuditSizes &z, uint32_t *flags,
+                         char *work, cudaStream_t s, int32_t *bad_array, int64_t *bad_pos);
 
 }  // namespace pgm

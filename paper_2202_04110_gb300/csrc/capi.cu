@@ -686,7 +686,16 @@ std::vector<AuditArray> device_audit_arrays(const pgm_graph *g) {
     add(G.lr_pos, E, 0, g->lr_slots, false, kAuditLrPos);
     add(G.paroff_pool, g->paroff_size, 0, E + 1, false, kAuditParOff);
     for (const VarLaunch &L : g->P.var) add(L.list, L.n, 0, V, false, kAuditVarList);
+    const LrGridPlan &p = g->P.grid;
+    if (p.nb > 0)
+        add(reinterpret_cast<const int32_t *>(p.off), 2 * ((int64_t)p.nb + 1), 0, std::max(E / 2, p.n_split) + 1, false, kAuditGridOff);
     return a;
+}
+
+// The blocks of a fused launch as the audit takes them.
+static AuditFuse audit_fuse(const FuseBlock *p, int n, int variant, int threads, int64_t n_list) {
+    const int K = variant == kPairT4 ? 4 : variant == kPairT8 ? 8 : 16;
+    return AuditFuse{p, n, K, threads / (K / 4), n_list};
 }
 
 // Checked mode (PGM_OPT_CHECKED): before a call's kernels, the device audit of every
@@ -713,10 +722,15 @@ pgm_status checked_gate(pgm_graph *g, void *stream) {
     if (g->adj_logic_launch.segs) logics.emplace_back(g->adj_logic_launch.segs, g->adj_logic_launch.n_seg);
     const DevGraph &G = g->G;
     const AuditSizes z{G.V, G.VS, G.E, G.ES, g->info.n_potentials, g->cfg_size, g->bs_size, g->paroff_size,
-                       G.cfg_pool, G.bs_pool, G.paroff_pool};
+                       G.cfg_pool, G.bs_pool, G.paroff_pool, (int64_t)g->members.size()};
+    std::vector<AuditFuse> fused;
+    for (const auto &f : g->fused) {
+        const FactorLaunch &L = g->P.factor[f.factor];
+        fused.push_back(audit_fuse(L.fuse, L.fuse_blocks, L.base_variant, L.fuse_threads, g->P.var[f.var].n));
+    }
     int32_t bad = -1;
     int64_t pos = -1;
-    cudaError_t e = audit_device(flat, enums, logics, z, G.flags, g->audit_mem, static_cast<cudaStream_t>(stream),
+    cudaError_t e = audit_device(flat, enums, logics, fused, z, G.flags, g->audit_mem, static_cast<cudaStream_t>(stream),
                                  &bad, &pos);
     if (e != cudaSuccess) return cuda_fail(e, "index audit");
     if (bad < 0) return PGM_OK;
@@ -2864,6 +2878,18 @@ pgm_status pgm_audit_desc(const pgm_graph_desc *desc, int32_t corrupt_array, int
     std::vector<std::vector<int32_t>> lists;
     for (int k = 0; k < kNumVarKinds; ++k)
         if (!H.var_bucket[k].empty() && !H.var_bucket_identity[k]) lists.push_back(H.var_bucket[k]);
+    // the plans of one-launch runs and of the fused form on a GB300
+    LrGridPlan grid;
+    std::vector<int2> off;
+    if (lr_eligible(H) && !H.vin_tab4.empty()) off = lr_grid_plan(H, kPlanSms, kPlanSmem, &grid);
+    std::vector<std::vector<FuseBlock>> blocks;
+    std::vector<AuditFuse> fused;
+    for (int variant : {kPairT4, kPairT8, kPairT16}) {
+        int kind = 0, threads = 0;
+        blocks.push_back(fuse_plan(H, variant, kPlanSms, &kind, &threads));
+        if (!blocks.back().empty())
+            fused.push_back(audit_fuse(blocks.back().data(), (int)blocks.back().size(), variant, threads, (int64_t)H.var_bucket[kind].size()));
+    }
     // the test's corruption of one entry (corrupt_array < 0: none)
     if (corrupt_array >= 0) {
         auto poke = [&](auto &vec, const char *name) -> pgm_status {
@@ -2896,6 +2922,14 @@ pgm_status pgm_audit_desc(const pgm_graph_desc *desc, int32_t corrupt_array, int
                 if (lists.empty()) return fail(PGM_EINVAL, "the graph has no variable lists");
                 st = poke(lists[0], "variable lists");
                 break;
+            case kAuditGridOff:
+                if (corrupt_pos < 0 || corrupt_pos >= 2 * (int64_t)off.size()) return fail(PGM_EINVAL, "no such entry");
+                reinterpret_cast<int32_t *>(off.data())[corrupt_pos] = (int32_t)corrupt_value;
+                break;
+            case kAuditFuse:
+                if (fused.empty() || corrupt_pos < 0 || corrupt_pos >= fused[0].n) return fail(PGM_EINVAL, "no such record");
+                const_cast<FuseBlock *>(fused[0].p)[corrupt_pos].pos = (int32_t)corrupt_value;
+                break;
             default: return fail(PGM_EINVAL, "unknown array id");
         }
         if (st != PGM_OK) return st;
@@ -2913,9 +2947,11 @@ pgm_status pgm_audit_desc(const pgm_graph_desc *desc, int32_t corrupt_array, int
     add(lr.data(), (int64_t)lr.size(), 0, lr_slot_count(H), false, kAuditLrPos);
     add(H.paroff_pool.data(), (int64_t)H.paroff_pool.size(), 0, H.E + 1, false, kAuditParOff);
     for (const auto &l : lists) add(l.data(), (int64_t)l.size(), 0, H.V, false, kAuditVarList);
+    add(reinterpret_cast<const int32_t *>(off.data()), 2 * (int64_t)off.size(), 0, std::max(H.E / 2, grid.n_split) + 1, false, kAuditGridOff);
     const AuditSizes z{H.V, H.VS, H.E, H.ES, H.P, (int64_t)H.cfg_pool.size(), (int64_t)H.bs_pool.size(),
-                       (int64_t)H.paroff_pool.size(), H.cfg_pool.data(), H.bs_pool.data(), H.paroff_pool.data()};
-    audit_host(flat, esegs, lsegs, z, bad_array, bad_pos);
+                       (int64_t)H.paroff_pool.size(), H.cfg_pool.data(), H.bs_pool.data(), H.paroff_pool.data(),
+                       (int64_t)H.members.size()};
+    audit_host(flat, esegs, lsegs, fused, z, bad_array, bad_pos);
     return PGM_OK;
 }
 
