@@ -287,7 +287,7 @@ pgm_status pgm_launch_times(pgm_graph *g, int32_t n, double *ms, int64_t *count,
  * own table, runs the call as one kernel launch where PGM_OPT_SMALL_RUN and PGM_OPT_CUDA_GRAPH
  * are on and the blocks of that option's forms hold it: each iteration's variable-to-factor
  * log-ratios are kept instead of checkpoints (16 bytes per variable and iteration beside the
- * scratch above, up to 1 GiB, else the launches). A table with a non-finite entry or an
+ * scratch above, up to 512 MiB, else the launches). A table with a non-finite entry or an
  * infinite message makes the same recorded call run the launches after all.
  * Every sum is taken in a fixed order, so repeated calls give the same bits: gradients of
  * log-potentials shared by a group of factors with a state sum up to 64 through warp

@@ -2516,9 +2516,7 @@ pgm_status pgm_grad(pgm_graph *g, const float *log_pot, const float *evidence, f
     const bool in_place = d_evidence < d_beliefs + g->info.n_var_states && d_beliefs < d_evidence + g->info.n_var_states;
     if (g->small_run != 0 && g->P.lr && g->G.vin_tab4 != nullptr && n_iters >= 1 && g->adj_nc_max == 0 && !in_place)
         one = lr_grad_plan(g->P.grid, g->G.V, g->G.E / 2, n_iters);
-    // (its lam of every iteration: up to 1 GiB; a longer run keeps the checkpoints' bound)
-    if (one.form != 0 && one.hist_bytes <= (size_t)1 << 30) total = align_up(launches, 256) + 256 + one.hist_bytes;
-    else one = LrGradPlan{};
+    if (one.form != 0) total = align_up(launches, 256) + 256 + one.hist_bytes;
     if (one.form != 0 && total >= g->grad_refused && g->grad_bytes < total) {
         // refused before: asking again would free the launches' buffers and drop the recorded calls
         size_t free_bytes = 0, all = 0;

@@ -1308,7 +1308,7 @@ LrGradPlan lr_grad_plan(const LrGridPlan &g, int V, int F, int n_iters) {
         return p;
     }
     p.hist_bytes = (size_t)n_iters * p.nb * 16 * (size_t)p.Vc;
-    if (p.hist_bytes > ((size_t)512 << 20)) p.form = 0;
+    if (p.hist_bytes > kLrGradHistory) p.form = 0;
     return p;
 }
 

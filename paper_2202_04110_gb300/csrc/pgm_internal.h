@@ -418,8 +418,10 @@ cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiP
                                 const float *log_pot, const float *ev, float *msgs, char *work, float T, float damping,
                                 int n_iters, const LrWait &wait, cudaStream_t s);
 // pgm_grad in one launch (lr_run.cu; every group with a table per factor): form 1 one block, 2 a
-// cluster, 3 the grid; 0: not taken. hist: hist_bytes of work; *bail (zeroed by the caller)
+// cluster, 3 the grid; 0: not taken. hist: hist_bytes of work, at most kLrGradHistory (a longer run
+// keeps the checkpoints' bound and makes the launches); *bail (zeroed by the caller)
 // is set when the launches have to do it after all. d_pot zeroed by the caller.
+constexpr size_t kLrGradHistory = (size_t)512 << 20;
 struct LrGradPlan {
     int form = 0, nb = 0, Vc = 0, f_cap = 0, h_cap = 0;
     size_t hist_bytes = 0;

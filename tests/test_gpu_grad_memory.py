@@ -63,3 +63,20 @@ def test_no_room_for_the_history(gpu):
         torch.cuda.synchronize()
         torch.cuda.empty_cache()
     assert all(torch.equal(a, b) for a, b in zip(grad(g), one))
+
+
+def test_history_limit(gpu):
+    """512 MiB of kept values (16 bytes per variable, 152 blocks of 264, and iteration): the one launch up
+    to there, whose bits differ from the launches', the launches above."""
+    import torch
+    p = W.ising_grid(200, 200, seed=1)
+    lp, ev = torch.as_tensor(p.log_pot).cuda(), torch.as_tensor(p.evidence).cuda()
+    cot = torch.as_tensor(np.random.default_rng(2).standard_normal(p.evidence.size).astype(np.float32)).cuda()
+    at_most = (512 << 20) // (152 * 264 * 16)
+    for n, same in ((at_most, False), (at_most + 1, True)):
+        out = []
+        for small in (1, 0):
+            g = gpu.Graph(p.graph)
+            g.set_option(gpu.OPT_SMALL_RUN, small)
+            out.append(g.grad(lp, ev, 1.0, 0.5, n, 30, cot)[0])
+        assert torch.equal(*out) == same, n
