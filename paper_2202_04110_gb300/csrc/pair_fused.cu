@@ -19,7 +19,7 @@
 // 16 on 181 x 181 17.9 -> 9.7; K = 8 on 178 x 178 9.3 -> 5.8; K = 4 on 64 x 64 6.0 -> 3.4 (two
 // launches' latency -> one); per launch on 128 uneven grids K = 16 (662,000 variables) 60 + 222
 // -> 178 us, K = 8 (800,000) 43 + 88 -> 101, K = 4 (672,000) 28 + 46 -> 51. What bounds it now:
-// issue slots (half of them) and the chain index -> messages -> weights -> targets of a round;
+// issue slots (half of them) and the chain index -> messages -> weights -> targets;
 // more resident blocks win against fewer spills (K = 16: 2, 3, 4 blocks of 256 per SM 232, 183,
 // 171 us).
 #include <cstdint>
@@ -310,10 +310,10 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
              const float *__restrict__ pot, const float *__restrict__ ev, const float *__restrict__ m_old,
              float *__restrict__ m_new, float T, float invT, float damping) {
     constexpr int L = K / 4;                  // lanes per variable
-    constexpr int kStep = NT / L;       // variables per round of the block
+    constexpr int kTeams = NT / L;            // the block's variables at most (fuse_plan, capi.cu)
     constexpr int kRow = K == 4 ? 8 : 2 * K + 4;  // a team's exchange row: few bank conflicts between teams
     __shared__ __align__(16) float S0[K * K], S1[K * K];
-    __shared__ __align__(16) float xch[2 * kStep * kRow];
+    __shared__ __align__(16) float xch[2 * kTeams * kRow];
     __shared__ float tab[K * K];
     __shared__ float red[2 * NT / 32];
     if constexpr (MS) {  // multi-sample launches: this block's sample
@@ -350,39 +350,32 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
     const bool al = ((reinterpret_cast<uintptr_t>(m_old + es_base) | reinterpret_cast<uintptr_t>(m_new + es_base) |
                       reinterpret_cast<uintptr_t>(ev + vs)) & 15u) == 0;
     const bool all_al = __syncthreads_and(al);
-    for (int j = team; j - team < n; j += kStep) {
-        float e4[4], q[4][4];
-        unsigned rare;
-        if (all_al) {
-            row_load<true>(e4, ev + vs + 4 * l);
+    float e4[4], q[4][4];
+    unsigned rare;
+    if (all_al) {
+        row_load<true>(e4, ev + vs + 4 * l);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (i < t.deg) row_load<true>(q[i], m_old + t.es[i] + 4 * l);
-                else q[i][0] = q[i][1] = q[i][2] = q[i][3] = 0.f;  // adds exactly nothing
-            }
-            rare = team_edges<K, MAXP, true>(t, e4, q, l, es_base, S0, S1, red[0], xs, kStep * kRow, m_old, m_new, T, invT,
-                                             damping);
-        } else {
-            row_load<false>(e4, ev + vs + 4 * l);
+        for (int i = 0; i < 4; ++i) {
+            if (i < t.deg) row_load<true>(q[i], m_old + t.es[i] + 4 * l);
+            else q[i][0] = q[i][1] = q[i][2] = q[i][3] = 0.f;  // adds exactly nothing
+        }
+        rare = team_edges<K, MAXP, true>(t, e4, q, l, es_base, S0, S1, red[0], xs, kTeams * kRow, m_old, m_new, T, invT,
+                                         damping);
+    } else {
+        row_load<false>(e4, ev + vs + 4 * l);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (i < t.deg) row_load<false>(q[i], m_old + t.es[i] + 4 * l);
-                else q[i][0] = q[i][1] = q[i][2] = q[i][3] = 0.f;
-            }
-            rare = team_edges<K, MAXP, false>(t, e4, q, l, es_base, S0, S1, red[0], xs, kStep * kRow, m_old, m_new, T, invT,
-                                             damping);
+        for (int i = 0; i < 4; ++i) {
+            if (i < t.deg) row_load<false>(q[i], m_old + t.es[i] + 4 * l);
+            else q[i][0] = q[i][1] = q[i][2] = q[i][3] = 0.f;
         }
-        if (rare != 0 && l == 0)
-#pragma unroll 1
-            for (int i = 0; i < t.deg; ++i)
-                if ((rare >> i) & 1) fused_edge<K, MAXP>(G, tab, ev, m_old, m_new, t.v, i, es_base, T, invT, damping);
-        if (j - team + kStep >= n && !pdl_small()) pdl_launch_dependents();
-        if (j - team + kStep < n) {  // the next round's variable
-            const int jn = j + kStep;
-            t = team_var(G, list, B.x + (jn < n ? jn : 0), jn < n, es_base);
-            vs = __ldg(G.vs_off + t.v);
-        }
+        rare = team_edges<K, MAXP, false>(t, e4, q, l, es_base, S0, S1, red[0], xs, kTeams * kRow, m_old, m_new, T, invT,
+                                          damping);
     }
+    if (rare != 0 && l == 0)
+#pragma unroll 1
+        for (int i = 0; i < t.deg; ++i)
+            if ((rare >> i) & 1) fused_edge<K, MAXP>(G, tab, ev, m_old, m_new, t.v, i, es_base, T, invT, damping);
+    if (!pdl_small()) pdl_launch_dependents();
 }
 
 template <int K, bool MAXP, bool MS>
