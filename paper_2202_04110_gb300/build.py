@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB_PATH = os.path.join(HERE, "libpgm.so")
 SOURCES = ["compile.cpp", "kernels.cu", "lr_run.cu", "lr_edge.cu", "pair_fused.cu", "capi.cu", "noalloc.cu", "serve.cu", "audit.cu"]
-HEADERS = [os.path.join(CSRC, "pgm_internal.h"), os.path.join(CSRC, "audit.h"), os.path.join(CSRC, "lr_math.cuh"), os.path.join(CSRC, "bp_common.cuh"),
+HEADERS = [os.path.join(CSRC, "pgm_internal.h"), os.path.join(CSRC, "audit.h"), os.path.join(CSRC, "lr_layout.h"), os.path.join(CSRC, "lr_math.cuh"), os.path.join(CSRC, "bp_common.cuh"),
            os.path.join(CSRC, "pair_math.cuh"), os.path.join(ROOT, "include", "pgm.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -55,9 +55,6 @@ namespace {
 
 constexpr uint32_t kFlagTimeout = PGM_FLAG_TIMEOUT;
 
-// Where a block's items and exchanged values live.
-enum Exchange : int { kAlone = 0, kCluster = 1, kGrid = 2 };
-
 struct LrRun {
     int32_t V, E;
     const int4 *tab4;       // each variable's incoming edge-states (DevGraph::vin_tab4)
@@ -981,14 +978,6 @@ RunKernel run_kernel(bool maxp, int x, bool res, bool lam) {
     return maxp ? run_kernel_t<true>(x, res, lam) : run_kernel_t<false>(x, res, lam);
 }
 
-// Shared memory of a block.
-size_t run_smem(int x, bool res, bool lam, int Vc, int f_cap, int h_cap) {
-    size_t n = (lam ? 32 : 24) * (size_t)Vc;
-    if (res) n += 8 * (size_t)Vc + 16 * (size_t)f_cap + 20 * (size_t)h_cap;
-    if (x == kCluster) n += 16 * (size_t)h_cap;
-    return n + 16;
-}
-
 // What the device offers, asked once: SMs, shared memory for a block, cluster size, whether
 // it takes cooperative launches. The kernels' attributes are set here too.
 struct RunDevice {
@@ -1055,16 +1044,6 @@ const RunDevice &run_device() {
     return R;
 }
 
-// Shared memory of a gradient block.
-size_t grad_smem(int x, int Vc, int f_cap, int h_cap) {
-    return 44 * (size_t)Vc + 32 * (size_t)f_cap + (x == kCluster ? 52 : 36) * (size_t)h_cap + 16;
-}
-
-int run_threads(int Vc, int items) {
-    const int per = std::max(Vc, items);
-    return std::min(kLrRunThreads, std::max(32, (per + 31) / 32 * 32));
-}
-
 template <class Args>
 cudaError_t launch(void (*kern)(const Args), const Args &A, int blocks, int threads, size_t smem, int x, cudaStream_t s) {
     cudaLaunchConfig_t cfg{};
@@ -1088,17 +1067,14 @@ cudaError_t launch(void (*kern)(const Args), const Args &A, int blocks, int thre
 }
 
 // The push form of one block per sample (lr_block_fits).
-constexpr int kPushOneE = 600;
 template <bool MAXP>
-RunKernel push_kernel(int E) {
-    if (E <= kPushOneE) return k_lr_push<MAXP, 1, false>;
-    return E <= kLrRunThreads ? k_lr_push<MAXP, 1, true> : E <= 2 * kLrRunThreads ? k_lr_push<MAXP, 2, true>
-                                                                                  : k_lr_push<MAXP, 4, true>;
+RunKernel push_kernel(const PushShape &p) {
+    if (!p.two) return k_lr_push<MAXP, 1, false>;
+    return p.edges == 1 ? k_lr_push<MAXP, 1, true> : p.edges == 2 ? k_lr_push<MAXP, 2, true> : k_lr_push<MAXP, 4, true>;
 }
 cudaError_t launch_push(const LrRun &A, bool maxp, int samples, cudaStream_t s) {
-    const int ne = A.E <= kLrRunThreads ? 1 : A.E <= 2 * kLrRunThreads ? 2 : 4;
-    return launch(maxp ? push_kernel<true>(A.E) : push_kernel<false>(A.E), A, samples,
-                  run_threads(A.V, (A.E + ne - 1) / ne), (A.E <= kPushOneE ? 32 : 40) * (size_t)A.V, kAlone, s);
+    const PushShape p = push_shape(A.V, A.E);
+    return launch(maxp ? push_kernel<true>(p) : push_kernel<false>(p), A, samples, p.threads, p.smem, kAlone, s);
 }
 
 LrRun run_args(const DevGraph &G, const EnumSeg *segs, int n_seg, const float *pot, const float *ev, float *msgs,
@@ -1164,13 +1140,6 @@ cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *l
 int lr_grid_device() { return run_device().coop ? run_device().n_sm : 0; }
 int lr_grid_smem() { return run_device().smem; }
 
-int lr_grid_blocks(int V, int n_sm, int smem) {
-    if (n_sm < 1 || V < 2) return 0;
-    const int Vc = std::max((V + n_sm - 1) / n_sm, kLrGridMinV);
-    const int nb = (V + Vc - 1) / Vc;
-    return nb >= 2 && run_smem(kGrid, false, false, Vc, 0, 0) <= (size_t)smem && Vc < (1 << 14) ? nb : 0;
-}
-
 bool lr_grid_fits(const LrGridPlan &g, int V, int F) {
     const RunDevice &R = run_device();
     if (g.nb < 2 || !R.coop || g.nb > R.n_sm) return false;
@@ -1221,29 +1190,7 @@ cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPla
 
 LrMultiPlan lr_multi_plan(int V, int S, bool local) {
     const RunDevice &R = run_device();
-    LrMultiPlan p;
-    if (R.n_sm < 1 || V < 1 || S < 1) return p;
-    const int v_max = std::min((1 << 14) - 1, (R.smem - 16) / 24);  // variables one block can own
-    const int nb_min = (V + v_max - 1) / v_max;
-    int nb = 1, Sc = S;
-    if (V > kLrAloneV && R.coop && local && nb_min <= R.n_sm) {
-        const int chunks = (S + R.n_sm / nb_min - 1) / (R.n_sm / nb_min);
-        Sc = (S + chunks - 1) / chunks;
-        nb = std::min(R.n_sm / Sc, (V + kLrGridMinV - 1) / kLrGridMinV);
-    } else if (nb_min > 1) {
-        return p;
-    }
-    p.Vc = (V + nb - 1) / nb;
-    p.nb = (V + p.Vc - 1) / p.Vc;
-    p.f_cap = 2 * p.Vc;
-    p.h_cap = p.nb > 1 ? 4 * p.Vc : 0;
-    const int x = p.nb > 1 ? kGrid : kAlone;
-    p.res = run_smem(x, true, true, p.Vc, p.f_cap, p.h_cap) <= (size_t)R.smem;
-    // per sample: lam and directory, then each block's items (run_multi's layout)
-    p.sample_bytes = 32 * (size_t)V + (size_t)p.nb * (16 * (size_t)p.h_cap + (p.res ? 0 : 16 * (size_t)p.f_cap + 20 * (size_t)p.h_cap));
-    if (p.nb == 1) Sc = (int)std::min<int64_t>(S, std::max<int64_t>(1, ((int64_t)1 << 28) / (int64_t)p.sample_bytes));
-    p.S = Sc;
-    return p;
+    return lr_multi_plan(V, S, local, R.n_sm, R.smem, R.coop);
 }
 
 cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiPlan &p, int S, int64_t pot_stride,

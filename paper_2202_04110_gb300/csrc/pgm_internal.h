@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/pgm.h"
+#include "lr_layout.h"
 
 namespace pgm {
 
@@ -365,14 +366,7 @@ struct LrWait {
     uint32_t *host;
 };
 constexpr int kLrWaitPolls = 1 << 22;
-constexpr int kLrRunThreads = 1024, kLrSmallMaxV = 1024, kLrSmallMaxF = 2048;
-constexpr int kLrClusterMax = 16;
 int lr_cluster_size();
-// Setting 1 of PGM_OPT_SMALL_RUN: one block up to this many variables and factors, the cluster
-// up to kLrClusterAutoV variables, the grid form above (us per iteration, T = 1, square grids:
-// 22 x 22 block 0.65, cluster 0.82; 24 x 24 1.03, 0.81; 90 x 90 cluster 1.17; 128 x 128 cluster
-// 1.75, grid 1.22).
-constexpr int kLrBlockAutoV = 700, kLrBlockAutoF = 1024, kLrClusterAutoV = 9000;
 inline bool lr_block_fits(int V, int F) { return V > 0 && V <= kLrSmallMaxV && F <= kLrSmallMaxF; }
 inline bool lr_cluster_fits(int V, int F) {
     const int C = lr_cluster_size();
@@ -390,29 +384,17 @@ cudaError_t launch_lr_small_run(const DevGraph &G, const Plan &P, const float *l
                                 float *msgs, float *lam, int32_t *dir, float T, float damping, int n_iters,
                                 bool cluster, const LrWait &wait, cudaStream_t s);
 // Larger graphs: a cooperative grid of nb blocks, block b owning variables b Vc ..
-// (b + 1) Vc - 1. lr_grid_blocks: nb for V variables on n_sm SMs with smem bytes a block (0: none);
-// the plan's other fields are counted from the graph (capi.cu). lr_grid_device, lr_grid_smem: this
-// device's (0 SMs: no cooperative launches). lr_grid_fits: the device takes the plan and the
-// graph's scratch holds its workspace.
-constexpr int kLrGridMinV = 256;  // variables per block at least
-int lr_grid_blocks(int V, int n_sm, int smem);
+// (b + 1) Vc - 1 (nb: lr_grid_blocks; the plan's other fields are counted from the graph, capi.cu).
+// lr_grid_device, lr_grid_smem: this device's SMs (0: no cooperative launches) and shared memory a
+// block. lr_grid_fits: the device takes the plan and the graph's scratch holds its workspace.
 int lr_grid_device();
 int lr_grid_smem();
-// A GB300's, for sizes that are stated without asking a device (pgm_check_desc, serving budgets).
-constexpr int kPlanSms = 152, kPlanSmem = 232448 - 256;
 bool lr_grid_fits(const LrGridPlan &g, int V, int F);
 cudaError_t launch_lr_grid_run(const DevGraph &G, const Plan &P, const LrGridPlan &g, const float *log_pot,
                                const float *ev, float *msgs, float *lam, float *m_tmp, float *b, float *d, float *prm,
                                float T, float damping, int n_iters, const LrWait &wait, cudaStream_t s);
 // S samples of one graph (pgm_run_bp_multi), nb blocks each, up to p.S samples a launch;
 // work: p.sample_bytes per sample. local: few factors join different blocks (LrGridPlan).
-constexpr int kLrAloneV = 1536;  // up to this many variables a sample takes one block
-struct LrMultiPlan {
-    int S = 0;  // samples per launch; 0: the device takes no such launch
-    int nb = 0, Vc = 0, f_cap = 0, h_cap = 0;
-    bool res = false;
-    size_t sample_bytes = 0;
-};
 LrMultiPlan lr_multi_plan(int V, int S, bool local);
 cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiPlan &p, int S, int64_t pot_stride,
                                 const float *log_pot, const float *ev, float *msgs, char *work, float T, float damping,
