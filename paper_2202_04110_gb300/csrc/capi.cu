@@ -376,7 +376,7 @@ std::vector<FuseBlock> fuse_plan(const HostLayout &H, int variant, int n_sm, int
     // would form the table less often, but a round's loads depend on one another and other
     // blocks hide them better (K = 16 on 128 uneven grids: 171 us with one round, 192 with
     // two). 128 threads; 256 for K = 16 from 6 such blocks per SM on, where the table counts
-    // (256 x 256: 16.6 against 17.2 us per iteration; 178 x 178: 9.9 against 9.4)
+    // (256 x 256, T = 0: 12.8 against 13.6 us per iteration, T = 1: 15.7 against 15.8)
     const int lanes = variant == kPairT4 ? 1 : variant == kPairT8 ? 2 : 4;
     const int threads = lanes == 4 && (int64_t)bucket.size() * lanes >= (int64_t)256 * 6 * n_sm ? 256 : 128;
     const int per = threads / lanes;
@@ -865,11 +865,12 @@ static pgm_status build_from_layout(const HostLayout &H, pgm_graph **out, cudaSt
     size_t vs_bytes = align_up(std::max<int64_t>(H.VS, 1) * sizeof(float), 256);
     size_t hd_bytes = H.var_bucket[kVarBlock].empty() ? 0 : 4 * vs_bytes;
     const size_t lr_bytes = g->P.lr ? align_up((size_t)g->lr_slots * sizeof(float), 256) : 0;
+    const size_t lam_bytes = g->P.lr ? align_up(lam_floats_max(g->lr_slots) * sizeof(float), 256) : 0;
     const size_t prm_bytes = g->P.lr ? align_up((size_t)3 * (H.E / 2) * sizeof(float), 256) : 0;
     const size_t blo_bytes = keeps_b_lo(H) ? vs_bytes : 0;
     const size_t tot_bytes = align_up((size_t)g->hd_tot_entries * sizeof(float4), 256) +
                              align_up((size_t)g->hd_vars * sizeof(int32_t), 256);
-    const size_t scratch_bytes = es_bytes + vs_bytes + 256 + hd_bytes + 2 * lr_bytes + prm_bytes + blo_bytes + tot_bytes;
+    const size_t scratch_bytes = es_bytes + vs_bytes + 256 + hd_bytes + lr_bytes + lam_bytes + prm_bytes + blo_bytes + tot_bytes;
     char *smem = nullptr;
     ce = ordered ? cudaMallocAsync(&smem, scratch_bytes, s) : cudaMalloc(&smem, scratch_bytes);
     if (ce != cudaSuccess) {
@@ -904,10 +905,10 @@ static pgm_status build_from_layout(const HostLayout &H, pgm_graph **out, cudaSt
     G.flags = flags;
     G.hd_b = hd_bytes ? reinterpret_cast<float *>(smem + es_bytes + vs_bytes + 256) : nullptr;
     G.lr_pos = g->P.lr ? reinterpret_cast<const int32_t *>(dmem + o_lr_pos) : nullptr;
-    G.b_lo = blo_bytes ? reinterpret_cast<float *>(smem + es_bytes + vs_bytes + 256 + hd_bytes + 2 * lr_bytes +
+    G.b_lo = blo_bytes ? reinterpret_cast<float *>(smem + es_bytes + vs_bytes + 256 + hd_bytes + lr_bytes + lam_bytes +
                                                     prm_bytes)
                        : nullptr;
-    G.hd_tot = tot_bytes ? reinterpret_cast<float4 *>(smem + es_bytes + vs_bytes + 256 + hd_bytes + 2 * lr_bytes +
+    G.hd_tot = tot_bytes ? reinterpret_cast<float4 *>(smem + es_bytes + vs_bytes + 256 + hd_bytes + lr_bytes + lam_bytes +
                                                       prm_bytes + blo_bytes)
                          : nullptr;
     G.hd_cnt = g->hd_vars ? reinterpret_cast<int32_t *>(reinterpret_cast<char *>(G.hd_tot) +
@@ -924,7 +925,7 @@ static pgm_status build_from_layout(const HostLayout &H, pgm_graph **out, cudaSt
     if (g->P.lr) {
         g->lr_d = reinterpret_cast<float *>(smem + es_bytes + vs_bytes + 256 + hd_bytes);
         g->lr_lam = reinterpret_cast<float *>(smem + es_bytes + vs_bytes + 256 + hd_bytes + lr_bytes);
-        g->lr_prm = reinterpret_cast<float *>(smem + es_bytes + vs_bytes + 256 + hd_bytes + 2 * lr_bytes);
+        g->lr_prm = reinterpret_cast<float *>(smem + es_bytes + vs_bytes + 256 + hd_bytes + lr_bytes + lam_bytes);
     }
     // attach device pointers of the launch lists / segments
     size_t vi = 0, fi = 0;
@@ -1007,7 +1008,8 @@ int64_t pgm::layout_device_bytes(const HostLayout &H) {
     size_t es_bytes = align_up(std::max<int64_t>(H.ES, 1) * sizeof(float), 256);
     const int nb_grid = lr_grid_plan_blocks(H.V, kPlanSms, kPlanSmem);
     if (lr_eligible(H))  // the slot map, the two log-ratio arrays, the table differences, the grid plan
-        idx += H.E * sizeof(int32_t) + 2 * align_up((size_t)lr_slot_count(H) * sizeof(float), 256) +
+        idx += H.E * sizeof(int32_t) + align_up((size_t)lr_slot_count(H) * sizeof(float), 256) +
+               align_up(lam_floats_max(lr_slot_count(H)) * sizeof(float), 256) +
                align_up((size_t)3 * (H.E / 2) * sizeof(float), 256) +
                (H.vin_tab4.empty() || nb_grid == 0 ? 0 : ((size_t)nb_grid + 1) * sizeof(int2));
     for (int variant : {kPairT4, kPairT8, kPairT16}) {

@@ -33,6 +33,12 @@ inline size_t run_smem(int x, bool res, bool lam, int Vc, int f_cap, int h_cap) 
     return n + 16;
 }
 
+// Explicit sums in global memory (the form with totals): 4 Vc a block, fewer than 4 nb floats more than
+// 4 V in all, of which a graph's scratch has room for up to kLrMaxBlocks blocks.
+constexpr int kLrMaxBlocks = 256;
+inline size_t lam_floats(int nb, int Vc) { return 4 * (size_t)nb * Vc; }
+inline size_t lam_floats_max(int64_t slots) { return (size_t)slots + 4 * kLrMaxBlocks; }
+
 // Shared memory of a gradient block.
 inline size_t grad_smem(int x, int Vc, int f_cap, int h_cap) {
     return 44 * (size_t)Vc + 32 * (size_t)f_cap + (x == kCluster ? 52 : 36) * (size_t)h_cap + 16;
@@ -60,6 +66,7 @@ inline PushShape push_shape(int V, int E) {
 // The grid form: blocks for V variables on n_sm SMs with smem bytes a block (0: none).
 inline int lr_grid_blocks(int V, int n_sm, int smem) {
     if (n_sm < 1 || V < 2) return 0;
+    n_sm = std::min(n_sm, kLrMaxBlocks);
     const int Vc = std::max((V + n_sm - 1) / n_sm, kLrGridMinV);
     const int nb = (V + Vc - 1) / Vc;
     return nb >= 2 && run_smem(kGrid, false, false, Vc, 0, 0) <= (size_t)smem && Vc < (1 << 14) ? nb : 0;
@@ -92,7 +99,7 @@ inline LrMultiPlan lr_multi_plan(int V, int S, bool local, int n_sm, int smem, b
     p.h_cap = p.nb > 1 ? 4 * p.Vc : 0;
     p.res = run_smem(p.nb > 1 ? kGrid : kAlone, true, true, p.Vc, p.f_cap, p.h_cap) <= (size_t)smem;
     // per sample: lam and directory, then each block's items (launch_lr_multi_run's layout)
-    p.sample_bytes = 32 * (size_t)V + (size_t)p.nb * (16 * (size_t)p.h_cap + (p.res ? 0 : 16 * (size_t)p.f_cap + 20 * (size_t)p.h_cap));
+    p.sample_bytes = 4 * lam_floats(p.nb, p.Vc) + 16 * (size_t)V + (size_t)p.nb * (16 * (size_t)p.h_cap + (p.res ? 0 : 16 * (size_t)p.f_cap + 20 * (size_t)p.h_cap));
     if (p.nb == 1) Sc = (int)std::min<int64_t>(S, std::max<int64_t>(1, ((int64_t)1 << 28) / (int64_t)p.sample_bytes));
     p.S = Sc;
     return p;

@@ -62,8 +62,9 @@ struct LrRun {
     const EnumSeg *segs;
     int n_seg;
     const float *pot, *ev;
-    float *msgs, *lam;      // lam: explicit sums of variables with infinite entries, [4 V] per sample
+    float *msgs, *lam;      // lam: explicit sums of variables with infinite entries, lam_floats per sample
     int64_t pot_stride, ev_stride, msg_stride;  // per sample (pot_stride 0: one table set)
+    int64_t lam_stride;                         // (lam_floats)
     uint32_t *flags;
     float k, Tln2, damping;
     int n_iters;
@@ -80,7 +81,7 @@ struct LrRun {
 };
 
 // A wait of this run has run out.
-__device__ __forceinline__ void wait_failed(const LrRun &A) {
+__device__ __noinline__ void wait_failed(const LrRun &A) {
     atomicOr(A.flags, kFlagTimeout);
     if (A.wait.host) {
         *(volatile uint32_t *)A.wait.host = 1u;
@@ -144,11 +145,18 @@ __device__ __noinline__ float run_exact(const LrRun &A, const float *pot, int v0
     return lr_dir_exact<MAXP>(phi, (es >> 1) & 1, l, mo, A.k, A.Tln2, A.damping, A.flags);
 }
 
-// A variable whose values do not come out finite: its four lam by the explicit sums, at lam[k step].
-__device__ __noinline__ void run_var_slow(float *lam, int step, float2 e, float d0, float d1, float d2, float d3) {
+// A variable whose values do not come out finite: its four lam by the explicit sums.
+__device__ __noinline__ void run_var_slow(float *lam, int lv, int Vc, float2 e, float d0, float d1, float d2, float d3) {
     const float dk[4] = {d0, d1, d2, d3};
-    const int pos[4] = {0, step, 2 * step, 3 * step};
+    const int pos[4] = {lv, Vc + lv, 2 * Vc + lv, 3 * Vc + lv};
     lr_var_slow(e, dk, pos, 4, lam);
+}
+
+// A block's explicit sums in global memory, by local slot: 4 Vc a block, so that the last one's, of
+// fewer variables, end inside. (Formed where it is used: the streamed forms are at 60 to 64 registers,
+// and an index by variable, or a call in the factor loop, cost 3 to 6 % on 32 samples of 256 x 256.)
+__device__ __forceinline__ float *run_sums(const LrRun &A, int smp, int v0) {
+    return A.lam + (size_t)smp * A.lam_stride + 4 * (size_t)v0;
 }
 
 __device__ __forceinline__ bool is_slow(float2 D) { return __float_as_uint(D.x) == kDvSlow; }
@@ -178,7 +186,6 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
     const float *pot = A.pot + (size_t)smp * A.pot_stride;
     const float2 *ev = reinterpret_cast<const float2 *>(A.ev + (size_t)smp * A.ev_stride) + v0;
     float *msgs = A.msgs + (size_t)smp * A.msg_stride;
-    float *lam_g = LAM ? nullptr : A.lam + (size_t)smp * 4 * V + 4 * (size_t)v0;  // explicit sums, 4 a variable
     int32_t *dir = A.dir + (size_t)smp * 4 * V;
     // shared memory: [records, split records,] lam or totals, [evidence,] [inbox,] slots, [addresses]
     char *sp = lr_sm;
@@ -220,10 +227,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
 
     // ---- prologue: slots from msgs, the block's items ----
     if (tid < 2) s_n[tid] = 0;
-    if (tid == 0) {
-        s_abort = X != kAlone && A.wait.polls == 0;
-        if (s_abort) wait_failed(A);
-    }
+    if (tid == 0) s_abort = X != kAlone && A.wait.polls == 0;
     __syncthreads();
     for (int l0 = 0; l0 < nv; l0 += nt) {
         const int lv = l0 + tid, v = v0 + lv;
@@ -307,9 +311,8 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
     auto lam_of = [&](int s, float dk) {
         if constexpr (LAM) return lam[s];
         else {
-            const int lv = var_of(s);
-            const float2 D = Dv[lv];
-            return is_slow(D) ? __ldcg(lam_g + 4 * (size_t)lv + (s - lv) / Vc) : lr_lam_from_D(D, dk);
+            const float2 D = Dv[var_of(s)];
+            return is_slow(D) ? __ldcg(run_sums(A, smp, v0) + s) : lr_lam_from_D(D, dk);
         }
     };
     // what the thread reads first in steps 1 and 3 is fixed for the run: in registers when the
@@ -338,9 +341,9 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
                          isfinite(l0) && isfinite(l1) && isfinite(l2) && isfinite(l3));
             if (slow) {
                 if constexpr (LAM) {
-                    run_var_slow(lam + lv, Vc, e, d0, d1, d2, d3);
+                    run_var_slow(lam, lv, Vc, e, d0, d1, d2, d3);
                 } else {
-                    run_var_slow(lam_g + 4 * (size_t)lv, 1, e, d0, d1, d2, d3);
+                    run_var_slow(run_sums(A, smp, v0), lv, Vc, e, d0, d1, d2, d3);
                     Dv[lv] = make_float2(__uint_as_float(kDvSlow), 0.f);
                 }
             } else if constexpr (LAM) {
@@ -415,7 +418,6 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
                     if ((uint32_t)(wd >> 32) == (uint32_t)it) break;
                     if (*(volatile int *)&s_abort) break;
                     if (++polls >= A.wait.polls) {
-                        wait_failed(A);
                         *(volatile int *)&s_abort = 1;
                         break;
                     }
@@ -430,6 +432,8 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
         }
         __syncthreads();
     }
+
+    if (X != kAlone && tid == 0 && s_abort) wait_failed(A);  // (here, not in the wait loop: 2 to 3 %)
 
     // ---- epilogue: every slot's two entries back into msgs (as k_lr_unpack) ----
     const bool aligned = (reinterpret_cast<uintptr_t>(msgs) & 7u) == 0;
@@ -667,7 +671,7 @@ __device__ __forceinline__ void grad_publish(const LrRun &A, const float *val, c
 }
 template <int X>
 __device__ __forceinline__ float grad_receive(const LrRun &A, const unsigned long long *box, size_t h_base, int h, int st,
-                                              int *s_abort, int *bail) {
+                                              int *s_abort) {
     unsigned long long wd = 0;
     int polls = 0;
     while (true) {
@@ -681,7 +685,6 @@ __device__ __forceinline__ float grad_receive(const LrRun &A, const unsigned lon
         if ((uint32_t)(wd >> 32) == (uint32_t)st) return __uint_as_float((uint32_t)wd);
         if (*(volatile int *)s_abort) break;
         if (++polls >= A.wait.polls) {
-            *(volatile int *)bail = 1;
             *(volatile int *)s_abort = 1;
             break;
         }
@@ -725,10 +728,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
     uint32_t *hdst = reinterpret_cast<uint32_t *>(sp);
 
     if (tid < 2) s_n[tid] = 0;
-    if (tid == 0) {
-        s_abort = X != kAlone && A.wait.polls == 0;
-        if (s_abort) *(volatile int *)P.bail = 1;
-    }
+    if (tid == 0) s_abort = X != kAlone && A.wait.polls == 0;
     for (int i = tid; i < A.f_cap; i += nt) racc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i = tid; i < A.h_cap; i += nt) hacc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
@@ -825,7 +825,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
                 lam[2 * Vc + lv] = lr_lam_from_D(Df, d2);
                 lam[3 * Vc + lv] = lr_lam_from_D(Df, d3);
             } else {
-                run_var_slow(lam + lv, Vc, e, d0, d1, d2, d3);
+                run_var_slow(lam, lv, Vc, e, d0, d1, d2, d3);
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) __stcg(H + q * Vc + lv, lam[q * Vc + lv]);
@@ -851,7 +851,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
             const uint32_t pk = __float_as_uint(r.w);
             const int s = pk & 0xffff;
             const bool one = (pk >> 16) != 0;  // the message into the factor's variable 1
-            const float mo = d[s], l = grad_receive<X>(A, box, h_base, h, it, &s_abort, P.bail);
+            const float mo = d[s], l = grad_receive<X>(A, box, h_base, h, it, &s_abort);
             float n = one ? grad_dir(r.z, r.y + r.x - r.z, r.x, l, mo, T, invT, damping, w)
                           : grad_dir(r.x, r.y, r.z, l, mo, T, invT, damping, w);
             if (lr_dir_rare(n, l)) n = rare(s, l, mo);
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
             const uint32_t pk = __float_as_uint(r.w);
             const int s = pk & 0xffff;
             const bool one = (pk >> 16) != 0;  // the source is variable 1: the message to variable 0
-            const float l = __ldcg(H + s), a = w * grad_receive<X>(A, box, h_base, h, st, &s_abort, P.bail);
+            const float l = __ldcg(H + s), a = w * grad_receive<X>(A, box, h_base, h, st, &s_abort);
             const DirGrad g = one ? dir_grad(r.y, r.z, l, a, invT) : dir_grad(r.y + r.x - r.z, r.x, l, a, invT);
             lam[s] = g.lam;
             float4 t = hacc[h];
@@ -956,7 +956,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
         atomicAdd(t + 2, a.z);
         atomicAdd(t + 3, a.w);
     }
-    if (bad) *P.bail = 1;
+    if (bad || (X != kAlone && s_abort)) *P.bail = 1;
     if constexpr (X == kCluster) cluster_barrier();
 }
 
@@ -1206,6 +1206,7 @@ cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiP
     A.msg_stride = G.ES;
     A.nb = p.nb;
     A.Vc = p.Vc;
+    A.lam_stride = (int64_t)lam_floats(p.nb, p.Vc);
     A.f_cap = p.f_cap;
     A.h_cap = p.h_cap;
     // 16-byte records first, then 8-byte inboxes, then words
@@ -1218,7 +1219,7 @@ cudaError_t launch_lr_multi_run(const DevGraph &G, const Plan &P, const LrMultiP
     A.box1 = A.box0 + blocks * p.h_cap;
     A.hdst = reinterpret_cast<uint32_t *>(A.box1 + blocks * p.h_cap);
     A.lam = reinterpret_cast<float *>(A.hdst + (p.res ? 0 : blocks * p.h_cap));
-    A.dir = reinterpret_cast<int32_t *>(A.lam + 4 * V * S);
+    A.dir = reinterpret_cast<int32_t *>(A.lam + lam_floats(p.nb, p.Vc) * S);
     if (p.nb == 1 && G.V <= kLrBlockAutoV && lr_block_fits(G.V, G.E / 2)) return launch_push(A, T == 0.f, S, s);
     const int x = p.nb > 1 ? kGrid : kAlone;
     const bool lam_sh = run_smem(x, false, true, p.Vc, 0, 0) <= (size_t)run_device().smem;

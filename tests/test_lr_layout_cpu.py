@@ -25,6 +25,7 @@ long constants(int i) {
 }
 long c_run_smem(int x, int res, int lam, int Vc, int f, int h) { return (long)run_smem(x, res, lam, Vc, f, h); }
 long c_grad_smem(int x, int Vc, int f, int h) { return (long)grad_smem(x, Vc, f, h); }
+long c_lam_max(long slots) { return (long)lam_floats_max(slots); }
 int c_run_threads(int Vc, int items) { return run_threads(Vc, items); }
 int c_grid_blocks(int V, int n_sm, int smem) { return lr_grid_blocks(V, n_sm, smem); }
 void c_push(int V, int E, long *o) {
@@ -46,7 +47,7 @@ def lib(tmp_path_factory):
     so = str(d / "wrap.so")
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-o", so, str(d / "wrap.cpp")], check=True)
     lib = ctypes.CDLL(so)
-    for f in ("constants", "c_run_smem", "c_grad_smem"):
+    for f in ("constants", "c_run_smem", "c_grad_smem", "c_lam_max"):
         getattr(lib, f).restype = ctypes.c_long
     return lib
 
@@ -117,6 +118,9 @@ def test_grid_blocks(lib, V):
     Vc = -(-V // nb)
     assert 2 <= nb <= SMS and nb * Vc >= V and 4 * Vc <= 1 << 16  # (slots are 16 bits)
     assert lib.c_run_smem(GRID, 0, 0, Vc, 0, 0) <= SMEM
+    # explicit sums: a last block's of fewer variables end inside the scratch
+    last = V - (nb - 1) * Vc
+    assert 4 * (nb - 1) * Vc + 3 * Vc + max(last, 1) <= lib.c_lam_max(ctypes.c_long(4 * V))
     assert (lib.c_run_smem(GRID, 0, 1, Vc, 0, 0) <= SMEM) == (V <= 1102760)  # lam per slot: 7,255 a block
     for f in (1, Vc, 2 * Vc):
         t = lib.c_run_threads(Vc, f)
@@ -150,4 +154,4 @@ def test_samples_per_launch(lib, V, S, local):
     assert res or lib.c_run_smem(x, 0, 0, Vc, 0, 0) <= SMEM
     # launch_lr_multi_run's layout: records, split records, two inboxes, addresses, explicit sums, directory
     parts = ([] if res else [(16, Sc * nb * f), (16, Sc * nb * h)]) + [(8, 2 * Sc * nb * h)] + ([] if res else [(4, Sc * nb * h)])
-    assert _walk(parts + [(4, 4 * V * Sc), (4, 4 * V * Sc)]) <= Sc * sample
+    assert _walk(parts + [(4, 4 * nb * Vc * Sc), (4, 4 * V * Sc)]) <= Sc * sample
