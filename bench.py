@@ -108,30 +108,11 @@ def measured_peaks():
     return FALLBACK_HBM_GBS, "fallback"
 
 
-LR_KERNELS = ("k_pair2_lr", "k_var_slot4_lr", "k_var_csr_lr")
-
-
 def kernel_source_hash(kernel: str) -> str:
-    """sha256 (16 hex digits) of the source a kernel is built from: for the log-ratio
-    kernels, lr_math.cuh, bp_common.cuh, the log-ratio section of kernels.cu and the
-    log-ratio launchers; for the others, the whole of kernels.cu and the headers."""
+    """sha256 (16 hex digits) of the source a kernel of the one-launch runs is built from."""
     csrc = os.path.join(ROOT, "paper_2202_04110_gb300", "csrc")
-
-    def read(name):
-        with open(os.path.join(csrc, name)) as f:
-            return f.read()
-
-    src = read("kernels.cu")
-    head = read("lr_math.cuh") + read("bp_common.cuh")
-    if kernel in LR_KERNELS:
-        a = src.index("// Binary pairwise graphs: log-ratio messages (Plan::lr)")
-        b = src.index("// Many evidence / potential sets on one binary pairwise graph")
-        c = src.index("static cudaError_t launch_pdl(")
-        d = src.index("cudaError_t launch_ms_prepare(")
-        src = head + src[a:b] + src[c:d]
-    else:
-        src += head + read("pair_math.cuh")
-    return hashlib.sha256(src.encode()).hexdigest()[:16]
+    src = "".join(open(os.path.join(csrc, name)).read() for name in ("lr_run.cu", "lr_math.cuh", "lr_layout.h"))
+    return hashlib.sha256((kernel + src).encode()).hexdigest()[:16]
 
 
 def profiled_traffic(kernel: str, workload: str):
@@ -983,7 +964,7 @@ def run_ours(args):
     lr = lr_min > 0 and args.iters >= lr_min
     # (a grid above the small forms whose 24 bytes per variable fit the SMs' shared
     # memories is one cooperative launch per run; beliefs and decode follow either way)
-    one_launch = lr and I["max_degree"] <= 4 and (g.get_option(binding.OPT_SMALL_RUN) != 0 or I["n_vars"] <= 1_450_000)
+    one_launch = lr and I["max_degree"] <= 4 and (g.get_option(binding.OPT_SMALL_RUN) != 0 or I["n_vars"] <= 1_470_448)
     launches_per_step = len(temps) * (2 + (1 if one_launch else args.iters * I["launches_per_iter"] + (3 if lr else 0)))
 
     if dist is not None:
@@ -1061,11 +1042,10 @@ def run_ours(args):
     dom_bytes, oth_bytes = (fac_bytes, var_bytes) if fac_dom else (var_bytes, fac_bytes)
     dom_impl, oth_impl = (impl_fac_bytes, impl_var_bytes) if fac_dom else (impl_var_bytes, impl_fac_bytes)
     dom_s, oth_s = (fac_avg_s, var_avg_s) if fac_dom else (var_avg_s, fac_avg_s)
-    roof = {"bound": "hbm", "kernel": dominant,
+    passes = {"bound": "hbm", "kernel": dominant,
             "achieved": round(dom_gbs, 1),
             "peak": peak, "unit": "GB/s", "peak_source": f"{peak_src} HBM copy bandwidth",
             "frac": round(dom_gbs / peak, 4),
-            "traffic": profiled_traffic(dominant, wl),
             "algorithmic_bytes_per_launch": dom_bytes,
             "algorithmic_bytes": "the factor pass's share of the per-iteration minimum 8 ES + 4 sum n_cfg + "
                                  "4 VS + 4 E (8 ES + 4 sum n_cfg + 4 E); the variable pass's share is 4 VS",
@@ -1077,22 +1057,35 @@ def run_ours(args):
                         "algorithmic_bytes_per_launch": oth_bytes,
                         "implementation_bytes_per_launch": oth_impl,
                         "implementation_frac": round(oth_impl / oth_s / 1e9 / peak, 4),
-                        "mean_launch_us": round(1e6 * oth_s, 2),
-                        "traffic": profiled_traffic(other, wl)}},
+                        "mean_launch_us": round(1e6 * oth_s, 2)}},
             "kernel_timing": "CUDA events on the launching stream around the passes of every "
                              f"{min(PROFILE_PERIOD, args.iters)}th iteration of runs after the timed ones, launch by "
-                             "launch (event nodes in their CUDA graphs); a timed run is one launch of both passes "
-                             "where the graph's size allows",
+                             "launch (event nodes in their CUDA graphs)",
             "nominal_peak": NOMINAL_HBM_GBS, "frac_of_nominal": round(dom_gbs / NOMINAL_HBM_GBS, 4),
-            "iteration": {"algorithmic_bytes": iter_bytes,
-                          "implementation_bytes": impl_fac_bytes + impl_var_bytes,
-                          "mean_us": round(1e6 * iter_run_s, 2),
-                          "achieved": round(iter_bytes / iter_run_s / 1e9, 1),
-                          "frac": round(iter_bytes / iter_run_s / 1e9 / peak, 4),
-                          "frac_of_nominal": round(iter_bytes / iter_run_s / 1e9 / NOMINAL_HBM_GBS, 4),
-                          "timing": "CUDA events around each pgm_run_bp call of the timed steps / "
-                                    "iterations; both passes back to back",
-                          "sum_of_pass_events_us": round(1e6 * iter_s, 2)}}
+            "sum_of_pass_events_us": round(1e6 * iter_s, 2)}
+    iteration = {"algorithmic_bytes": iter_bytes,
+                 "implementation_bytes": impl_fac_bytes + impl_var_bytes,
+                 "mean_us": round(1e6 * iter_run_s, 2),
+                 "achieved": round(iter_bytes / iter_run_s / 1e9, 1),
+                 "frac": round(iter_bytes / iter_run_s / 1e9 / peak, 4),
+                 "frac_of_nominal": round(iter_bytes / iter_run_s / 1e9 / NOMINAL_HBM_GBS, 4),
+                 "timing": "CUDA events around each pgm_run_bp call of the timed steps / iterations"}
+    if one_launch:
+        # what runs in the timed region: one k_lr_run per run, its messages on the chip. A factor's two
+        # messages are four softplus values, an exponential and a logarithm each (T = 1 runs).
+        sm_mhz = float((clocks or {}).get("sm_max_mhz") or 2070.0)
+        mufu_peak = torch.cuda.get_device_properties(dev).multi_processor_count * 16 * sm_mhz * 1e6
+        t1_s = statistics.mean(run_ms[0::len(temps)]) / 1e3
+        mufu = 8.0 * F * args.iters / t1_s
+        roof = {"bound": "issue slots, then MUFU", "kernel": "k_lr_run", "achieved": round(mufu / 1e9, 1),
+                "peak": round(mufu_peak / 1e9, 1), "unit": "Gop/s (exp2 and log2)",
+                "peak_source": "SMs x 16 per clock x maximum SM clock", "frac": round(mufu / mufu_peak, 4),
+                "mean_launch_us": round(1e6 * t1_s, 1), "traffic": profiled_traffic("k_lr_run", wl),
+                "algorithmic_bytes_note": "the per-iteration minimum 8 ES + 4 sum n_cfg + 4 VS + 4 E does not cross HBM: "
+                                          "the iteration below can exceed the copy peak",
+                "iteration": iteration, "launch_per_pass": passes}
+    else:
+        roof = {**passes, "traffic": None, "iteration": iteration}
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
