@@ -535,13 +535,12 @@ pgm_status pgm_run_bp_until_members(pgm_graph *g, const float *log_pot, const fl
 /*
  * PGM_OPT_SMALL_RUN (default 1): a log-ratio run (PGM_OPT_LOG_RATIO) of a graph whose
  * variables have at most 4 factors each is one kernel launch: one thread block for at most
- * 700 variables (and 2,048 factors), else a cluster of C thread blocks on C SMs, whose
- * shared memories together hold the run's state, for at most 1,024 C variables and 2,048 C
- * factors: C = 16 where the device places a cluster of 16 such blocks (GB300: up to 16,384
- * variables), else 8 where it places 8, else no cluster form. 2 takes the cluster at every
- * size up to its limits. Above the cluster's limits pgm_run_bp is one cooperative launch of
- * up to one block per SM while 24 bytes per variable fit the SMs' shared memories (152 SMs:
- * up to 1.45 million variables) and few enough factors join two blocks' ranges of
+ * 700 variables and 1,024 factors, else a cluster of C thread blocks on C SMs for at most 9,000
+ * variables (where the form below does not apply: at most 1,024 C variables and 2,048 C factors):
+ * C = 16 where the device places a cluster of 16 such blocks (GB300), else 8 where it places 8,
+ * else no cluster form. 2 takes the cluster at every size up to its limits. Above, pgm_run_bp is
+ * one cooperative launch of up to one block per SM while 24 bytes per variable fit the SMs' shared
+ * memories (152 SMs: up to 1.47 million variables) and few enough factors join two blocks' ranges of
  * consecutive variables that the graph's scratch holds the exchange; pgm_run_bp_multi runs
  * chunks of samples in one such launch each. The launch converts msgs, runs every iteration
  * with the messages in shared memory, and writes msgs back, instead of 2 launches per
@@ -550,8 +549,9 @@ pgm_status pgm_run_bp_until_members(pgm_graph *g, const float *log_pot, const fl
  * iterations, so the messages and flags are bitwise the same. 0 turns all of it off. Per-pass
  * profiling (pgm_set_profiling) keeps the multi-launch form, which is also the one that
  * launches_per_iter and pgm_launch_info describe. Changing it drops the cached CUDA
- * graphs. pgm_get_option returns the setting where a log-ratio run of the graph takes
- * the one-block or cluster form, else 0 (it asks the device once whether the cluster fits).
+ * graphs. pgm_get_option returns the setting where the graph is within the limits of the
+ * one-block or cluster form, else 0 (it asks the device once whether the cluster fits). Where the
+ * stream's context has too few SMs for a cooperative launch, the calls take their launches per pass.
  * A block's wait for another block is bounded (PGM_OPT_WAIT_POLLS). One that runs out raises
  * PGM_FLAG_TIMEOUT in the status word and ends the run with msgs undefined: pgm_run_bp and
  * pgm_run_bp_multi have returned by then, calls that return results to the host (pgm_infer_host,

@@ -44,8 +44,9 @@ __device__ __forceinline__ float edge_ratio(const float *__restrict__ d, const f
 __device__ __forceinline__ bool aligned16(const float *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // The next launch may be scheduled once every block of this one has its inputs: where they are
-// all resident (784 x 500: 164,000 and 196,000 threads). Blocks that still queue need the places
-// (pdl_launch_if_small).
+// all resident (784 x 500: 164,000 and 196,000 threads; 152 SMs hold 311,000). Blocks that still queue
+// need the places. (By threads, since these kernels' blocks have 128 to 1,024; the edge-state
+// kernels' rule, pdl_launch_if_small, counts blocks of mostly 256 and more registers.)
 __device__ __forceinline__ void pdl_launch_if_one_wave() {
     if ((int64_t)gridDim.x * gridDim.y * blockDim.x <= 300000) pdl_launch_dependents();
 }

@@ -24,7 +24,7 @@
 // with a block barrier after 1 and after 4. Step 3 runs while the values travel.
 // Measured against the multi-launch run (whole calls, GB300): 1000 x 1000, 200 iterations
 // 3.65 -> 1.80 ms (8.9 us per iteration), 317 x 241 max-product, 50 iterations 213 -> 87 us,
-// 32 evidence sets of 256 x 256, 100 iterations 4.22 -> 2.14 ms.
+// 32 evidence sets of 256 x 256, 100 iterations 4.22 -> 2.16 ms.
 //
 // Inbox words carry their iteration: one 8-byte store holds (value, iteration), and the
 // reader polls its own word until the iteration is the one it is in; no fence, flag or
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_push(const LrRun A) {
 // fine: its sigmas are 0 or 1) set *bail, and so does a wait that runs out: the caller's launches
 // take over.
 // Measured (GB300, whole calls): 64 x 64, 100 iterations, checkpoints every 10: 1.59 ms as ~590
-// dependent launches of 2.4 us, 0.32 in one (0.31 with plain sums over a variable's factors, which
+// dependent launches of 2.4 us, 0.313 in one (0.311 with plain sums over a variable's factors, which
 // lose what cancelling adjoints leave); with lr_dir's SFU forms 0.28, but the table gradients' error
 // against 64 bits rose from 2.3e-7 to 2.7e-7 (mean of 15 grids). What bounds it:
 // two barriers and an exchange per step of 200.
