@@ -79,6 +79,12 @@ struct LrMultiPlan {
     bool res = false;
     size_t sample_bytes = 0;
 };
+// A sample that several blocks do not divide well still takes one block up to kLrAloneMaxV variables, and
+// above that where S >= (V / 800)^2 samples keep as many SMs busy: one block is slower than the launches
+// of all samples together until they are that many (us per iteration, grids numbered at random, launches
+// against one block: 3,600 variables 3.7 / 4.5 with 8 samples, 5.1 / 4.5 with 32; 5,625 6.1 / 7.2 with 32,
+// 9.1 / 7.2 with 64; 9,409 13.5 / 14.2 with 64, 29 / 14.5 with 152).
+constexpr int kLrAloneMaxV = 3000;
 // coop: the device takes cooperative launches; local: few factors join different blocks (LrGridPlan).
 inline LrMultiPlan lr_multi_plan(int V, int S, bool local, int n_sm, int smem, bool coop) {
     LrMultiPlan p;
@@ -90,7 +96,7 @@ inline LrMultiPlan lr_multi_plan(int V, int S, bool local, int n_sm, int smem, b
         const int chunks = (S + n_sm / nb_min - 1) / (n_sm / nb_min);
         Sc = (S + chunks - 1) / chunks;
         nb = std::min(n_sm / Sc, (V + kLrGridMinV - 1) / kLrGridMinV);
-    } else if (nb_min > 1) {
+    } else if (nb_min > 1 || (V > kLrAloneMaxV && (int64_t)V * V > (int64_t)640000 * S)) {
         return p;
     }
     p.Vc = (V + nb - 1) / nb;

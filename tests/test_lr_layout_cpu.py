@@ -140,12 +140,15 @@ def test_one_block(lib, V, E):
 
 @pytest.mark.parametrize("V,S,local", [(100, 32, 1), (1536, 7, 1), (1537, 3, 1), (5000, 16, 1), (5000, 16, 0), (9000, 40, 1),
                                        (65536, 32, 1), (65536, 5, 1), (250000, 7, 1), (602175, 2, 1), (1000000, 3, 1),
-                                       (1480000, 2, 1), (20000, 3, 0), (100, 100000, 1)])
+                                       (1480000, 2, 1), (20000, 3, 0), (100, 100000, 1),
+                                       (2025, 2, 0), (3000, 2, 0), (3001, 2, 0), (3600, 20, 0), (3600, 21, 0), (9409, 32, 0),
+                                       (9409, 138, 0), (9409, 139, 0)])
 def test_samples_per_launch(lib, V, S, local):
     Sc, nb, Vc, f, h, res, sample = _out(lib.c_multi, 7, V, S, local)
-    if Sc == 0:  # (more than a block holds and the numbering is not local, or more than all blocks hold)
-        assert V > 9674 and (not local or V > 9674 * SMS)
+    if Sc == 0:  # (the numbering is not local and one block a sample does not pay; or no room)
+        assert V > 9674 * SMS if local else V > 9674 or (V > 3000 and S < (V / 800) ** 2)
         return
+    assert local or V <= 3000 or S >= (V / 800) ** 2
     assert 1 <= Sc <= S and nb * Vc >= V and (nb - 1) * Vc < V and 4 * Vc <= 1 << 16
     assert nb == 1 or Sc * nb <= SMS
     assert f == 2 * Vc and h == (4 * Vc if nb > 1 else 0)
