@@ -16,12 +16,13 @@
 // lane reads the four targets' part of the table, once for two edges of the same side. A block
 // loads its indices and table before it waits for the previous launch.
 // Measured against the two passes it replaces (GB300, T = 1, whole calls, us per iteration): K =
-// 16 on 181 x 181 17.9 -> 8.7; K = 8 on 178 x 178 9.3 -> 5.5; K = 4 on 64 x 64 6.0 -> 3.3 (two
+// 16 on 181 x 181 17.9 -> 9.0; K = 8 on 178 x 178 9.3 -> 5.5; K = 4 on 64 x 64 6.0 -> 3.3 (two
 // launches' latency -> one); per launch on 128 uneven grids K = 16 (662,000 variables) 60 + 222
 // -> 160 us, K = 8 (800,000) 43 + 88 -> 93, K = 4 (672,000) 28 + 46 -> 48. What bounds it now: the
 // L1's data path (wavefronts 70 to 75 % of its rate) and issue slots (49 % at K = 4, 64 % at K = 16);
 // more resident blocks win against fewer spills (K = 16: 2, 3, 4 blocks of 256 per SM 232, 183,
-// 171 us, when the kernel had a second round that no plan reached; without it 160).
+// 171 us, when the kernel had a second round that no plan reached; without it 160). Edges with entries
+// that are -inf, large or NaN, and tables of range above 60 T, go to team_rare.
 #include <cstdint>
 
 #include "pair_math.cuh"
@@ -55,44 +56,6 @@ __device__ __forceinline__ void row_load(float (&d)[4], const float *p) {
     }
 }
 
-// One outgoing edge by one thread, with the beliefs formed here: a sum-product table of range
-// above 60 T, entry by entry, and the guarded arithmetic (pair_dir_rare). tab: the table.
-template <int K, bool MAXP>
-__device__ __noinline__ void fused_edge(const DevGraph &G, const float *tab, const float *ev, const float *m_old,
-                                        float *m_new, int v, int i, int es_base, float T, float invT, float damping) {
-    const int k0 = G.vin_off[v], k1 = G.vin_off[v + 1], vs = G.vs_off[v];
-    const int es = G.vin_es[k0 + i], side = ((es - es_base) / K) & 1, es_t = side ? es - K : es + K;
-    float m[K], x[K], o[K];
-    load_n<K>(m, m_old + es);
-    bool odd = false;
-    for (int y = 0; y < K; ++y) odd |= needs_exact(m[y]);
-    if (odd) {
-        pair_dir_rare<K, MAXP>(G, tab, side ? 1 : K, side ? K : 1, nullptr, ev, m_old, m_new, vs, es, es_t, T, invT, damping);
-        return;
-    }
-    FF s[K];
-    float mx = kNegInf;
-    int arg = 0;
-    for (int y = 0; y < K; ++y) {
-        s[y] = ff_make(ev[vs + y]);
-        for (int k = k0; k < k1; ++k) s[y] = ff_add(s[y], m_old[G.vin_es[k] + y]);
-        if (s[y].hi + s[y].lo > mx) {
-            mx = s[y].hi + s[y].lo;
-            arg = y;
-        }
-    }
-    const FF best = s[arg];
-    for (int y = 0; y < K; ++y)
-        x[y] = (best.hi == kNegInf ? kNegInf : y == arg ? 0.f : ff_diff(s[y], best)) - m[y];
-    pair_entries<K, MAXP>(x, o, tab, side ? 1 : K, side ? K : 1, T, invT);
-    F2 o2[K / 2], m2[K / 2];
-#pragma unroll
-    for (int y = 0; y < K / 2; ++y) o2[y] = f2(o[2 * y], o[2 * y + 1]);
-    f2_load<K>(m2, m_old + es_t);
-    pair_finish<K>(o2, m2, damping, G.flags);
-    f2_store<K>(m_new + es_t, o2);
-}
-
 // A team's variable: its incoming edges (es_base where there is none) and their number.
 struct TeamVar {
     int v, deg, es[4];
@@ -107,9 +70,137 @@ __device__ __forceinline__ TeamVar team_var(const DevGraph &G, const int32_t *li
     return t;
 }
 
+// The edges that team_edges leaves out (bits of mask, the same for the team; every lane of the warp
+// calls): all of them with a sum-product table of range above 60 T, else those whose stored entries
+// are -inf, large or NaN, or that met a maximum of -inf. The variable-to-factor values of an edge with
+// such entries are the explicit sums without its own message (v2f_slow_edge's), of another the beliefs
+// less the message, and each target's sum runs over the table's entries (lse_row): the operations of
+// pair_dir_rare and of the two passes' entry form, lane by lane, so the same bits. Out of line: its
+// registers are not the main path's. us per iteration on 181 x 181 by the two passes, by one thread
+// per edge, which this replaces, and so: T = 0.02 (a range of 100 T and more) K = 4 8.1, 19.6, 8.3, K = 8
+// 13.5, 21.2, 13.0, K = 16 35.3, 45.0, 29.3; max-product with messages above 128 K = 4 16.8, 25.9, 8.9, K =
+// 16 68, 91, 21.6. What bounds it: the accurate exponentials (K^2 per edge) and the edges one after
+// the other.
+template <int K, bool MAXP>
+__device__ __noinline__ void team_rare(const DevGraph &G, const float *tab, const float *ev, const float *m_old,
+                                       float *m_new, const TeamVar &t, int l, int es_base, float *xs, unsigned mask,
+                                       float T, float invT, float damping) {
+    constexpr int L = K / 4;
+    mask &= (1u << t.deg) - 1u;  // (a maximum of -inf marks edges that are not there, too)
+    const float *e = ev + __ldg(G.vs_off + t.v) + 4 * l;
+    // beliefs relative to the best state (the largest rounded sum, lowest state on ties). The messages
+    // are read again where they are used: held, they would spill
+    unsigned odd = 0;
+    float b[4];
+    {
+        FF sum[4];
+        float e4[4], mx = kNegInf;
+        int arg = 4 * l;
+        load_n<4>(e4, e);
+#pragma unroll
+        for (int x = 0; x < 4; ++x) sum[x] = ff_make(e4[x]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < t.deg) {
+                float q[4];
+                load_n<4>(q, m_old + t.es[i] + 4 * l);
+                if (needs_exact(q[0]) | needs_exact(q[1]) | needs_exact(q[2]) | needs_exact(q[3])) odd |= 1u << i;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) sum[x] = ff_add(sum[x], q[x]);
+            }
+        FF best = sum[0];
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+            if (sum[x].hi + sum[x].lo > mx) {
+                mx = sum[x].hi + sum[x].lo;
+                arg = 4 * l + x;
+                best = sum[x];
+            }
+#pragma unroll
+        for (int d = L / 2; d > 0; d >>= 1) {
+            odd |= __shfl_xor_sync(0xffffffffu, odd, d, L);
+            const float ov = __shfl_xor_sync(0xffffffffu, mx, d, L), oh = __shfl_xor_sync(0xffffffffu, best.hi, d, L),
+                        ol = __shfl_xor_sync(0xffffffffu, best.lo, d, L);
+            const int oi = __shfl_xor_sync(0xffffffffu, arg, d, L);
+            if (ov > mx || (ov == mx && oi < arg)) {
+                mx = ov;
+                arg = oi;
+                best = FF{oh, ol};
+            }
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x) b[x] = best.hi == kNegInf ? kNegInf : 4 * l + x == arg ? 0.f : ff_diff(sum[x], best);
+    }
+    const float w = 1.f - damping;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool mine = (mask >> i) & 1;
+        if (!__any_sync(0xffffffffu, mine)) continue;
+        const int side = ((t.es[i] - es_base) / K) & 1, es_t = side ? t.es[i] - K : t.es[i] + K;
+        F2 mo[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        if (mine) {
+            f2_load<4>(mo, m_old + es_t + 4 * l);
+            if ((odd >> i) & 1) {  // the explicit sums
+                float q[4];
+                FF s[4];
+                load_n<4>(q, e);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) s[x] = ff_make(q[x]);
+                for (int k = 0; k < t.deg; ++k)
+                    if (k != i) {
+                        load_n<4>(q, m_old + t.es[k] + 4 * l);
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) s[x] = ff_add(s[x], q[x]);
+                    }
+#pragma unroll
+                for (int x = 0; x < 4; ++x) v[x] = s[x].hi + s[x].lo;
+            } else {
+                load_n<4>(v, m_old + t.es[i] + 4 * l);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) v[x] = b[x] - v[x];
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int x = 0; x < 4; ++x) xs[4 * l + x] = v[x];
+        __syncwarp();
+        const float *p = tab + (side ? 4 * l * K : 4 * l);  // phi(s, 4 l + j) at p[s ss + j sj]
+        const int ss = side ? 1 : K, sj = side ? K : 1;
+        float mx[4];
+        constexpr int N = K == 4 ? 2 : 1;  // targets at a time: N K values in registers
+#pragma unroll
+        for (int j = 0; j < 4; j += N) {
+            float z[N][K];
+#pragma unroll
+            for (int s = 0; s < K; ++s) {
+                const float v = xs[s];
+#pragma unroll
+                for (int n = 0; n < N; ++n) z[n][s] = p[s * ss + (j + n) * sj] + v;
+            }
+#pragma unroll
+            for (int n = 0; n < N; ++n) mx[j + n] = lse_row<K, MAXP>(z[n], T, invT);
+        }
+        // pair_finish
+        F2 o[2] = {f2(mx[0], mx[1]), f2(mx[2], mx[3])};
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            if (team_normalise<L>(o) == kNegInf) {
+                if (mine && l == 0) atomicOr(G.flags, kFlagContradiction);
+                o[0] = o[1] = f2(0.f, 0.f);
+            }
+            if (r == 0 && damping != 0.f) {
+                o[0] = f2_fma(f2(damping, damping), mo[0], f2_mul(f2(w, w), o[0]));
+                o[1] = f2_fma(f2(damping, damping), mo[1], f2_mul(f2(w, w), o[1]));
+            }
+        }
+        if (mine) f2_store<4>(m_new + es_t + 4 * l, o);
+    }
+}
+
 // The four states of lane l (of a team of K / 4): the beliefs' sums s + evidence and the stored
 // messages q, then the message that leaves each edge. Returns the edges (bit i, the same for
-// the whole team) that fused_edge has to take: stored entries that are -inf, large or NaN, or
+// the whole team) that team_rare has to take: stored entries that are -inf, large or NaN, or
 // a maximum of -inf on the way (contradictions and their flags are left to it).
 template <int K, bool MAXP, bool AL>
 __device__ __forceinline__ unsigned team_edges(const TeamVar &t, const float (&e4)[4], const float (&q)[4][4], int l,
@@ -338,11 +429,7 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
     if (member_skip<MAXP>(G, __ldg(&blocks[blockIdx.x].member), T, invT, damping)) return;  // the whole block
     const bool lin = pair_tables_make<K, MAXP, NT>(tab, S0, S1, red, invT);
     if (!MAXP && !lin) {
-        for (int k = threadIdx.x; k < 4 * n; k += NT) {
-            const int pos = B.x + (k >> 2), v = list ? __ldg(list + pos) : pos;
-            if ((k & 3) < __ldg(G.vin_off + v + 1) - __ldg(G.vin_off + v))
-                fused_edge<K, MAXP>(G, tab, ev, m_old, m_new, v, k & 3, es_base, T, invT, damping);
-        }
+        team_rare<K, MAXP>(G, tab, ev, m_old, m_new, t, l, es_base, xs, (1u << t.deg) - 1u, T, invT, damping);
         return;
     }
     pdl_launch_if_small();  // the next launch may be scheduled (it waits likewise)
@@ -371,10 +458,8 @@ k_pair_fused(const __grid_constant__ DevGraph G, const FuseBlock *__restrict__ b
         rare = team_edges<K, MAXP, false>(t, e4, q, l, es_base, S0, S1, red[0], xs, kTeams * kRow, m_old, m_new, T, invT,
                                           damping);
     }
-    if (rare != 0 && l == 0)
-#pragma unroll 1
-        for (int i = 0; i < t.deg; ++i)
-            if ((rare >> i) & 1) fused_edge<K, MAXP>(G, tab, ev, m_old, m_new, t.v, i, es_base, T, invT, damping);
+    if (__any_sync(0xffffffffu, rare != 0))
+        team_rare<K, MAXP>(G, tab, ev, m_old, m_new, t, l, es_base, xs, rare, T, invT, damping);
     if (!pdl_small()) pdl_launch_dependents();
 }
 
