@@ -58,6 +58,17 @@ __device__ __forceinline__ void add_term(FF &s, float &c, float q) {
     else s = ff_add(s, q);
 }
 
+// A clamped variable -- one state's evidence -inf, the other's finite -- whose messages are finite and
+// far from overflow has every leave-one-out log-ratio at that infinity, whatever the messages: its
+// total says so (edge_lam), without the explicit sums (784 x 500, all visible variables clamped: 20.6 us per
+// iteration with them, 10.4 so; the edge-state form takes 22.4). 0: not such a variable.
+constexpr float kClampedMax = 1e30f;  // (times the largest degree far below the largest number)
+__device__ __forceinline__ float clamped_ratio(float2 e) {
+    if (e.x == kNegInf && isfinite(e.y)) return CUDART_INF_F;
+    if (e.y == kNegInf && isfinite(e.x)) return kNegInf;
+    return 0.f;
+}
+
 // Block per variable of more than kVarBlockDegree factors, 128 threads (1024 on graphs with
 // variables of more than kLrEdgeMaxDegree) with 8 edges each in flight. The gathers' latency bounds it: every block is resident at once (1284 blocks for 784 x
 // 500), the edge list is read before the previous pass ends, and each thread adds its edges in
@@ -91,7 +102,7 @@ __global__ void __launch_bounds__(B) k_edge_var_block(DevGraph G, const int32_t 
     pdl_launch_if_one_wave();
     const float2 e = make_float2(__ldg(ev + 2 * (size_t)v), __ldg(ev + 2 * (size_t)v + 1));
     FF s = ff_make(0.f);
-    bool fin = isfinite(e.x) & isfinite(e.y);
+    bool fin = true, big = false;
     for (int base = k0;;) {
         float q[N];
 #pragma unroll
@@ -99,18 +110,24 @@ __global__ void __launch_bounds__(B) k_edge_var_block(DevGraph G, const int32_t 
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             fin &= isfinite(q[i]);
+            big |= fabsf(q[i]) > kClampedMax;
             s = ff_add_nc(s, q[i]);
         }
         base += N * B;
         if (base >= k1) break;
         load_es(base);
     }
-    float c = fin ? 0.f : 1.f;
+    float c = !fin ? 1.f : big ? 1.f / 65536.f : 0.f;  // below 1: every thread's are finite
     const FF tot = block_sum_count(s, c, sh);
     FF D = ff_add_nc(ff_make(e.y), -e.x);
     D = ff_add(D, tot);
-    if (c == 0.f && isfinite(D.hi) && isfinite(D.lo)) {
+    if (c < 1.f && isfinite(D.hi) && isfinite(D.lo)) {
         if (threadIdx.x == 0) Dv[v] = make_float2(D.hi, D.lo);
+        return;
+    }
+    const float inf = c == 0.f ? clamped_ratio(e) : 0.f;
+    if (inf != 0.f) {
+        if (threadIdx.x == 0) Dv[v] = make_float2(inf, 0.f);
         return;
     }
     // an infinite (or NaN) term, the same for the whole block: the two states' totals apart
@@ -146,7 +163,7 @@ __global__ void __launch_bounds__(256) k_edge_var_thread(DevGraph G, const int32
     if (i >= n) return;
     const float2 e = make_float2(__ldg(ev + 2 * (size_t)v), __ldg(ev + 2 * (size_t)v + 1));
     FF D = ff_add_nc(ff_make(e.y), -e.x);
-    bool fin = isfinite(e.x) & isfinite(e.y);
+    bool fin = true, big = false;
     for (int k = k0; k < k1; k += 4) {
         float q[4];
 #pragma unroll
@@ -154,11 +171,17 @@ __global__ void __launch_bounds__(256) k_edge_var_thread(DevGraph G, const int32
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             fin &= isfinite(q[j]);
+            big |= fabsf(q[j]) > kClampedMax;
             D = ff_add_nc(D, q[j]);
         }
     }
     if (fin && isfinite(D.hi) && isfinite(D.lo)) {
         Dv[v] = make_float2(D.hi, D.lo);
+        return;
+    }
+    const float inf = fin && !big ? clamped_ratio(e) : 0.f;
+    if (inf != 0.f) {
+        Dv[v] = make_float2(inf, 0.f);
         return;
     }
     // an infinite (or NaN) term: each edge's explicit sums without its own message
