@@ -2436,7 +2436,7 @@ static pgm_status one_launch_grad(pgm_graph *g, const LrGradPlan &one, const flo
     e = cudaStreamBeginCaptureToGraph(cs, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return failed(e, "cudaStreamBeginCaptureToGraph");
     cudaGraph_t captured = nullptr;
-    e = cudaMemsetAsync(bail, 0, sizeof(int), cs);
+    e = cudaMemsetAsync(bail, 0, 2 * sizeof(int), cs);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_log_pot, 0, (size_t)g->info.n_potentials * sizeof(float), cs);
     if (e == cudaSuccess)
         e = launch_lr_grad(g->G, g->P, one, log_pot, evidence, d_beliefs, d_log_pot, d_evidence, hist, bail, g->m_tmp,

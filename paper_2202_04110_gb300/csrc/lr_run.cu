@@ -606,7 +606,9 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_push(const LrRun A) {
 // two terms: the same bits in either order), so repeated calls give the same bits.
 // Tables with non-finite entries, contradictions and infinite messages (a lam of +-inf is
 // fine: its sigmas are 0 or 1) set *bail, and so does a wait that runs out: the caller's launches
-// take over.
+// take over. What shows in the inputs -- tables, evidence of -inf in both states -- ends the kernel in
+// its prologue (64 x 64, 60 iterations, a table with -inf: 894 us by the launches alone, 1,097 with the
+// kernel run to its end first, 941 so).
 // Measured (GB300, whole calls): 64 x 64, 100 iterations, checkpoints every 10: 1.59 ms as ~590
 // dependent launches of 2.4 us, 0.313 in one (0.311 with plain sums over a variable's factors, which
 // lose what cancelling adjoints leave); with lr_dir's SFU forms 0.28, but the table gradients' error
@@ -617,7 +619,7 @@ struct LrGrad {
     const float *gnb;       // [2 V] cotangent of the normalised log-beliefs
     float *d_pot, *d_ev;
     float *hist;            // [n_iters][blocks][4 Vc]
-    int *bail;
+    int *bail;              // and, at bail + 1, whether it was set in the prologue (both zeroed by the caller)
     float T;
 };
 
@@ -736,7 +738,11 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
     for (int l0 = 0; l0 < nv; l0 += nt) {  // as k_lr_run's prologue
         const int lv = l0 + tid, v = v0 + lv;
         const int4 t = lv < nv ? __ldg(A.tab4 + v) : make_int4(-1, -1, -1, -1);
-        if (lv < nv) es_sh[lv] = __ldg(reinterpret_cast<const float2 *>(A.ev) + v);
+        if (lv < nv) {
+            const float2 e = __ldg(reinterpret_cast<const float2 *>(A.ev) + v);
+            es_sh[lv] = e;
+            bad |= (e.x == kNegInf && e.y == kNegInf) | (e.x != e.x) | (e.y != e.y);
+        }
         const int es[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -775,7 +781,16 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
             }
         }
     }
-    __syncthreads();
+    // tables and evidence that the kernel hands back show here: every block learns of them at the
+    // barrier, and none begins
+    if (__syncthreads_or(bad)) {
+        if (tid == 0) {
+            *(volatile int *)P.bail = 1;
+            *(volatile int *)(P.bail + 1) = 1;
+            __threadfence();
+        }
+        if (X == kAlone) return;
+    }
     const int nF = s_n[0], nH = X == kAlone ? 0 : s_n[1];
     bool ok = true;
     if constexpr (X == kCluster) {
@@ -792,6 +807,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_grad(const __grid_const
         if (tid == 0) *(volatile int *)P.bail = 1;
         return;
     }
+    if (X != kAlone && *(volatile int *)(P.bail + 1) != 0) return;  // (written before the barrier only)
     for (int h = tid; h < nH; h += nt) {
         const int s = (int)(__float_as_uint(hrec[h].w) & 0xffff), q = s / Vc, lv = s - q * Vc;
         const int4 t = __ldg(A.tab4 + v0 + lv);
