@@ -24,7 +24,12 @@
 // with a block barrier after 1 and after 4. Step 3 runs while the values travel.
 // Measured against the multi-launch run (whole calls, GB300): 1000 x 1000, 200 iterations
 // 3.65 -> 1.80 ms (8.9 us per iteration), 317 x 241 max-product, 50 iterations 213 -> 87 us,
-// 32 evidence sets of 256 x 256, 100 iterations 4.22 -> 2.16 ms.
+// 32 evidence sets of 256 x 256, 100 iterations 4.22 -> 2.16 ms. Messages that need the guarded
+// arithmetic (towards or from clamped variables, tables with -inf) are done where they are met, each
+// three dependent loads away from its table at half the warps of the launches: where records are
+// streamed that costs more than the launches from some per cent of such messages on (1000 x 1000, T = 1,
+// 10 % of the tables with -inf: 49.6 us per iteration against 30.6). Putting them on a list that all
+// threads take up after the loop was measured: 24.7 us there, but 1.80 -> 1.89 ms on finite inputs; dropped.
 //
 // Inbox words carry their iteration: one 8-byte store holds (value, iteration), and the
 // reader polls its own word until the iteration is the one it is in; no fence, flag or
@@ -145,8 +150,24 @@ __device__ __noinline__ float run_exact(const LrRun &A, const float *pot, int v0
     return lr_dir_exact<MAXP>(phi, (es >> 1) & 1, l, mo, A.k, A.Tln2, A.damping, A.flags);
 }
 
-// A variable whose values do not come out finite: its four lam by the explicit sums.
+// A clamped variable -- one state's evidence -inf, the other's finite -- whose messages are finite and
+// far from overflow has every leave-one-out log-ratio at that infinity; 0: not such a variable.
+__device__ __forceinline__ float clamped_ratio(float2 e, float d0, float d1, float d2, float d3) {
+    const float big = fmaxf(fmaxf(fabsf(d0), fabsf(d1)), fmaxf(fabsf(d2), fabsf(d3))), sum = d0 + d1 + d2 + d3;
+    if (!(big < 1e37f) || sum != sum) return 0.f;
+    if (e.x == kNegInf && fabsf(e.y) < 1e37f) return CUDART_INF_F;
+    if (e.y == kNegInf && fabsf(e.x) < 1e37f) return kNegInf;
+    return 0.f;
+}
+
+// A variable whose values do not come out finite: its four lam by the explicit sums, or, clamped, without
+// (30 % of the variables clamped, us per iteration, the launches per pass / sums / so: 64 x 64 3.75 / 4.2 /
+// 3.8, 317 x 241 8.7 / 5.5 / 4.8, 1000 x 1000 38.7 / 64.8 / 56.4).
 __device__ __noinline__ void run_var_slow(float *lam, int lv, int Vc, float2 e, float d0, float d1, float d2, float d3) {
+    if (const float inf = clamped_ratio(e, d0, d1, d2, d3); inf != 0.f) {
+        lam[lv] = lam[Vc + lv] = lam[2 * Vc + lv] = lam[3 * Vc + lv] = inf;
+        return;
+    }
     const float dk[4] = {d0, d1, d2, d3};
     const int pos[4] = {lv, Vc + lv, 2 * Vc + lv, 3 * Vc + lv};
     lr_var_slow(e, dk, pos, 4, lam);
@@ -466,6 +487,7 @@ __global__ void __launch_bounds__(kLrRunThreads, 1) k_lr_run(const __grid_consta
 //   TWO = true: a thread per variable forms the totals, a barrier, then the edges. Two chains,
 //     but 1.6x fewer instructions, which is what bounds a block of 1,024 threads.
 __device__ __noinline__ float push_lam_slow(float2 e, float d0, float d1, float d2, float d3, int k) {
+    if (const float inf = clamped_ratio(e, d0, d1, d2, d3); inf != 0.f) return inf;
     const float dk[4] = {d0, d1, d2, d3};
     FF l0 = ff_make(e.x), l1 = ff_make(e.y);
     for (int j = 0; j < 4; ++j) {  // as lr_var_slow
