@@ -16,7 +16,7 @@
 // lane reads the four targets' part of the table, once for two edges of the same side. A block
 // loads its indices and table before it waits for the previous launch.
 // Measured against the two passes it replaces (GB300, T = 1, whole calls, us per iteration): K =
-// 16 on 181 x 181 17.9 -> 9.0; K = 8 on 178 x 178 9.3 -> 5.5; K = 4 on 64 x 64 6.0 -> 3.3 (two
+// 16 on 181 x 181 17.9 -> 9.1; K = 8 on 178 x 178 9.3 -> 5.5; K = 4 on 64 x 64 6.0 -> 3.3 (two
 // launches' latency -> one); per launch on 128 uneven grids K = 16 (662,000 variables) 60 + 222
 // -> 160 us, K = 8 (800,000) 43 + 88 -> 93, K = 4 (672,000) 28 + 46 -> 48. What bounds it now: the
 // L1's data path (wavefronts 70 to 75 % of its rate) and issue slots (49 % at K = 4, 64 % at K = 16);
